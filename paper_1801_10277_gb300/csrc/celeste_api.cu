@@ -238,7 +238,7 @@ celeste_status run(celeste_problem* pr, const double* d_theta, int precision, in
         return CELESTE_OK;
     }
     CEL_CUDA(timed(pr, "prep", st, [&] { return launch_prep(P, d_theta, precision, st); }));
-    CEL_CUDA(timed(pr, "contrib", st, [&] { return launch_contrib(P, precision, st); }));
+    CEL_CUDA(timed(pr, "contrib", st, [&] { return launch_contrib(P, precision, st, true); }));
     CEL_CUDA(timed(pr, "gather", st, [&] { return launch_gather(P, precision, st); }));
     if (mode == MODE_HESS)
         CEL_CUDA(timed(pr, "hess_adjoint", st, [&] { return launch_hess_pixels(P, precision, st); }));
@@ -865,8 +865,9 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     P.queue = (int32_t*)p;
     prime_persistent_grids();
     {
-        const cudaError_t pe = prime_items_kernels();
-        if (pe != cudaSuccess) return bail(fail(CELESTE_ERR_CUDA, "item kernel set-up: %s", cudaGetErrorString(pe)));
+        cudaError_t pe = prime_items_kernels();
+        if (pe == cudaSuccess) pe = prime_hess_kernels();
+        if (pe != cudaSuccess) return bail(fail(CELESTE_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(pe)));
     }
     if (cudaMemset(P.queue, 0, 2 * sizeof(int32_t)) != cudaSuccess) return bail(fail(CELESTE_ERR_CUDA, "memset"));
     if ((st = dalloc(pr, &p, sizeof(int32_t)))) return bail(st);

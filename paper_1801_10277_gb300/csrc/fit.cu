@@ -1151,7 +1151,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
         // the stage-start E_s / Var_s in this phase's precision
         const size_t bytes = (size_t)P.n_sp * (prec == CELESTE_FP64 ? sizeof(double) : sizeof(float));
         FIT_CUDA(launch_prep(P, d_th0, prec, st));
-        FIT_CUDA(launch_contrib(P, prec, st));
+        FIT_CUDA(launch_contrib(P, prec, st, true));
         FIT_CUDA(cudaMemcpyAsync(d_se0, P.spE, bytes, cudaMemcpyDeviceToDevice, st));
         FIT_CUDA(cudaMemcpyAsync(d_sv0, P.spE2, bytes, cudaMemcpyDeviceToDevice, st));
     }
@@ -1164,7 +1164,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             if (nb == 0) continue;
             // current E_s / Var_s of every source (global buffers)
             FIT_CUDA(launch_prep(P, pr->d_theta, prec, st));
-            FIT_CUDA(launch_contrib(P, prec, st));
+            FIT_CUDA(launch_contrib(P, prec, st, true));
             FIT_CUDA(cudaMemcpyAsync(d_bsrc, B.src.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice, st));
             FIT_CUDA(cudaMemcpyAsync(d_bpo, B.patch_off.data(), sizeof(int32_t) * (nb + 1), cudaMemcpyHostToDevice, st));
             FIT_CUDA(cudaMemcpyAsync(d_bgeo, B.geo.data(), sizeof(PatchGeo) * B.geo.size(), cudaMemcpyHostToDevice, st));

@@ -20,6 +20,7 @@
 
 #include <type_traits>
 
+#include "fp64_profile.cuh"
 #include "internal.cuh"
 #include "source_math.cuh"
 
@@ -28,7 +29,6 @@ namespace cel {
 namespace {
 
 __device__ __forceinline__ float ex2h(float x) { return exp2f(x); }
-__device__ __forceinline__ double ex2h(double x) { return exp2(x); }
 __device__ __forceinline__ float lgh(float x) { return logf(x); }
 __device__ __forceinline__ double lgh(double x) { return log(x); }
 
@@ -62,7 +62,7 @@ __device__ __forceinline__ void warp_reduce_scatter(R (&v)[HVP], int lane) {
     }
 }
 
-// ---- The galaxy components in the frame that whitens PSF component k (FP32 path).
+// ---- The galaxy components in the frame that whitens PSF component k.
 // T_k maps a pixel offset d to z = T_k d with T_k Sigma_k T_k' = I and T_k G T_k' =
 // diag(g1, g2), so component j's precision is T_k' diag(lam1, lam2) T_k with
 // lam_a = 1 / (1 + nu_j g_a).  With r = lam z and E~ = T_k E T_k', every derivative of
@@ -88,18 +88,37 @@ constexpr int WS_N = 0,    // N
               WS_BE = 30,  // dN/de_dev nu lam
               WS_AE = 32,  // dN/de_dev nu lam lam
               NWS = 35;
-constexpr int WROW = 40;   // floats per (k, j): exponent coefficients of z1^2, z2^2, constant; 35 weights; pad
-constexpr int WFR = 16;    // floats per k: T (row-major), K (3 x 3), g1, g2, pad
+// Of these, with lam_a (1 + nu g_a) = 1, the ones of lower degree follow from 19 (all terms
+// positive, so nothing cancels):  A_0 = C_0 + g1 D3_0, A_1 = C_1 + g1 D3_1, A_2 = C_3 + g2 D3_3,
+// B = A + g D2, L = LL + g A, N = L_0 + g1 B_0; and the e_dev sums are the difference of the
+// dev and the exp components' sums at unit weight.  So the kernel accumulates 19 sums over
+// the exp components, then over the dev components, and forms the 35 once per (pixel, k).
+constexpr int BS_LL = 0, BS_C = 3, BS_D2 = 7, BS_D3 = 10, BS_D4 = 14, NBS = 19;
+constexpr int WROW = 40;   // a full row: exponent coefficients of z1^2, z2^2, constant; 35 weights; pad
+constexpr int BROW = 24;   // a kernel row: the exponent's three coefficients, 19 weights, pad
+constexpr int WFR = 16;    // entries per k: T (row-major), K (3 x 3), g1, g2, pad
 // K[e][p] = (T E_e T')_p for the pixel-frame shape directions E_e = (xx, xy + yx, yy)
 // and the whitened pairs p = (11, 12, 22)
 constexpr int WF_K = 4, WF_G = 13;
-static_assert(3 + NWS <= WROW && WROW % 4 == 0 && WFR % 4 == 0 && WF_G + 2 <= WFR,
-              "whitened rows are read as float4 from a 16-byte aligned array");
+static_assert(3 + NWS <= WROW && 3 + NBS <= BROW && BROW % 4 == 0 && WFR % 4 == 0 && WF_G + 2 <= WFR,
+              "whitened rows are read as 16-byte vectors from a 16-byte aligned array");
 
 __host__ __device__ __forceinline__ int wpa(int p) { return p == 2 ? 1 : 0; }
 __host__ __device__ __forceinline__ int wpb(int p) { return p == 0 ? 0 : 1; }
-__host__ __device__ __forceinline__ float wmult(int p) { return p == 1 ? 2.f : 1.f; }
-__host__ __device__ __forceinline__ float wdl(int a, int b) { return a == b ? 1.f : 0.f; }
+
+// K of a frame whose T is in place
+template <class R>
+__host__ __device__ __forceinline__ void whiten_shape_map(R* fr) {
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const R* Ta = fr + 2 * wpa(p);
+        const R* Tb = fr + 2 * wpb(p);
+        fr[WF_K + 0 * 3 + p] = Ta[0] * Tb[0];
+        fr[WF_K + 1 * 3 + p] = Ta[0] * Tb[1] + Ta[1] * Tb[0];
+        fr[WF_K + 2 * 3 + p] = Ta[1] * Tb[1];
+    }
+    fr[15] = 0;
+}
 
 // T_k from the Cholesky factor of the component's precision and one Jacobi rotation, in
 // FP32 (a few threads per work item, before its pixels: FP64 square roots and divisions
@@ -129,70 +148,106 @@ __host__ __device__ void whiten_frame(const float* sT, int k, float* fr) {
         const float v0 = T[a][0] * gxx + T[a][1] * gxy, v1 = T[a][0] * gxy + T[a][1] * gyy;
         fr[WF_G + a] = fmaxf(v0 * T[a][0] + v1 * T[a][1], 0.f);
     }
+    whiten_shape_map(fr);
+}
+
+// lam1^(deg - i) lam2^i, i = 0 .. deg, times w
+template <class R>
+__host__ __device__ __forceinline__ void monomials(R w, R l1, R l2, int deg, R* c) {
 #pragma unroll
-    for (int p = 0; p < 3; ++p) {
-        const int a = wpa(p), b = wpb(p);
-        fr[WF_K + 0 * 3 + p] = T[a][0] * T[b][0];
-        fr[WF_K + 1 * 3 + p] = T[a][0] * T[b][1] + T[a][1] * T[b][0];
-        fr[WF_K + 2 * 3 + p] = T[a][1] * T[b][1];
+    for (int i = 0; i <= deg; ++i) {
+        R v = w;
+#pragma unroll
+        for (int u = 0; u < deg; ++u) v *= u < i ? l2 : l1;
+        c[i] = v;
     }
-    fr[15] = 0.f;
 }
 
 // the row of galaxy component (k, j): exponent in z and the 35 monomial weights
 __host__ __device__ void whiten_row(const float* G, const float* fr, float* row) {
     const float nu = G[9], w = G[7], dw = G[8];
     const float l1 = 1.f / (1.f + nu * fr[WF_G]), l2 = 1.f / (1.f + nu * fr[WF_G + 1]);
-    float p1[5], p2[5];
-    p1[0] = p2[0] = 1.f;
-#pragma unroll
-    for (int i = 1; i < 5; ++i) {
-        p1[i] = p1[i - 1] * l1;
-        p2[i] = p2[i - 1] * l2;
-    }
-    auto mono = [&](int deg, int i) { return p1[deg - i] * p2[i]; };
-    const float wn = w * nu, wn2 = wn * nu, dwn = dw * nu;
     row[0] = -0.5f * (float)LOG2E_H * l1;
     row[1] = -0.5f * (float)LOG2E_H * l2;
     row[2] = G[3];
     float* c = row + 3;
     c[WS_N] = w;
     c[WS_NE] = dw;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        c[WS_L + i] = w * mono(1, i);
-        c[WS_B + i] = wn * mono(1, i);
-        c[WS_LE + i] = dw * mono(1, i);
-        c[WS_BE + i] = dwn * mono(1, i);
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        c[WS_LL + i] = w * mono(2, i);
-        c[WS_A + i] = wn * mono(2, i);
-        c[WS_D2 + i] = wn2 * mono(2, i);
-        c[WS_AE + i] = dwn * mono(2, i);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        c[WS_C + i] = wn * mono(3, i);
-        c[WS_D3 + i] = wn2 * mono(3, i);
-    }
-#pragma unroll
-    for (int i = 0; i < 5; ++i) c[WS_D4 + i] = wn2 * mono(4, i);
+    monomials(w, l1, l2, 1, c + WS_L);
+    monomials(w, l1, l2, 2, c + WS_LL);
+    monomials(w * nu, l1, l2, 1, c + WS_B);
+    monomials(w * nu, l1, l2, 2, c + WS_A);
+    monomials(w * nu, l1, l2, 3, c + WS_C);
+    monomials(w * nu * nu, l1, l2, 2, c + WS_D2);
+    monomials(w * nu * nu, l1, l2, 3, c + WS_D3);
+    monomials(w * nu * nu, l1, l2, 4, c + WS_D4);
+    monomials(dw, l1, l2, 1, c + WS_LE);
+    monomials(dw * nu, l1, l2, 1, c + WS_BE);
+    monomials(dw * nu, l1, l2, 2, c + WS_AE);
     row[3 + NWS] = 0.f;
     row[4 + NWS] = 0.f;
 }
 
+// the kernel's row: three exponent coefficients (given) and the 19 weights at weight w
+template <class R>
+__host__ __device__ __forceinline__ void base_row(R w, R nu, R l1, R l2, R* c) {
+    monomials(w, l1, l2, 2, c + BS_LL);
+    monomials(w * nu, l1, l2, 3, c + BS_C);
+    monomials(w * nu * nu, l1, l2, 2, c + BS_D2);
+    monomials(w * nu * nu, l1, l2, 3, c + BS_D3);
+    monomials(w * nu * nu, l1, l2, 4, c + BS_D4);
+}
+
+// adds f times the sums over one group's components (b, at unit weight) to the 27 sums of
+// N and fe times them to the 8 e_dev sums
+template <class R>
+__host__ __device__ __forceinline__ void add_group(const R (&b)[NBS], R g1, R g2, R f, R fe, R (&s)[NWS]) {
+    R A[3], B[2], L[2];
+    A[0] = b[BS_C] + g1 * b[BS_D3];
+    A[1] = b[BS_C + 1] + g1 * b[BS_D3 + 1];
+    A[2] = b[BS_C + 3] + g2 * b[BS_D3 + 3];
+    B[0] = A[0] + g1 * b[BS_D2];
+    B[1] = A[2] + g2 * b[BS_D2 + 2];
+    L[0] = b[BS_LL] + g1 * A[0];
+    L[1] = b[BS_LL + 2] + g2 * A[2];
+    const R N = L[0] + g1 * B[0];
+    s[WS_N] += f * N;
+    s[WS_NE] += fe * N;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        s[WS_L + i] += f * L[i];
+        s[WS_LE + i] += fe * L[i];
+        s[WS_B + i] += f * B[i];
+        s[WS_BE + i] += fe * B[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        s[WS_A + i] += f * A[i];
+        s[WS_AE + i] += fe * A[i];
+        s[WS_LL + i] += f * b[BS_LL + i];
+        s[WS_D2 + i] += f * b[BS_D2 + i];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        s[WS_C + i] += f * b[BS_C + i];
+        s[WS_D3 + i] += f * b[BS_D3 + i];
+    }
+#pragma unroll
+    for (int i = 0; i < 5; ++i) s[WS_D4 + i] += f * b[BS_D4 + i];
+}
+
 // adds PSF component k's galaxy terms at one pixel, from its 35 sums, to the pixel-frame
-// value, gradient (mx, my, Gxx, Gxy, Gyy), e_dev derivatives and packed 5 x 5 Hessian
-__host__ __device__ __forceinline__ void whitened_add(const float (&s)[NWS], float z1, float z2,
-                                             const float* fr, float& g1, float (&d1)[5],
-                                             float& de, float (&h1)[15], float (&he)[5]) {
-    const float z[2] = {z1, z2};
-    const float Z2[3] = {z1 * z1, z1 * z2, z2 * z2};
-    const float Z3[4] = {z1 * Z2[0], z1 * Z2[1], z1 * Z2[2], z2 * Z2[2]};
-    const float Z4[5] = {Z2[0] * Z2[0], Z2[0] * Z2[1], Z2[0] * Z2[2], Z2[1] * Z2[2], Z2[2] * Z2[2]};
-    float T[2][2], K[3][3];
+// value, gradient (mx, my, Gxx, Gxy, Gyy), e_dev derivatives and packed 5 x 5 Hessian.
+// (The Kronecker deltas are branches on constants: a product with a constant 0 would be
+// computed.)
+template <class R>
+__host__ __device__ __forceinline__ void whitened_add(const R (&s)[NWS], R z1, R z2, const R* fr, R& g1, R (&d1)[5],
+                                                      R& de, R (&h1)[15], R (&he)[5]) {
+    const R z[2] = {z1, z2};
+    const R Z2[3] = {z1 * z1, z1 * z2, z2 * z2};
+    const R Z3[4] = {z1 * Z2[0], z1 * Z2[1], z1 * Z2[2], z2 * Z2[2]};
+    const R Z4[5] = {Z2[0] * Z2[0], Z2[0] * Z2[1], Z2[0] * Z2[2], Z2[1] * Z2[2], Z2[2] * Z2[2]};
+    R T[2][2], K[3][3];
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
         T[a][0] = fr[2 * a];
@@ -205,14 +260,19 @@ __host__ __device__ __forceinline__ void whitened_add(const float (&s)[NWS], flo
     g1 += s[WS_N];
     de += s[WS_NE];
     // d/dmu = T' r-sums; d/dG[E] = K (W11, 2 W12, W22), W_ab = (z_a z_b A_ab - delta_ab B_a) / 2
-    const float gm[2] = {z1 * s[WS_L], z2 * s[WS_L + 1]};
-    const float ge[2] = {z1 * s[WS_LE], z2 * s[WS_LE + 1]};
-    float Wv[3], Wev[3];
+    const R gm[2] = {z1 * s[WS_L], z2 * s[WS_L + 1]};
+    const R ge[2] = {z1 * s[WS_LE], z2 * s[WS_LE + 1]};
+    R Wv[3], Wev[3];
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
         const int a = wpa(p), b = wpb(p);
-        Wv[p] = 0.5f * wmult(p) * (Z2[a + b] * s[WS_A + a + b] - wdl(a, b) * s[WS_B + a]);
-        Wev[p] = 0.5f * wmult(p) * (Z2[a + b] * s[WS_AE + a + b] - wdl(a, b) * s[WS_BE + a]);
+        R v = Z2[a + b] * s[WS_A + a + b], u = Z2[a + b] * s[WS_AE + a + b];
+        if (a == b) {
+            v = (R)0.5 * (v - s[WS_B + a]);
+            u = (R)0.5 * (u - s[WS_BE + a]);
+        }
+        Wv[p] = v;
+        Wev[p] = u;
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -224,33 +284,27 @@ __host__ __device__ __forceinline__ void whitened_add(const float (&s)[NWS], flo
         d1[2 + e] += K[e][0] * Wv[0] + K[e][1] * Wv[1] + K[e][2] * Wv[2];
         he[2 + e] += K[e][0] * Wev[0] + K[e][1] * Wev[1] + K[e][2] * Wev[2];
     }
-    // (mu, mu) = T' X T, X_ab = z_a z_b LL_ab - delta_ab L_a
-    float XT[2][2];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            float v = 0.f;
-#pragma unroll
-            for (int b = 0; b < 2; ++b)
-                v += (Z2[a + b] * s[WS_LL + a + b] - wdl(a, b) * s[WS_L + a]) * T[b][k];
-            XT[a][k] = v;
-        }
-    h1[0] += T[0][0] * XT[0][0] + T[1][0] * XT[1][0];
-    h1[1] += T[0][0] * XT[0][1] + T[1][0] * XT[1][1];
-    h1[5] += T[0][1] * XT[0][1] + T[1][1] * XT[1][1];
+    // (mu, mu) = T' X T, X_ab = z_a z_b LL_ab - delta_ab L_a: the pixel-frame entries are K X
+    {
+        const R X[3] = {Z2[0] * s[WS_LL] - s[WS_L], Z2[1] * s[WS_LL + 1], Z2[2] * s[WS_LL + 2] - s[WS_L + 1]};
+        h1[0] += K[0][0] * X[0] + (R)2 * K[0][1] * X[1] + K[0][2] * X[2];
+        h1[1] += (R)0.5 * (K[1][0] * X[0] + K[1][2] * X[2]) + K[1][1] * X[1];
+        h1[5] += K[2][0] * X[0] + (R)2 * K[2][1] * X[1] + K[2][2] * X[2];
+    }
     // (mu, G): T' (Yv K'), Y_{a,bc} = (z_a z_b z_c C_abc - delta_bc z_a A_ab - delta_ab z_c A_ac
     //                                  - delta_ac z_b A_ab) / 2
-    float YK[2][3];
+    R YK[2][3];
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-        float Yv[3];
+        R Yv[3];
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
             const int b = wpa(p), c = wpb(p);
-            Yv[p] = 0.5f * wmult(p) *
-                    (Z3[a + b + c] * s[WS_C + a + b + c] - wdl(b, c) * z[a] * s[WS_A + a + b] -
-                     wdl(a, b) * z[c] * s[WS_A + a + c] - wdl(a, c) * z[b] * s[WS_A + a + b]);
+            R v = Z3[a + b + c] * s[WS_C + a + b + c];
+            if (b == c && a == b) v -= (R)3 * z[a] * s[WS_A + 2 * a];
+            else if (b == c) v -= z[a] * s[WS_A + 1];
+            else v -= z[1 - a] * s[WS_A + 1];   // p = (1, 2): a is one of the two
+            Yv[p] = b == c ? (R)0.5 * v : v;
         }
 #pragma unroll
         for (int e = 0; e < 3; ++e) YK[a][e] = K[e][0] * Yv[0] + K[e][1] * Yv[1] + K[e][2] * Yv[2];
@@ -260,30 +314,30 @@ __host__ __device__ __forceinline__ void whitened_add(const float (&s)[NWS], flo
         h1[2 + e] += T[0][0] * YK[0][e] + T[1][0] * YK[1][e];
         h1[6 + e] += T[0][1] * YK[0][e] + T[1][1] * YK[1][e];
     }
-    // (G, G) = K Vm K', Vm_pq = m_p m_q V_{ab,cd} (pairs p = ab, q = cd)
-    float KV[3][3];
+    // (G, G) = K Vm K', Vm_pq = m_p m_q V_{ab,cd} / 4 (pairs p = ab, q = cd; symmetric):
+    //   V = z_a z_b z_c z_d D4 - delta_cd z_a z_b D3_abc - delta_ab z_c z_d D3_acd + delta_ab delta_cd D2_ac
+    //       - (delta_bc z_a z_d + delta_bd z_a z_c) D3 - (delta_ac z_b z_d + delta_ad z_b z_c) D3
+    //       + (delta_bc delta_ad + delta_ac delta_bd) D2_ab
+    R Vm[3][3];
     {
-        float Vm[3][3];
-#pragma unroll
-        for (int p = 0; p < 3; ++p)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const int a = wpa(p), b = wpb(p), c = wpa(q), d = wpb(q);
-                const float* D2 = s + WS_D2;
-                const float* D3 = s + WS_D3;
-                const float v =
-                    Z4[a + b + c + d] * s[WS_D4 + a + b + c + d] - wdl(c, d) * Z2[a + b] * D3[a + b + c] -
-                    wdl(a, b) * Z2[c + d] * D3[a + c + d] + wdl(a, b) * wdl(c, d) * D2[a + c] -
-                    wdl(b, c) * Z2[a + d] * D3[a + b + d] - wdl(a, c) * Z2[b + d] * D3[a + b + d] -
-                    wdl(b, d) * Z2[a + c] * D3[a + b + c] - wdl(a, d) * Z2[b + c] * D3[a + b + c] +
-                    (wdl(b, c) * wdl(a, d) + wdl(a, c) * wdl(b, d)) * D2[a + b];
-                Vm[p][q] = 0.25f * wmult(p) * wmult(q) * v;
-            }
-#pragma unroll
-        for (int e = 0; e < 3; ++e)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) KV[e][q] = K[e][0] * Vm[0][q] + K[e][1] * Vm[1][q] + K[e][2] * Vm[2][q];
+        const R* D2 = s + WS_D2;
+        const R* D3 = s + WS_D3;
+        const R* D4 = s + WS_D4;
+        Vm[0][0] = (R)0.25 * (Z4[0] * D4[0] + (R)3 * D2[0]) - (R)1.5 * Z2[0] * D3[0];
+        Vm[2][2] = (R)0.25 * (Z4[4] * D4[4] + (R)3 * D2[2]) - (R)1.5 * Z2[2] * D3[3];
+        Vm[0][2] = (R)0.25 * (Z4[2] * D4[2] - Z2[0] * D3[1] - Z2[2] * D3[2] + D2[1]);
+        Vm[0][1] = (R)0.5 * Z4[1] * D4[1] - (R)1.5 * Z2[1] * D3[1];
+        Vm[1][2] = (R)0.5 * Z4[3] * D4[3] - (R)1.5 * Z2[1] * D3[2];
+        Vm[1][1] = Z4[2] * D4[2] - Z2[0] * D3[1] - Z2[2] * D3[2] + D2[1];
+        Vm[1][0] = Vm[0][1];
+        Vm[2][0] = Vm[0][2];
+        Vm[2][1] = Vm[1][2];
     }
+    R KV[3][3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) KV[e][q] = K[e][0] * Vm[0][q] + K[e][1] * Vm[1][q] + K[e][2] * Vm[2][q];
     int c = 9;
 #pragma unroll
     for (int e = 0; e < 3; ++e)
@@ -291,54 +345,100 @@ __host__ __device__ __forceinline__ void whitened_add(const float (&s)[NWS], flo
         for (int f = e; f < 3; ++f, ++c) h1[c] += KV[e][0] * K[f][0] + KV[e][1] * K[f][1] + KV[e][2] * K[f][2];
 }
 
+// Shared memory of k_hess (bytes): the patch's table (R), per PSF component its frame, the
+// component rows and, FP64, the table of 2^x; the warps' sums take the rows' place at the end.
+template <class R>
+struct HessLay {
+    static constexpr int tbl = 0;
+    static constexpr int fr = tbl + TBL_STRIDE * (int)sizeof(R);
+    static constexpr int rows = fr + MAXPSF * WFR * (int)sizeof(R);
+    static constexpr int rows_bytes = MAXPSF * MAXPROF * BROW * (int)sizeof(R);
+    static constexpr int red_bytes = (CHUNK / 32) * HV * 8;
+    static constexpr int tab = rows + (rows_bytes > red_bytes ? rows_bytes : red_bytes);
+    static constexpr int bytes = tab + (sizeof(R) == 8 ? EX_N * 8 : 0);
+    static_assert(fr % 16 == 0 && rows % 16 == 0 && tab % 16 == 0, "16-byte alignment");
+};
+
+// Per work item: the sums over its pixels of ll, d ll / d y and d2 ll / dy2.  The mixture in
+// the whitened frame (above); FP64 as in fp64_profile.cuh, E and Var of a singly covered
+// pixel (single, FP64 only) formed here, those of the others from the maps.
+// Bound by the FP32 or the FP64 pipe: 22 / 25 of its instructions per component, where the
+// 35 sums accumulated one by one took 38 (FP32: 500 sources, 909,100 source-pixels, 180 ->
+// 140 us) and the pixel-frame formulas about 140 (FP64: fp64_profile.cuh has the figures).
 template <class R>
 __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ items,
                                                 const PatchGeo* __restrict__ geo,
-                                                const ImgMeta* __restrict__ img, int nprof,
+                                                const ImgMeta* __restrict__ img, int nprof, int n_exp,
                                                 const float* __restrict__ pixels,
+                                                const float* __restrict__ sky_map,
                                                 const R* __restrict__ tbl,
+                                                const uint8_t* __restrict__ single,
                                                 const R* __restrict__ emap,
                                                 const R* __restrict__ vmap,
                                                 double* __restrict__ part,
                                                 const int32_t* __restrict__ src_active) {
-    // FP32: the galaxy terms in the frame that whitens each PSF component
-    constexpr bool WHITE = std::is_same<R, float>::value;
-    __shared__ R sT[TBL_STRIDE];
-    __shared__ double red[CHUNK / 32][HV];
-    __shared__ __align__(16) float wsm[WHITE ? MAXPSF * WFR + MAXPSF * MAXPROF * WROW : 4];
+    constexpr bool DBL = std::is_same<R, double>::value;
+    using Lay = HessLay<R>;
+    extern __shared__ __align__(16) unsigned char smem[];
+    R* sT = reinterpret_cast<R*>(smem + Lay::tbl);
+    R* frames = reinterpret_cast<R*>(smem + Lay::fr);
+    R* rows = reinterpret_cast<R*>(smem + Lay::rows);
+    double* tab = reinterpret_cast<double*>(smem + Lay::tab);
     const WorkItem it = items[blockIdx.x];
     const PatchGeo g = geo[it.patch];
     if (src_active && !src_active[g.src]) return;
     const ImgMeta& im = img[g.img];
     const int npsf = im.npsf;
+    const int t = threadIdx.x;
     {
         const R* gT = tbl + (size_t)it.patch * TBL_STRIDE;
         const int n = T_GAL + npsf * nprof * GAL_STRIDE;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) sT[i] = gT[i];
+        for (int i = t; i < n; i += blockDim.x) sT[i] = gT[i];
+        if constexpr (DBL) load_exp2_table(tab);
         __syncthreads();
     }
-    if constexpr (WHITE) {
-        if ((int)threadIdx.x < npsf) whiten_frame(sT, threadIdx.x, wsm + threadIdx.x * WFR);
-        __syncthreads();
-        for (int i = threadIdx.x; i < npsf * nprof; i += blockDim.x)
-            whiten_row(sT + T_GAL + i * GAL_STRIDE, wsm + (i / nprof) * WFR, wsm + MAXPSF * WFR + i * WROW);
-        __syncthreads();
+    if (t < npsf) {
+        if constexpr (DBL) {
+            const R* F = sT + T_STAR + t * STAR_STRIDE;
+            R* fr = frames + t * WFR;
+            for (int i = 0; i < 4; ++i) fr[i] = F[i];
+            fr[WF_G] = F[4];
+            fr[WF_G + 1] = F[5];
+            whiten_shape_map(fr);
+        } else {
+            whiten_frame(sT, t, frames + t * WFR);
+        }
     }
+    __syncthreads();
+    for (int i = t; i < npsf * nprof; i += blockDim.x) {
+        // the exponent's coefficients and the 19 weights at unit e_dev weight
+        const R* G = sT + T_GAL + i * GAL_STRIDE;
+        const R* fr = frames + (i / nprof) * WFR;
+        R* row = rows + i * BROW;
+        R l1, l2, w;
+        const R nu = G[9];
+        if constexpr (DBL) {
+            l1 = G[0] * EX_IHALF;
+            l2 = G[1] * EX_IHALF;
+            w = G[3];
+        } else {
+            l1 = 1.f / (1.f + nu * fr[WF_G]);
+            l2 = 1.f / (1.f + nu * fr[WF_G + 1]);
+            w = i % nprof >= n_exp ? G[8] : -G[8];
+        }
+        row[0] = DBL ? G[0] : (R)(-0.5 * LOG2E_H) * l1;
+        row[1] = DBL ? G[1] : (R)(-0.5 * LOG2E_H) * l2;
+        row[2] = DBL ? G[2] : G[3];
+        base_row(w, nu, l1, l2, row + 3);
+        row[3 + NBS] = row[4 + NBS] = 0;
+    }
+    __syncthreads();
     R out[HV];
 #pragma unroll
     for (int i = 0; i < HV; ++i) out[i] = 0;
-    const int t = threadIdx.x;
     if (t < it.n) {
         const int q = it.q0 + t;
         const int yy = q / g.w, xx = q - yy * g.w;
-        const int64_t m = im.px_off + (int64_t)(g.y0 + yy) * im.W + (g.x0 + xx);
-        const R x = (R)pixels[m], E = emap[m], V = vmap[m];
-        const R iE = (R)1 / E, iE2 = iE * iE;
-        const R cE = x * (iE + V * iE2 * iE) - (R)1;
-        const R cV = (R)-0.5 * x * iE2;
-        const R hEE = -x * iE2 * ((R)1 + (R)3 * V * iE2);
-        const R hEV = x * iE2 * iE;
-        out[0] = x * (lgh(E) - (R)0.5 * V * iE2) - E;
         // star: value, gradient (mx, my), Hessian (xx, xy, yy)
         R g0 = 0, d0[2] = {0, 0}, h0[3] = {0, 0, 0};
         // galaxy: value; gradient over z5 = (mx, my, Gxx, Gxy, Gyy); e_dev derivative;
@@ -346,195 +446,228 @@ __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ ite
         R g1 = 0, d1[5] = {0, 0, 0, 0, 0}, de = 0, h1[15], he[5] = {0, 0, 0, 0, 0};
 #pragma unroll
         for (int i = 0; i < 15; ++i) h1[i] = 0;
+        const R edev = sT[H_EDEV];
         for (int k = 0; k < npsf; ++k) {
             const R dx = (R)xx - sT[T_MEAN + 2 * k], dy = (R)yy - sT[T_MEAN + 2 * k + 1];
-            const R dxx = dx * dx, dxy = dx * dy, dyy = dy * dy;
+            const R* fr = frames + k * WFR;
+            const R z1 = fr[0] * dx + fr[1] * dy, z2 = fr[2] * dx + fr[3] * dy;
+            const R z1s = z1 * z1, z2s = z2 * z2;
+            float f1 = 0.f, f2 = 0.f;
+            if constexpr (DBL) {
+                f1 = (float)z1s;
+                f2 = (float)z2s;
+            }
             {
+                // P d = T' z and P = T' T
                 const R* S = sT + T_STAR + k * STAR_STRIDE;
-                const R n = S[7] * ex2h(S[0] * dxx + S[1] * dxy + S[2] * dyy + S[3]);
-                const R qx = S[4] * dx + S[5] * dy, qy = S[5] * dx + S[6] * dy;
+                R n, qx, qy, pxx, pxy, pyy;
+                if constexpr (DBL) {
+                    n = S[6] * ex2_quad(EX_HALF, z1s, EX_HALF, z2s, (float)EX_HALF, f1, (float)EX_HALF, f2, tab);
+                    qx = fr[0] * z1 + fr[2] * z2;
+                    qy = fr[1] * z1 + fr[3] * z2;
+                    pxx = fr[WF_K] + fr[WF_K + 2];
+                    pxy = (R)0.5 * (fr[WF_K + 3] + fr[WF_K + 5]);
+                    pyy = fr[WF_K + 6] + fr[WF_K + 8];
+                } else {
+                    n = S[7] * ex2h(S[0] * (dx * dx) + S[1] * (dx * dy) + S[2] * (dy * dy) + S[3]);
+                    qx = S[4] * dx + S[5] * dy;
+                    qy = S[5] * dx + S[6] * dy;
+                    pxx = S[4];
+                    pxy = S[5];
+                    pyy = S[6];
+                }
                 g0 += n;
                 d0[0] += n * qx;
                 d0[1] += n * qy;
-                h0[0] += n * (qx * qx - S[4]);
-                h0[1] += n * (qx * qy - S[5]);
-                h0[2] += n * (qy * qy - S[6]);
+                h0[0] += n * (qx * qx - pxx);
+                h0[1] += n * (qx * qy - pxy);
+                h0[2] += n * (qy * qy - pyy);
             }
-            if constexpr (WHITE) {
-                const float* fr = wsm + k * WFR;
-                const float z1 = fr[0] * dx + fr[1] * dy, z2 = fr[2] * dx + fr[3] * dy;
-                const float z1s = z1 * z1, z2s = z2 * z2;
-                float sw[NWS];
+            R s[NWS];
 #pragma unroll
-                for (int m = 0; m < NWS; ++m) sw[m] = 0.f;
-                const float4* row = reinterpret_cast<const float4*>(wsm + MAXPSF * WFR + k * nprof * WROW);
-                for (int j = 0; j < nprof; ++j, row += WROW / 4) {
-                    float cw[WROW];
+            for (int m = 0; m < NWS; ++m) s[m] = 0;
+            const R* row = rows + k * nprof * BROW;
+            // the exp components at weight 1 - e_dev, then the dev components at e_dev
+            auto group = [&](int n, R f, R fe) {
+                R b[NBS];
 #pragma unroll
-                    for (int u = 0; u < WROW / 4; ++u) {
-                        const float4 v = row[u];
-                        cw[4 * u] = v.x;
-                        cw[4 * u + 1] = v.y;
-                        cw[4 * u + 2] = v.z;
-                        cw[4 * u + 3] = v.w;
+                for (int m = 0; m < NBS; ++m) b[m] = 0;
+                for (int j = 0; j < n; ++j, row += BROW) {
+                    R cw[BROW], e;
+                    if constexpr (DBL) {
+#pragma unroll
+                        for (int u = 0; u < (3 + NBS + 1) / 2; ++u) {
+                            const double2 v = reinterpret_cast<const double2*>(row)[u];
+                            cw[2 * u] = v.x;
+                            cw[2 * u + 1] = v.y;
+                        }
+                        const float2 ab = as_float2(cw[2]);
+                        e = ex2_quad(cw[0], z1s, cw[1], z2s, ab.x, f1, ab.y, f2, tab);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < (3 + NBS + 3) / 4; ++u) {
+                            const float4 v = reinterpret_cast<const float4*>(row)[u];
+                            cw[4 * u] = v.x;
+                            cw[4 * u + 1] = v.y;
+                            cw[4 * u + 2] = v.z;
+                            cw[4 * u + 3] = v.w;
+                        }
+                        e = ex2h(fmaf(cw[0], z1s, fmaf(cw[1], z2s, cw[2])));
                     }
-                    const float e = ex2h(fmaf(cw[0], z1s, fmaf(cw[1], z2s, cw[2])));
 #pragma unroll
-                    for (int m = 0; m < NWS; ++m) sw[m] = fmaf(e, cw[3 + m], sw[m]);
+                    for (int m = 0; m < NBS; ++m) b[m] += e * cw[3 + m];
                 }
-                whitened_add(sw, z1, z2, fr, g1, d1, de, h1, he);
-                continue;
-            }
-            // FP64: the galaxy components one by one in the pixel frame
-            const R* G = sT + T_GAL + k * nprof * GAL_STRIDE;
-            for (int j = 0; j < nprof; ++j, G += GAL_STRIDE) {
-                const R e = ex2h(G[0] * dxx + G[1] * dxy + G[2] * dyy + G[3]);
-                const R n = G[7] * e, ne = G[8] * e;
-                const R pxx = G[4], pxy = G[5], pyy = G[6], nu = G[9];
-                const R qx = pxx * dx + pxy * dy, qy = pxy * dx + pyy * dy;
-                R l[5];
-                l[0] = qx;
-                l[1] = qy;
-                l[2] = (R)0.5 * nu * (qx * qx - pxx);
-                l[3] = nu * (qx * qy - pxy);
-                l[4] = (R)0.5 * nu * (qy * qy - pyy);
-                const R nu2 = nu * nu;
-                const R Pqy_x = pxx * qy + pxy * qx;   // (P (qy, qx))_x
-                const R Pqy_y = pxy * qy + pyy * qx;   // (P (qy, qx))_y
-                R L[15];
-                L[0] = -pxx;                  // (mx, mx)
-                L[1] = -pxy;                  // (mx, my)
-                L[2] = -nu * pxx * qx;        // (mx, Gxx)
-                L[3] = -nu * Pqy_x;           // (mx, Gxy)
-                L[4] = -nu * pxy * qy;        // (mx, Gyy)
-                L[5] = -pyy;                  // (my, my)
-                L[6] = -nu * pxy * qx;        // (my, Gxx)
-                L[7] = -nu * Pqy_y;           // (my, Gxy)
-                L[8] = -nu * pyy * qy;        // (my, Gyy)
-                L[9] = nu2 * ((R)0.5 * pxx * pxx - pxx * qx * qx);                           // (Gxx, Gxx)
-                L[10] = nu2 * (pxx * pxy - qx * Pqy_x);                                      // (Gxx, Gxy)
-                L[11] = nu2 * ((R)0.5 * pxy * pxy - pxy * qx * qy);                          // (Gxx, Gyy)
-                L[12] = nu2 * (pxy * pxy + pxx * pyy - (qy * Pqy_x + qx * Pqy_y));            // (Gxy, Gxy)
-                L[13] = nu2 * (pxy * pyy - qy * Pqy_y);                                      // (Gxy, Gyy)
-                L[14] = nu2 * ((R)0.5 * pyy * pyy - pyy * qy * qy);                          // (Gyy, Gyy)
-                g1 += n;
-                de += ne;
-                int c = 0;
-#pragma unroll
-                for (int a = 0; a < 5; ++a) {
-                    d1[a] += n * l[a];
-                    he[a] += ne * l[a];
-#pragma unroll
-                    for (int b = a; b < 5; ++b, ++c) h1[c] += n * (l[a] * l[b] + L[c]);
-                }
-            }
+                add_group(b, fr[WF_G], fr[WF_G + 1], f, fe, s);
+            };
+            group(n_exp, (R)1 - edev, (R)-1);
+            group(nprof - n_exp, edev, (R)1);
+            whitened_add(s, z1, z2, fr, g1, d1, de, h1, he);
         }
-        // ---- assemble the pixel's y-derivatives
+        // ---- E, Var and the pixel's weights
         const R iota = sT[H_IOTA], a0 = sT[H_A0], a1 = sT[H_A1];
         const R el0 = sT[H_EL0], el20 = sT[H_EL20], el1 = sT[H_EL1], el21 = sT[H_EL21];
         const R i2 = iota * iota;
         const R f0 = iota * el0 * g0, f1 = iota * el1 * g1;
         const R Es = a0 * f0 + a1 * f1;
+        const int64_t m = im.px_off + (int64_t)(g.y0 + yy) * im.W + (g.x0 + xx);
+        const R x = (R)pixels[m];
+        R E, V;
+        if (DBL && single && single[g.sp_off + q]) {
+            if constexpr (DBL) {
+                double em0, em1, es;
+                moment_ratios64(sT, em0, em1);
+                source_ev64(sT, em0, em1, g0, g1, es, V);
+                E = (im.has_sky_map ? (double)sky_map[m] : im.sky) + es;
+            }
+        } else {
+            E = emap[m];
+            V = vmap[m];
+        }
+        const R iE = (R)1 / E, iE2 = iE * iE;
+        const R cE = x * (iE + V * iE2 * iE) - (R)1;
+        const R cV = (R)-0.5 * x * iE2;
+        const R hEE = -x * iE2 * ((R)1 + (R)3 * V * iE2);
+        const R hEV = x * iE2 * iE;
+        out[0] = x * (lgh(E) - (R)0.5 * V * iE2) - E;
+        // ---- assemble the pixel's y-derivatives (entries known to be zero are left out: a
+        // product with a constant 0 would be computed)
         const R w1 = cE - (R)2 * cV * Es, w2 = cV;
-        // gradient of g_i over y (index 6..11), zero elsewhere
-        R dg0[6] = {d0[0], d0[1], 0, 0, 0, 0};
-        R dg1[6] = {d1[0], d1[1], de, d1[2], d1[3], d1[4]};
-        // e = dE_s/dy, v2 = dE2_s/dy
+        // gradient of g_1 over y (index 6..11); g_0's is (d0[0], d0[1], 0, 0, 0, 0)
+        const R dg1[6] = {d1[0], d1[1], de, d1[2], d1[3], d1[4]};
+        // e = dE_s/dy (0 for Y_EL20, Y_EL21), v2 = dE2_s/dy (0 for Y_EL0, Y_EL1)
         R e[NY], v2[NY];
+        const R g00 = i2 * g0 * g0, g11 = i2 * g1 * g1;
         e[Y_A0] = f0;
         e[Y_A1] = f1;
         e[Y_EL0] = a0 * iota * g0;
-        e[Y_EL20] = 0;
         e[Y_EL1] = a1 * iota * g1;
-        e[Y_EL21] = 0;
-        v2[Y_A0] = i2 * el20 * g0 * g0;
-        v2[Y_A1] = i2 * el21 * g1 * g1;
-        v2[Y_EL0] = 0;
-        v2[Y_EL20] = a0 * i2 * g0 * g0;
-        v2[Y_EL1] = 0;
-        v2[Y_EL21] = a1 * i2 * g1 * g1;
+        v2[Y_A0] = el20 * g00;
+        v2[Y_A1] = el21 * g11;
+        v2[Y_EL20] = a0 * g00;
+        v2[Y_EL21] = a1 * g11;
         const R k0 = a0 * iota * el0, k1 = a1 * iota * el1;
         const R m0 = (R)2 * a0 * i2 * el20, m1 = (R)2 * a1 * i2 * el21;
+        const R n0 = m0 * g0, n1 = m1 * g1;
 #pragma unroll
         for (int z = 0; z < 6; ++z) {
-            e[Y_MX + z] = k0 * dg0[z] + k1 * dg1[z];
-            v2[Y_MX + z] = m0 * g0 * dg0[z] + m1 * g1 * dg1[z];
+            e[Y_MX + z] = k1 * dg1[z];
+            v2[Y_MX + z] = n1 * dg1[z];
+            if (z < 2) {
+                e[Y_MX + z] += k0 * d0[z];
+                v2[Y_MX + z] += n0 * d0[z];
+            }
         }
-        // gradient
+        auto has_e = [](int y) { return y != Y_EL20 && y != Y_EL21; };
+        auto has_v2 = [](int y) { return y != Y_EL0 && y != Y_EL1; };
+        // gradient, and the outer-product part of the Hessian: with v = v2 - 2 E_s e,
+        //   (h_EE - 2 c_V) e e' + h_EV (e v' + v e') = e p' + p e',
+        //   p = (h_EE / 2 - c_V - 2 h_EV E_s) e + h_EV v2
+        const R c1 = (R)0.5 * hEE - cV - (R)2 * hEV * Es;
+        R pv[NY];
 #pragma unroll
-        for (int y = 0; y < NY; ++y) out[1 + y] = w1 * e[y] + w2 * v2[y];
-        // Hessian: outer-product part
-        R v[NY];
-#pragma unroll
-        for (int y = 0; y < NY; ++y) v[y] = v2[y] - (R)2 * Es * e[y];
-        const R c1 = hEE - (R)2 * cV;
+        for (int y = 0; y < NY; ++y) {
+            if (!has_e(y)) {
+                out[1 + y] = w2 * v2[y];
+                pv[y] = hEV * v2[y];
+            } else if (!has_v2(y)) {
+                out[1 + y] = w1 * e[y];
+                pv[y] = c1 * e[y];
+            } else {
+                out[1 + y] = w1 * e[y] + w2 * v2[y];
+                pv[y] = c1 * e[y] + hEV * v2[y];
+            }
+        }
         R* H = out + 1 + NY;
 #pragma unroll
         for (int a = 0; a < NY; ++a)
 #pragma unroll
-            for (int b = a; b < NY; ++b)
-                H[yh_index(a, b)] = c1 * e[a] * e[b] + hEV * (e[a] * v[b] + v[a] * e[b]);
+            for (int b = a; b < NY; ++b) {
+                R h = 0;
+                if (has_e(a) && has_e(b)) h = e[a] * pv[b] + pv[a] * e[b];
+                else if (has_e(a)) h = e[a] * pv[b];
+                else if (has_e(b)) h = pv[a] * e[b];
+                H[yh_index(a, b)] = h;
+            }
         // second-derivative part  w1 DE + w2 DE2
         H[P2(Y_A0, Y_EL0)] += w1 * iota * g0;
         H[P2(Y_A1, Y_EL1)] += w1 * iota * g1;
-        H[P2(Y_A0, Y_EL20)] += w2 * i2 * g0 * g0;
-        H[P2(Y_A1, Y_EL21)] += w2 * i2 * g1 * g1;
+        H[P2(Y_A0, Y_EL20)] += w2 * g00;
+        H[P2(Y_A1, Y_EL21)] += w2 * g11;
         const R p0 = w1 * iota * el0 + (R)2 * w2 * i2 * el20 * g0;
         const R p1 = w1 * iota * el1 + (R)2 * w2 * i2 * el21 * g1;
         const R u0 = a0 * p0, u1 = a1 * p1;
         const R b0 = w2 * m0, b1 = w2 * m1;
+        const R l0 = w1 * a0 * iota, l1 = w1 * a1 * iota;
+        const R r0 = w2 * (R)2 * a0 * i2 * g0, r1 = w2 * (R)2 * a1 * i2 * g1;
+        R bd1[6];
 #pragma unroll
         for (int z = 0; z < 6; ++z) {
             const int yz = Y_MX + z;
-            H[P2(Y_A0, yz)] += p0 * dg0[z];
             H[P2(Y_A1, yz)] += p1 * dg1[z];
-            H[P2(Y_EL0, yz)] += w1 * a0 * iota * dg0[z];
-            H[P2(Y_EL1, yz)] += w1 * a1 * iota * dg1[z];
-            H[P2(Y_EL20, yz)] += w2 * (R)2 * a0 * i2 * g0 * dg0[z];
-            H[P2(Y_EL21, yz)] += w2 * (R)2 * a1 * i2 * g1 * dg1[z];
+            H[P2(Y_EL1, yz)] += l1 * dg1[z];
+            H[P2(Y_EL21, yz)] += r1 * dg1[z];
+            if (z < 2) {
+                H[P2(Y_A0, yz)] += p0 * d0[z];
+                H[P2(Y_EL0, yz)] += l0 * d0[z];
+                H[P2(Y_EL20, yz)] += r0 * d0[z];
+            }
+            bd1[z] = b1 * dg1[z];
         }
         // z-z block: u0 d2g0 + b0 dg0 dg0' + u1 d2g1 + b1 dg1 dg1'
-        // d2g1 over (mx, my, edev, Gxx, Gxy, Gyy) from h1 (z5 packed) and he (edev x z5)
+        // d2g1 over (mx, my, edev, Gxx, Gxy, Gyy) from h1 (z5 packed) and he (edev x z5;
+        // the e_dev diagonal is zero)
         const int zmap[5] = {0, 1, 3, 4, 5};   // z5 position -> position among the six
-        R d2g1[6][6];
-#pragma unroll
-        for (int a = 0; a < 6; ++a)
-#pragma unroll
-            for (int b = 0; b < 6; ++b) d2g1[a][b] = 0;
         {
             int c = 0;
 #pragma unroll
             for (int a = 0; a < 5; ++a) {
-                d2g1[zmap[a]][2] = he[a];
-                d2g1[2][zmap[a]] = he[a];
+                H[P2(Y_EDEV, Y_MX + zmap[a])] += u1 * he[a];
 #pragma unroll
-                for (int b = a; b < 5; ++b, ++c) {
-                    d2g1[zmap[a]][zmap[b]] = h1[c];
-                    d2g1[zmap[b]][zmap[a]] = h1[c];
-                }
+                for (int b = a; b < 5; ++b, ++c) H[yh_index(Y_MX + zmap[a], Y_MX + zmap[b])] += u1 * h1[c];
             }
         }
-        const R d2g0[3] = {h0[0], h0[1], h0[2]};
 #pragma unroll
         for (int a = 0; a < 6; ++a)
 #pragma unroll
             for (int b = a; b < 6; ++b) {
-                R s = u1 * d2g1[a][b] + b1 * dg1[a] * dg1[b] + b0 * dg0[a] * dg0[b];
-                if (a < 2 && b < 2) s += u0 * d2g0[a + b];
-                H[yh_index(Y_MX + a, Y_MX + b)] += s;
+                R v = bd1[a] * dg1[b];
+                if (a < 2 && b < 2) v += b0 * d0[a] * d0[b] + u0 * h0[a + b];
+                H[yh_index(Y_MX + a, Y_MX + b)] += v;
             }
     }
     // ---- CTA reduction: in R within a warp (a reduce-scatter), FP64 across warps
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = t & 31, warp = t >> 5;
+    double(*red)[HV] = reinterpret_cast<double(*)[HV]>(smem + Lay::rows);
     R v[HVP];
 #pragma unroll
     for (int i = 0; i < HVP; ++i) v[i] = i < HV ? out[i] : (R)0;
     warp_reduce_scatter(v, lane);
+    __syncthreads();   // every warp is past its reads of the rows
 #pragma unroll
     for (int u = 0; u < HVP / 32; ++u)
         if (3 * lane + u < HV) red[warp][3 * lane + u] = (double)v[u];
     __syncthreads();
-    for (int i = threadIdx.x; i < HV; i += blockDim.x) {
+    for (int i = t; i < HV; i += blockDim.x) {
         double s = 0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][i];
         part[(size_t)blockIdx.x * NPART + i] = s;
@@ -862,17 +995,26 @@ k_finalize_hess(int n_src, const double* __restrict__ theta, const PatchGeo* __r
     }
 }
 
+template <class R>
+static cudaError_t hess_pixels(const DevProblem& P, const R* tbl, cudaStream_t st) {
+    k_hess<R><<<P.n_item, CHUNK, HessLay<R>::bytes, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.pixels, P.sky_map, tbl,
+                                              P.single, (const R*)P.emap, (const R*)P.vmap, P.item_part, P.src_active);
+    return cudaGetLastError();
+}
+
+// shared-memory limits of the Hessian kernels on the current device, set at problem
+// creation (outside any stream capture)
+cudaError_t prime_hess_kernels() {
+    cudaError_t e = cudaFuncSetAttribute(k_hess<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         HessLay<float>::bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_hess<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, HessLay<double>::bytes);
+    return e;
+}
+
 cudaError_t launch_hess_pixels(const DevProblem& P, int precision, cudaStream_t st) {
     if (P.n_item == 0) return cudaSuccess;
-    if (precision == CELESTE_FP64)
-        k_hess<double><<<P.n_item, CHUNK, 0, st>>>(P.items, P.geo, P.img, P.nprof, P.pixels,
-                                                   P.tbl64, (const double*)P.emap,
-                                                   (const double*)P.vmap, P.item_part, P.src_active);
-    else
-        k_hess<float><<<P.n_item, CHUNK, 0, st>>>(P.items, P.geo, P.img, P.nprof, P.pixels,
-                                                  P.tbl32, (const float*)P.emap,
-                                                  (const float*)P.vmap, P.item_part, P.src_active);
-    return cudaGetLastError();
+    return precision == CELESTE_FP64 ? hess_pixels<double>(P, P.tbl64, st) : hess_pixels<float>(P, P.tbl32, st);
 }
 
 cudaError_t launch_finalize_hess(const DevProblem& P, const double* d_theta, double* d_local,

@@ -60,13 +60,20 @@ constexpr int ZPCOLS = 2 + NP;
 //   galaxy [64 + 12 (k nprof + j)]: qa qb qc qd pxx pxy pyy c dc nu 0 0
 // Component density: c * exp2(qa dx^2 + qb dx dy + qc dy^2 + qd) with
 // (qa, qb, qc) = -log2(e) (Pxx/2, Pxy, Pyy/2) and qd = -log2(2 pi sqrt(det C)).
+// The FP64 table holds the same slots in the frame that whitens each PSF component
+// (fp64_profile.cuh; T, D, l as in item_kernels.cu): e_dev in header slot 7, and
+//   star   [16 + 8k]: T11 T12 T21 T22 D1 D2 c_star 0, c_star = alpha_k / (2 pi sqrt(det Sigma_k))
+//   galaxy [64 + 12 (k nprof + j)]: A B (A, B in FP32) U0 U1 U2 Wa Wb W12 nu Va Vb, with
+//     (A, B) = -1024 log2(e) (l1, l2), U0 = c_star w_j sqrt(l1 l2), c = U0 times 1 - e_dev (exp)
+//     or e_dev (dev), (U1, U2) = c (l1, l2), (Wa, Wb) = c nu (l1^2, -l1), W12 = c nu l1 l2,
+//     (Va, Vb) = c nu (l2^2, -l2)
 constexpr int T_HDR = 0, T_MEAN = 8, T_STAR = 16, STAR_STRIDE = 8, T_DG = 48, T_G = 57, T_GAL = 64,
               GAL_STRIDE = 12;
 constexpr int TBL_STRIDE = T_GAL + MAXPSF * MAXPROF * GAL_STRIDE;   // 832
 static_assert(T_MEAN + 2 * MAXPSF <= T_STAR && T_STAR + MAXPSF * STAR_STRIDE <= T_DG &&
                   T_DG + 9 <= T_G && T_G + 3 <= T_GAL,
               "mixture-table fields overlap");
-constexpr int H_A0 = 0, H_A1 = 1, H_EL0 = 2, H_EL20 = 3, H_EL1 = 4, H_EL21 = 5, H_IOTA = 6;
+constexpr int H_A0 = 0, H_A1 = 1, H_EL0 = 2, H_EL20 = 3, H_EL1 = 4, H_EL21 = 5, H_IOTA = 6, H_EDEV = 7;
 
 // floats of one patch's whitened-frame table (item_kernels.cu): a value part (header 16,
 // per PSF component 8 + 8 per pair of profile components) and a gradient part (per PSF
@@ -98,6 +105,10 @@ struct ImgMeta {
     float psf_cs[MAXPSF];
     float psf_sg[MAXPSF];
     float psf_dm[MAXPSF];
+    // the same in FP64, with c_star = alpha_k / (2 pi sqrt(det Sigma_k))
+    double psf_li64[MAXPSF][3];
+    double psf_c64[MAXPSF];
+    double psf_dm64[MAXPSF];
     float sky_f;
     float iota_f;
 };
@@ -205,6 +216,8 @@ inline void fill_float_copies(ImgMeta& im) {
     im.iota_f = (float)im.iota;
     const double detA = im.A[0] * im.A[3] - im.A[1] * im.A[2];
     for (int k = 0; k < MAXPSF; ++k) {
+        for (int c = 0; c < 3; ++c) im.psf_li64[k][c] = 0.0;
+        im.psf_c64[k] = im.psf_dm64[k] = 0.0;
         im.psf_li[k][0] = im.psf_li[k][1] = im.psf_li[k][2] = 0.f;
         im.psf_cs[k] = -INFINITY;
         im.psf_sg[k] = 1.f;
@@ -213,12 +226,15 @@ inline void fill_float_copies(ImgMeta& im) {
         const double* ps = im.psf[k];
         const double l11 = std::sqrt(ps[3]), l21 = ps[4] / l11, l22 = std::sqrt(ps[5] - l21 * l21);
         const double det = ps[3] * ps[5] - ps[4] * ps[4];
-        im.psf_li[k][0] = (float)(1.0 / l11);
-        im.psf_li[k][1] = (float)(-l21 / (l11 * l22));
-        im.psf_li[k][2] = (float)(1.0 / l22);
+        im.psf_li64[k][0] = 1.0 / l11;
+        im.psf_li64[k][1] = -l21 / (l11 * l22);
+        im.psf_li64[k][2] = 1.0 / l22;
+        for (int c = 0; c < 3; ++c) im.psf_li[k][c] = (float)im.psf_li64[k][c];
+        im.psf_c64[k] = ps[0] / (6.283185307179586 * std::sqrt(det));
+        im.psf_dm64[k] = detA * detA / det;
         im.psf_cs[k] = (float)(std::log2(std::fabs(ps[0])) - 2.6514961294723187 /* log2(2 pi) */ - 0.5 * std::log2(det));
         im.psf_sg[k] = ps[0] < 0 ? -1.f : 1.f;
-        im.psf_dm[k] = (float)(detA * detA / det);
+        im.psf_dm[k] = (float)im.psf_dm64[k];
     }
 }
 
@@ -366,14 +382,16 @@ celeste_status fit_sources_checked(celeste_problem* pr, double* theta_inout, con
 
 void prime_persistent_grids();
 cudaError_t prime_items_kernels();
+cudaError_t prime_hess_kernels();
 // total = tile ll sums + item ll sums - KL (after the gather and every item ll)
 cudaError_t launch_total(const DevProblem& P, double* d_total, cudaStream_t st);
 // tables (and, with_kl, the KL value / gradient and the domain check) of every source
 cudaError_t launch_prep(const DevProblem& P, const double* d_theta, int precision,
                         cudaStream_t st, bool with_kl = true);
-// contrib / adjoint over the items idx[0 .. n) (idx null: items 0 .. n; n < 0: all items)
-cudaError_t launch_contrib(const DevProblem& P, int precision, cudaStream_t st,
-                           const int32_t* idx = nullptr, int n = -1);
+// E_s and Var_s at every item pixel, singly covered ones (P.single) finished into the maps;
+// multi_only (FP64): at the multiply covered pixels alone, the others being left to the
+// kernels that evaluate the source there anyway
+cudaError_t launch_contrib(const DevProblem& P, int precision, cudaStream_t st, bool multi_only = false);
 // The FP32 value (MODE_LL) or value + gradient (MODE_GRAD) evaluation (item_kernels.cu):
 // the patches' whitened-frame tables, the KL value / gradient and the domain check of
 // theta, every item, the per-source epilogue (local objective, gradient; each nullable)
@@ -385,8 +403,7 @@ cudaError_t launch_items(const DevProblem& P, int mode, cudaStream_t st, const d
 cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStream_t st, const double* d_theta,
                                double* d_local, double* d_grad, double* d_total);
 cudaError_t launch_gather(const DevProblem& P, int precision, cudaStream_t st);
-cudaError_t launch_adjoint(const DevProblem& P, int precision, int mode, cudaStream_t st,
-                           const int32_t* idx = nullptr, int n = -1);
+cudaError_t launch_adjoint(const DevProblem& P, int precision, int mode, cudaStream_t st);
 cudaError_t launch_hess_pixels(const DevProblem& P, int precision, cudaStream_t st);
 cudaError_t launch_finalize(const DevProblem& P, const double* d_theta, int precision, int mode,
                             double* d_total, double* d_local, double* d_grad, double* d_hess,

@@ -190,6 +190,8 @@ extern "C" celeste_status celeste_patch_elbo_grad_noalloc(
     P.n_img_rec = 1;
     P.npsf_max = im->n_psf;
     P.nprof = model->n_exp + model->n_dev;
+    P.model_ne = model->n_exp;
+    P.model_nd = model->n_dev;
     P.n_px = (int64_t)w * h;
     P.n_sp = (int64_t)w * h;
     P.img = (const ImgMeta*)(base + OFF_IMG);

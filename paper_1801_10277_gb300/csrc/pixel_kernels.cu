@@ -13,7 +13,8 @@
 //              wrt the twelve intermediate variables y of the (source, patch)
 //
 // R = float: mixture and likelihood arithmetic in FP32, warp sums in FP32, every
-// sum across warps in FP64.  R = double: FP64 throughout.
+// sum across warps in FP64.  The FP64 path has map and adjoint kernels of its own
+// (k_contrib64, k_adjoint64, FP64 throughout); k_prep and k_gather serve both.
 #include <math.h>
 
 #include <map>
@@ -23,6 +24,7 @@
 #include "internal.cuh"
 #include "async_copy.cuh"
 #include "epilogue.cuh"
+#include "fp64_profile.cuh"
 
 namespace cel {
 
@@ -37,7 +39,6 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ double ex2(double x) { return exp2(x); }
 __device__ __forceinline__ float lg(float x) { return logf(x); }
 __device__ __forceinline__ double lg(double x) { return log(x); }
 
@@ -88,6 +89,8 @@ __device__ __forceinline__ void load_table(R* sT, const R* gT, int n) {
 //   galaxy component (k, j): weight alpha_k w_j (1 - e_dev) [exp] or alpha_k w_j e_dev [dev],
 //                            covariance Sigma_k + nu_j G,  G = A W A^T,
 //                            W = sigma^2 R(phi) diag(1, rho^2) R(phi)^T
+// R = float: the components in the pixel frame.  R = double: in the frame that whitens each
+// PSF component (internal.cuh lists the slots), one frame per (patch, PSF component).
 // Positions are formed in FP64 and stored relative to the patch origin (so FP32
 // differences stay exact); the galaxy covariance, the brightness moments and the
 // per-component algebra run in the table's precision R, spread over lanes (a lone
@@ -153,6 +156,61 @@ __device__ __forceinline__ void prep_kl(int s, const double* th, const R* thr,
     for (int i = lane; i < NP; i += 32) klg_out[(size_t)NP * s + i] = kg[i];
 }
 
+// The FP64 table.  PSF component k's whitened frame (the FP64 table's star slots): T = Q^T L^-1 with
+// Q diagonalising M = L^-1 G L^-T (one Jacobi rotation), D the eigenvalues, the smaller one
+// from det M = psf_dm (sigma^2 rho)^2 (no cancellation)
+__device__ __forceinline__ void whiten_frame64(const ImgMeta& im, int k, const double* G, double s2rho, double* F,
+                                               double* D) {
+    const double gxx = G[0], gxy = G[1], gyy = G[2];
+    const double a = im.psf_li64[k][0], b = im.psf_li64[k][1], c = im.psf_li64[k][2];
+    const double bxc = b * gxx + c * gxy, byc = b * gxy + c * gyy;
+    const double m11 = a * a * gxx, m12 = a * bxc, m22 = bxc * b + byc * c;
+    double cs = 1.0, sn = 0.0, d1 = m11, d2 = m22;
+    if (m12 != 0.0) {
+        const double tau = (m22 - m11) / (2.0 * m12);
+        const double t = copysign(1.0, tau) / (fabs(tau) + sqrt(1.0 + tau * tau));   // 0 for an infinite tau
+        cs = rsqrt(1.0 + t * t);
+        sn = t * cs;
+        d1 = m11 - t * m12;
+        d2 = m22 + t * m12;
+    }
+    const double detm = im.psf_dm64[k] * s2rho * s2rho;
+    if (d1 >= d2 && d1 > 0.0) d2 = detm / d1;
+    else if (d2 > d1 && d2 > 0.0) d1 = detm / d2;
+    D[0] = fmax(d1, 0.0);
+    D[1] = fmax(d2, 0.0);
+    F[0] = cs * a - sn * b;
+    F[1] = -sn * c;
+    F[2] = sn * a + cs * b;
+    F[3] = cs * c;
+    F[4] = D[0];
+    F[5] = D[1];
+    F[6] = im.psf_c64[k];
+    F[7] = 0.0;
+}
+
+// the FP64 table's row of galaxy component j of a PSF component
+__device__ __forceinline__ void galaxy_row64(const ModelDev& md, double c_star, int j, double edev, const double* D,
+                                             double* row) {
+    const double nu = md.prof_nu[j];
+    const double l1 = 1.0 / (1.0 + nu * D[0]), l2 = 1.0 / (1.0 + nu * D[1]);
+    const double u0 = c_star * md.prof_w[j] * sqrt(l1 * l2);
+    const double c = u0 * (j >= md.n_exp ? edev : 1.0 - edev), cn1 = c * nu * l1, cn2 = c * nu * l2;
+    const double A = EX_HALF * l1, B = EX_HALF * l2;
+    row[0] = A;
+    row[1] = B;
+    row[2] = pack_float2((float)A, (float)B);
+    row[3] = u0;
+    row[4] = c * l1;
+    row[5] = c * l2;
+    row[6] = cn1 * l1;
+    row[7] = -cn1;
+    row[8] = cn1 * l2;
+    row[9] = nu;
+    row[10] = cn2 * l2;
+    row[11] = -cn2;
+}
+
 template <class R>
 __global__ void __launch_bounds__(PREP_THREADS)
 k_prep(const double* __restrict__ theta, const PatchGeo* __restrict__ geo,
@@ -170,6 +228,8 @@ k_prep(const double* __restrict__ theta, const PatchGeo* __restrict__ geo,
     __shared__ double th[NP];
     __shared__ R thr[NP];
     __shared__ R gsh[PREP_THREADS / PREP_HDR][4];   // gxx gxy gyy e_dev per patch of a round
+    constexpr bool WHITE = std::is_same<R, double>::value;   // the FP64 table's whitened frame
+    __shared__ double dsh[WHITE ? PREP_THREADS / PREP_HDR : 1][MAXPSF][2];   // D1 D2
     const int t = threadIdx.x;
     if (t < NP) {
         const double v = theta[(size_t)NP * s + t];
@@ -248,7 +308,7 @@ k_prep(const double* __restrict__ theta, const PatchGeo* __restrict__ geo,
                 T[H_A0] = thr[P_A];
                 T[H_A1] = thr[P_A + 1];
                 T[H_IOTA] = (R)im.iota;
-                T[7] = (R)0;
+                T[H_EDEV] = thr[P_EDEV];
             }
         }
         if (r0 == 0 && kl_here) {
@@ -258,6 +318,17 @@ k_prep(const double* __restrict__ theta, const PatchGeo* __restrict__ geo,
         __syncthreads();
         // components of the patches of this round
         const int nr = min(np - r0, PREP_THREADS / PREP_HDR);
+        if constexpr (WHITE) {
+            // one thread per (patch, PSF component): the frame T_k and D
+            for (int idx = t; idx < nr * MAXPSF; idx += blockDim.x) {
+                const int pj = idx / MAXPSF, k = idx % MAXPSF;
+                const ImgMeta& im = img[geo[p0 + r0 + pj].img];
+                if (k >= im.npsf) continue;
+                whiten_frame64(im, k, gsh[pj], thr[P_SCALE] * thr[P_SCALE] * thr[P_AXIS],
+                               tbl + (size_t)(p0 + r0 + pj) * TBL_STRIDE + T_STAR + k * STAR_STRIDE, dsh[pj][k]);
+            }
+            __syncthreads();
+        }
         const R log2e = (R)LOG2E, log2_2pi = (R)2.6514961294723187;   // log2(2 pi)
         for (int idx = t; ; idx += blockDim.x) {
             // component idx of the round: patch pj = first patch whose running count exceeds idx
@@ -277,6 +348,11 @@ k_prep(const double* __restrict__ theta, const PatchGeo* __restrict__ geo,
             const R* Gp = gsh[pj];
             const R gxx = Gp[0], gxy = Gp[1], gyy = Gp[2], edev = Gp[3];
             const int k = base_c / per_k, j = base_c % per_k - 1;
+            if constexpr (WHITE) {
+                if (j >= 0)
+                    galaxy_row64(*md, im.psf_c64[k], j, edev, dsh[pj][k], T + T_GAL + (k * nprof + j) * GAL_STRIDE);
+                continue;
+            }
             const R* ps = psf_row(im, k, R());
             R cxx = ps[3], cxy = ps[4], cyy = ps[5], w = ps[0], dw = 0, nu = 0;
             if (j >= 0) {
@@ -606,6 +682,184 @@ __global__ void __launch_bounds__(CHUNK / PPT) k_adjoint(const WorkItem* __restr
                             &c0, &y1, &c1, &y2, &c2);
             out[PART_TH + j] = (double)c0 * tot[1 + y0] + (double)c1 * tot[1 + y1] +
                                (double)c2 * tot[1 + y2];
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------
+// The FP64 passes (fp64_profile.cuh: the mixture in the whitened frame, 2^x by table).
+// Bound by the FP64 pipe: one pixel per thread, the table and the 16 KB table of 2^x in
+// shared memory.  A source's E_s / Var_s are needed before the adjoint only where another
+// patch covers the pixel, so the map pass runs at those pixels alone (multi_only) and the
+// adjoint, which evaluates the mixture anyway, forms E = sky + E_s itself at the others.
+
+// Sums v over the warp's lanes (a butterfly: the same tree for every entry); lane l is left
+// with the sum of entry l / 2.  16 additions instead of 5 per entry.
+__device__ __forceinline__ double warp_reduce16(double (&v)[16], int lane) {
+#pragma unroll
+    for (int m = 16, n = 16; m > 1; m >>= 1, n >>= 1) {
+        const bool up = (lane & m) != 0;
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) {
+            const double send = up ? v[i] : v[i + n / 2], keep = up ? v[i + n / 2] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+__global__ void __launch_bounds__(CHUNK)
+k_contrib64(const WorkItem* __restrict__ items, const PatchGeo* __restrict__ geo, const ImgMeta* __restrict__ img,
+            int nprof, int n_exp, const double* __restrict__ tbl, double* __restrict__ spE, double* __restrict__ spV,
+            const uint8_t* __restrict__ single, const float* __restrict__ sky_map, double* __restrict__ emap,
+            double* __restrict__ vmap, bool multi_only, const int32_t* __restrict__ src_active) {
+    __shared__ __align__(16) double sT[TBL_STRIDE];
+    __shared__ __align__(16) double tab[EX_N];
+    const int item = (int)blockIdx.x;
+    const WorkItem it = items[item];
+    const PatchGeo g = geo[it.patch];
+    if (src_active && !src_active[g.src]) return;
+    const ImgMeta& im = img[g.img];
+    const int t = threadIdx.x, q = it.q0 + (t < it.n ? t : 0);
+    const int64_t sp = g.sp_off + q;
+    const bool alone = single && single[sp], need = t < it.n && !(alone && multi_only);
+    if (!__syncthreads_or(need)) return;
+    load_exp2_table(tab);
+    load_table(sT, tbl + (size_t)it.patch * TBL_STRIDE, T_GAL + im.npsf * nprof * GAL_STRIDE);
+    if (!__any_sync(0xffffffffu, need)) return;
+    const int yy = q / g.w, xx = q - yy * g.w;
+    Profile64 o;
+    profile64<false>(sT, nullptr, tab, im.npsf, nprof, n_exp, (double)xx, (double)yy, o);
+    double em0, em1, e, v;
+    moment_ratios64(sT, em0, em1);
+    source_ev64(sT, em0, em1, o.g0, galaxy64(sT, o), e, v);
+    if (!need) return;
+    if (alone) {
+        const int64_t m = im.px_off + (int64_t)(g.y0 + yy) * im.W + (g.x0 + xx);
+        emap[m] = (im.has_sky_map ? (double)sky_map[m] : im.sky) + e;
+        vmap[m] = v;
+    } else {
+        spE[sp] = e;
+        spV[sp] = v;
+    }
+}
+
+// Per item: the sums of ll and (MODE_GRAD) of d ll / d y over its pixels, the chain rule to
+// theta, and the ll of its singly covered pixels (item_ll, its share of the total).
+template <int MODE>
+__global__ void __launch_bounds__(CHUNK)
+k_adjoint64(const WorkItem* __restrict__ items, const PatchGeo* __restrict__ geo, const ImgMeta* __restrict__ img,
+            int nprof, int n_exp, const float* __restrict__ pixels, const float* __restrict__ sky_map,
+            const double* __restrict__ tbl, const uint8_t* __restrict__ single, const double* __restrict__ emap,
+            const double* __restrict__ vmap, double* __restrict__ part, double* __restrict__ item_ll) {
+    constexpr bool GRAD = MODE >= MODE_GRAD;
+    constexpr int V_ONE = 1 + NY;   // sums: ll, d ll / d y, ll of the singly covered pixels
+    __shared__ __align__(16) double sT[TBL_STRIDE];
+    __shared__ __align__(16) double tab[EX_N];
+    __shared__ double KG[MAXPSF * KG_STRIDE];
+    __shared__ double red[CHUNK / 32][16], tot[16];
+    const int item = (int)blockIdx.x;
+    const WorkItem it = items[item];
+    const PatchGeo g = geo[it.patch];
+    const ImgMeta& im = img[g.img];
+    const int npsf = im.npsf;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const bool ok = t < it.n;
+    const int q = it.q0 + (ok ? t : 0);
+    const int yy = q / g.w, xx = q - yy * g.w;
+    const int64_t m = im.px_off + (int64_t)(g.y0 + yy) * im.W + (g.x0 + xx);
+    const double x = (double)pixels[m];
+    const bool alone = single && single[g.sp_off + q];
+    double E = 0.0, V = 0.0;
+    if (alone) E = im.has_sky_map ? (double)sky_map[m] : im.sky;
+    else {
+        E = emap[m];
+        V = vmap[m];
+    }
+    if (GRAD || __syncthreads_or(alone)) {
+        load_exp2_table(tab);
+        load_table(sT, tbl + (size_t)it.patch * TBL_STRIDE, T_GAL + npsf * nprof * GAL_STRIDE);
+    }
+    if constexpr (GRAD) {
+        load_shape_maps(KG, sT, npsf);
+        __syncthreads();
+    }
+    double v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = 0.0;
+    const bool work = __any_sync(0xffffffffu, GRAD ? ok : ok && alone);
+    Profile64 o;
+    double g1 = 0.0, Es = 0.0;
+    if (work) {
+        double em0, em1, Vs;
+        profile64<GRAD>(sT, KG, tab, npsf, nprof, n_exp, (double)xx, (double)yy, o);
+        moment_ratios64(sT, em0, em1);
+        g1 = galaxy64(sT, o);
+        source_ev64(sT, em0, em1, o.g0, g1, Es, Vs);
+        if (alone) {
+            E = __dadd_rn(E, Es);
+            V = Vs;
+        }
+    }
+    if (ok) {
+        const double iE = __drcp_rn(E);
+        v[0] = pixel_ll64(x, E, V, iE);
+        if (alone) v[V_ONE] = v[0];
+        if constexpr (GRAD) {
+            const double iE2 = iE * iE, w2 = -0.5 * x * iE2;
+            const double w1 = x * (iE + V * iE2 * iE) - 1.0 - 2.0 * w2 * Es;
+            const double iota = sT[H_IOTA], a0 = sT[H_A0], a1 = sT[H_A1];
+            const double el0 = sT[H_EL0], el20 = sT[H_EL20], el1 = sT[H_EL1], el21 = sT[H_EL21];
+            const double h0 = iota * o.g0, h1 = iota * g1;
+            const double s0 = w2 * h0 * h0, s1 = w2 * h1 * h1, r0 = w1 * h0, r1 = w1 * h1;
+            v[1 + Y_A0] = r0 * el0 + s0 * el20;
+            v[1 + Y_A1] = r1 * el1 + s1 * el21;
+            v[1 + Y_EL0] = r0 * a0;
+            v[1 + Y_EL20] = s0 * a0;
+            v[1 + Y_EL1] = r1 * a1;
+            v[1 + Y_EL21] = s1 * a1;
+            const double u0 = a0 * iota * (w1 * el0 + 2.0 * w2 * el20 * h0);
+            const double u1 = a1 * iota * (w1 * el1 + 2.0 * w2 * el21 * h1);
+            v[1 + Y_MX] = u0 * o.gx0 + u1 * o.gx1;
+            v[1 + Y_MY] = u0 * o.gy0 + u1 * o.gy1;
+            v[1 + Y_EDEV] = u1 * (o.gd - o.ge);
+            v[1 + Y_GXX] = 0.5 * u1 * o.sxx;
+            v[1 + Y_GXY] = u1 * o.sxy;
+            v[1 + Y_GYY] = 0.5 * u1 * o.syy;
+        }
+    }
+    if constexpr (GRAD) {
+        const double s = warp_reduce16(v, lane);
+        if (!(lane & 1)) red[warp][lane >> 1] = s;
+    } else {
+        // the same butterfly for the two sums of the value
+        const double a = warp_sum(v[0]), b = warp_sum(v[V_ONE]);
+        if (lane == 0) {
+            red[warp][0] = a;
+            red[warp][V_ONE] = b;
+        }
+    }
+    __syncthreads();
+    if (t < (GRAD ? V_ONE + 1 : 1) || t == V_ONE) {
+        double s = 0.0;
+        for (int w = 0; w < CHUNK / 32; ++w) s += red[w][t];
+        tot[t] = s;
+    }
+    __syncthreads();
+    double* out = part + (size_t)item * NPART;
+    if (t == 0) {
+        out[PART_LL] = tot[0];
+        if (item_ll) item_ll[item] = tot[V_ONE];
+    }
+    if constexpr (GRAD) {
+        // chain rule of this item's y-gradient: d/dtheta_j = sum_y dy/dtheta_j d/dy
+        for (int j = t; j < NP; j += CHUNK) {
+            const double el[2] = {sT[H_EL0], sT[H_EL1]}, el2[2] = {sT[H_EL20], sT[H_EL21]};
+            int y0, y1, y2;
+            double c0, c1, c2;
+            chain_column<double>(j, im.band, wcs_row<double>(im), el, el2, (const double(*)[3])(sT + T_DG), &y0,
+                                 &c0, &y1, &c1, &y2, &c2);
+            out[PART_TH + j] = c0 * tot[1 + y0] + c1 * tot[1 + y1] + c2 * tot[1 + y2];
         }
     }
 }
@@ -1261,18 +1515,13 @@ cudaError_t launch_prep(const DevProblem& P, const double* d_theta, int precisio
     return cudaGetLastError();
 }
 
-static ItemSet item_set(const DevProblem& P, const int32_t* idx, int n) {
-    return ItemSet{idx, n < 0 ? P.n_item : n};
-}
-
-cudaError_t launch_contrib(const DevProblem& P, int precision, cudaStream_t st, const int32_t* idx, int n) {
-    const ItemSet S = item_set(P, idx, n);
+cudaError_t launch_contrib(const DevProblem& P, int precision, cudaStream_t st, bool multi_only) {
+    const ItemSet S{nullptr, P.n_item};
     if (S.n == 0) return cudaSuccess;
     if (precision == CELESTE_FP64)
-        k_contrib<double, 1><<<S.n, CHUNK, 0, st>>>(P.items, S.idx, P.geo, P.img, P.nprof, P.tbl64,
-                                                    (double*)P.spE, (double*)P.spE2, P.single,
-                                                    P.pixels, P.sky_map, (double*)P.emap,
-                                                    (double*)P.vmap, P.item_ll, P.src_active);
+        k_contrib64<<<S.n, CHUNK, 0, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.tbl64, (double*)P.spE,
+                                           (double*)P.spE2, P.single, P.sky_map, (double*)P.emap, (double*)P.vmap,
+                                           multi_only, P.src_active);
     else
         switch (ppt_contrib(P)) {
 #define CEL_CONTRIB32(N)                                                                          \
@@ -1321,12 +1570,13 @@ static void adjoint_impl(const DevProblem& P, const R* tbl, int mode, ItemSet S,
             P.items, S.idx, P.geo, P.img, P.nprof, P.pixels, tbl, em, vm, P.item_part);
 }
 
-cudaError_t launch_adjoint(const DevProblem& P, int precision, int mode, cudaStream_t st,
-                           const int32_t* idx, int n) {
-    const ItemSet S = item_set(P, idx, n);
+cudaError_t launch_adjoint(const DevProblem& P, int precision, int mode, cudaStream_t st) {
+    const ItemSet S{nullptr, P.n_item};
     if (S.n == 0) return cudaSuccess;
     if (precision == CELESTE_FP64) {
-        adjoint_impl<double, 1>(P, P.tbl64, mode, S, st);
+        auto* fn = mode == MODE_LL ? k_adjoint64<MODE_LL> : k_adjoint64<MODE_GRAD>;
+        fn<<<S.n, CHUNK, 0, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.pixels, P.sky_map, P.tbl64, P.single,
+                                  (const double*)P.emap, (const double*)P.vmap, P.item_part, P.item_ll);
     } else {
         switch (ppt_adjoint(P)) {
             case 1: adjoint_impl<float, 1>(P, P.tbl32, mode, S, st); break;
