@@ -237,11 +237,12 @@ celeste_status run(celeste_problem* pr, const double* d_theta, int precision, in
             }));
         return CELESTE_OK;
     }
-    CEL_CUDA(timed(pr, "prep", st, [&] { return launch_prep(P, d_theta, precision, st); }));
+    // (the Hessian pass takes the KL terms itself)
+    CEL_CUDA(timed(pr, "prep", st, [&] { return launch_prep(P, d_theta, precision, st, mode != MODE_HESS); }));
     CEL_CUDA(timed(pr, "contrib", st, [&] { return launch_contrib(P, precision, st, true); }));
     CEL_CUDA(timed(pr, "gather", st, [&] { return launch_gather(P, precision, st); }));
     if (mode == MODE_HESS)
-        CEL_CUDA(timed(pr, "hess_adjoint", st, [&] { return launch_hess_pixels(P, precision, st); }));
+        CEL_CUDA(timed(pr, "hess_adjoint", st, [&] { return launch_hess_pixels(P, precision, d_theta, d_hess, st); }));
     else
         CEL_CUDA(timed(pr, mode == MODE_LL ? "ll_sum" : "adjoint", st,
                        [&] { return launch_adjoint(P, precision, mode, st); }));
@@ -853,6 +854,8 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     P.kl_grad = (double*)p;
     if ((st = dalloc(pr, &p, sizeof(double) * (size_t)n_src))) return bail(st);
     P.src_total = (double*)p;
+    if ((st = dalloc(pr, &p, sizeof(double) * HREC * (size_t)n_src))) return bail(st);
+    P.hsrc = (double*)p;
     if ((st = dalloc(pr, &p, sizeof(int32_t)))) return bail(st);
     P.done = (int32_t*)p;
     if (cudaMemset(P.done, 0, sizeof(int32_t)) != cudaSuccess) return bail(fail(CELESTE_ERR_CUDA, "memset"));

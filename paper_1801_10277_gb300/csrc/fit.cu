@@ -34,9 +34,6 @@
 
 namespace cel {
 
-cudaError_t launch_finalize_hess(const DevProblem& P, const double* d_theta, double* d_local,
-                                 double* d_grad, double* d_hess, cudaStream_t st);
-
 namespace {
 
 // K_LO: added to every softmax weight, so that a weight whose softmax underflows keeps
@@ -1079,7 +1076,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
     int32_t *d_bsrc, *d_bpo, *d_active, *d_srcact;
     PatchGeo* d_bgeo;
     WorkItem* d_bitems;
-    double *d_bth, *d_bthc, *d_bt, *d_btc, *d_f, *d_g, *d_h, *d_kl, *d_part, *d_dll, *d_tbl64;
+    double *d_bth, *d_bthc, *d_bt, *d_btc, *d_f, *d_g, *d_h, *d_kl, *d_hsrc, *d_part, *d_dll, *d_tbl64;
     float* d_tbl32;
     TrState* d_st;
     unsigned char *d_eo, *d_vo, *d_se, *d_sv, *d_ce, *d_cv;
@@ -1097,6 +1094,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
     FIT_CUDA(mem.alloc(&d_g, maxB * NP));
     FIT_CUDA(mem.alloc(&d_h, maxB * NP * NP));
     FIT_CUDA(mem.alloc(&d_kl, maxB));
+    FIT_CUDA(mem.alloc(&d_hsrc, maxB * HREC));
     FIT_CUDA(mem.alloc(&d_part, maxI * NPART));
     FIT_CUDA(mem.alloc(&d_dll, maxI));
     FIT_CUDA(mem.alloc(&d_tbl64, maxP * TBL_STRIDE));
@@ -1204,7 +1202,8 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             Pb.spE2 = d_sv;
             Pb.item_part = d_part;
             Pb.kl = d_kl;
-            Pb.kl_grad = nullptr;   // k_finalize_hess and k_tr_accept take the KL themselves
+            Pb.hsrc = d_hsrc;
+            Pb.kl_grad = nullptr;   // the Hessian pass and k_tr_accept take the KL themselves
             Pb.single = nullptr;    // batch buffers keep every E_s / Var_s
             Pb.item_ll = nullptr;
             Pb.status = nullptr;
@@ -1236,8 +1235,8 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
                                                               (const float*)d_sv, (float*)P.emap, (float*)P.vmap,
                                                               d_srcact);
             }
-            chk(launch_hess_pixels(Pb, prec, st));
-            chk(launch_finalize_hess(Pb, d_bth, d_f, d_g, d_h, st));
+            chk(launch_hess_pixels(Pb, prec, d_bth, d_h, st));
+            chk(launch_finalize_hess(Pb, d_f, d_g, d_h, st));
             k_tr_step<<<nb, TR_THREADS, TR_DYN_BYTES, st>>>(nb, d_bth, d_bt, d_f, d_g, d_h, d_kl, d_bthc, d_btc,
                                                  d_st, *opts, d_active);
             // only sources with a candidate evaluate it

@@ -36,7 +36,7 @@ constexpr double EX_C1 = 0x1.62e42fefa39efp-12, EX_C2 = 0x1.ebfbdff82c58fp-25, E
 // below 2^-1020 the value is taken as 0
 constexpr float EX_MIN = -1020.f * EX_N;
 
-struct Exp2Table {
+struct alignas(16) Exp2Table {
     double v[EX_N];
 };
 struct DoubleDouble {

@@ -3,10 +3,11 @@
 //
 //   k_hess           per work item: value, gradient and Hessian of the pixel terms
 //                    wrt the twelve intermediate variables y of the (source, patch);
-//                    the mixture terms are recomputed here, nothing is stored.
-//   k_finalize_hess  one CTA per source: sparse chain rule y -> theta over the
-//                    source's patches, plus the KL Hessian; writes the full
-//                    symmetric 44 x 44 matrix, the gradient and the local objective.
+//                    the mixture terms are recomputed here, nothing is stored.  Its first
+//                    CTAs take the sources' KL terms and parameter-only derivatives.
+//   k_finalize_hess  one CTA per source: chain rule y -> theta over the source's patches,
+//                    added to the KL Hessian; the full symmetric 44 x 44 matrix, the
+//                    gradient and the local objective.
 //
 // With e = dE_s/dy, v = dVar_s/dy = dE2_s/dy - 2 E_s e and the second derivatives
 // DE = d2E_s/dy2, DE2 = d2E2_s/dy2 (E2_s = sum_i a_i iota^2 E[l_i^2] g_i^2):
@@ -345,6 +346,221 @@ __host__ __device__ __forceinline__ void whitened_add(const R (&s)[NWS], R z1, R
         for (int f = e; f < 3; ++f, ++c) h1[c] += KV[e][0] * K[f][0] + KV[e][1] * K[f][1] + KV[e][2] * K[f][2];
 }
 
+// The pixel-frame ellipse is G = A W A' with W = ah I + bh (cos 2phi, sin 2phi; sin 2phi,
+// -cos 2phi), ah = sigma^2 (1 + rho^2) / 2, bh = sigma^2 (1 - rho^2) / 2.  Its first and
+// second derivatives over s = (e_axis, e_angle, e_scale) are A (dW) A' and A (d2W) A':
+// dW and d2W depend on theta alone (computed once per source, by one thread), and each
+// patch maps them through its own A (one output per thread).  Host-callable for tests.
+__host__ __device__ void shape_w_derivs(const double* th, double dW[3][3], double d2W[3][3][3]) {
+    const double rho = th[P_AXIS], phi = th[P_ANGLE], sg = th[P_SCALE];
+    const double bh = 0.5 * sg * sg * (1.0 - rho * rho);
+    double s2, c2;
+    sincos(2.0 * phi, &s2, &c2);
+    // first derivatives (index order rho = 0, phi = 1, sigma = 2; W as xx, xy, yy)
+    {
+        const double da = sg * sg * rho, db = -sg * sg * rho;
+        dW[0][0] = da + db * c2; dW[0][1] = db * s2; dW[0][2] = da - db * c2;
+    }
+    dW[1][0] = -2.0 * bh * s2; dW[1][1] = 2.0 * bh * c2; dW[1][2] = 2.0 * bh * s2;
+    {
+        const double da = sg * (1.0 + rho * rho), db = sg * (1.0 - rho * rho);
+        dW[2][0] = da + db * c2; dW[2][1] = db * s2; dW[2][2] = da - db * c2;
+    }
+    // second derivatives of ah, bh over (rho, sigma)
+    const double bh_r = -sg * sg * rho, bh_s = sg * (1.0 - rho * rho);
+    const double ah_rr = sg * sg, ah_ss = 1.0 + rho * rho, ah_rs = 2.0 * sg * rho;
+    const double bh_rr = -sg * sg, bh_ss = 1.0 - rho * rho, bh_rs = -2.0 * sg * rho;
+    auto set = [&](int a, int b, double xx, double xy, double yy) {
+        d2W[a][b][0] = d2W[b][a][0] = xx;
+        d2W[a][b][1] = d2W[b][a][1] = xy;
+        d2W[a][b][2] = d2W[b][a][2] = yy;
+    };
+    set(0, 0, ah_rr + bh_rr * c2, bh_rr * s2, ah_rr - bh_rr * c2);
+    set(2, 2, ah_ss + bh_ss * c2, bh_ss * s2, ah_ss - bh_ss * c2);
+    set(0, 2, ah_rs + bh_rs * c2, bh_rs * s2, ah_rs - bh_rs * c2);
+    set(0, 1, -2.0 * bh_r * s2, 2.0 * bh_r * c2, 2.0 * bh_r * s2);
+    set(2, 1, -2.0 * bh_s * s2, 2.0 * bh_s * c2, 2.0 * bh_s * s2);
+    set(1, 1, -4.0 * bh * c2, -4.0 * bh * s2, 4.0 * bh * c2);
+}
+
+// component c (xx, xy, yy) of A w A' for a symmetric w = (wxx, wxy, wyy)
+__host__ __device__ __forceinline__ double a_transform(const double* A, const double* w, int c) {
+    const double wxx = w[0], wxy = w[1], wyy = w[2];
+    if (c == 0) return A[0] * A[0] * wxx + 2.0 * A[0] * A[1] * wxy + A[1] * A[1] * wyy;
+    if (c == 1) return A[0] * A[2] * wxx + (A[0] * A[3] + A[1] * A[2]) * wxy + A[1] * A[3] * wyy;
+    return A[2] * A[2] * wxx + 2.0 * A[2] * A[3] * wxy + A[3] * A[3] * wyy;
+}
+
+// ---- The terms of a source that depend on its parameters alone, by the first CTAs of
+// k_hess (their FP64 latencies then pass behind the pixel work): the KL value, gradient and
+// Hessian, the brightness moments of the five bands and the world-frame shape derivatives.
+// hess_out receives -KL'' and zeros; the rest goes to the source's record.
+constexpr int HR_KL = 0, HR_KLG = 1, HR_MOM = HR_KLG + NP, HR_DW = HR_MOM + 20, HR_D2W = HR_DW + 9;
+static_assert(HR_D2W + 27 <= HREC && HREC % 2 == 0, "the source's record");
+constexpr int TERM_SRC = CHUNK / 64;   // sources per CTA: two warps each
+
+struct SourceTerms {
+    int n_src;
+    const double* theta;
+    const ModelDev* md;
+    double* hsrc;        // [n_src][HREC]
+    double* kl;
+    double* hess;        // [n_src][NP][NP]
+    int32_t* status;     // nullable: no domain check
+};
+
+// KL value, gradient and Hessian of one source by one warp (the closed forms of
+// kl_value_grad and their derivatives).  One logarithm and one reciprocal per lane (lanes
+// 8 i + d: k_id; 16 + 4 i + j: c2; 24 + i: a_i; 26 + i: r2_i), the 4 x 4 algebra of
+// colour-prior component (i, d) on lane 8 i + d, the sums over components by shuffles, and
+// then every entry written by one lane.
+__device__ __forceinline__ void kl_terms_warp(const ModelDev& md, const double* th, double* rec, double* kl_out,
+                                              double* H) {
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    const int i = (lane >> 3) & 1, d = lane & 7;
+    auto put = [&](int p, int q, double v) {
+        H[p * NP + q] = -v;
+        if (p != q) H[q * NP + p] = -v;
+    };
+    double x = 1.0;
+    if (lane < 16) x = th[P_K + lane];
+    else if (lane < 24) x = th[P_C2 + lane - 16];
+    else if (lane < 26) x = th[P_A + lane - 24];
+    else if (lane < 28) x = th[P_R2 + lane - 26];
+    double lv = log(x);
+    const double rv = 1.0 / x;
+    if (lane < 16) lv -= md.prior_logw[i][d];
+    else if (lane >= 24 && lane < 26) lv -= md.prior_logphi[lane - 24];
+    else if (lane >= 26 && lane < 28) lv = md.prior_logpv[lane - 26] - lv;
+    double slog = 0.0, ic2[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        slog += __shfl_sync(full, lv, 16 + 4 * i + j);
+        ic2[j] = __shfl_sync(full, rv, 16 + 4 * i + j);
+    }
+    const double a = th[P_A + i];
+    // sums over the components of: k (log k / w + KL_d), k, k P diff, k diag P, k P (upper)
+    double sum[20];
+#pragma unroll
+    for (int u = 0; u < 20; ++u) sum[u] = 0.0;
+    if (lane < 16) {
+        const double k = th[P_K + lane];
+        const double* Pm = md.prior_P[i][d];
+        const double* mu = md.prior_mu[i][d];
+        double diff[4], quad = 0.0, tr = 0.0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) diff[j] = th[P_C1 + 4 * i + j] - mu[j];
+        const int ik = P_K + lane;
+        int c = 10;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            double pd = 0.0;
+#pragma unroll
+            for (int l = 0; l < 4; ++l) pd += Pm[4 * j + l] * diff[l];
+            quad += diff[j] * pd;
+            tr += Pm[5 * j] * th[P_C2 + 4 * i + j];
+            sum[2 + j] = k * pd;
+            sum[6 + j] = k * Pm[5 * j];
+            put(ik, P_C1 + 4 * i + j, a * pd);
+            put(ik, P_C2 + 4 * i + j, 0.5 * a * (Pm[5 * j] - ic2[j]));
+#pragma unroll
+            for (int l = j; l < 4; ++l, ++c) sum[c] = k * Pm[4 * j + l];
+        }
+        const double klc = 0.5 * (tr + quad - 4.0 + md.prior_logdet[i][d] - slog);
+        sum[0] = k * (lv + klc);
+        sum[1] = k;
+        const double dk = lv + 1.0 + klc;
+        rec[HR_KLG + ik] = a * dk;
+        put(P_A + i, ik, dk);
+        put(ik, ik, a * rv);
+    }
+#pragma unroll
+    for (int u = 0; u < 20; ++u)
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) sum[u] += __shfl_xor_sync(full, sum[u], o);
+    const double la = __shfl_sync(full, lv, 24 + i), ia = __shfl_sync(full, rv, 24 + i);
+    const double lpr = __shfl_sync(full, lv, 26 + i), ir2 = __shfl_sync(full, rv, 26 + i);
+    double klv = 0.0;
+    if (lane < 16) {
+        const int iA = P_A + i;
+        if (d < 4) {
+            // colour j = d; the row's upper entries of sum_d k_d P_d
+            double kp = sum[2], kd = sum[6], ic = ic2[0], row[4] = {sum[10], sum[11], sum[12], sum[13]};
+            if (d == 1) { kp = sum[3]; kd = sum[7]; ic = ic2[1]; row[1] = sum[14]; row[2] = sum[15]; row[3] = sum[16]; }
+            if (d == 2) { kp = sum[4]; kd = sum[8]; ic = ic2[2]; row[2] = sum[17]; row[3] = sum[18]; }
+            if (d == 3) { kp = sum[5]; kd = sum[9]; ic = ic2[3]; row[3] = sum[19]; }
+            const int c1 = P_C1 + 4 * i + d, c2 = P_C2 + 4 * i + d;
+            const double sc2 = 0.5 * (kd - sum[1] * ic);
+            rec[HR_KLG + c1] = a * kp;
+            rec[HR_KLG + c2] = a * sc2;
+            put(iA, c1, kp);
+            put(iA, c2, sc2);
+            put(c2, c2, 0.5 * a * sum[1] * ic * ic);
+#pragma unroll
+            for (int l = 0; l < 4; ++l)
+                if (l >= d) put(c1, P_C1 + 4 * i + l, a * row[l]);
+        } else {
+            const double r1 = th[P_R1 + i], r2 = th[P_R2 + i];
+            const double dr = r1 - md.prior_r[i][0], ipv = md.prior_inv_pv[i];
+            if (d == 4) {
+                const double K = 0.5 * (lpr + (r2 + dr * dr) * ipv - 1.0) + sum[0];
+                klv = a * (la + K);
+                rec[HR_KLG + iA] = la + 1.0 + K;
+                put(iA, iA, ia);
+            } else if (d == 5) {
+                rec[HR_KLG + P_R1 + i] = a * dr * ipv;
+                put(iA, P_R1 + i, dr * ipv);
+                put(P_R1 + i, P_R1 + i, a * ipv);
+            } else if (d == 6) {
+                const double v = 0.5 * (ipv - ir2);
+                rec[HR_KLG + P_R2 + i] = a * v;
+                put(iA, P_R2 + i, v);
+                put(P_R2 + i, P_R2 + i, 0.5 * a * ir2 * ir2);
+            }
+        }
+    }
+    if (lane < 6) rec[HR_KLG + lane] = 0.0;   // position and shape carry no prior
+    klv += __shfl_xor_sync(full, klv, 8);
+    klv = __shfl_sync(full, klv, 4);
+    if (lane == 0) {
+        rec[HR_KL] = klv;
+        *kl_out = klv;
+    }
+}
+
+// the terms of sources s0 .. s0 + TERM_SRC, one CTA of k_hess; sm: TERM_SRC NP doubles
+__device__ __forceinline__ void source_terms(const SourceTerms& a, int s0, const int32_t* __restrict__ src_active,
+                                             double* sm) {
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int n = min(TERM_SRC, a.n_src - s0);
+    for (int u = 0; u < n; ++u) {
+        if (src_active && !src_active[s0 + u]) continue;
+        double* H = a.hess + (size_t)NP * NP * (s0 + u);   // the caller's: 8-byte aligned
+        for (int i = t; i < NP * NP; i += CHUNK) H[i] = 0.0;
+    }
+    for (int i = t; i < n * NP; i += CHUNK) {
+        sm[i] = a.theta[(size_t)NP * s0 + i];
+        if (a.status) theta_domain_check(i % NP, sm[i], a.status);
+    }
+    __syncthreads();
+    const int u = warp % TERM_SRC, s = s0 + u;
+    if (u >= n || (src_active && !src_active[s])) return;
+    const double* th = sm + u * NP;
+    double* rec = a.hsrc + (size_t)HREC * s;
+    if (warp < TERM_SRC) {
+        kl_terms_warp(*a.md, th, rec, a.kl + s, a.hess + (size_t)NP * NP * s);
+        return;
+    }
+    if (lane < 10) band_moments(th, lane >> 1, lane & 1, rec[HR_MOM + 2 * lane], rec[HR_MOM + 2 * lane + 1]);
+    if (lane == 10) {
+        double dW[3][3], d2W[3][3][3];
+        shape_w_derivs(th, dW, d2W);
+        for (int i = 0; i < 9; ++i) rec[HR_DW + i] = dW[i / 3][i % 3];
+        for (int i = 0; i < 27; ++i) rec[HR_D2W + i] = d2W[i / 9][i / 3 % 3][i % 3];
+    }
+}
+
 // Shared memory of k_hess (bytes): the patch's table (R), per PSF component its frame, the
 // component rows and, FP64, the table of 2^x; the warps' sums take the rows' place at the end.
 template <class R>
@@ -376,7 +592,7 @@ __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ ite
                                                 const R* __restrict__ emap,
                                                 const R* __restrict__ vmap,
                                                 double* __restrict__ part,
-                                                const int32_t* __restrict__ src_active) {
+                                                const int32_t* __restrict__ src_active, SourceTerms src) {
     constexpr bool DBL = std::is_same<R, double>::value;
     using Lay = HessLay<R>;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -384,7 +600,14 @@ __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ ite
     R* frames = reinterpret_cast<R*>(smem + Lay::fr);
     R* rows = reinterpret_cast<R*>(smem + Lay::rows);
     double* tab = reinterpret_cast<double*>(smem + Lay::tab);
-    const WorkItem it = items[blockIdx.x];
+    // the first CTAs take the sources' terms that do not depend on the pixels
+    const int n_term_cta = (src.n_src + TERM_SRC - 1) / TERM_SRC;
+    if ((int)blockIdx.x < n_term_cta) {
+        source_terms(src, (int)blockIdx.x * TERM_SRC, src_active, reinterpret_cast<double*>(smem));
+        return;
+    }
+    const int item = (int)blockIdx.x - n_term_cta;
+    const WorkItem it = items[item];
     const PatchGeo g = geo[it.patch];
     if (src_active && !src_active[g.src]) return;
     const ImgMeta& im = img[g.img];
@@ -670,335 +893,199 @@ __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ ite
     for (int i = t; i < HV; i += blockDim.x) {
         double s = 0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][i];
-        part[(size_t)blockIdx.x * NPART + i] = s;
+        part[(size_t)item * NPART + i] = s;
     }
 }
 
 // ---------------------------------------------------------------------------------
-// per-source chain rule and KL Hessian
+// per-source chain rule
 
-
-// The pixel-frame ellipse is G = A W A' with W = ah I + bh (cos 2phi, sin 2phi; sin 2phi,
-// -cos 2phi), ah = sigma^2 (1 + rho^2) / 2, bh = sigma^2 (1 - rho^2) / 2.  Its first and
-// second derivatives over s = (e_axis, e_angle, e_scale) are A (dW) A' and A (d2W) A':
-// dW and d2W depend on theta alone (computed once per source, by one thread), and each
-// patch maps them through its own A (one output per thread).  Host-callable for tests.
-__host__ __device__ void shape_w_derivs(const double* th, double dW[3][3], double d2W[3][3][3]) {
-    const double rho = th[P_AXIS], phi = th[P_ANGLE], sg = th[P_SCALE];
-    const double bh = 0.5 * sg * sg * (1.0 - rho * rho);
-    double s2, c2;
-    sincos(2.0 * phi, &s2, &c2);
-    // first derivatives (index order rho = 0, phi = 1, sigma = 2; W as xx, xy, yy)
-    {
-        const double da = sg * sg * rho, db = -sg * sg * rho;
-        dW[0][0] = da + db * c2; dW[0][1] = db * s2; dW[0][2] = da - db * c2;
-    }
-    dW[1][0] = -2.0 * bh * s2; dW[1][1] = 2.0 * bh * c2; dW[1][2] = 2.0 * bh * s2;
-    {
-        const double da = sg * (1.0 + rho * rho), db = sg * (1.0 - rho * rho);
-        dW[2][0] = da + db * c2; dW[2][1] = db * s2; dW[2][2] = da - db * c2;
-    }
-    // second derivatives of ah, bh over (rho, sigma)
-    const double bh_r = -sg * sg * rho, bh_s = sg * (1.0 - rho * rho);
-    const double ah_rr = sg * sg, ah_ss = 1.0 + rho * rho, ah_rs = 2.0 * sg * rho;
-    const double bh_rr = -sg * sg, bh_ss = 1.0 - rho * rho, bh_rs = -2.0 * sg * rho;
-    auto set = [&](int a, int b, double xx, double xy, double yy) {
-        d2W[a][b][0] = d2W[b][a][0] = xx;
-        d2W[a][b][1] = d2W[b][a][1] = xy;
-        d2W[a][b][2] = d2W[b][a][2] = yy;
-    };
-    set(0, 0, ah_rr + bh_rr * c2, bh_rr * s2, ah_rr - bh_rr * c2);
-    set(2, 2, ah_ss + bh_ss * c2, bh_ss * s2, ah_ss - bh_ss * c2);
-    set(0, 2, ah_rs + bh_rs * c2, bh_rs * s2, ah_rs - bh_rs * c2);
-    set(0, 1, -2.0 * bh_r * s2, 2.0 * bh_r * c2, 2.0 * bh_r * s2);
-    set(2, 1, -2.0 * bh_s * s2, 2.0 * bh_s * c2, 2.0 * bh_s * s2);
-    set(1, 1, -4.0 * bh * c2, -4.0 * bh * s2, 4.0 * bh * c2);
+// The chain rule goes through twelve variables w per (source, patch) that stand in the
+// places of y: a_0, a_1, then per type i the mean m_i and variance v_i of the log brightness
+// in the patch's band (places Y_EL0, Y_EL20, Y_EL1, Y_EL21), u_0, u_1, e_dev, and e_axis,
+// e_angle, e_scale.  A parameter theta_j < P_K enters exactly one of them, with a factor of
+// the band alone that is -1, 0 or 1, so the w-Hessians of a band's patches are added first
+// and spread over the 28 x 28 block once per source by additions.
+__device__ __forceinline__ int w_of_param(int j) {
+    if (j < 2) return Y_MX + j;
+    if (j == P_EDEV) return Y_EDEV;
+    if (j <= P_SCALE) return Y_GXX + j - P_AXIS;
+    if (j >= P_A) return j == P_A ? Y_A0 : Y_A1;
+    const bool var = (j >= P_R2 && j < P_C1) || j >= P_C2;
+    const int i = j < P_R2 ? j - P_R1 : j < P_C1 ? j - P_R2 : j < P_C2 ? (j - P_C1) >> 2 : (j - P_C2) >> 2;
+    return (i == 0 ? Y_EL0 : Y_EL1) + (var ? 1 : 0);
+}
+__device__ __forceinline__ int w_factor(int band, int j) {
+    if (j < P_C1 || j >= P_A) return 1;
+    const int c = (j - P_C1) & 3, ref = 2;   // color_beta as an integer
+    const int beta = band < ref ? (c >= band && c < ref ? -1 : 0) : band > ref ? (c >= ref && c < band ? 1 : 0) : 0;
+    return j < P_C2 ? beta : beta * beta;
 }
 
-// component c (xx, xy, yy) of A w A' for a symmetric w = (wxx, wxy, wyy)
-__host__ __device__ __forceinline__ double a_transform(const double* A, const double* w, int c) {
-    const double wxx = w[0], wxy = w[1], wyy = w[2];
-    if (c == 0) return A[0] * A[0] * wxx + 2.0 * A[0] * A[1] * wxy + A[1] * A[1] * wyy;
-    if (c == 1) return A[0] * A[2] * wxx + (A[0] * A[3] + A[1] * A[2]) * wxy + A[1] * A[3] * wyy;
-    return A[2] * A[2] * wxx + 2.0 * A[2] * A[3] * wxy + A[3] * A[3] * wyy;
-}
-
-// Full KL Hessian (44 x 44, row-major) added into H (zeroed by the caller), by one warp
-// (every lane calls it).  Lanes 8 i + d (i < 2, d < 8) hold the terms of type i's
-// colour-prior component d, which touch disjoint entries (the k_d rows); the sums over
-// components are shuffled within each group of eight, and lane 8 i then writes the
-// type's a / r / c entries.  Every entry is written by exactly one lane.
-__device__ void kl_hessian_warp(const ModelDev& md, const double* th, double* H) {
-    const int lane = threadIdx.x & 31;
-    const unsigned full = 0xffffffffu;
-    const int i = (lane >> 3) & 1, d = lane & 7;
-    auto add = [&](int p, int q, double v) {
-        H[p * NP + q] += v;
-        if (p != q) H[q * NP + p] += v;
-    };
-    double c1[4], c2[4], ic2[4], slog = 0.0;
-    for (int j = 0; j < 4; ++j) {
-        c1[j] = th[P_C1 + 4 * i + j];
-        c2[j] = th[P_C2 + 4 * i + j];
-    }
-    double sc1[4] = {0, 0, 0, 0}, sc2[4] = {0, 0, 0, 0}, Pk[16], ks = 0.0;
-    for (int j = 0; j < 16; ++j) Pk[j] = 0.0;
-    const double a = th[P_A + i];
-    if (lane < 16) {
-        for (int j = 0; j < 4; ++j) {
-            slog += log(c2[j]);
-            ic2[j] = 1.0 / c2[j];
-        }
-        const double k = th[P_K + NCOMP * i + d];
-        const double* Pm = md.prior_P[i][d];
-        const double* mu = md.prior_mu[i][d];
-        double diff[4], Pd[4], quad = 0.0, tr = 0.0;
-        for (int j = 0; j < 4; ++j) diff[j] = c1[j] - mu[j];
-        for (int j = 0; j < 4; ++j) {
-            double sj = 0.0;
-            for (int l = 0; l < 4; ++l) sj += Pm[4 * j + l] * diff[l];
-            Pd[j] = sj;
-            quad += diff[j] * sj;
-            tr += Pm[5 * j] * c2[j];
-        }
-        const double klc = 0.5 * (tr + quad - 4.0 + md.prior_logdet[i][d] - slog);
-        const int ik = P_K + NCOMP * i + d;
-        add(P_A + i, ik, log(k / md.prior_w[i][d]) + 1.0 + klc);
-        add(ik, ik, a / k);
-        for (int j = 0; j < 4; ++j) {
-            add(ik, P_C1 + 4 * i + j, a * Pd[j]);
-            add(ik, P_C2 + 4 * i + j, a * 0.5 * (Pm[5 * j] - ic2[j]));
-            sc1[j] = k * Pd[j];
-            sc2[j] = 0.5 * k * (Pm[5 * j] - ic2[j]);
-        }
-        for (int j = 0; j < 16; ++j) Pk[j] = k * Pm[j];
-        ks = k;
-    }
-    for (int o = 1; o < 8; o <<= 1) {
-        ks += __shfl_xor_sync(full, ks, o);
-        for (int j = 0; j < 4; ++j) {
-            sc1[j] += __shfl_xor_sync(full, sc1[j], o);
-            sc2[j] += __shfl_xor_sync(full, sc2[j], o);
-        }
-        for (int j = 0; j < 16; ++j) Pk[j] += __shfl_xor_sync(full, Pk[j], o);
-    }
-    if (lane < 16 && d == 0) {
-        const double r1 = th[P_R1 + i], r2 = th[P_R2 + i];
-        const double pm = md.prior_r[i][0], pv = md.prior_r[i][1];
-        const int ia = P_A + i, ir1 = P_R1 + i, ir2 = P_R2 + i;
-        add(ia, ia, 1.0 / a);
-        add(ia, ir1, (r1 - pm) / pv);
-        add(ia, ir2, 0.5 * (1.0 / pv - 1.0 / r2));
-        add(ir1, ir1, a / pv);
-        add(ir2, ir2, a * 0.5 / (r2 * r2));
-        for (int j = 0; j < 4; ++j) {
-            add(ia, P_C1 + 4 * i + j, sc1[j]);
-            add(ia, P_C2 + 4 * i + j, sc2[j]);
-            add(P_C2 + 4 * i + j, P_C2 + 4 * i + j, a * 0.5 * ks * ic2[j] * ic2[j]);
-            for (int l = j; l < 4; ++l) add(P_C1 + 4 * i + j, P_C1 + 4 * i + l, a * Pk[4 * j + l]);
-        }
-    }
-    __syncwarp();
-}
-
-constexpr int FH_THREADS = 256;
-// packed order of the 44 x 44 upper triangle (a << 8 | b, b <= a)
-__device__ const PackedTriangle<NP> g_pkq = packed_triangle<NP>();
-
-// d(m + v/2) / d theta_j (second = false) or d(2m + 2v) / d theta_j (second = true) of
-// type ty in band `band`, where log l | ty ~ N(m, v), m = r1 + beta . c1, v = r2 + beta^2 . c2
-__device__ __forceinline__ double bright_d(int band, int ty, int j, bool second) {
-    if (j == P_R1 + ty) return second ? 2.0 : 1.0;
-    if (j == P_R2 + ty) return second ? 2.0 : 0.5;
-    if (j >= P_C1 + 4 * ty && j < P_C1 + 4 * ty + 4) {
-        const double b = color_beta(band, j - P_C1 - 4 * ty);
-        return second ? 2.0 * b : b;
-    }
-    if (j >= P_C2 + 4 * ty && j < P_C2 + 4 * ty + 4) {
-        const double b = color_beta(band, j - P_C2 - 4 * ty);
-        return second ? 2.0 * b * b : 0.5 * b * b;
-    }
-    return 0.0;
-}
+// One CTA per source, two warps per band: a warp takes every second patch of its band, adds
+// the 91 sums of the patch's items (item order), maps them to w (X = H_y J, then J' X, J at
+// most three entries per column) and adds the result to the warp's shared accumulator; then
+// the block is spread and added to the -KL terms that source_terms left in hess_out.
+// Latency-bound, so the patches of a source run side by side and a patch costs about 50 FP64
+// instructions; per-patch loops over the 44 x 44 entries with the KL and its Hessian in the
+// same CTA took 119 us for 500 sources and 49 us for 64.
+constexpr int FH_SPLIT = 2, FH_WARPS = 5 * FH_SPLIT, FH_THREADS = 32 * FH_WARPS;
+constexpr int NPIX = P_K;                         // parameters that the pixels depend on
+constexpr int NPIXH = NPIX * (NPIX + 1) / 2;
+__device__ const PackedTriangle<NPIX> g_pix = packed_triangle<NPIX>();
+__device__ const PackedTriangle<NY> g_ypk = packed_triangle<NY>();
 
 __global__ void __launch_bounds__(FH_THREADS)
-k_finalize_hess(int n_src, const double* __restrict__ theta, const PatchGeo* __restrict__ geo,
-                const int32_t* __restrict__ patch_off, const ImgMeta* __restrict__ img,
-                const ModelDev* __restrict__ md, const double* __restrict__ part,
-                double* __restrict__ kl_out, double* __restrict__ local_out,
-                double* __restrict__ grad_out, double* __restrict__ hess_out,
-                int32_t* __restrict__ status, const int32_t* __restrict__ src_active) {
+k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __restrict__ patch_off,
+                const ImgMeta* __restrict__ img, const double* __restrict__ part, const double* __restrict__ hsrc,
+                double* __restrict__ local_out, double* __restrict__ grad_out, double* __restrict__ hess_out,
+                const int32_t* __restrict__ src_active) {
     const int s = blockIdx.x;
     if (s >= n_src || (src_active && !src_active[s])) return;
-    __shared__ double th[NP];
-    __shared__ double Hy[NY][NY];
-    __shared__ double Gy[NY + 1];
-    __shared__ int nzn[NP];
-    __shared__ int nzy[NP][3];
-    __shared__ double nzv[NP][3];
-    __shared__ double bmom[5][2][2];              // E[l_b | i], E[l_b^2 | i] per band and type
-    __shared__ double dG[3][3], d2G[3][3][3];     // the patch map's shape derivatives
-    __shared__ double dW[3][3], d2W[3][3][3];     // the same in the world frame (theta only)
-    __shared__ double wd[2], we[2];
-    __shared__ double S2[3][3];
-    __shared__ double klH[NP * NP];
-    __shared__ double Hacc[NP * NP];              // the pixel part of the 44 x 44 Hessian
-    __shared__ double bd[2][2][NP];               // bright_d(band, type, j, second) of this patch
-    __shared__ int act[NP], nact;                 // parameters this patch touches
-    __shared__ double klg[NP];
-    __shared__ double klv;
-    // packed upper-triangle order of the active block: q = a (a + 1) / 2 + b, b <= a,
-    // stored as a << 8 | b
-    constexpr int NPK = NP * (NP + 1) / 2;
-    __shared__ uint16_t pkq[NPK];
+    __shared__ double acc[FH_WARPS][HV];     // ll, d/dw, d2/dw2 (packed) of the warp's patches
+    __shared__ double rec[HREC];
+    __shared__ double sy[FH_WARPS][HV + 1];  // the patch's sums over y
+    __shared__ double sx[FH_WARPS][NY][NY];  // H_y J
+    __shared__ double sj[FH_WARPS][NY][3];   // J: column w's entries ...
+    __shared__ uint8_t si[FH_WARPS][NY][3];  // ... and their y
+    __shared__ double sg[FH_WARPS][36];      // dG, d2G of the patch
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    for (int q = t; q < NPK; q += blockDim.x) pkq[q] = g_pkq.v[q];
-    if (t < NP) {
-        th[t] = theta[(size_t)NP * s + t];
-        if (status) theta_domain_check(t, th[t], status);
-    }
-    for (int i = t; i < NP * NP; i += blockDim.x) {
-        klH[i] = 0.0;
-        Hacc[i] = 0.0;
-    }
+    const int band = warp % 5, half = warp / 5;
+    for (int i = t; i < HREC; i += FH_THREADS) rec[i] = hsrc[(size_t)HREC * s + i];
+    for (int i = lane; i < HV; i += 32) acc[warp][i] = 0.0;
     __syncthreads();
-    // the KL (warp 0: value and gradient; warp 1: Hessian) and the band moments of the
-    // five bands (warp 2), each lane-parallel: the FP64 pipe costs a warp instruction
-    // the same however few of its lanes are active
-    if (warp == 0) {
-        const double v = kl_warp<double>(*md, th, th, klg);
-        if (lane == 0) klv = v;
-    } else if (warp == 1) {
-        kl_hessian_warp(*md, th, klH);
-    } else if (warp == 2 && lane < 10) {
-        const int b = lane >> 1, i = lane & 1;
-        band_moments(th, b, i, bmom[b][i][0], bmom[b][i][1]);
-    } else if (warp == 3 && lane == 0) {
-        shape_w_derivs(th, dW, d2W);
-    }
-    double gacc = 0.0, lacc = 0.0;
-    for (int p = patch_off[s]; p < patch_off[s + 1]; ++p) {
-        __syncthreads();
-        const PatchGeo g = geo[p];
-        const ImgMeta& im = img[g.img];
-        const double* A = im.A;
-        if (t < 1 + NY + NYH) {
-            // the patch's items in order, loaded eight at a time before any is added
-            double v = 0.0;
+    const int p0 = patch_off[s], p1 = patch_off[s + 1];
+    int seen = 0;   // patches of this band so far
+    for (int pb = p0; pb < p1; pb += 32) {
+        const int pl = pb + lane;
+        unsigned mine = __ballot_sync(0xffffffffu, pl < p1 && img[geo[pl < p1 ? pl : p0].img].band == band);
+        for (; mine; mine &= mine - 1) {
+            if ((seen++ & (FH_SPLIT - 1)) != half) continue;
+            const int p = pb + __ffs(mine) - 1;
+            const PatchGeo g = geo[p];
+            const double* A = img[g.img].A;
+            // the patch's items in order, loaded four at a time before any is added
+            double v[3] = {0.0, 0.0, 0.0};
             const int i1 = g.item0 + g.nitem;
-            for (int i0 = g.item0; i0 < i1; i0 += 8) {
-                double x[8];
+            for (int i0 = g.item0; i0 < i1; i0 += 4) {
+                double x[4][3];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) x[u] = i0 + u < i1 ? part[(size_t)(i0 + u) * NPART + t] : 0.0;
+                for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (i0 + u < i1) v += x[u];
+                    for (int c = 0; c < 3; ++c)
+                        x[u][c] = i0 + u < i1 && lane + 32 * c < HV
+                                      ? part[(size_t)(i0 + u) * NPART + lane + 32 * c] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (i0 + u < i1)
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) v[c] += x[u][c];
             }
-            if (t == 0) lacc += v;
-            else if (t < 1 + NY) Gy[t - 1] = v;
-            else {
-                // unpack the packed upper triangle
-                int idx = t - 1 - NY, a = 0;
-                while (idx >= NY - a) { idx -= NY - a; ++a; }
-                const int b = a + idx;
-                Hy[a][b] = v;
-                Hy[b][a] = v;
+            // the shape derivatives through the patch's map
+            for (int i = lane; i < 36; i += 32)
+                sg[warp][i] = a_transform(A, rec + HR_DW + 3 * (i / 3), i % 3);
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                if (lane + 32 * c < HV) sy[warp][lane + 32 * c] = v[c];
+            __syncwarp();
+            const double* m = rec + HR_MOM + 4 * band;   // E[l_0], E[l_0^2], E[l_1], E[l_1^2]
+            if (lane < NY) {
+                const int w = lane;
+                int y0 = w, y1 = 0, y2 = 0;
+                double c0 = 1.0, c1 = 0.0, c2 = 0.0;
+                if (w >= Y_EL0 && w <= Y_EL21) {
+                    const int i = (w - Y_EL0) >> 1, var = (w - Y_EL0) & 1;
+                    y0 = Y_EL0 + 2 * i;
+                    y1 = y0 + 1;
+                    c0 = var ? 0.5 * m[2 * i] : m[2 * i];
+                    c1 = 2.0 * m[2 * i + 1];
+                } else if (w == Y_MX || w == Y_MY) {
+                    y0 = Y_MX;
+                    y1 = Y_MY;
+                    c0 = A[w - Y_MX];
+                    c1 = A[2 + w - Y_MX];
+                } else if (w >= Y_GXX) {
+                    const double* d = sg[warp] + 3 * (w - Y_GXX);
+                    y0 = Y_GXX; y1 = Y_GXY; y2 = Y_GYY;
+                    c0 = d[0]; c1 = d[1]; c2 = d[2];
+                }
+                sj[warp][w][0] = c0; sj[warp][w][1] = c1; sj[warp][w][2] = c2;
+                si[warp][w][0] = (uint8_t)y0; si[warp][w][1] = (uint8_t)y1; si[warp][w][2] = (uint8_t)y2;
+                acc[warp][1 + w] += c0 * sy[warp][1 + y0] + c1 * sy[warp][1 + y1] + c2 * sy[warp][1 + y2];
             }
-        } else if (t >= 128 && t < 128 + 9 + 27) {
-            // the patch's shape derivatives through its map, one output per thread
-            const int i = t - 128;
-            if (i < 9) {
-                dG[i / 3][i % 3] = a_transform(A, dW[i / 3], i % 3);
-            } else {
-                const int r = i - 9, a = r / 9, b = (r / 3) % 3, c = r % 3;
-                d2G[a][b][c] = a_transform(A, d2W[a][b], c);
+            if (lane == 0) acc[warp][0] += sy[warp][0];
+            __syncwarp();
+            const double* Gy = sy[warp] + 1;
+            const double* Hy = sy[warp] + 1 + NY;
+            for (int i = lane; i < NY * NY; i += 32) {
+                const int y = i / NY, w = i % NY;
+                double x = 0.0;
+#pragma unroll
+                for (int e = 0; e < 3; ++e) x += Hy[P2(y, si[warp][w][e])] * sj[warp][w][e];
+                sx[warp][y][w] = x;
             }
-        }
-        __syncthreads();
-        if (t < NP) {
-            // column t of the sparse Jacobian dy / dtheta for this patch
-            const int j = t;
-            int n = 0;
-            auto put = [&](int y, double val) {
-                nzy[j][n] = y;
-                nzv[j][n] = val;
-                ++n;
-            };
-            if (j == 0) { put(Y_MX, A[0]); put(Y_MY, A[2]); }
-            else if (j == 1) { put(Y_MX, A[1]); put(Y_MY, A[3]); }
-            else if (j == P_EDEV) put(Y_EDEV, 1.0);
-            else if (j >= P_AXIS && j <= P_SCALE) {
-                const int q = j - P_AXIS;
-                put(Y_GXX, dG[q][0]);
-                put(Y_GXY, dG[q][1]);
-                put(Y_GYY, dG[q][2]);
-            } else if (j == P_A || j == P_A + 1) put(j == P_A ? Y_A0 : Y_A1, 1.0);
-            else if (j < P_A) {
-                const int i = (j < P_C1) ? ((j - P_R1) & 1) : (((j - (j >= P_C2 ? P_C2 : P_C1)) >> 2) & 1);
-                const double dv = bright_d(im.band, i, j, false), ev = bright_d(im.band, i, j, true);
-                if (dv != 0.0) put(i == 0 ? Y_EL0 : Y_EL1, bmom[im.band][i][0] * dv);
-                if (ev != 0.0) put(i == 0 ? Y_EL20 : Y_EL21, bmom[im.band][i][1] * ev);
+            __syncwarp();
+            for (int i = lane; i < NYH; i += 32) {
+                const int b = g_ypk.v[i] >> 8, a = g_ypk.v[i] & 255;   // a <= b
+                double h = 0.0;
+#pragma unroll
+                for (int e = 0; e < 3; ++e) h += sj[warp][a][e] * sx[warp][si[warp][a][e]][b];
+                // second derivatives of y over w: E[l] = e^{m + v/2}, E[l^2] = e^{2m + 2v} (type i), and G
+                if (a >= Y_EL0 && b <= Y_EL21 && (a - Y_EL0) >> 1 == (b - Y_EL0) >> 1) {
+                    const int k = (a - Y_EL0) & ~1;
+                    const double f = ((a - Y_EL0) & 1 ? 0.5 : 1.0) * ((b - Y_EL0) & 1 ? 0.5 : 1.0);
+                    h += f * m[k] * Gy[Y_EL0 + k] + 4.0 * m[k + 1] * Gy[Y_EL0 + k + 1];
+                } else if (a >= Y_GXX) {
+                    const double* d = sg[warp] + 9 + 9 * (a - Y_GXX) + 3 * (b - Y_GXX);
+                    h += Gy[Y_GXX] * d[0] + Gy[Y_GXY] * d[1] + Gy[Y_GYY] * d[2];
+                }
+                acc[warp][1 + NY + yh_index(a, b)] += h;
             }
-            nzn[j] = n;
-            for (int ty = 0; ty < 2; ++ty) {
-                bd[ty][0][j] = bright_d(im.band, ty, j, false);
-                bd[ty][1][j] = bright_d(im.band, ty, j, true);
-            }
-        } else if (t >= 64 && t < 73) {
-            const int a = (t - 64) / 3, b = (t - 64) % 3;
-            S2[a][b] = Gy[Y_GXX] * d2G[a][b][0] + Gy[Y_GXY] * d2G[a][b][1] + Gy[Y_GYY] * d2G[a][b][2];
-        } else if (t >= 96 && t < 98) {
-            const int i = t - 96;
-            wd[i] = bmom[im.band][i][0] * Gy[i == 0 ? Y_EL0 : Y_EL1];
-            we[i] = bmom[im.band][i][1] * Gy[i == 0 ? Y_EL20 : Y_EL21];
-        }
-        __syncthreads();
-        if (t < NP)
-            for (int n = 0; n < nzn[t]; ++n) gacc += nzv[t][n] * Gy[nzy[t][n]];
-        if (warp == 0) {
-            // the parameters with a nonzero Jacobian column, ascending: the only rows and
-            // columns this patch adds to (every brightness and shape term lies among them)
-            const unsigned b0 = __ballot_sync(0xffffffffu, nzn[lane] > 0);
-            const unsigned b1 = __ballot_sync(0xffffffffu, lane + 32 < NP && nzn[lane + 32] > 0);
-            const unsigned below = (1u << lane) - 1u;
-            if (b0 >> lane & 1u) act[__popc(b0 & below)] = lane;
-            if (b1 >> lane & 1u) act[__popc(b0) + __popc(b1 & below)] = lane + 32;
-            if (lane == 0) nact = __popc(b0) + __popc(b1);
-        }
-        __syncthreads();
-        // the upper triangle of the active block, each entry (and its mirror) by one thread
-        const int na = nact, npair = na * (na + 1) / 2;
-        for (int q = t; q < npair; q += blockDim.x) {
-            const int a = pkq[q] >> 8, b = pkq[q] & 255;   // b <= a
-            const int i = act[a], j = act[b];
-            double h = 0.0;
-            for (int u = 0; u < nzn[i]; ++u)
-                for (int v = 0; v < nzn[j]; ++v)
-                    h += nzv[i][u] * Hy[nzy[i][u]][nzy[j][v]] * nzv[j][v];
-            // second derivatives of log E[l] and log E[l^2] (linear in the brightness
-            // parameters, so only their products appear): w (dm)(dm)'
-            for (int ty = 0; ty < 2; ++ty)
-                h += wd[ty] * bd[ty][0][i] * bd[ty][0][j] + we[ty] * bd[ty][1][i] * bd[ty][1][j];
-            if (i >= P_AXIS && i <= P_SCALE && j >= P_AXIS && j <= P_SCALE)
-                h += S2[i - P_AXIS][j - P_AXIS];
-            Hacc[i * NP + j] += h;
-            if (i != j) Hacc[j * NP + i] += h;
+            __syncwarp();
         }
     }
     __syncthreads();
+    // the band's warps together, in order
+    for (int i = t; i < 5 * HV; i += FH_THREADS)
+#pragma unroll
+        for (int h = 1; h < FH_SPLIT; ++h) acc[i / HV][i % HV] += acc[i / HV + 5 * h][i % HV];
+    __syncthreads();
+    auto band_sum = [&](int col, int i, int j) {
+        double h = 0.0;
+#pragma unroll
+        for (int b = 0; b < 5; ++b) {
+            const int f = w_factor(b, i) * w_factor(b, j);
+            if (f != 0) h += f > 0 ? acc[b][col] : -acc[b][col];
+        }
+        return h;
+    };
     double* Ho = hess_out + (size_t)NP * NP * s;
-    for (int idx = t; idx < NP * NP; idx += blockDim.x) Ho[idx] = Hacc[idx] - klH[idx];
-    if (t < NP && grad_out) grad_out[(size_t)NP * s + t] = gacc - klg[t];
-    if (t == 0) {
-        kl_out[s] = klv;
-        if (local_out) local_out[s] = lacc - klv;
+    for (int q = t; q < NPIXH; q += FH_THREADS) {
+        const int i = g_pix.v[q] >> 8, j = g_pix.v[q] & 255;   // j <= i
+        const int wi = w_of_param(i), wj = w_of_param(j);
+        const double h = Ho[i * NP + j] + band_sum(1 + NY + P2(wi, wj), i, j);
+        Ho[i * NP + j] = h;
+        if (i != j) Ho[j * NP + i] = h;
+    }
+    if (t < NP && grad_out)
+        grad_out[(size_t)NP * s + t] =
+            (t < NPIX ? band_sum(1 + w_of_param(t), t, P_U) : 0.0) - rec[HR_KLG + t];
+    if (t == 0 && local_out) {
+        double l = 0.0;
+        for (int b = 0; b < 5; ++b) l += acc[b][0];
+        local_out[s] = l - rec[HR_KL];
     }
 }
 
 template <class R>
-static cudaError_t hess_pixels(const DevProblem& P, const R* tbl, cudaStream_t st) {
-    k_hess<R><<<P.n_item, CHUNK, HessLay<R>::bytes, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.pixels, P.sky_map, tbl,
-                                              P.single, (const R*)P.emap, (const R*)P.vmap, P.item_part, P.src_active);
+static cudaError_t hess_pixels(const DevProblem& P, const R* tbl, const double* d_theta, double* d_hess,
+                               cudaStream_t st) {
+    const SourceTerms src{P.n_src, d_theta, P.model, P.hsrc, P.kl, d_hess, P.status};
+    const int grid = P.n_item + (P.n_src + TERM_SRC - 1) / TERM_SRC;
+    if (grid == 0) return cudaSuccess;
+    k_hess<R><<<grid, CHUNK, HessLay<R>::bytes, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.pixels, P.sky_map,
+                                                      tbl, P.single, (const R*)P.emap, (const R*)P.vmap, P.item_part,
+                                                      P.src_active, src);
     return cudaGetLastError();
 }
 
@@ -1012,17 +1099,17 @@ cudaError_t prime_hess_kernels() {
     return e;
 }
 
-cudaError_t launch_hess_pixels(const DevProblem& P, int precision, cudaStream_t st) {
-    if (P.n_item == 0) return cudaSuccess;
-    return precision == CELESTE_FP64 ? hess_pixels<double>(P, P.tbl64, st) : hess_pixels<float>(P, P.tbl32, st);
+cudaError_t launch_hess_pixels(const DevProblem& P, int precision, const double* d_theta, double* d_hess,
+                               cudaStream_t st) {
+    return precision == CELESTE_FP64 ? hess_pixels<double>(P, P.tbl64, d_theta, d_hess, st)
+                                     : hess_pixels<float>(P, P.tbl32, d_theta, d_hess, st);
 }
 
-cudaError_t launch_finalize_hess(const DevProblem& P, const double* d_theta, double* d_local,
-                                 double* d_grad, double* d_hess, cudaStream_t st) {
+cudaError_t launch_finalize_hess(const DevProblem& P, double* d_local, double* d_grad, double* d_hess,
+                                 cudaStream_t st) {
     if (P.n_src == 0) return cudaSuccess;
-    k_finalize_hess<<<P.n_src, FH_THREADS, 0, st>>>(P.n_src, d_theta, P.geo, P.patch_off, P.img,
-                                                    P.model, P.item_part, P.kl, d_local, d_grad,
-                                                    d_hess, P.status, P.src_active);
+    k_finalize_hess<<<P.n_src, FH_THREADS, 0, st>>>(P.n_src, P.geo, P.patch_off, P.img, P.item_part, P.hsrc, d_local,
+                                                    d_grad, d_hess, P.src_active);
     return cudaGetLastError();
 }
 

@@ -50,6 +50,9 @@ constexpr int NPART = 1 + NY + NYH;
 // item's pixels, [1] ll of the pixels the item owns (its share of the total), [2 .. 2 + NP)
 // d ll / d theta of its source (the patch's chain rule applied per item).
 constexpr int ZPCOLS = 2 + NP;
+// A source's record in the Hessian pass (doubles; hess_kernels.cu): KL, its gradient, the bands'
+// brightness moments, the world-frame shape derivatives
+constexpr int HREC = 102;
 
 // Mixture table of one (source, patch), in units of the pixel precision R:
 //   header [0..7]: a0 a1 E[l|star] E[l^2|star] E[l|gal] E[l^2|gal] iota 0
@@ -295,6 +298,7 @@ struct DevProblem {
     double* kl;
     double* kl_grad;         // [n_src][44] KL gradient, written by k_prep (nullable: no KL in prep)
     double* src_total;       // [n_src] each source's share of the total ELBO (k_finalize)
+    double* hsrc;            // [n_src][HREC] the Hessian pass's parameter-only terms
     int32_t* done;           // k_finalize completion counter, 0 between launches
     double* tot_part;        // [64] k_total slice sums
     int32_t* tot_done;       // k_total completion counter, 0 between launches
@@ -404,7 +408,12 @@ cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStr
                                double* d_local, double* d_grad, double* d_total);
 cudaError_t launch_gather(const DevProblem& P, int precision, cudaStream_t st);
 cudaError_t launch_adjoint(const DevProblem& P, int precision, int mode, cudaStream_t st);
-cudaError_t launch_hess_pixels(const DevProblem& P, int precision, cudaStream_t st);
+// the Hessian's pixel sums, and the sources' terms that do not depend on the pixels (P.hsrc,
+// P.kl, -KL'' into d_hess); launch_finalize_hess then adds the pixel part
+cudaError_t launch_hess_pixels(const DevProblem& P, int precision, const double* d_theta, double* d_hess,
+                               cudaStream_t st);
+cudaError_t launch_finalize_hess(const DevProblem& P, double* d_local, double* d_grad, double* d_hess,
+                                 cudaStream_t st);
 cudaError_t launch_finalize(const DevProblem& P, const double* d_theta, int precision, int mode,
                             double* d_total, double* d_local, double* d_grad, double* d_hess,
                             cudaStream_t st);

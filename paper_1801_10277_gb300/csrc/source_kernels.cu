@@ -31,9 +31,6 @@ k_total(const double* __restrict__ tile_ll, int n_tile, const double* __restrict
     total_reduce(tile_ll, n_tile, item_ll, n_item, kl, n_src, part, done, out);
 }
 
-cudaError_t launch_finalize_hess(const DevProblem& P, const double* d_theta, double* d_local,
-                                 double* d_grad, double* d_hess, cudaStream_t st);
-
 // total = tile ll sums + item ll sums - KL (fixed order, TOTAL_CTAS slices)
 cudaError_t launch_total(const DevProblem& P, double* d_total, cudaStream_t st) {
     k_total<<<TOTAL_CTAS, TOTAL_THREADS, 0, st>>>(P.tile_ll, P.n_tile, P.item_ll,
@@ -46,7 +43,7 @@ cudaError_t launch_finalize(const DevProblem& P, const double* d_theta, int prec
                             double* d_total, double* d_local, double* d_grad, double* d_hess,
                             cudaStream_t st) {
     if (mode == MODE_HESS) {
-        cudaError_t e = launch_finalize_hess(P, d_theta, d_local, d_grad, d_hess, st);
+        cudaError_t e = launch_finalize_hess(P, d_local, d_grad, d_hess, st);
         if (e != cudaSuccess) return e;
     } else if (P.n_src > 0) {
         // the KL value and gradient come from k_prep of the same theta
