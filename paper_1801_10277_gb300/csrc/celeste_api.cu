@@ -841,7 +841,7 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     if ((st = dalloc(pr, &P.spE2, sizeof(double) * (size_t)n_sp))) return bail(st);
     if ((st = dalloc(pr, &P.emap, sizeof(double) * (size_t)n_px))) return bail(st);
     if ((st = dalloc(pr, &P.vmap, sizeof(double) * (size_t)n_px))) return bail(st);
-    if ((st = dalloc(pr, &p, sizeof(double) * NPART * (size_t)P.n_item))) return bail(st);
+    if ((st = dalloc(pr, &p, sizeof(double) * ITEM_PART * (size_t)P.n_item))) return bail(st);
     P.item_part = (double*)p;
     if ((st = dalloc(pr, &p, sizeof(double) * (size_t)P.n_tile))) return bail(st);
     P.tile_ll = (double*)p;

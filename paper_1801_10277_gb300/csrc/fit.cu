@@ -1095,7 +1095,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
     FIT_CUDA(mem.alloc(&d_h, maxB * NP * NP));
     FIT_CUDA(mem.alloc(&d_kl, maxB));
     FIT_CUDA(mem.alloc(&d_hsrc, maxB * HREC));
-    FIT_CUDA(mem.alloc(&d_part, maxI * NPART));
+    FIT_CUDA(mem.alloc(&d_part, maxI * ITEM_PART));
     FIT_CUDA(mem.alloc(&d_dll, maxI));
     FIT_CUDA(mem.alloc(&d_tbl64, maxP * TBL_STRIDE));
     FIT_CUDA(mem.alloc(&d_tbl32, maxP * TBL_STRIDE));

@@ -1,17 +1,22 @@
 // Per-source exact Hessians (Section IV-D: Newton steps need the exact 44 x 44
 // Hessian of each source's block).
 //
-//   k_hess           per work item: value, gradient and Hessian of the pixel terms
-//                    wrt the twelve intermediate variables y of the (source, patch);
+//   k_hess           per part of a work item: value, gradient and Hessian of the pixel
+//                    terms wrt ten intermediate variables z of the (source, patch);
 //                    the mixture terms are recomputed here, nothing is stored.  Its first
 //                    CTAs take the sources' KL terms and parameter-only derivatives.
-//   k_finalize_hess  one CTA per source: chain rule y -> theta over the source's patches,
+//   k_finalize_hess  one CTA per source: chain rule z -> theta over the source's patches,
 //                    added to the KL Hessian; the full symmetric 44 x 44 matrix, the
 //                    gradient and the local objective.
 //
-// With e = dE_s/dy, v = dVar_s/dy = dE2_s/dy - 2 E_s e and the second derivatives
-// DE = d2E_s/dy2, DE2 = d2E2_s/dy2 (E2_s = sum_i a_i iota^2 E[l_i^2] g_i^2):
-//   d2 ll/dy2 = (h_EE - 2 c_V) e e' + h_EV (e v' + v e') + (c_E - 2 c_V E_s) DE + c_V DE2
+// The pixel terms depend on theta through ten variables z of the (source, patch): with
+// k_i = a_i iota E[l_i] and q_i = a_i iota^2 E[l_i^2] (i = star, galaxy),
+//   E_s = k_0 g_0 + k_1 g_1,  E2_s = q_0 g_0^2 + q_1 g_1^2,  Var_s = E2_s - E_s^2,
+// z = (k_0, k_1, q_0, q_1, the mean, e_dev, G).  (The twelve y of the gradient passes hold
+// a_i, E[l_i] and E[l_i^2] apart: their rows of the Hessian are multiples of each other.)
+// With e = dE_s/dz, v = dVar_s/dz = dE2_s/dz - 2 E_s e and the second derivatives
+// DE = d2E_s/dz2, DE2 = d2E2_s/dz2:
+//   d2 ll/dz2 = (h_EE - 2 c_V) e e' + h_EV (e v' + v e') + (c_E - 2 c_V E_s) DE + c_V DE2
 //   h_EE = -x (1/E^2 + 3 Var/E^4),  h_EV = x / E^3,  h_VV = 0.
 // Per Gaussian component N (log-density derivatives, q = P d, C = Sigma_psf + nu G):
 //   dlogN/dmu = q,  d2logN/dmu2 = -P,
@@ -29,30 +34,35 @@ namespace cel {
 
 namespace {
 
-__device__ __forceinline__ float ex2h(float x) { return exp2f(x); }
+// 2^x on the SFU (results below 2^-126 become 0)
+__device__ __forceinline__ float ex2h(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ float lgh(float x) { return logf(x); }
 __device__ __forceinline__ double lgh(double x) { return log(x); }
 
 constexpr double LOG2E_H = 1.4426950408889634;   // log2(e)
 
-// packed index of the symmetric 12 x 12 (a <= b not required)
-__device__ __forceinline__ int P2(int a, int b) { return a <= b ? yh_index(a, b) : yh_index(b, a); }
+// packed index of a symmetric N x N (upper triangle by rows; a <= b not required)
+template <int N>
+__host__ __device__ __forceinline__ constexpr int sym(int a, int b) {
+    return a <= b ? a * N - a * (a - 1) / 2 + b - a : b * N - b * (b - 1) / 2 + a - b;
+}
 
 }  // namespace
 
-constexpr int HV = 1 + NY + NYH;   // values reduced per work item
-constexpr int HVP = 96;            // HV padded to three per lane
-static_assert(HV <= HVP && HVP == 3 * 32, "the reduce-scatter leaves three sums per lane");
-
-// Sums v over the warp's 32 lanes and leaves lane l holding the sums of entries
-// 3 l, 3 l + 1, 3 l + 2 in v[0..2].  Five halving steps: at the step on lane bit m the
-// two lanes that differ in m hold the same index range; the one with m set keeps the
-// upper half and adds its partner's upper half, the other keeps and adds the lower
-// half.  93 shuffles instead of 5 per entry.
+// Sums v[0 .. 64) over the warp's 32 lanes: lane l is left with the sums of entries 2 l,
+// 2 l + 1 in v[0], v[1].  Five halving steps: at the step on lane bit m the two lanes that
+// differ in m hold the same index range; the one with m set keeps the upper half and adds
+// its partner's upper half, the other keeps and adds the lower half.  62 shuffles instead
+// of 5 per entry.  v[64], v[65] are summed onto every lane.
+static_assert(HV == 66, "64 scattered sums and two");
 template <class R>
-__device__ __forceinline__ void warp_reduce_scatter(R (&v)[HVP], int lane) {
+__device__ __forceinline__ void warp_reduce_scatter(R (&v)[HV], int lane) {
 #pragma unroll
-    for (int m = 16, n = HVP; m > 0; m >>= 1, n >>= 1) {
+    for (int m = 16, n = 64; m > 0; m >>= 1, n >>= 1) {
         const bool up = (lane & m) != 0;
 #pragma unroll
         for (int i = 0; i < n / 2; ++i) {
@@ -60,6 +70,8 @@ __device__ __forceinline__ void warp_reduce_scatter(R (&v)[HVP], int lane) {
             const R keep = up ? v[i + n / 2] : v[i];
             v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
         }
+#pragma unroll
+        for (int i = 64; i < HV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], m);
     }
 }
 
@@ -96,12 +108,12 @@ constexpr int WS_N = 0,    // N
 // the exp components, then over the dev components, and forms the 35 once per (pixel, k).
 constexpr int BS_LL = 0, BS_C = 3, BS_D2 = 7, BS_D3 = 10, BS_D4 = 14, NBS = 19;
 constexpr int WROW = 40;   // a full row: exponent coefficients of z1^2, z2^2, constant; 35 weights; pad
-constexpr int BROW = 24;   // a kernel row: the exponent's three coefficients, 19 weights, pad
+constexpr int BROW = 24;   // a kernel row: the exponent's three coefficients, (FP32: a pad,) 19 weights, pad
 constexpr int WFR = 16;    // entries per k: T (row-major), K (3 x 3), g1, g2, pad
 // K[e][p] = (T E_e T')_p for the pixel-frame shape directions E_e = (xx, xy + yx, yy)
 // and the whitened pairs p = (11, 12, 22)
 constexpr int WF_K = 4, WF_G = 13;
-static_assert(3 + NWS <= WROW && 3 + NBS <= BROW && BROW % 4 == 0 && WFR % 4 == 0 && WF_G + 2 <= WFR,
+static_assert(3 + NWS <= WROW && 4 + NBS < BROW && BROW % 4 == 0 && WFR % 4 == 0 && WF_G + 2 <= WFR,
               "whitened rows are read as 16-byte vectors from a 16-byte aligned array");
 
 __host__ __device__ __forceinline__ int wpa(int p) { return p == 2 ? 1 : 0; }
@@ -199,11 +211,10 @@ __host__ __device__ __forceinline__ void base_row(R w, R nu, R l1, R l2, R* c) {
     monomials(w * nu * nu, l1, l2, 4, c + BS_D4);
 }
 
-// adds f times the sums over one group's components (b, at unit weight) to the 27 sums of
-// N and fe times them to the 8 e_dev sums
+// the sums of lower degree: A (3), B (2), L (2), N from the base sums
 template <class R>
-__host__ __device__ __forceinline__ void add_group(const R (&b)[NBS], R g1, R g2, R f, R fe, R (&s)[NWS]) {
-    R A[3], B[2], L[2];
+__host__ __device__ __forceinline__ void derived_sums(const R (&b)[NBS], R g1, R g2, R (&A)[3], R (&B)[2], R (&L)[2],
+                                                      R& N) {
     A[0] = b[BS_C] + g1 * b[BS_D3];
     A[1] = b[BS_C + 1] + g1 * b[BS_D3 + 1];
     A[2] = b[BS_C + 3] + g2 * b[BS_D3 + 3];
@@ -211,30 +222,49 @@ __host__ __device__ __forceinline__ void add_group(const R (&b)[NBS], R g1, R g2
     B[1] = A[2] + g2 * b[BS_D2 + 2];
     L[0] = b[BS_LL] + g1 * A[0];
     L[1] = b[BS_LL + 2] + g2 * A[2];
-    const R N = L[0] + g1 * B[0];
-    s[WS_N] += f * N;
-    s[WS_NE] += fe * N;
+    N = L[0] + g1 * B[0];
+}
+
+// the 35 sums from the base sums over the exp components and over the dev components (each
+// at unit e_dev weight): N's at weights 1 - e_dev and e_dev, the e_dev sums their difference
+template <class R>
+__host__ __device__ __forceinline__ void combine_groups(const R (&be)[NBS], const R (&bd)[NBS], R g1, R g2, R edev,
+                                                        R (&s)[NWS]) {
+    R c[NBS], A[3], B[2], L[2], N;
+    const R fe = (R)1 - edev;
+#pragma unroll
+    for (int i = 0; i < NBS; ++i) c[i] = fe * be[i] + edev * bd[i];
+    derived_sums(c, g1, g2, A, B, L, N);
+    s[WS_N] = N;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        s[WS_L + i] += f * L[i];
-        s[WS_LE + i] += fe * L[i];
-        s[WS_B + i] += f * B[i];
-        s[WS_BE + i] += fe * B[i];
+        s[WS_L + i] = L[i];
+        s[WS_B + i] = B[i];
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        s[WS_A + i] += f * A[i];
-        s[WS_AE + i] += fe * A[i];
-        s[WS_LL + i] += f * b[BS_LL + i];
-        s[WS_D2 + i] += f * b[BS_D2 + i];
+        s[WS_A + i] = A[i];
+        s[WS_LL + i] = c[BS_LL + i];
+        s[WS_D2 + i] = c[BS_D2 + i];
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        s[WS_C + i] += f * b[BS_C + i];
-        s[WS_D3 + i] += f * b[BS_D3 + i];
+        s[WS_C + i] = c[BS_C + i];
+        s[WS_D3 + i] = c[BS_D3 + i];
     }
 #pragma unroll
-    for (int i = 0; i < 5; ++i) s[WS_D4 + i] += f * b[BS_D4 + i];
+    for (int i = 0; i < 5; ++i) s[WS_D4 + i] = c[BS_D4 + i];
+#pragma unroll
+    for (int i = 0; i < NBS; ++i) c[i] = bd[i] - be[i];   // those that the e_dev sums need
+    derived_sums(c, g1, g2, A, B, L, N);
+    s[WS_NE] = N;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        s[WS_LE + i] = L[i];
+        s[WS_BE + i] = B[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) s[WS_AE + i] = A[i];
 }
 
 // adds PSF component k's galaxy terms at one pixel, from its 35 sums, to the pixel-frame
@@ -395,9 +425,10 @@ __host__ __device__ __forceinline__ double a_transform(const double* A, const do
 // k_hess (their FP64 latencies then pass behind the pixel work): the KL value, gradient and
 // Hessian, the brightness moments of the five bands and the world-frame shape derivatives.
 // hess_out receives -KL'' and zeros; the rest goes to the source's record.
-constexpr int HR_KL = 0, HR_KLG = 1, HR_MOM = HR_KLG + NP, HR_DW = HR_MOM + 20, HR_D2W = HR_DW + 9;
-static_assert(HR_D2W + 27 <= HREC && HREC % 2 == 0, "the source's record");
-constexpr int TERM_SRC = CHUNK / 64;   // sources per CTA: two warps each
+constexpr int HR_KL = 0, HR_KLG = 1, HR_MOM = HR_KLG + NP, HR_DW = HR_MOM + 20, HR_D2W = HR_DW + 9,
+              HR_A = HR_D2W + 27;
+static_assert(HR_A + 2 <= HREC && HREC % 2 == 0, "the source's record");
+constexpr int TERM_SRC = HCHUNK / 64;   // sources per CTA: two warps each
 
 struct SourceTerms {
     int n_src;
@@ -537,9 +568,9 @@ __device__ __forceinline__ void source_terms(const SourceTerms& a, int s0, const
     for (int u = 0; u < n; ++u) {
         if (src_active && !src_active[s0 + u]) continue;
         double* H = a.hess + (size_t)NP * NP * (s0 + u);   // the caller's: 8-byte aligned
-        for (int i = t; i < NP * NP; i += CHUNK) H[i] = 0.0;
+        for (int i = t; i < NP * NP; i += HCHUNK) H[i] = 0.0;
     }
-    for (int i = t; i < n * NP; i += CHUNK) {
+    for (int i = t; i < n * NP; i += HCHUNK) {
         sm[i] = a.theta[(size_t)NP * s0 + i];
         if (a.status) theta_domain_check(i % NP, sm[i], a.status);
     }
@@ -553,6 +584,7 @@ __device__ __forceinline__ void source_terms(const SourceTerms& a, int s0, const
         return;
     }
     if (lane < 10) band_moments(th, lane >> 1, lane & 1, rec[HR_MOM + 2 * lane], rec[HR_MOM + 2 * lane + 1]);
+    if (lane >= 30) rec[HR_A + lane - 30] = th[P_A + lane - 30];
     if (lane == 10) {
         double dW[3][3], d2W[3][3][3];
         shape_w_derivs(th, dW, d2W);
@@ -569,20 +601,20 @@ struct HessLay {
     static constexpr int fr = tbl + TBL_STRIDE * (int)sizeof(R);
     static constexpr int rows = fr + MAXPSF * WFR * (int)sizeof(R);
     static constexpr int rows_bytes = MAXPSF * MAXPROF * BROW * (int)sizeof(R);
-    static constexpr int red_bytes = (CHUNK / 32) * HV * 8;
+    static constexpr int red_bytes = (HCHUNK / 32) * HV * 8;
     static constexpr int tab = rows + (rows_bytes > red_bytes ? rows_bytes : red_bytes);
     static constexpr int bytes = tab + (sizeof(R) == 8 ? EX_N * 8 : 0);
     static_assert(fr % 16 == 0 && rows % 16 == 0 && tab % 16 == 0, "16-byte alignment");
 };
 
-// Per work item: the sums over its pixels of ll, d ll / d y and d2 ll / dy2.  The mixture in
+// Per part of a work item: the sums over its pixels of ll, d ll / d y and d2 ll / dy2.  The mixture in
 // the whitened frame (above); FP64 as in fp64_profile.cuh, E and Var of a singly covered
 // pixel (single, FP64 only) formed here, those of the others from the maps.
 // Bound by the FP32 or the FP64 pipe: 22 / 25 of its instructions per component, where the
 // 35 sums accumulated one by one took 38 (FP32: 500 sources, 909,100 source-pixels, 180 ->
 // 140 us) and the pixel-frame formulas about 140 (FP64: fp64_profile.cuh has the figures).
 template <class R>
-__global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ items,
+__global__ void __launch_bounds__(HCHUNK, sizeof(R) == 8 ? 2 : 4) k_hess(const WorkItem* __restrict__ items,
                                                 const PatchGeo* __restrict__ geo,
                                                 const ImgMeta* __restrict__ img, int nprof, int n_exp,
                                                 const float* __restrict__ pixels,
@@ -606,8 +638,11 @@ __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ ite
         source_terms(src, (int)blockIdx.x * TERM_SRC, src_active, reinterpret_cast<double*>(smem));
         return;
     }
-    const int item = (int)blockIdx.x - n_term_cta;
-    const WorkItem it = items[item];
+    // one HCHUNK-pixel part of an item
+    const int rec = (int)blockIdx.x - n_term_cta, sub = rec % HSPLIT * HCHUNK;
+    const WorkItem it = items[rec / HSPLIT];
+    const int n_px = it.n - sub;
+    if (n_px <= 0) return;
     const PatchGeo g = geo[it.patch];
     if (src_active && !src_active[g.src]) return;
     const ImgMeta& im = img[g.img];
@@ -652,15 +687,16 @@ __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ ite
         row[0] = DBL ? G[0] : (R)(-0.5 * LOG2E_H) * l1;
         row[1] = DBL ? G[1] : (R)(-0.5 * LOG2E_H) * l2;
         row[2] = DBL ? G[2] : G[3];
-        base_row(w, nu, l1, l2, row + 3);
-        row[3 + NBS] = row[4 + NBS] = 0;
+        constexpr int W0 = DBL ? 3 : 4;   // FP32: the weights on a 16-byte boundary
+        base_row(w, nu, l1, l2, row + W0);
+        row[W0 + NBS] = 0;
     }
     __syncthreads();
     R out[HV];
 #pragma unroll
     for (int i = 0; i < HV; ++i) out[i] = 0;
-    if (t < it.n) {
-        const int q = it.q0 + t;
+    if (t < n_px) {
+        const int q = it.q0 + sub + t;
         const int yy = q / g.w, xx = q - yy * g.w;
         // star: value, gradient (mx, my), Hessian (xx, xy, yy)
         R g0 = 0, d0[2] = {0, 0}, h0[3] = {0, 0, 0};
@@ -706,18 +742,13 @@ __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ ite
                 h0[1] += n * (qx * qy - pxy);
                 h0[2] += n * (qy * qy - pyy);
             }
-            R s[NWS];
-#pragma unroll
-            for (int m = 0; m < NWS; ++m) s[m] = 0;
             const R* row = rows + k * nprof * BROW;
-            // the exp components at weight 1 - e_dev, then the dev components at e_dev
-            auto group = [&](int n, R f, R fe) {
-                R b[NBS];
+            auto group = [&](int n, R (&b)[NBS]) {
+                if constexpr (DBL) {
 #pragma unroll
-                for (int m = 0; m < NBS; ++m) b[m] = 0;
-                for (int j = 0; j < n; ++j, row += BROW) {
-                    R cw[BROW], e;
-                    if constexpr (DBL) {
+                    for (int m = 0; m < NBS; ++m) b[m] = 0;
+                    for (int j = 0; j < n; ++j, row += BROW) {
+                        double cw[BROW];
 #pragma unroll
                         for (int u = 0; u < (3 + NBS + 1) / 2; ++u) {
                             const double2 v = reinterpret_cast<const double2*>(row)[u];
@@ -725,33 +756,43 @@ __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ ite
                             cw[2 * u + 1] = v.y;
                         }
                         const float2 ab = as_float2(cw[2]);
-                        e = ex2_quad(cw[0], z1s, cw[1], z2s, ab.x, f1, ab.y, f2, tab);
-                    } else {
+                        const double e = ex2_quad(cw[0], z1s, cw[1], z2s, ab.x, f1, ab.y, f2, tab);
 #pragma unroll
-                        for (int u = 0; u < (3 + NBS + 3) / 4; ++u) {
-                            const float4 v = reinterpret_cast<const float4*>(row)[u];
-                            cw[4 * u] = v.x;
-                            cw[4 * u + 1] = v.y;
-                            cw[4 * u + 2] = v.z;
-                            cw[4 * u + 3] = v.w;
+                        for (int m = 0; m < NBS; ++m) b[m] += e * cw[3 + m];
+                    }
+                } else {
+                    // packed FP32x2: the 19 weights as ten pairs (half the issue slots)
+                    constexpr int NPR = (NBS + 1) / 2;
+                    float2 bb[NPR];
+#pragma unroll
+                    for (int m = 0; m < NPR; ++m) bb[m] = make_float2(0.f, 0.f);
+                    for (int j = 0; j < n; ++j, row += BROW) {
+                        float4 cw[BROW / 4];
+#pragma unroll
+                        for (int u = 0; u < BROW / 4; ++u) cw[u] = reinterpret_cast<const float4*>(row)[u];
+                        const float e = ex2h(fmaf(cw[0].x, z1s, fmaf(cw[0].y, z2s, cw[0].z)));
+                        const float2 ee = make_float2(e, e);
+#pragma unroll
+                        for (int m = 0; m < NPR; ++m) {
+                            const float4 w = cw[1 + m / 2];
+                            bb[m] = __ffma2_rn(ee, m & 1 ? make_float2(w.z, w.w) : make_float2(w.x, w.y), bb[m]);
                         }
-                        e = ex2h(fmaf(cw[0], z1s, fmaf(cw[1], z2s, cw[2])));
                     }
 #pragma unroll
-                    for (int m = 0; m < NBS; ++m) b[m] += e * cw[3 + m];
+                    for (int m = 0; m < NBS; ++m) b[m] = m & 1 ? bb[m / 2].y : bb[m / 2].x;
                 }
-                add_group(b, fr[WF_G], fr[WF_G + 1], f, fe, s);
             };
-            group(n_exp, (R)1 - edev, (R)-1);
-            group(nprof - n_exp, edev, (R)1);
+            R be[NBS], bd[NBS], s[NWS];
+            group(n_exp, be);
+            group(nprof - n_exp, bd);
+            combine_groups(be, bd, fr[WF_G], fr[WF_G + 1], edev, s);
             whitened_add(s, z1, z2, fr, g1, d1, de, h1, he);
         }
         // ---- E, Var and the pixel's weights
         const R iota = sT[H_IOTA], a0 = sT[H_A0], a1 = sT[H_A1];
-        const R el0 = sT[H_EL0], el20 = sT[H_EL20], el1 = sT[H_EL1], el21 = sT[H_EL21];
-        const R i2 = iota * iota;
-        const R f0 = iota * el0 * g0, f1 = iota * el1 * g1;
-        const R Es = a0 * f0 + a1 * f1;
+        const R k0 = a0 * iota * sT[H_EL0], k1 = a1 * iota * sT[H_EL1];
+        const R q0 = a0 * iota * iota * sT[H_EL20], q1 = a1 * iota * iota * sT[H_EL21];
+        const R Es = k0 * g0 + k1 * g1;
         const int64_t m = im.px_off + (int64_t)(g.y0 + yy) * im.W + (g.x0 + xx);
         const R x = (R)pixels[m];
         R E, V;
@@ -772,101 +813,84 @@ __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ ite
         const R hEE = -x * iE2 * ((R)1 + (R)3 * V * iE2);
         const R hEV = x * iE2 * iE;
         out[0] = x * (lgh(E) - (R)0.5 * V * iE2) - E;
-        // ---- assemble the pixel's y-derivatives (entries known to be zero are left out: a
+        // ---- assemble the pixel's z-derivatives (entries known to be zero are left out: a
         // product with a constant 0 would be computed)
         const R w1 = cE - (R)2 * cV * Es, w2 = cV;
-        // gradient of g_1 over y (index 6..11); g_0's is (d0[0], d0[1], 0, 0, 0, 0)
+        // gradient of g_1 over (mx, my, e_dev, Gxx, Gxy, Gyy); g_0's is (d0[0], d0[1], 0, 0, 0, 0)
         const R dg1[6] = {d1[0], d1[1], de, d1[2], d1[3], d1[4]};
-        // e = dE_s/dy (0 for Y_EL20, Y_EL21), v2 = dE2_s/dy (0 for Y_EL0, Y_EL1)
-        R e[NY], v2[NY];
-        const R g00 = i2 * g0 * g0, g11 = i2 * g1 * g1;
-        e[Y_A0] = f0;
-        e[Y_A1] = f1;
-        e[Y_EL0] = a0 * iota * g0;
-        e[Y_EL1] = a1 * iota * g1;
-        v2[Y_A0] = el20 * g00;
-        v2[Y_A1] = el21 * g11;
-        v2[Y_EL20] = a0 * g00;
-        v2[Y_EL21] = a1 * g11;
-        const R k0 = a0 * iota * el0, k1 = a1 * iota * el1;
-        const R m0 = (R)2 * a0 * i2 * el20, m1 = (R)2 * a1 * i2 * el21;
-        const R n0 = m0 * g0, n1 = m1 * g1;
+        // e = dE_s/dz (0 for q), v2 = dE2_s/dz (0 for k)
+        R e[NZ], v2[NZ];
+        e[Z_K0] = g0;
+        e[Z_K1] = g1;
+        v2[Z_Q0] = g0 * g0;
+        v2[Z_Q1] = g1 * g1;
+        const R m0 = (R)2 * q0, m1 = (R)2 * q1, n0 = m0 * g0, n1 = m1 * g1;
 #pragma unroll
         for (int z = 0; z < 6; ++z) {
-            e[Y_MX + z] = k1 * dg1[z];
-            v2[Y_MX + z] = n1 * dg1[z];
+            e[Z_MX + z] = k1 * dg1[z];
+            v2[Z_MX + z] = n1 * dg1[z];
             if (z < 2) {
-                e[Y_MX + z] += k0 * d0[z];
-                v2[Y_MX + z] += n0 * d0[z];
+                e[Z_MX + z] += k0 * d0[z];
+                v2[Z_MX + z] += n0 * d0[z];
             }
         }
-        auto has_e = [](int y) { return y != Y_EL20 && y != Y_EL21; };
-        auto has_v2 = [](int y) { return y != Y_EL0 && y != Y_EL1; };
+        auto has_e = [](int z) { return z != Z_Q0 && z != Z_Q1; };
+        auto has_v2 = [](int z) { return z != Z_K0 && z != Z_K1; };
         // gradient, and the outer-product part of the Hessian: with v = v2 - 2 E_s e,
         //   (h_EE - 2 c_V) e e' + h_EV (e v' + v e') = e p' + p e',
         //   p = (h_EE / 2 - c_V - 2 h_EV E_s) e + h_EV v2
         const R c1 = (R)0.5 * hEE - cV - (R)2 * hEV * Es;
-        R pv[NY];
+        R pv[NZ];
 #pragma unroll
-        for (int y = 0; y < NY; ++y) {
-            if (!has_e(y)) {
-                out[1 + y] = w2 * v2[y];
-                pv[y] = hEV * v2[y];
-            } else if (!has_v2(y)) {
-                out[1 + y] = w1 * e[y];
-                pv[y] = c1 * e[y];
+        for (int z = 0; z < NZ; ++z) {
+            if (!has_e(z)) {
+                out[1 + z] = w2 * v2[z];
+                pv[z] = hEV * v2[z];
+            } else if (!has_v2(z)) {
+                out[1 + z] = w1 * e[z];
+                pv[z] = c1 * e[z];
             } else {
-                out[1 + y] = w1 * e[y] + w2 * v2[y];
-                pv[y] = c1 * e[y] + hEV * v2[y];
+                out[1 + z] = w1 * e[z] + w2 * v2[z];
+                pv[z] = c1 * e[z] + hEV * v2[z];
             }
         }
-        R* H = out + 1 + NY;
+        R* H = out + 1 + NZ;
 #pragma unroll
-        for (int a = 0; a < NY; ++a)
+        for (int a = 0; a < NZ; ++a)
 #pragma unroll
-            for (int b = a; b < NY; ++b) {
+            for (int b = a; b < NZ; ++b) {
                 R h = 0;
                 if (has_e(a) && has_e(b)) h = e[a] * pv[b] + pv[a] * e[b];
                 else if (has_e(a)) h = e[a] * pv[b];
                 else if (has_e(b)) h = pv[a] * e[b];
-                H[yh_index(a, b)] = h;
+                H[sym<NZ>(a, b)] = h;
             }
         // second-derivative part  w1 DE + w2 DE2
-        H[P2(Y_A0, Y_EL0)] += w1 * iota * g0;
-        H[P2(Y_A1, Y_EL1)] += w1 * iota * g1;
-        H[P2(Y_A0, Y_EL20)] += w2 * g00;
-        H[P2(Y_A1, Y_EL21)] += w2 * g11;
-        const R p0 = w1 * iota * el0 + (R)2 * w2 * i2 * el20 * g0;
-        const R p1 = w1 * iota * el1 + (R)2 * w2 * i2 * el21 * g1;
-        const R u0 = a0 * p0, u1 = a1 * p1;
         const R b0 = w2 * m0, b1 = w2 * m1;
-        const R l0 = w1 * a0 * iota, l1 = w1 * a1 * iota;
-        const R r0 = w2 * (R)2 * a0 * i2 * g0, r1 = w2 * (R)2 * a1 * i2 * g1;
+        const R u0 = w1 * k0 + b0 * g0, u1 = w1 * k1 + b1 * g1;
+        const R r0 = (R)2 * w2 * g0, r1 = (R)2 * w2 * g1;
         R bd1[6];
 #pragma unroll
         for (int z = 0; z < 6; ++z) {
-            const int yz = Y_MX + z;
-            H[P2(Y_A1, yz)] += p1 * dg1[z];
-            H[P2(Y_EL1, yz)] += l1 * dg1[z];
-            H[P2(Y_EL21, yz)] += r1 * dg1[z];
+            H[sym<NZ>(Z_K1, Z_MX + z)] += w1 * dg1[z];
+            H[sym<NZ>(Z_Q1, Z_MX + z)] += r1 * dg1[z];
             if (z < 2) {
-                H[P2(Y_A0, yz)] += p0 * d0[z];
-                H[P2(Y_EL0, yz)] += l0 * d0[z];
-                H[P2(Y_EL20, yz)] += r0 * d0[z];
+                H[sym<NZ>(Z_K0, Z_MX + z)] += w1 * d0[z];
+                H[sym<NZ>(Z_Q0, Z_MX + z)] += r0 * d0[z];
             }
             bd1[z] = b1 * dg1[z];
         }
-        // z-z block: u0 d2g0 + b0 dg0 dg0' + u1 d2g1 + b1 dg1 dg1'
-        // d2g1 over (mx, my, edev, Gxx, Gxy, Gyy) from h1 (z5 packed) and he (edev x z5;
-        // the e_dev diagonal is zero)
-        const int zmap[5] = {0, 1, 3, 4, 5};   // z5 position -> position among the six
+        // mean / shape block: u0 d2g0 + b0 dg0 dg0' + u1 d2g1 + b1 dg1 dg1', d2g1 over
+        // (mx, my, e_dev, Gxx, Gxy, Gyy) from h1 (packed without e_dev) and he (the e_dev row;
+        // its diagonal is zero)
+        const int zmap[5] = {0, 1, 3, 4, 5};   // position without e_dev -> position among the six
         {
             int c = 0;
 #pragma unroll
             for (int a = 0; a < 5; ++a) {
-                H[P2(Y_EDEV, Y_MX + zmap[a])] += u1 * he[a];
+                H[sym<NZ>(Z_ED, Z_MX + zmap[a])] += u1 * he[a];
 #pragma unroll
-                for (int b = a; b < 5; ++b, ++c) H[yh_index(Y_MX + zmap[a], Y_MX + zmap[b])] += u1 * h1[c];
+                for (int b = a; b < 5; ++b, ++c) H[sym<NZ>(Z_MX + zmap[a], Z_MX + zmap[b])] += u1 * h1[c];
             }
         }
 #pragma unroll
@@ -875,32 +899,29 @@ __global__ void __launch_bounds__(CHUNK) k_hess(const WorkItem* __restrict__ ite
             for (int b = a; b < 6; ++b) {
                 R v = bd1[a] * dg1[b];
                 if (a < 2 && b < 2) v += b0 * d0[a] * d0[b] + u0 * h0[a + b];
-                H[yh_index(Y_MX + a, Y_MX + b)] += v;
+                H[sym<NZ>(Z_MX + a, Z_MX + b)] += v;
             }
     }
     // ---- CTA reduction: in R within a warp (a reduce-scatter), FP64 across warps
     const int lane = t & 31, warp = t >> 5;
     double(*red)[HV] = reinterpret_cast<double(*)[HV]>(smem + Lay::rows);
-    R v[HVP];
-#pragma unroll
-    for (int i = 0; i < HVP; ++i) v[i] = i < HV ? out[i] : (R)0;
-    warp_reduce_scatter(v, lane);
+    warp_reduce_scatter(out, lane);
     __syncthreads();   // every warp is past its reads of the rows
-#pragma unroll
-    for (int u = 0; u < HVP / 32; ++u)
-        if (3 * lane + u < HV) red[warp][3 * lane + u] = (double)v[u];
+    red[warp][2 * lane] = (double)out[0];
+    red[warp][2 * lane + 1] = (double)out[1];
+    if (lane < HV - 64) red[warp][64 + lane] = (double)(lane == 0 ? out[64] : out[65]);
     __syncthreads();
     for (int i = t; i < HV; i += blockDim.x) {
         double s = 0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][i];
-        part[(size_t)item * NPART + i] = s;
+        part[(size_t)rec * HV + i] = s;
     }
 }
 
 // ---------------------------------------------------------------------------------
 // per-source chain rule
 
-// The chain rule goes through twelve variables w per (source, patch) that stand in the
+// The chain rule goes from z to twelve variables w per (source, patch) that stand in the
 // places of y: a_0, a_1, then per type i the mean m_i and variance v_i of the log brightness
 // in the patch's band (places Y_EL0, Y_EL20, Y_EL1, Y_EL21), u_0, u_1, e_dev, and e_axis,
 // e_angle, e_scale.  A parameter theta_j < P_K enters exactly one of them, with a factor of
@@ -923,7 +944,7 @@ __device__ __forceinline__ int w_factor(int band, int j) {
 }
 
 // One CTA per source, two warps per band: a warp takes every second patch of its band, adds
-// the 91 sums of the patch's items (item order), maps them to w (X = H_y J, then J' X, J at
+// the 66 sums of the patch's records (in order), maps them to w (X = H_z J, then J' X, J at
 // most three entries per column) and adds the result to the warp's shared accumulator; then
 // the block is spread and added to the -KL terms that source_terms left in hess_out.
 // Latency-bound, so the patches of a source run side by side and a patch costs about 50 FP64
@@ -942,17 +963,18 @@ k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __re
                 const int32_t* __restrict__ src_active) {
     const int s = blockIdx.x;
     if (s >= n_src || (src_active && !src_active[s])) return;
-    __shared__ double acc[FH_WARPS][HV];     // ll, d/dw, d2/dw2 (packed) of the warp's patches
+    constexpr int NACC = 1 + NY + NYH;
+    __shared__ double acc[FH_WARPS][NACC];   // ll, d/dw, d2/dw2 (packed) of the warp's patches
     __shared__ double rec[HREC];
-    __shared__ double sy[FH_WARPS][HV + 1];  // the patch's sums over y
-    __shared__ double sx[FH_WARPS][NY][NY];  // H_y J
+    __shared__ double sy[FH_WARPS][HV];      // the patch's sums over z
+    __shared__ double sx[FH_WARPS][NZ][NY];  // H_z J
     __shared__ double sj[FH_WARPS][NY][3];   // J: column w's entries ...
-    __shared__ uint8_t si[FH_WARPS][NY][3];  // ... and their y
+    __shared__ uint8_t si[FH_WARPS][NY][3];  // ... and their z
     __shared__ double sg[FH_WARPS][36];      // dG, d2G of the patch
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int band = warp % 5, half = warp / 5;
     for (int i = t; i < HREC; i += FH_THREADS) rec[i] = hsrc[(size_t)HREC * s + i];
-    for (int i = lane; i < HV; i += 32) acc[warp][i] = 0.0;
+    for (int i = lane; i < NACC; i += 32) acc[warp][i] = 0.0;
     __syncthreads();
     const int p0 = patch_off[s], p1 = patch_off[s + 1];
     int seen = 0;   // patches of this band so far
@@ -964,17 +986,18 @@ k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __re
             const int p = pb + __ffs(mine) - 1;
             const PatchGeo g = geo[p];
             const double* A = img[g.img].A;
-            // the patch's items in order, loaded four at a time before any is added
+            // the patch's records in order (items cut into HCHUNK-pixel parts, so one per HCHUNK
+            // pixels), loaded four at a time before any is added
             double v[3] = {0.0, 0.0, 0.0};
-            const int i1 = g.item0 + g.nitem;
-            for (int i0 = g.item0; i0 < i1; i0 += 4) {
+            const int r0 = g.item0 * HSPLIT, i1 = r0 + (g.w * g.h + HCHUNK - 1) / HCHUNK;
+            for (int i0 = r0; i0 < i1; i0 += 4) {
                 double x[4][3];
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
 #pragma unroll
                     for (int c = 0; c < 3; ++c)
                         x[u][c] = i0 + u < i1 && lane + 32 * c < HV
-                                      ? part[(size_t)(i0 + u) * NPART + lane + 32 * c] : 0.0;
+                                      ? part[(size_t)(i0 + u) * HV + lane + 32 * c] : 0.0;
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     if (i0 + u < i1)
@@ -988,41 +1011,49 @@ k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __re
             for (int c = 0; c < 3; ++c)
                 if (lane + 32 * c < HV) sy[warp][lane + 32 * c] = v[c];
             __syncwarp();
-            const double* m = rec + HR_MOM + 4 * band;   // E[l_0], E[l_0^2], E[l_1], E[l_1^2]
+            // iota E[l_i] and iota^2 E[l_i^2] of type i
+            const double iota = img[g.img].iota;
+            const double* mom = rec + HR_MOM + 4 * band;
+            const double m[4] = {iota * mom[0], iota * iota * mom[1], iota * mom[2], iota * iota * mom[3]};
+            const double* Gz = sy[warp] + 1;
+            const double* Hz = sy[warp] + 1 + NZ;
             if (lane < NY) {
                 const int w = lane;
-                int y0 = w, y1 = 0, y2 = 0;
+                int z0 = Z_ED, z1 = 0, z2 = 0;
                 double c0 = 1.0, c1 = 0.0, c2 = 0.0;
-                if (w >= Y_EL0 && w <= Y_EL21) {
-                    const int i = (w - Y_EL0) >> 1, var = (w - Y_EL0) & 1;
-                    y0 = Y_EL0 + 2 * i;
-                    y1 = y0 + 1;
-                    c0 = var ? 0.5 * m[2 * i] : m[2 * i];
-                    c1 = 2.0 * m[2 * i + 1];
+                if (w <= Y_EL21) {
+                    // k_i = a_i iota E[l_i], q_i = a_i iota^2 E[l_i^2] over a_i, m_i, v_i
+                    const int i = w == Y_A1 || w >= Y_EL1;
+                    z0 = Z_K0 + i;
+                    z1 = Z_Q0 + i;
+                    c0 = i ? m[2] : m[0];
+                    c1 = i ? m[3] : m[1];
+                    if (w >= Y_EL0) {
+                        c0 *= rec[HR_A + i] * ((w - Y_EL0) & 1 ? 0.5 : 1.0);
+                        c1 *= 2.0 * rec[HR_A + i];
+                    }
                 } else if (w == Y_MX || w == Y_MY) {
-                    y0 = Y_MX;
-                    y1 = Y_MY;
+                    z0 = Z_MX;
+                    z1 = Z_MY;
                     c0 = A[w - Y_MX];
                     c1 = A[2 + w - Y_MX];
                 } else if (w >= Y_GXX) {
                     const double* d = sg[warp] + 3 * (w - Y_GXX);
-                    y0 = Y_GXX; y1 = Y_GXY; y2 = Y_GYY;
+                    z0 = Z_GXX; z1 = Z_GXX + 1; z2 = Z_GXX + 2;
                     c0 = d[0]; c1 = d[1]; c2 = d[2];
                 }
                 sj[warp][w][0] = c0; sj[warp][w][1] = c1; sj[warp][w][2] = c2;
-                si[warp][w][0] = (uint8_t)y0; si[warp][w][1] = (uint8_t)y1; si[warp][w][2] = (uint8_t)y2;
-                acc[warp][1 + w] += c0 * sy[warp][1 + y0] + c1 * sy[warp][1 + y1] + c2 * sy[warp][1 + y2];
+                si[warp][w][0] = (uint8_t)z0; si[warp][w][1] = (uint8_t)z1; si[warp][w][2] = (uint8_t)z2;
+                acc[warp][1 + w] += c0 * Gz[z0] + c1 * Gz[z1] + c2 * Gz[z2];
             }
             if (lane == 0) acc[warp][0] += sy[warp][0];
             __syncwarp();
-            const double* Gy = sy[warp] + 1;
-            const double* Hy = sy[warp] + 1 + NY;
-            for (int i = lane; i < NY * NY; i += 32) {
-                const int y = i / NY, w = i % NY;
+            for (int i = lane; i < NZ * NY; i += 32) {
+                const int z = i / NY, w = i % NY;
                 double x = 0.0;
 #pragma unroll
-                for (int e = 0; e < 3; ++e) x += Hy[P2(y, si[warp][w][e])] * sj[warp][w][e];
-                sx[warp][y][w] = x;
+                for (int e = 0; e < 3; ++e) x += Hz[sym<NZ>(z, si[warp][w][e])] * sj[warp][w][e];
+                sx[warp][z][w] = x;
             }
             __syncwarp();
             for (int i = lane; i < NYH; i += 32) {
@@ -1030,14 +1061,20 @@ k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __re
                 double h = 0.0;
 #pragma unroll
                 for (int e = 0; e < 3; ++e) h += sj[warp][a][e] * sx[warp][si[warp][a][e]][b];
-                // second derivatives of y over w: E[l] = e^{m + v/2}, E[l^2] = e^{2m + 2v} (type i), and G
-                if (a >= Y_EL0 && b <= Y_EL21 && (a - Y_EL0) >> 1 == (b - Y_EL0) >> 1) {
-                    const int k = (a - Y_EL0) & ~1;
-                    const double f = ((a - Y_EL0) & 1 ? 0.5 : 1.0) * ((b - Y_EL0) & 1 ? 0.5 : 1.0);
-                    h += f * m[k] * Gy[Y_EL0 + k] + 4.0 * m[k + 1] * Gy[Y_EL0 + k + 1];
+                // second derivatives of z over w: k = a iota e^{m + v/2}, q = a iota^2 e^{2m + 2v}, and G
+                const int ia = a == Y_A1 || a >= Y_EL1, ib = b == Y_A1 || b >= Y_EL1;
+                if (b <= Y_EL21 && b >= Y_EL0 && ia == ib) {
+                    const double Gk = Gz[Z_K0 + ia] * (ia ? m[2] : m[0]), Gq = Gz[Z_Q0 + ia] * (ia ? m[3] : m[1]);
+                    const double fb = (b - Y_EL0) & 1 ? 0.5 : 1.0;
+                    if (a >= Y_EL0) {
+                        const double fa = (a - Y_EL0) & 1 ? 0.5 : 1.0;
+                        h += rec[HR_A + ia] * (fa * fb * Gk + 4.0 * Gq);
+                    } else {
+                        h += fb * Gk + 2.0 * Gq;
+                    }
                 } else if (a >= Y_GXX) {
                     const double* d = sg[warp] + 9 + 9 * (a - Y_GXX) + 3 * (b - Y_GXX);
-                    h += Gy[Y_GXX] * d[0] + Gy[Y_GXY] * d[1] + Gy[Y_GYY] * d[2];
+                    h += Gz[Z_GXX] * d[0] + Gz[Z_GXX + 1] * d[1] + Gz[Z_GXX + 2] * d[2];
                 }
                 acc[warp][1 + NY + yh_index(a, b)] += h;
             }
@@ -1046,9 +1083,9 @@ k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __re
     }
     __syncthreads();
     // the band's warps together, in order
-    for (int i = t; i < 5 * HV; i += FH_THREADS)
+    for (int i = t; i < 5 * NACC; i += FH_THREADS)
 #pragma unroll
-        for (int h = 1; h < FH_SPLIT; ++h) acc[i / HV][i % HV] += acc[i / HV + 5 * h][i % HV];
+        for (int h = 1; h < FH_SPLIT; ++h) acc[i / NACC][i % NACC] += acc[i / NACC + 5 * h][i % NACC];
     __syncthreads();
     auto band_sum = [&](int col, int i, int j) {
         double h = 0.0;
@@ -1063,7 +1100,7 @@ k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __re
     for (int q = t; q < NPIXH; q += FH_THREADS) {
         const int i = g_pix.v[q] >> 8, j = g_pix.v[q] & 255;   // j <= i
         const int wi = w_of_param(i), wj = w_of_param(j);
-        const double h = Ho[i * NP + j] + band_sum(1 + NY + P2(wi, wj), i, j);
+        const double h = Ho[i * NP + j] + band_sum(1 + NY + sym<NY>(wi, wj), i, j);
         Ho[i * NP + j] = h;
         if (i != j) Ho[j * NP + i] = h;
     }
@@ -1081,9 +1118,9 @@ template <class R>
 static cudaError_t hess_pixels(const DevProblem& P, const R* tbl, const double* d_theta, double* d_hess,
                                cudaStream_t st) {
     const SourceTerms src{P.n_src, d_theta, P.model, P.hsrc, P.kl, d_hess, P.status};
-    const int grid = P.n_item + (P.n_src + TERM_SRC - 1) / TERM_SRC;
+    const int grid = P.n_item * HSPLIT + (P.n_src + TERM_SRC - 1) / TERM_SRC;
     if (grid == 0) return cudaSuccess;
-    k_hess<R><<<grid, CHUNK, HessLay<R>::bytes, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.pixels, P.sky_map,
+    k_hess<R><<<grid, HCHUNK, HessLay<R>::bytes, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.pixels, P.sky_map,
                                                       tbl, P.single, (const R*)P.emap, (const R*)P.vmap, P.item_part,
                                                       P.src_active, src);
     return cudaGetLastError();

@@ -41,18 +41,17 @@ enum : int { Y_A0 = 0, Y_A1, Y_EL0, Y_EL20, Y_EL1, Y_EL21, Y_MX, Y_MY, Y_EDEV, Y
              Y_GYY, NY };
 constexpr int NYH = NY * (NY + 1) / 2;   // packed upper triangle of the y-Hessian
 
-// Work-item partial record (doubles): [0] sum of ll over the item's pixels; gradient
-// mode: [1..44] gradient wrt theta (the chain rule applied per item); Hessian mode:
-// [1..NY] gradient wrt y, [1+NY ..) packed y-Hessian.
-constexpr int PART_LL = 0, PART_G = 1, PART_H = 1 + NY, PART_TH = 1;
-constexpr int NPART = 1 + NY + NYH;
+// Work-item partial record (doubles) of the FP64 value / gradient path: [0] sum of ll over
+// the item's pixels, [1..44] gradient wrt theta (the chain rule applied per item).
+constexpr int PART_LL = 0, PART_TH = 1;
+constexpr int NPART = 1 + NP;
 // Per-item partial record of the FP32 value / gradient kernel (doubles): [0] ll of the
 // item's pixels, [1] ll of the pixels the item owns (its share of the total), [2 .. 2 + NP)
 // d ll / d theta of its source (the patch's chain rule applied per item).
 constexpr int ZPCOLS = 2 + NP;
 // A source's record in the Hessian pass (doubles; hess_kernels.cu): KL, its gradient, the bands'
 // brightness moments, the world-frame shape derivatives
-constexpr int HREC = 102;
+constexpr int HREC = 104;
 
 // Mixture table of one (source, patch), in units of the pixel precision R:
 //   header [0..7]: a0 a1 E[l|star] E[l^2|star] E[l|gal] E[l^2|gal] iota 0
@@ -83,6 +82,15 @@ constexpr int H_A0 = 0, H_A1 = 1, H_EL0 = 2, H_EL20 = 3, H_EL1 = 4, H_EL21 = 5, 
 // component 12 + 12 per pair); each profile group padded to an even count
 constexpr int ZFULL_FLOATS = 16 + MAXPSF * (8 + ((MAXPROF + 2) / 2) * 8) + MAXPSF * (12 + ((MAXPROF + 2) / 2) * 12);
 constexpr int CHUNK = 256;   // pixels per work item (one CTA)
+// The Hessian pass takes an item in parts of HCHUNK pixels, a CTA and a record of item_part
+// each: its CTAs are heavy in registers, and small ones overlap one's set-up and reduction
+// with the others' pixels and even out the last wave.
+constexpr int HCHUNK = 128, HSPLIT = CHUNK / HCHUNK;
+// Its ten variables z per (source, patch) (hess_kernels.cu) and a part's record: ll, d/dz, the
+// packed upper triangle of d2/dz2
+enum : int { Z_K0 = 0, Z_K1, Z_Q0, Z_Q1, Z_MX, Z_MY, Z_ED, Z_GXX, Z_GXY, Z_GYY, NZ };
+constexpr int HV = 1 + NZ + NZ * (NZ + 1) / 2;
+constexpr int ITEM_PART = HSPLIT * HV > NPART ? HSPLIT * HV : NPART;   // doubles of item_part per item
 constexpr int ZIMAX = 512;   // most pixels per item of the FP32 value / gradient kernel
 constexpr int ZMAXC = 4;     // other covering patches named inline in such an item's queue record
 constexpr int ZSTAGE = 12;   // other covering patches whose value records an item stages (more are
