@@ -238,7 +238,7 @@ celeste_status run(celeste_problem* pr, const double* d_theta, int precision, in
         return CELESTE_OK;
     }
     // (the Hessian pass takes the KL terms itself)
-    CEL_CUDA(timed(pr, "prep", st, [&] { return launch_prep(P, d_theta, precision, st, mode != MODE_HESS); }));
+    CEL_CUDA(timed(pr, "prep", st, [&] { return launch_prep(P, d_theta, precision, st, mode != MODE_HESS, mode == MODE_HESS); }));
     CEL_CUDA(timed(pr, "contrib", st, [&] { return launch_contrib(P, precision, st, true); }));
     CEL_CUDA(timed(pr, "gather", st, [&] { return launch_gather(P, precision, st); }));
     if (mode == MODE_HESS)
@@ -455,6 +455,7 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     if (n_patch > 0 && !patches) return fail(CELESTE_ERR_ARG, "patches is null");
     std::vector<PatchGeo> geo(n_patch);
     std::vector<WorkItem> items;
+    std::vector<HItem> hitems;   // the Hessian pass's parts
     int64_t n_sp = 0;
     for (int s = 0; s < n_src; ++s)
         for (int p = patch_offsets[s]; p < patch_offsets[s + 1]; ++p) {
@@ -474,6 +475,8 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
             g.nitem = (int)items.size() - g.item0;
             n_sp += npx;
         }
+    const int hchunk = hess_chunk(n_sp, sm_count());
+    for (int p = 0; p < n_patch; ++p) push_parts(hitems, geo[p], p, im[geo[p].img], hchunk);
     // per-(source, pixel) flag: 1 when no other patch covers the pixel (those pixels are
     // finished by k_contrib; k_gather visits only cells that two or more patches touch)
     std::vector<uint8_t> single((size_t)n_sp, 0);
@@ -776,6 +779,11 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     if ((st = dupload(pr, &d_img, im.data(), im.size()))) return bail(st);
     if ((st = dupload(pr, &d_geo, geo.data(), geo.size()))) return bail(st);
     if ((st = dupload(pr, &d_items, items.data(), items.size()))) return bail(st);
+    HItem* d_hitems;
+    if ((st = dupload(pr, &d_hitems, hitems.data(), hitems.size()))) return bail(st);
+    P.hitems = d_hitems;
+    P.n_hitem = (int)hitems.size();
+    P.hchunk = hchunk;
     if ((st = dupload(pr, &d_tiles, tiles.data(), tiles.size()))) return bail(st);
     if ((st = dupload(pr, &d_tl, tile_list.data(), tile_list.size()))) return bail(st);
     if ((st = dupload(pr, &d_tg, tile_grid.data(), tile_grid.size()))) return bail(st);
@@ -841,7 +849,8 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     if ((st = dalloc(pr, &P.spE2, sizeof(double) * (size_t)n_sp))) return bail(st);
     if ((st = dalloc(pr, &P.emap, sizeof(double) * (size_t)n_px))) return bail(st);
     if ((st = dalloc(pr, &P.vmap, sizeof(double) * (size_t)n_px))) return bail(st);
-    if ((st = dalloc(pr, &p, sizeof(double) * ITEM_PART * (size_t)P.n_item))) return bail(st);
+    if ((st = dalloc(pr, &p, sizeof(double) * std::max(NPART * (size_t)P.n_item, HV * (size_t)P.n_hitem))))
+        return bail(st);
     P.item_part = (double*)p;
     if ((st = dalloc(pr, &p, sizeof(double) * (size_t)P.n_tile))) return bail(st);
     P.tile_ll = (double*)p;
@@ -866,6 +875,9 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     if (cudaMemset(P.tot_done, 0, sizeof(int32_t)) != cudaSuccess) return bail(fail(CELESTE_ERR_CUDA, "memset"));
     if ((st = dalloc(pr, &p, 2 * sizeof(int32_t)))) return bail(st);
     P.queue = (int32_t*)p;
+    if ((st = dalloc(pr, &p, 2 * sizeof(int32_t)))) return bail(st);
+    P.hqueue = (int32_t*)p;
+    if (cudaMemset(P.hqueue, 0, 2 * sizeof(int32_t)) != cudaSuccess) return bail(fail(CELESTE_ERR_CUDA, "memset"));
     prime_persistent_grids();
     {
         cudaError_t pe = prime_items_kernels();

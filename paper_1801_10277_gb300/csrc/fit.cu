@@ -850,7 +850,9 @@ struct Batch {
     std::vector<int32_t> patch_off;  // batch CSR
     std::vector<PatchGeo> geo;       // batch patches (src = batch index, sp_off batch-local)
     std::vector<WorkItem> items;     // patch = batch patch, src = GLOBAL id
+    std::vector<HItem> parts;        // the Hessian pass's, src = batch index
     int64_t n_sp = 0;
+    int hchunk = 0;                  // pixels of a part
 };
 
 Batch make_batch(const celeste_problem* pr, const std::vector<int32_t>& members) {
@@ -873,6 +875,9 @@ Batch make_batch(const celeste_problem* pr, const std::vector<int32_t>& members)
         }
         B.patch_off.push_back((int)B.geo.size());
     }
+    B.hchunk = hess_chunk(B.n_sp, sm_count());
+    for (int p = 0; p < (int)B.geo.size(); ++p)
+        push_parts(B.parts, B.geo[p], p, pr->imgs[B.geo[p].img], B.hchunk);
     return B;
 }
 
@@ -1016,27 +1021,30 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
     }
     // device buffers for the largest batch: a colour, or (Cyclades: at most one source
     // per component of a sample) the sample_size moving sources with the most work
-    size_t maxB = 1, maxP = 1, maxI = 1;
+    size_t maxB = 1, maxP = 1, maxI = 1, maxH = 1;   // sources, patches, items, Hessian parts
     int64_t maxSp = 1;
     if (!cyclades) {
         for (const Batch& B : colour_batches) {
             maxB = std::max(maxB, B.src.size());
             maxP = std::max(maxP, B.geo.size());
             maxI = std::max(maxI, B.items.size());
+            maxH = std::max(maxH, B.parts.size());
             maxSp = std::max(maxSp, B.n_sp);
         }
     } else {
-        std::vector<int64_t> np_, ni_, nsp_;
+        std::vector<int64_t> np_, ni_, nh_, nsp_;
         for (int s : moving) {
-            int64_t a = 0, b = 0, c = 0;
+            int64_t a = 0, b = 0, h = 0, c = 0;
             for (int p = pr->patch_off[s]; p < pr->patch_off[s + 1]; ++p) {
                 const int64_t npx = (int64_t)pr->geo[p].w * pr->geo[p].h;
                 ++a;
                 b += (npx + CHUNK - 1) / CHUNK;
+                h += (npx + 31) / 32;   // the smallest parts a batch may have
                 c += npx;
             }
             np_.push_back(a);
             ni_.push_back(b);
+            nh_.push_back(h);
             nsp_.push_back(c);
         }
         const size_t top = std::min<size_t>((size_t)opts->sample_size, moving.size());
@@ -1049,6 +1057,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
         maxB = std::max<size_t>(1, top);
         maxP = std::max<size_t>(1, (size_t)top_sum(np_));
         maxI = std::max<size_t>(1, (size_t)top_sum(ni_));
+        maxH = std::max<size_t>(1, (size_t)top_sum(nh_));
         maxSp = std::max<int64_t>(1, top_sum(nsp_));
     }
     // the batches of sweep g (counted over both precision phases)
@@ -1076,6 +1085,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
     int32_t *d_bsrc, *d_bpo, *d_active, *d_srcact;
     PatchGeo* d_bgeo;
     WorkItem* d_bitems;
+    HItem* d_bparts;
     double *d_bth, *d_bthc, *d_bt, *d_btc, *d_f, *d_g, *d_h, *d_kl, *d_hsrc, *d_part, *d_dll, *d_tbl64;
     float* d_tbl32;
     TrState* d_st;
@@ -1095,7 +1105,8 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
     FIT_CUDA(mem.alloc(&d_h, maxB * NP * NP));
     FIT_CUDA(mem.alloc(&d_kl, maxB));
     FIT_CUDA(mem.alloc(&d_hsrc, maxB * HREC));
-    FIT_CUDA(mem.alloc(&d_part, maxI * ITEM_PART));
+    FIT_CUDA(mem.alloc(&d_part, maxH * HV));
+    FIT_CUDA(mem.alloc(&d_bparts, maxH));
     FIT_CUDA(mem.alloc(&d_dll, maxI));
     FIT_CUDA(mem.alloc(&d_tbl64, maxP * TBL_STRIDE));
     FIT_CUDA(mem.alloc(&d_tbl32, maxP * TBL_STRIDE));
@@ -1167,6 +1178,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             FIT_CUDA(cudaMemcpyAsync(d_bpo, B.patch_off.data(), sizeof(int32_t) * (nb + 1), cudaMemcpyHostToDevice, st));
             FIT_CUDA(cudaMemcpyAsync(d_bgeo, B.geo.data(), sizeof(PatchGeo) * B.geo.size(), cudaMemcpyHostToDevice, st));
             FIT_CUDA(cudaMemcpyAsync(d_bitems, B.items.data(), sizeof(WorkItem) * B.items.size(), cudaMemcpyHostToDevice, st));
+            FIT_CUDA(cudaMemcpyAsync(d_bparts, B.parts.data(), sizeof(HItem) * B.parts.size(), cudaMemcpyHostToDevice, st));
             const int nI = (int)B.items.size();
             if (nI > 0) {
                 if (prec == CELESTE_FP64)
@@ -1195,6 +1207,9 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             Pb.n_sp = B.n_sp;
             Pb.geo = d_bgeo;
             Pb.items = d_bitems;
+            Pb.hitems = d_bparts;
+            Pb.n_hitem = (int)B.parts.size();
+            Pb.hchunk = B.hchunk;
             Pb.patch_off = d_bpo;
             Pb.tbl64 = d_tbl64;
             Pb.tbl32 = d_tbl32;
@@ -1221,7 +1236,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
                 if (ce == cudaSuccess && e != cudaSuccess) ce = e;
             };
             chk(cudaMemsetAsync(d_active, 0, sizeof(int32_t), st));
-            chk(launch_prep(Pb, d_bth, prec, st));
+            chk(launch_prep(Pb, d_bth, prec, st, true, true));
             chk(launch_contrib(Pb, prec, st));
             if (nI > 0) {
                 if (prec == CELESTE_FP64)

@@ -18,7 +18,7 @@
 // Measured (500 sources, 909,100 source-pixels): the adjoint 3.64 -> 1.51 ms, about 800 FP64
 // instructions per warp, which is the pipe's rate; the map pass, now at the 59,000 multiply
 // covered pixels alone, 2.13 -> 0.14 ms; the Hessian pass of 64 crowded sources (118,800
-// source-pixels) 1.53 -> 0.70 ms.  Error of the gradient against 64-bit autograd unchanged.
+// source-pixels) 1.53 -> 0.58 ms.  Error of the gradient against 64-bit autograd unchanged.
 #pragma once
 
 #include "internal.cuh"

@@ -24,11 +24,14 @@
 //   d2logN/dC[E]dC[F] = -q'E P F q + tr(P E P F)/2,   d2N = N (dlogN dlogN' + d2logN).
 #include <math.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "fp64_profile.cuh"
 #include "internal.cuh"
+#include "async_copy.cuh"
 #include "source_math.cuh"
+#include "whiten.cuh"
 
 namespace cel {
 
@@ -42,8 +45,6 @@ __device__ __forceinline__ float ex2h(float x) {
 }
 __device__ __forceinline__ float lgh(float x) { return logf(x); }
 __device__ __forceinline__ double lgh(double x) { return log(x); }
-
-constexpr double LOG2E_H = 1.4426950408889634;   // log2(e)
 
 // packed index of a symmetric N x N (upper triangle by rows; a <= b not required)
 template <int N>
@@ -73,142 +74,6 @@ __device__ __forceinline__ void warp_reduce_scatter(R (&v)[HV], int lane) {
 #pragma unroll
         for (int i = 64; i < HV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], m);
     }
-}
-
-// ---- The galaxy components in the frame that whitens PSF component k.
-// T_k maps a pixel offset d to z = T_k d with T_k Sigma_k T_k' = I and T_k G T_k' =
-// diag(g1, g2), so component j's precision is T_k' diag(lam1, lam2) T_k with
-// lam_a = 1 / (1 + nu_j g_a).  With r = lam z and E~ = T_k E T_k', every derivative of
-// N_kj over (mu, G) is N_kj times T_k' (a polynomial in z) T_k:
-//   d/dmu: r;   d/dG[E]: (nu/2)(r' E~ r - tr(lam E~));   d2/dmu2: r r' - lam;
-//   d2/dmu dG[E]: r d/dG[E] - nu lam E~ r;
-//   d2/dG[E] dG[F]: d/dG[E] d/dG[F] - nu^2 r' E~ lam F~ r + (nu^2/2) tr(lam E~ lam F~).
-// A pixel therefore needs, per k, 35 sums over j of N_kj (or of its e_dev derivative)
-// times a monomial in (nu, lam1, lam2); the z-polynomials and the maps back to the
-// pixel frame are applied once per (pixel, k) instead of once per component.
-// Sums (monomial lam1^(deg - i) lam2^i at offset i):
-constexpr int WS_N = 0,    // N
-              WS_L = 1,    // N lam            (deg 1)
-              WS_LL = 3,   // N lam lam        (deg 2)
-              WS_B = 6,    // N nu lam         (deg 1)
-              WS_A = 8,    // N nu lam lam     (deg 2)
-              WS_C = 11,   // N nu lam^3       (deg 3)
-              WS_D2 = 15,  // N nu^2 lam^2
-              WS_D3 = 18,  // N nu^2 lam^3
-              WS_D4 = 22,  // N nu^2 lam^4
-              WS_NE = 27,  // dN/de_dev
-              WS_LE = 28,  // dN/de_dev lam
-              WS_BE = 30,  // dN/de_dev nu lam
-              WS_AE = 32,  // dN/de_dev nu lam lam
-              NWS = 35;
-// Of these, with lam_a (1 + nu g_a) = 1, the ones of lower degree follow from 19 (all terms
-// positive, so nothing cancels):  A_0 = C_0 + g1 D3_0, A_1 = C_1 + g1 D3_1, A_2 = C_3 + g2 D3_3,
-// B = A + g D2, L = LL + g A, N = L_0 + g1 B_0; and the e_dev sums are the difference of the
-// dev and the exp components' sums at unit weight.  So the kernel accumulates 19 sums over
-// the exp components, then over the dev components, and forms the 35 once per (pixel, k).
-constexpr int BS_LL = 0, BS_C = 3, BS_D2 = 7, BS_D3 = 10, BS_D4 = 14, NBS = 19;
-constexpr int WROW = 40;   // a full row: exponent coefficients of z1^2, z2^2, constant; 35 weights; pad
-constexpr int BROW = 24;   // a kernel row: the exponent's three coefficients, (FP32: a pad,) 19 weights, pad
-constexpr int WFR = 16;    // entries per k: T (row-major), K (3 x 3), g1, g2, pad
-// K[e][p] = (T E_e T')_p for the pixel-frame shape directions E_e = (xx, xy + yx, yy)
-// and the whitened pairs p = (11, 12, 22)
-constexpr int WF_K = 4, WF_G = 13;
-static_assert(3 + NWS <= WROW && 4 + NBS < BROW && BROW % 4 == 0 && WFR % 4 == 0 && WF_G + 2 <= WFR,
-              "whitened rows are read as 16-byte vectors from a 16-byte aligned array");
-
-__host__ __device__ __forceinline__ int wpa(int p) { return p == 2 ? 1 : 0; }
-__host__ __device__ __forceinline__ int wpb(int p) { return p == 0 ? 0 : 1; }
-
-// K of a frame whose T is in place
-template <class R>
-__host__ __device__ __forceinline__ void whiten_shape_map(R* fr) {
-#pragma unroll
-    for (int p = 0; p < 3; ++p) {
-        const R* Ta = fr + 2 * wpa(p);
-        const R* Tb = fr + 2 * wpb(p);
-        fr[WF_K + 0 * 3 + p] = Ta[0] * Tb[0];
-        fr[WF_K + 1 * 3 + p] = Ta[0] * Tb[1] + Ta[1] * Tb[0];
-        fr[WF_K + 2 * 3 + p] = Ta[1] * Tb[1];
-    }
-    fr[15] = 0;
-}
-
-// T_k from the Cholesky factor of the component's precision and one Jacobi rotation, in
-// FP32 (a few threads per work item, before its pixels: FP64 square roots and divisions
-// there would hold every warp of the item at the barrier; host-callable for tests)
-__host__ __device__ void whiten_frame(const float* sT, int k, float* fr) {
-    const float* S = sT + T_STAR + k * STAR_STRIDE;
-    const float pxx = S[4], pxy = S[5], pyy = S[6];
-    const float gxx = sT[T_G], gxy = sT[T_G + 1], gyy = sT[T_G + 2];
-    // T0 = [[r11, r21], [0, r22]] with T0 Sigma T0' = I (r the lower factor of Sigma^-1)
-    const float r11 = sqrtf(pxx), r21 = pxy / r11, r22 = sqrtf(fmaxf(pyy - r21 * r21, 0.f));
-    const float u0 = r11 * gxx + r21 * gxy, u1 = r11 * gxy + r21 * gyy;
-    const float b11 = u0 * r11 + u1 * r21, b12 = u1 * r22, b22 = r22 * gyy * r22;
-    // Q = [[c, s], [-s, c]] with Q B Q' diagonal, B = T0 G T0' (the smaller rotation; an
-    // infinite tau gives t = 0)
-    float c = 1.f, s = 0.f;
-    if (b12 != 0.f) {
-        const float tau = (b22 - b11) / (2.f * b12);
-        const float t = tau == 0.f ? 1.f : -copysignf(1.f, tau) / (fabsf(tau) + sqrtf(1.f + tau * tau));
-        c = 1.f / sqrtf(1.f + t * t);
-        s = t * c;
-    }
-    const float T[2][2] = {{c * r11, c * r21 + s * r22}, {-s * r11, -s * r21 + c * r22}};
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-        fr[2 * a] = T[a][0];
-        fr[2 * a + 1] = T[a][1];
-        const float v0 = T[a][0] * gxx + T[a][1] * gxy, v1 = T[a][0] * gxy + T[a][1] * gyy;
-        fr[WF_G + a] = fmaxf(v0 * T[a][0] + v1 * T[a][1], 0.f);
-    }
-    whiten_shape_map(fr);
-}
-
-// lam1^(deg - i) lam2^i, i = 0 .. deg, times w
-template <class R>
-__host__ __device__ __forceinline__ void monomials(R w, R l1, R l2, int deg, R* c) {
-#pragma unroll
-    for (int i = 0; i <= deg; ++i) {
-        R v = w;
-#pragma unroll
-        for (int u = 0; u < deg; ++u) v *= u < i ? l2 : l1;
-        c[i] = v;
-    }
-}
-
-// the row of galaxy component (k, j): exponent in z and the 35 monomial weights
-__host__ __device__ void whiten_row(const float* G, const float* fr, float* row) {
-    const float nu = G[9], w = G[7], dw = G[8];
-    const float l1 = 1.f / (1.f + nu * fr[WF_G]), l2 = 1.f / (1.f + nu * fr[WF_G + 1]);
-    row[0] = -0.5f * (float)LOG2E_H * l1;
-    row[1] = -0.5f * (float)LOG2E_H * l2;
-    row[2] = G[3];
-    float* c = row + 3;
-    c[WS_N] = w;
-    c[WS_NE] = dw;
-    monomials(w, l1, l2, 1, c + WS_L);
-    monomials(w, l1, l2, 2, c + WS_LL);
-    monomials(w * nu, l1, l2, 1, c + WS_B);
-    monomials(w * nu, l1, l2, 2, c + WS_A);
-    monomials(w * nu, l1, l2, 3, c + WS_C);
-    monomials(w * nu * nu, l1, l2, 2, c + WS_D2);
-    monomials(w * nu * nu, l1, l2, 3, c + WS_D3);
-    monomials(w * nu * nu, l1, l2, 4, c + WS_D4);
-    monomials(dw, l1, l2, 1, c + WS_LE);
-    monomials(dw * nu, l1, l2, 1, c + WS_BE);
-    monomials(dw * nu, l1, l2, 2, c + WS_AE);
-    row[3 + NWS] = 0.f;
-    row[4 + NWS] = 0.f;
-}
-
-// the kernel's row: three exponent coefficients (given) and the 19 weights at weight w
-template <class R>
-__host__ __device__ __forceinline__ void base_row(R w, R nu, R l1, R l2, R* c) {
-    monomials(w, l1, l2, 2, c + BS_LL);
-    monomials(w * nu, l1, l2, 3, c + BS_C);
-    monomials(w * nu * nu, l1, l2, 2, c + BS_D2);
-    monomials(w * nu * nu, l1, l2, 3, c + BS_D3);
-    monomials(w * nu * nu, l1, l2, 4, c + BS_D4);
 }
 
 // the sums of lower degree: A (3), B (2), L (2), N from the base sums
@@ -421,14 +286,13 @@ __host__ __device__ __forceinline__ double a_transform(const double* A, const do
     return A[2] * A[2] * wxx + 2.0 * A[2] * A[3] * wxy + A[3] * A[3] * wyy;
 }
 
-// ---- The terms of a source that depend on its parameters alone, by the first CTAs of
-// k_hess (their FP64 latencies then pass behind the pixel work): the KL value, gradient and
+// ---- The terms of a source that depend on its parameters alone, two tasks ahead of the pixel
+// work in k_hess's queue (their FP64 latencies then pass behind it): the KL value, gradient and
 // Hessian, the brightness moments of the five bands and the world-frame shape derivatives.
 // hess_out receives -KL'' and zeros; the rest goes to the source's record.
 constexpr int HR_KL = 0, HR_KLG = 1, HR_MOM = HR_KLG + NP, HR_DW = HR_MOM + 20, HR_D2W = HR_DW + 9,
               HR_A = HR_D2W + 27;
 static_assert(HR_A + 2 <= HREC && HREC % 2 == 0, "the source's record");
-constexpr int TERM_SRC = HCHUNK / 64;   // sources per CTA: two warps each
 
 struct SourceTerms {
     int n_src;
@@ -560,361 +424,442 @@ __device__ __forceinline__ void kl_terms_warp(const ModelDev& md, const double* 
     }
 }
 
-// the terms of sources s0 .. s0 + TERM_SRC, one CTA of k_hess; sm: TERM_SRC NP doubles
-__device__ __forceinline__ void source_terms(const SourceTerms& a, int s0, const int32_t* __restrict__ src_active,
-                                             double* sm) {
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int n = min(TERM_SRC, a.n_src - s0);
-    for (int u = 0; u < n; ++u) {
-        if (src_active && !src_active[s0 + u]) continue;
-        double* H = a.hess + (size_t)NP * NP * (s0 + u);   // the caller's: 8-byte aligned
-        for (int i = t; i < NP * NP; i += HCHUNK) H[i] = 0.0;
+// task 0 or 1 of source s by one warp; sm: NP doubles of the warp's shared memory
+__device__ __forceinline__ void source_terms(const SourceTerms& a, int s, int task, double* sm) {
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < NP; i += 32) {
+        sm[i] = a.theta[(size_t)NP * s + i];
+        if (a.status && task == 0) theta_domain_check(i, sm[i], a.status);
     }
-    for (int i = t; i < n * NP; i += HCHUNK) {
-        sm[i] = a.theta[(size_t)NP * s0 + i];
-        if (a.status) theta_domain_check(i % NP, sm[i], a.status);
-    }
-    __syncthreads();
-    const int u = warp % TERM_SRC, s = s0 + u;
-    if (u >= n || (src_active && !src_active[s])) return;
-    const double* th = sm + u * NP;
+    __syncwarp();
     double* rec = a.hsrc + (size_t)HREC * s;
-    if (warp < TERM_SRC) {
-        kl_terms_warp(*a.md, th, rec, a.kl + s, a.hess + (size_t)NP * NP * s);
-        return;
+    if (task == 0) {
+        double* H = a.hess + (size_t)NP * NP * s;   // the caller's: 8-byte aligned
+        for (int i = lane; i < NP * NP; i += 32) H[i] = 0.0;
+        __syncwarp();
+        kl_terms_warp(*a.md, sm, rec, a.kl + s, H);
+    } else {
+        if (lane < 10) band_moments(sm, lane >> 1, lane & 1, rec[HR_MOM + 2 * lane], rec[HR_MOM + 2 * lane + 1]);
+        if (lane >= 30) rec[HR_A + lane - 30] = sm[P_A + lane - 30];
+        if (lane == 10) {
+            double dW[3][3], d2W[3][3][3];
+            shape_w_derivs(sm, dW, d2W);
+            for (int i = 0; i < 9; ++i) rec[HR_DW + i] = dW[i / 3][i % 3];
+            for (int i = 0; i < 27; ++i) rec[HR_D2W + i] = d2W[i / 9][i / 3 % 3][i % 3];
+        }
     }
-    if (lane < 10) band_moments(th, lane >> 1, lane & 1, rec[HR_MOM + 2 * lane], rec[HR_MOM + 2 * lane + 1]);
-    if (lane >= 30) rec[HR_A + lane - 30] = th[P_A + lane - 30];
-    if (lane == 10) {
-        double dW[3][3], d2W[3][3][3];
-        shape_w_derivs(th, dW, d2W);
-        for (int i = 0; i < 9; ++i) rec[HR_DW + i] = dW[i / 3][i % 3];
-        for (int i = 0; i < 27; ++i) rec[HR_D2W + i] = d2W[i / 9][i / 3 % 3][i % 3];
-    }
+    __syncwarp();
 }
 
-// Shared memory of k_hess (bytes): the patch's table (R), per PSF component its frame, the
-// component rows and, FP64, the table of 2^x; the warps' sums take the rows' place at the end.
+// Shared memory of k_hess: in FP64 the CTA's table of 2^x; then per warp two stages, each a
+// part's record, its patch's table and (FP32) frames, the part's frames (FP64) and rows, and the
+// part's sums.  In bytes, for tables of n_comp components.
+constexpr int HESS_WARPS = 4;
 template <class R>
 struct HessLay {
-    static constexpr int tbl = 0;
-    static constexpr int fr = tbl + TBL_STRIDE * (int)sizeof(R);
-    static constexpr int rows = fr + MAXPSF * WFR * (int)sizeof(R);
-    static constexpr int rows_bytes = MAXPSF * MAXPROF * BROW * (int)sizeof(R);
-    static constexpr int red_bytes = (HCHUNK / 32) * HV * 8;
-    static constexpr int tab = rows + (rows_bytes > red_bytes ? rows_bytes : red_bytes);
-    static constexpr int bytes = tab + (sizeof(R) == 8 ? EX_N * 8 : 0);
-    static_assert(fr % 16 == 0 && rows % 16 == 0 && tab % 16 == 0, "16-byte alignment");
+    static constexpr bool DBL = sizeof(R) == 8;
+    static constexpr int tab_bytes = DBL ? EX_N * 8 : 0;
+    static constexpr int tbl = (int)sizeof(HItem);   // in the stage
+    int sfr, stage, fr, rows, sums, warp;
+    __host__ __device__ explicit HessLay(int n_comp) {
+        sfr = tbl + (T_GAL + n_comp * GAL_STRIDE) * (int)sizeof(R);
+        stage = sfr + (DBL ? 0 : MAXPSF * WFR * 4);
+        fr = 2 * stage;
+        rows = fr + (DBL ? MAXPSF * WFR * 8 : 0);
+        sums = rows + n_comp * BROW * (int)sizeof(R);
+        warp = sums + HV * 8;
+    }
+    __host__ __device__ int bytes() const { return tab_bytes + HESS_WARPS * warp; }
+};
+static_assert(sizeof(HItem) % 16 == 0 && GAL_STRIDE % 4 == 0 && BROW % 4 == 0 && HV % 2 == 0,
+              "every piece starts on a 16-byte boundary");
+
+// 16 bytes from global to shared memory, asynchronously
+__device__ __forceinline__ void copy16_async(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+
+// Per part of a work item: the sums over its pixels of ll, d ll / dz and d2 ll / dz2.  The
+// mixture in the whitened frame; FP64 as in fp64_profile.cuh.  E and Var of a singly covered
+// pixel (single) are formed here, those of the others come from the maps.
+// Persistent warps take tasks from a queue, warp w's first two being tasks w and w + W (W warps):
+// the sources' parameter-only terms, then the parts.  While a part is computed the next one's
+// record and table are on their way to the warp's other stage.  A warp goes through its part 32
+// pixels at a time and shares nothing with the others, so it waits neither for memory nor at a
+// barrier; one CTA per part had its warps waiting for loads and barriers 40 % of the time.
+// 500 sources, FP32: 125 -> 112 us (issue slots 63 % used, FMA pipe 52 %; 56 us at that pipe's
+// peak); 64 crowded sources, FP64: 608 -> 584 us (FP64 pipe 88 %).
+// Bound by the FP32 or the FP64 pipe: 12 (packed) / 25 of its instructions per component, where
+// the 35 sums accumulated one by one took 38 and the pixel-frame formulas about 140.
+template <class R>
+struct HessArgs {
+    const HItem* parts;
+    int n_part;
+    const ImgMeta* img;
+    const PatchGeo* geo;
+    int n_comp, nprof, n_exp;   // components of the largest table; profile components
+    const float* pixels;
+    const float* sky_map;
+    const R* tbl;
+    const float* hframe;
+    const uint8_t* single;
+    const R* emap;
+    const R* vmap;
+    double* part;
+    const int32_t* src_active;
+    int32_t* queue;
+    SourceTerms src;
 };
 
-// Per part of a work item: the sums over its pixels of ll, d ll / d y and d2 ll / dy2.  The mixture in
-// the whitened frame (above); FP64 as in fp64_profile.cuh, E and Var of a singly covered
-// pixel (single, FP64 only) formed here, those of the others from the maps.
-// Bound by the FP32 or the FP64 pipe: 22 / 25 of its instructions per component, where the
-// 35 sums accumulated one by one took 38 (FP32: 500 sources, 909,100 source-pixels, 180 ->
-// 140 us) and the pixel-frame formulas about 140 (FP64: fp64_profile.cuh has the figures).
-template <class R>
-__global__ void __launch_bounds__(HCHUNK, sizeof(R) == 8 ? 2 : 4) k_hess(const WorkItem* __restrict__ items,
-                                                const PatchGeo* __restrict__ geo,
-                                                const ImgMeta* __restrict__ img, int nprof, int n_exp,
-                                                const float* __restrict__ pixels,
-                                                const float* __restrict__ sky_map,
-                                                const R* __restrict__ tbl,
-                                                const uint8_t* __restrict__ single,
-                                                const R* __restrict__ emap,
-                                                const R* __restrict__ vmap,
-                                                double* __restrict__ part,
-                                                const int32_t* __restrict__ src_active, SourceTerms src) {
+// NE, ND: the exp and dev components of the model where they are known (the paper's model and
+// the synthetic workloads: 6 and 8), else 0.
+template <class R, int NE, int ND>
+__global__ void __launch_bounds__(32 * HESS_WARPS, sizeof(R) == 8 ? 2 : 4) k_hess(const HessArgs<R> a) {
     constexpr bool DBL = std::is_same<R, double>::value;
-    using Lay = HessLay<R>;
     extern __shared__ __align__(16) unsigned char smem[];
-    R* sT = reinterpret_cast<R*>(smem + Lay::tbl);
-    R* frames = reinterpret_cast<R*>(smem + Lay::fr);
-    R* rows = reinterpret_cast<R*>(smem + Lay::rows);
-    double* tab = reinterpret_cast<double*>(smem + Lay::tab);
-    // the first CTAs take the sources' terms that do not depend on the pixels
-    const int n_term_cta = (src.n_src + TERM_SRC - 1) / TERM_SRC;
-    if ((int)blockIdx.x < n_term_cta) {
-        source_terms(src, (int)blockIdx.x * TERM_SRC, src_active, reinterpret_cast<double*>(smem));
-        return;
-    }
-    // one HCHUNK-pixel part of an item
-    const int rec = (int)blockIdx.x - n_term_cta, sub = rec % HSPLIT * HCHUNK;
-    const WorkItem it = items[rec / HSPLIT];
-    const int n_px = it.n - sub;
-    if (n_px <= 0) return;
-    const PatchGeo g = geo[it.patch];
-    if (src_active && !src_active[g.src]) return;
-    const ImgMeta& im = img[g.img];
-    const int npsf = im.npsf;
-    const int t = threadIdx.x;
-    {
-        const R* gT = tbl + (size_t)it.patch * TBL_STRIDE;
-        const int n = T_GAL + npsf * nprof * GAL_STRIDE;
-        for (int i = t; i < n; i += blockDim.x) sT[i] = gT[i];
-        if constexpr (DBL) load_exp2_table(tab);
+    const HessLay<R> L(a.n_comp);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double* tab = reinterpret_cast<double*>(smem);
+    unsigned char* sm = smem + HessLay<R>::tab_bytes + warp * L.warp;   // this warp's
+    R* rows = reinterpret_cast<R*>(sm + L.rows);
+    double* sums = reinterpret_cast<double*>(sm + L.sums);
+    const int nprof = a.nprof, n_exp = a.n_exp;
+    if constexpr (DBL) {
+        load_exp2_table(tab);
         __syncthreads();
     }
-    if (t < npsf) {
-        if constexpr (DBL) {
-            const R* F = sT + T_STAR + t * STAR_STRIDE;
-            R* fr = frames + t * WFR;
+    // tasks [0, n_term): the sources' terms; then the parts
+    const int W = (int)gridDim.x * HESS_WARPS, n_term = 2 * a.src.n_src, n_task = n_term + a.n_part;
+    auto patch_of = [&](int task) {   // -1: not a part
+        return task >= n_term && task < n_task ? a.parts[task - n_term].patch : -1;
+    };
+    // the copies of one part: its record, its patch's table and (FP32) frames
+    auto fetch = [&](int task, int patch, int b) {
+        unsigned char* st = sm + b * L.stage;
+        auto copy = [&](int to, const void* from, int n) {
+            for (int i = lane; i < n; i += 32)
+                copy16_async(st + to + 16 * i, reinterpret_cast<const unsigned char*>(from) + 16 * i);
+        };
+        if (patch >= 0) {
+            copy(0, a.parts + (task - n_term), (int)sizeof(HItem) / 16);
+            copy(HessLay<R>::tbl, a.tbl + (size_t)patch * TBL_STRIDE, (L.sfr - HessLay<R>::tbl) / 16);
+            if (!DBL) copy(L.sfr, a.hframe + (size_t)patch * HF_STRIDE, MAXPSF * WFR / 4);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int task = warp * (int)gridDim.x + (int)blockIdx.x, next = task + W;
+    fetch(task, patch_of(task), 0);
+    int next_patch = patch_of(next);
+    for (int b = 0; task < n_task; b ^= 1) {
+        const int cur = task;
+        fetch(next, next_patch, b ^ 1);   // the stage was last read in the previous task
+        int claim = 0;
+        if (lane == 0) claim = 2 * W + atomicAdd(a.queue, 1);
+        task = next;
+        if (cur < n_term) {
+            const int s = cur >> 1;
+            if (!a.src_active || a.src_active[s]) source_terms(a.src, s, cur & 1, sums);
+            next = __shfl_sync(0xffffffffu, claim, 0);
+            next_patch = patch_of(next);
+            continue;
+        }
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        const HItem& it = *reinterpret_cast<const HItem*>(sm + b * L.stage);
+        if (a.src_active && !a.src_active[it.src]) {
+            __syncwarp();
+            next = __shfl_sync(0xffffffffu, claim, 0);
+            next_patch = patch_of(next);
+            continue;
+        }
+        const R* sT = reinterpret_cast<const R*>(sm + b * L.stage + HessLay<R>::tbl);
+        R* frames = reinterpret_cast<R*>(DBL ? sm + L.fr : sm + b * L.stage + L.sfr);
+        const int npsf = it.npsf;
+        if (DBL && lane < npsf) {
+            const R* F = sT + T_STAR + lane * STAR_STRIDE;
+            R* fr = frames + lane * WFR;
             for (int i = 0; i < 4; ++i) fr[i] = F[i];
             fr[WF_G] = F[4];
             fr[WF_G + 1] = F[5];
             whiten_shape_map(fr);
-        } else {
-            whiten_frame(sT, t, frames + t * WFR);
+            fr[15] = F[6];
         }
-    }
-    __syncthreads();
-    for (int i = t; i < npsf * nprof; i += blockDim.x) {
-        // the exponent's coefficients and the 19 weights at unit e_dev weight
-        const R* G = sT + T_GAL + i * GAL_STRIDE;
-        const R* fr = frames + (i / nprof) * WFR;
-        R* row = rows + i * BROW;
-        R l1, l2, w;
-        const R nu = G[9];
-        if constexpr (DBL) {
-            l1 = G[0] * EX_IHALF;
-            l2 = G[1] * EX_IHALF;
-            w = G[3];
-        } else {
-            l1 = 1.f / (1.f + nu * fr[WF_G]);
-            l2 = 1.f / (1.f + nu * fr[WF_G + 1]);
-            w = i % nprof >= n_exp ? G[8] : -G[8];
-        }
-        row[0] = DBL ? G[0] : (R)(-0.5 * LOG2E_H) * l1;
-        row[1] = DBL ? G[1] : (R)(-0.5 * LOG2E_H) * l2;
-        row[2] = DBL ? G[2] : G[3];
-        constexpr int W0 = DBL ? 3 : 4;   // FP32: the weights on a 16-byte boundary
-        base_row(w, nu, l1, l2, row + W0);
-        row[W0 + NBS] = 0;
-    }
-    __syncthreads();
-    R out[HV];
-#pragma unroll
-    for (int i = 0; i < HV; ++i) out[i] = 0;
-    if (t < n_px) {
-        const int q = it.q0 + sub + t;
-        const int yy = q / g.w, xx = q - yy * g.w;
-        // star: value, gradient (mx, my), Hessian (xx, xy, yy)
-        R g0 = 0, d0[2] = {0, 0}, h0[3] = {0, 0, 0};
-        // galaxy: value; gradient over z5 = (mx, my, Gxx, Gxy, Gyy); e_dev derivative;
-        // Hessian over z5 (packed 15); e_dev x z5
-        R g1 = 0, d1[5] = {0, 0, 0, 0, 0}, de = 0, h1[15], he[5] = {0, 0, 0, 0, 0};
-#pragma unroll
-        for (int i = 0; i < 15; ++i) h1[i] = 0;
-        const R edev = sT[H_EDEV];
-        for (int k = 0; k < npsf; ++k) {
-            const R dx = (R)xx - sT[T_MEAN + 2 * k], dy = (R)yy - sT[T_MEAN + 2 * k + 1];
-            const R* fr = frames + k * WFR;
-            const R z1 = fr[0] * dx + fr[1] * dy, z2 = fr[2] * dx + fr[3] * dy;
-            const R z1s = z1 * z1, z2s = z2 * z2;
-            float f1 = 0.f, f2 = 0.f;
+        for (int i = lane; i < npsf * nprof; i += 32) {
+            // the exponent's coefficients and the 19 weights at unit e_dev weight
+            const R* Gr = sT + T_GAL + i * GAL_STRIDE;
+            R* row = rows + i * BROW;
             if constexpr (DBL) {
-                f1 = (float)z1s;
-                f2 = (float)z2s;
-            }
-            {
-                // P d = T' z and P = T' T
-                const R* S = sT + T_STAR + k * STAR_STRIDE;
-                R n, qx, qy, pxx, pxy, pyy;
-                if constexpr (DBL) {
-                    n = S[6] * ex2_quad(EX_HALF, z1s, EX_HALF, z2s, (float)EX_HALF, f1, (float)EX_HALF, f2, tab);
-                    qx = fr[0] * z1 + fr[2] * z2;
-                    qy = fr[1] * z1 + fr[3] * z2;
-                    pxx = fr[WF_K] + fr[WF_K + 2];
-                    pxy = (R)0.5 * (fr[WF_K + 3] + fr[WF_K + 5]);
-                    pyy = fr[WF_K + 6] + fr[WF_K + 8];
-                } else {
-                    n = S[7] * ex2h(S[0] * (dx * dx) + S[1] * (dx * dy) + S[2] * (dy * dy) + S[3]);
-                    qx = S[4] * dx + S[5] * dy;
-                    qy = S[5] * dx + S[6] * dy;
-                    pxx = S[4];
-                    pxy = S[5];
-                    pyy = S[6];
-                }
-                g0 += n;
-                d0[0] += n * qx;
-                d0[1] += n * qy;
-                h0[0] += n * (qx * qx - pxx);
-                h0[1] += n * (qx * qy - pxy);
-                h0[2] += n * (qy * qy - pyy);
-            }
-            const R* row = rows + k * nprof * BROW;
-            auto group = [&](int n, R (&b)[NBS]) {
-                if constexpr (DBL) {
-#pragma unroll
-                    for (int m = 0; m < NBS; ++m) b[m] = 0;
-                    for (int j = 0; j < n; ++j, row += BROW) {
-                        double cw[BROW];
-#pragma unroll
-                        for (int u = 0; u < (3 + NBS + 1) / 2; ++u) {
-                            const double2 v = reinterpret_cast<const double2*>(row)[u];
-                            cw[2 * u] = v.x;
-                            cw[2 * u + 1] = v.y;
-                        }
-                        const float2 ab = as_float2(cw[2]);
-                        const double e = ex2_quad(cw[0], z1s, cw[1], z2s, ab.x, f1, ab.y, f2, tab);
-#pragma unroll
-                        for (int m = 0; m < NBS; ++m) b[m] += e * cw[3 + m];
-                    }
-                } else {
-                    // packed FP32x2: the 19 weights as ten pairs (half the issue slots)
-                    constexpr int NPR = (NBS + 1) / 2;
-                    float2 bb[NPR];
-#pragma unroll
-                    for (int m = 0; m < NPR; ++m) bb[m] = make_float2(0.f, 0.f);
-                    for (int j = 0; j < n; ++j, row += BROW) {
-                        float4 cw[BROW / 4];
-#pragma unroll
-                        for (int u = 0; u < BROW / 4; ++u) cw[u] = reinterpret_cast<const float4*>(row)[u];
-                        const float e = ex2h(fmaf(cw[0].x, z1s, fmaf(cw[0].y, z2s, cw[0].z)));
-                        const float2 ee = make_float2(e, e);
-#pragma unroll
-                        for (int m = 0; m < NPR; ++m) {
-                            const float4 w = cw[1 + m / 2];
-                            bb[m] = __ffma2_rn(ee, m & 1 ? make_float2(w.z, w.w) : make_float2(w.x, w.y), bb[m]);
-                        }
-                    }
-#pragma unroll
-                    for (int m = 0; m < NBS; ++m) b[m] = m & 1 ? bb[m / 2].y : bb[m / 2].x;
-                }
-            };
-            R be[NBS], bd[NBS], s[NWS];
-            group(n_exp, be);
-            group(nprof - n_exp, bd);
-            combine_groups(be, bd, fr[WF_G], fr[WF_G + 1], edev, s);
-            whitened_add(s, z1, z2, fr, g1, d1, de, h1, he);
-        }
-        // ---- E, Var and the pixel's weights
-        const R iota = sT[H_IOTA], a0 = sT[H_A0], a1 = sT[H_A1];
-        const R k0 = a0 * iota * sT[H_EL0], k1 = a1 * iota * sT[H_EL1];
-        const R q0 = a0 * iota * iota * sT[H_EL20], q1 = a1 * iota * iota * sT[H_EL21];
-        const R Es = k0 * g0 + k1 * g1;
-        const int64_t m = im.px_off + (int64_t)(g.y0 + yy) * im.W + (g.x0 + xx);
-        const R x = (R)pixels[m];
-        R E, V;
-        if (DBL && single && single[g.sp_off + q]) {
-            if constexpr (DBL) {
-                double em0, em1, es;
-                moment_ratios64(sT, em0, em1);
-                source_ev64(sT, em0, em1, g0, g1, es, V);
-                E = (im.has_sky_map ? (double)sky_map[m] : im.sky) + es;
-            }
-        } else {
-            E = emap[m];
-            V = vmap[m];
-        }
-        const R iE = (R)1 / E, iE2 = iE * iE;
-        const R cE = x * (iE + V * iE2 * iE) - (R)1;
-        const R cV = (R)-0.5 * x * iE2;
-        const R hEE = -x * iE2 * ((R)1 + (R)3 * V * iE2);
-        const R hEV = x * iE2 * iE;
-        out[0] = x * (lgh(E) - (R)0.5 * V * iE2) - E;
-        // ---- assemble the pixel's z-derivatives (entries known to be zero are left out: a
-        // product with a constant 0 would be computed)
-        const R w1 = cE - (R)2 * cV * Es, w2 = cV;
-        // gradient of g_1 over (mx, my, e_dev, Gxx, Gxy, Gyy); g_0's is (d0[0], d0[1], 0, 0, 0, 0)
-        const R dg1[6] = {d1[0], d1[1], de, d1[2], d1[3], d1[4]};
-        // e = dE_s/dz (0 for q), v2 = dE2_s/dz (0 for k)
-        R e[NZ], v2[NZ];
-        e[Z_K0] = g0;
-        e[Z_K1] = g1;
-        v2[Z_Q0] = g0 * g0;
-        v2[Z_Q1] = g1 * g1;
-        const R m0 = (R)2 * q0, m1 = (R)2 * q1, n0 = m0 * g0, n1 = m1 * g1;
-#pragma unroll
-        for (int z = 0; z < 6; ++z) {
-            e[Z_MX + z] = k1 * dg1[z];
-            v2[Z_MX + z] = n1 * dg1[z];
-            if (z < 2) {
-                e[Z_MX + z] += k0 * d0[z];
-                v2[Z_MX + z] += n0 * d0[z];
-            }
-        }
-        auto has_e = [](int z) { return z != Z_Q0 && z != Z_Q1; };
-        auto has_v2 = [](int z) { return z != Z_K0 && z != Z_K1; };
-        // gradient, and the outer-product part of the Hessian: with v = v2 - 2 E_s e,
-        //   (h_EE - 2 c_V) e e' + h_EV (e v' + v e') = e p' + p e',
-        //   p = (h_EE / 2 - c_V - 2 h_EV E_s) e + h_EV v2
-        const R c1 = (R)0.5 * hEE - cV - (R)2 * hEV * Es;
-        R pv[NZ];
-#pragma unroll
-        for (int z = 0; z < NZ; ++z) {
-            if (!has_e(z)) {
-                out[1 + z] = w2 * v2[z];
-                pv[z] = hEV * v2[z];
-            } else if (!has_v2(z)) {
-                out[1 + z] = w1 * e[z];
-                pv[z] = c1 * e[z];
+                row[0] = Gr[0];
+                row[1] = Gr[1];
+                row[2] = Gr[2];
+                base_row(Gr[3], Gr[9], Gr[0] * EX_IHALF, Gr[1] * EX_IHALF, row + 3);
+                row[3 + NBS] = 0;
             } else {
-                out[1 + z] = w1 * e[z] + w2 * v2[z];
-                pv[z] = c1 * e[z] + hEV * v2[z];
+                const float* fr = frames + (i / nprof) * WFR;
+                const float nu = Gr[9], l1 = 1.f / (1.f + nu * fr[WF_G]), l2 = 1.f / (1.f + nu * fr[WF_G + 1]);
+                row[0] = (float)(-0.5 * LOG2E_W) * l1;
+                row[1] = (float)(-0.5 * LOG2E_W) * l2;
+                row[2] = Gr[3];
+                base_row(i % nprof >= n_exp ? Gr[8] : -Gr[8], nu, l1, l2, row + 4);   // on a 16-byte boundary
+                row[4 + NBS] = 0;
             }
         }
-        R* H = out + 1 + NZ;
-#pragma unroll
-        for (int a = 0; a < NZ; ++a)
-#pragma unroll
-            for (int b = a; b < NZ; ++b) {
-                R h = 0;
-                if (has_e(a) && has_e(b)) h = e[a] * pv[b] + pv[a] * e[b];
-                else if (has_e(a)) h = e[a] * pv[b];
-                else if (has_e(b)) h = pv[a] * e[b];
-                H[sym<NZ>(a, b)] = h;
+        for (int i = lane; i < HV; i += 32) sums[i] = 0.0;
+        __syncwarp();
+        for (int c0 = 0; c0 < it.n; c0 += 32) {
+            // the pixel's data, asked for before the mixture
+            const bool ok = c0 + lane < it.n;
+            const int q = it.q0 + (ok ? c0 + lane : 0);
+            const int yy = q / it.w, xx = q - yy * it.w;
+            const int64_t m = it.m0 + (int64_t)yy * it.W + xx;
+            const R x = (R)a.pixels[m];
+            const bool alone = a.single && a.single[it.sp0 + q];
+            R E, V = 0;
+            if (alone) {
+                const ImgMeta& im = a.img[a.geo[it.patch].img];
+                E = im.has_sky_map ? (R)a.sky_map[m] : (R)im.sky;
+            } else {
+                E = a.emap[m];
+                V = a.vmap[m];
             }
-        // second-derivative part  w1 DE + w2 DE2
-        const R b0 = w2 * m0, b1 = w2 * m1;
-        const R u0 = w1 * k0 + b0 * g0, u1 = w1 * k1 + b1 * g1;
-        const R r0 = (R)2 * w2 * g0, r1 = (R)2 * w2 * g1;
-        R bd1[6];
+            R out[HV];
 #pragma unroll
-        for (int z = 0; z < 6; ++z) {
-            H[sym<NZ>(Z_K1, Z_MX + z)] += w1 * dg1[z];
-            H[sym<NZ>(Z_Q1, Z_MX + z)] += r1 * dg1[z];
-            if (z < 2) {
-                H[sym<NZ>(Z_K0, Z_MX + z)] += w1 * d0[z];
-                H[sym<NZ>(Z_Q0, Z_MX + z)] += r0 * d0[z];
+            for (int i = 0; i < HV; ++i) out[i] = 0;
+            if (ok) {
+                // star: value, gradient (mx, my), Hessian (xx, xy, yy)
+                R g0 = 0, d0[2] = {0, 0}, h0[3] = {0, 0, 0};
+                // galaxy: value; gradient over z5 = (mx, my, Gxx, Gxy, Gyy); e_dev derivative;
+                // Hessian over z5 (packed 15); e_dev x z5
+                R g1 = 0, d1[5] = {0, 0, 0, 0, 0}, de = 0, h1[15], he[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+                for (int i = 0; i < 15; ++i) h1[i] = 0;
+                const R edev = sT[H_EDEV];
+                for (int k = 0; k < npsf; ++k) {
+                    const R dx = (R)xx - sT[T_MEAN + 2 * k], dy = (R)yy - sT[T_MEAN + 2 * k + 1];
+                    const R* fr = frames + k * WFR;
+                    const R z1 = fr[0] * dx + fr[1] * dy, z2 = fr[2] * dx + fr[3] * dy;
+                    const R z1s = z1 * z1, z2s = z2 * z2;
+                    float f1 = 0.f, f2 = 0.f;
+                    if constexpr (DBL) {
+                        f1 = (float)z1s;
+                        f2 = (float)z2s;
+                    }
+                    {
+                        // P d = T' z and P = T' T
+                        R n;
+                        if constexpr (DBL)
+                            n = ex2_quad(EX_HALF, z1s, EX_HALF, z2s, (float)EX_HALF, f1, (float)EX_HALF, f2, tab);
+                        else
+                            n = ex2h((float)(-0.5 * LOG2E_W) * (z1s + z2s));
+                        n *= fr[15];
+                        const R qx = fr[0] * z1 + fr[2] * z2, qy = fr[1] * z1 + fr[3] * z2;
+                        const R pxx = fr[WF_K] + fr[WF_K + 2], pxy = (R)0.5 * (fr[WF_K + 3] + fr[WF_K + 5]),
+                                pyy = fr[WF_K + 6] + fr[WF_K + 8];
+                        g0 += n;
+                        d0[0] += n * qx;
+                        d0[1] += n * qy;
+                        h0[0] += n * (qx * qx - pxx);
+                        h0[1] += n * (qx * qy - pxy);
+                        h0[2] += n * (qy * qy - pyy);
+                    }
+                    const R* row = rows + k * nprof * BROW;
+                    // the base sums over one group's components (N of them where N > 0, else n)
+                    auto group = [&](auto N, int n, R (&b)[NBS]) {
+                        if constexpr (DBL) {
+#pragma unroll
+                            for (int m = 0; m < NBS; ++m) b[m] = 0;
+                            for (int j = 0; j < n; ++j, row += BROW) {
+                                double cw[BROW];
+#pragma unroll
+                                for (int u = 0; u < (3 + NBS + 1) / 2; ++u) {
+                                    const double2 v = reinterpret_cast<const double2*>(row)[u];
+                                    cw[2 * u] = v.x;
+                                    cw[2 * u + 1] = v.y;
+                                }
+                                const float2 ab = as_float2(cw[2]);
+                                const double e = ex2_quad(cw[0], z1s, cw[1], z2s, ab.x, f1, ab.y, f2, tab);
+#pragma unroll
+                                for (int m = 0; m < NBS; ++m) b[m] += e * cw[3 + m];
+                            }
+                        } else {
+                            // packed FP32x2: the 19 weights as ten pairs (half the issue slots)
+                            constexpr int NPR = (NBS + 1) / 2;
+                            float2 bb[NPR];
+#pragma unroll
+                            for (int m = 0; m < NPR; ++m) bb[m] = make_float2(0.f, 0.f);
+                            auto value = [&](const R* r) {
+                                const float4 c = *reinterpret_cast<const float4*>(r);
+                                return ex2h(fmaf(c.x, z1s, fmaf(c.y, z2s, c.z)));
+                            };
+                            auto add = [&](const R* r, float e) {
+                                const float2 ee = make_float2(e, e);
+#pragma unroll
+                                for (int u = 0; u < NPR / 2; ++u) {
+                                    const float4 w = reinterpret_cast<const float4*>(r)[1 + u];
+                                    bb[2 * u] = __ffma2_rn(ee, make_float2(w.x, w.y), bb[2 * u]);
+                                    bb[2 * u + 1] = __ffma2_rn(ee, make_float2(w.z, w.w), bb[2 * u + 1]);
+                                }
+                            };
+                            if constexpr (decltype(N)::value > 0) {
+                                // a known count: the values first, so that their latency overlaps, then the sums
+                                constexpr int n_c = decltype(N)::value;
+                                float ev[n_c];
+#pragma unroll
+                                for (int j = 0; j < n_c; ++j) ev[j] = value(row + j * BROW);
+#pragma unroll
+                                for (int j = 0; j < n_c; ++j) add(row + j * BROW, ev[j]);
+                                row += n_c * BROW;
+                            } else {
+                                for (int j = 0; j < n; ++j, row += BROW) add(row, value(row));
+                            }
+#pragma unroll
+                            for (int m = 0; m < NBS; ++m) b[m] = m & 1 ? bb[m / 2].y : bb[m / 2].x;
+                        }
+                    };
+                    R be[NBS], bd[NBS], s[NWS];
+                    group(std::integral_constant<int, NE>{}, n_exp, be);
+                    group(std::integral_constant<int, ND>{}, nprof - n_exp, bd);
+                    combine_groups(be, bd, fr[WF_G], fr[WF_G + 1], edev, s);
+                    whitened_add(s, z1, z2, fr, g1, d1, de, h1, he);
+                }
+                // ---- E, Var and the pixel's weights
+                const R iota = sT[H_IOTA], a0 = sT[H_A0], a1 = sT[H_A1];
+                const R k0 = a0 * iota * sT[H_EL0], k1 = a1 * iota * sT[H_EL1];
+                const R q0 = a0 * iota * iota * sT[H_EL20], q1 = a1 * iota * iota * sT[H_EL21];
+                const R Es = k0 * g0 + k1 * g1;
+                if (alone) {
+                    if constexpr (DBL) {
+                        double em0, em1, es;
+                        moment_ratios64(sT, em0, em1);
+                        source_ev64(sT, em0, em1, g0, g1, es, V);
+                        E += es;
+                    } else {
+                        // Var_s in the form that does not cancel (k_contrib's)
+                        const float f0 = iota * sT[H_EL0] * g0, f1 = iota * sT[H_EL1] * g1;
+                        const float em0 = sT[H_EL20] / (sT[H_EL0] * sT[H_EL0]) - 1.f;
+                        const float em1 = sT[H_EL21] / (sT[H_EL1] * sT[H_EL1]) - 1.f;
+                        V = a0 * f0 * f0 * (em0 + (1.f - a0)) + a1 * f1 * f1 * (em1 + (1.f - a1)) -
+                            2.f * a0 * a1 * f0 * f1;
+                        E += Es;
+                    }
+                }
+                const R iE = (R)1 / E, iE2 = iE * iE;
+                const R cE = x * (iE + V * iE2 * iE) - (R)1;
+                const R cV = (R)-0.5 * x * iE2;
+                const R hEE = -x * iE2 * ((R)1 + (R)3 * V * iE2);
+                const R hEV = x * iE2 * iE;
+                out[0] = x * (lgh(E) - (R)0.5 * V * iE2) - E;
+                // ---- assemble the pixel's z-derivatives (entries known to be zero are left out: a
+                // product with a constant 0 would be computed)
+                const R w1 = cE - (R)2 * cV * Es, w2 = cV;
+                // gradient of g_1 over (mx, my, e_dev, Gxx, Gxy, Gyy); g_0's is (d0[0], d0[1], 0, 0, 0, 0)
+                const R dg1[6] = {d1[0], d1[1], de, d1[2], d1[3], d1[4]};
+                // e = dE_s/dz (0 for q), v2 = dE2_s/dz (0 for k)
+                R e[NZ], v2[NZ];
+                e[Z_K0] = g0;
+                e[Z_K1] = g1;
+                v2[Z_Q0] = g0 * g0;
+                v2[Z_Q1] = g1 * g1;
+                const R m0 = (R)2 * q0, m1 = (R)2 * q1, n0 = m0 * g0, n1 = m1 * g1;
+#pragma unroll
+                for (int z = 0; z < 6; ++z) {
+                    e[Z_MX + z] = k1 * dg1[z];
+                    v2[Z_MX + z] = n1 * dg1[z];
+                    if (z < 2) {
+                        e[Z_MX + z] += k0 * d0[z];
+                        v2[Z_MX + z] += n0 * d0[z];
+                    }
+                }
+                auto has_e = [](int z) { return z != Z_Q0 && z != Z_Q1; };
+                auto has_v2 = [](int z) { return z != Z_K0 && z != Z_K1; };
+                // gradient, and the outer-product part of the Hessian: with v = v2 - 2 E_s e,
+                //   (h_EE - 2 c_V) e e' + h_EV (e v' + v e') = e p' + p e',
+                //   p = (h_EE / 2 - c_V - 2 h_EV E_s) e + h_EV v2
+                const R c1 = (R)0.5 * hEE - cV - (R)2 * hEV * Es;
+                R pv[NZ];
+#pragma unroll
+                for (int z = 0; z < NZ; ++z) {
+                    if (!has_e(z)) {
+                        out[1 + z] = w2 * v2[z];
+                        pv[z] = hEV * v2[z];
+                    } else if (!has_v2(z)) {
+                        out[1 + z] = w1 * e[z];
+                        pv[z] = c1 * e[z];
+                    } else {
+                        out[1 + z] = w1 * e[z] + w2 * v2[z];
+                        pv[z] = c1 * e[z] + hEV * v2[z];
+                    }
+                }
+                R* H = out + 1 + NZ;
+#pragma unroll
+                for (int a = 0; a < NZ; ++a)
+#pragma unroll
+                    for (int b = a; b < NZ; ++b) {
+                        R h = 0;
+                        if (has_e(a) && has_e(b)) h = e[a] * pv[b] + pv[a] * e[b];
+                        else if (has_e(a)) h = e[a] * pv[b];
+                        else if (has_e(b)) h = pv[a] * e[b];
+                        H[sym<NZ>(a, b)] = h;
+                    }
+                // second-derivative part  w1 DE + w2 DE2
+                const R b0 = w2 * m0, b1 = w2 * m1;
+                const R u0 = w1 * k0 + b0 * g0, u1 = w1 * k1 + b1 * g1;
+                const R r0 = (R)2 * w2 * g0, r1 = (R)2 * w2 * g1;
+                R bd1[6];
+#pragma unroll
+                for (int z = 0; z < 6; ++z) {
+                    H[sym<NZ>(Z_K1, Z_MX + z)] += w1 * dg1[z];
+                    H[sym<NZ>(Z_Q1, Z_MX + z)] += r1 * dg1[z];
+                    if (z < 2) {
+                        H[sym<NZ>(Z_K0, Z_MX + z)] += w1 * d0[z];
+                        H[sym<NZ>(Z_Q0, Z_MX + z)] += r0 * d0[z];
+                    }
+                    bd1[z] = b1 * dg1[z];
+                }
+                // mean / shape block: u0 d2g0 + b0 dg0 dg0' + u1 d2g1 + b1 dg1 dg1', d2g1 over
+                // (mx, my, e_dev, Gxx, Gxy, Gyy) from h1 (packed without e_dev) and he (the e_dev row;
+                // its diagonal is zero)
+                const int zmap[5] = {0, 1, 3, 4, 5};   // position without e_dev -> position among the six
+                {
+                    int c = 0;
+#pragma unroll
+                    for (int a = 0; a < 5; ++a) {
+                        H[sym<NZ>(Z_ED, Z_MX + zmap[a])] += u1 * he[a];
+#pragma unroll
+                        for (int b = a; b < 5; ++b, ++c) H[sym<NZ>(Z_MX + zmap[a], Z_MX + zmap[b])] += u1 * h1[c];
+                    }
+                }
+#pragma unroll
+                for (int a = 0; a < 6; ++a)
+#pragma unroll
+                    for (int b = a; b < 6; ++b) {
+                        R v = bd1[a] * dg1[b];
+                        if (a < 2 && b < 2) v += b0 * d0[a] * d0[b] + u0 * h0[a + b];
+                        H[sym<NZ>(Z_MX + a, Z_MX + b)] += v;
+                    }
             }
-            bd1[z] = b1 * dg1[z];
+            // ---- the 32 pixels' sums in R (a reduce-scatter), added to the part's in FP64
+            warp_reduce_scatter(out, lane);
+            sums[2 * lane] += (double)out[0];
+            sums[2 * lane + 1] += (double)out[1];
+            if (lane < HV - 64) sums[64 + lane] += (double)(lane == 0 ? out[64] : out[65]);
         }
-        // mean / shape block: u0 d2g0 + b0 dg0 dg0' + u1 d2g1 + b1 dg1 dg1', d2g1 over
-        // (mx, my, e_dev, Gxx, Gxy, Gyy) from h1 (packed without e_dev) and he (the e_dev row;
-        // its diagonal is zero)
-        const int zmap[5] = {0, 1, 3, 4, 5};   // position without e_dev -> position among the six
-        {
-            int c = 0;
-#pragma unroll
-            for (int a = 0; a < 5; ++a) {
-                H[sym<NZ>(Z_ED, Z_MX + zmap[a])] += u1 * he[a];
-#pragma unroll
-                for (int b = a; b < 5; ++b, ++c) H[sym<NZ>(Z_MX + zmap[a], Z_MX + zmap[b])] += u1 * h1[c];
-            }
-        }
-#pragma unroll
-        for (int a = 0; a < 6; ++a)
-#pragma unroll
-            for (int b = a; b < 6; ++b) {
-                R v = bd1[a] * dg1[b];
-                if (a < 2 && b < 2) v += b0 * d0[a] * d0[b] + u0 * h0[a + b];
-                H[sym<NZ>(Z_MX + a, Z_MX + b)] += v;
-            }
+        __syncwarp();
+        double* rec = a.part + (size_t)(cur - n_term) * HV;
+        for (int i = lane; i < HV; i += 32) rec[i] = sums[i];
+        next = __shfl_sync(0xffffffffu, claim, 0);
+        next_patch = patch_of(next);
+        __syncwarp();
     }
-    // ---- CTA reduction: in R within a warp (a reduce-scatter), FP64 across warps
-    const int lane = t & 31, warp = t >> 5;
-    double(*red)[HV] = reinterpret_cast<double(*)[HV]>(smem + Lay::rows);
-    warp_reduce_scatter(out, lane);
-    __syncthreads();   // every warp is past its reads of the rows
-    red[warp][2 * lane] = (double)out[0];
-    red[warp][2 * lane + 1] = (double)out[1];
-    if (lane < HV - 64) red[warp][64 + lane] = (double)(lane == 0 ? out[64] : out[65]);
     __syncthreads();
-    for (int i = t; i < HV; i += blockDim.x) {
-        double s = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][i];
-        part[(size_t)rec * HV + i] = s;
+    if (threadIdx.x == 0) {
+        // the last CTA resets the queue for the next launch
+        __threadfence();
+        if (atomicAdd(a.queue + 1, 1) == (int)gridDim.x - 1) {
+            a.queue[0] = 0;
+            a.queue[1] = 0;
+            __threadfence();
+        }
     }
 }
 
@@ -943,21 +888,23 @@ __device__ __forceinline__ int w_factor(int band, int j) {
     return j < P_C2 ? beta : beta * beta;
 }
 
-// One CTA per source, two warps per band: a warp takes every second patch of its band, adds
-// the 66 sums of the patch's records (in order), maps them to w (X = H_z J, then J' X, J at
-// most three entries per column) and adds the result to the warp's shared accumulator; then
-// the block is spread and added to the -KL terms that source_terms left in hess_out.
+// One CTA per source, two warps per band, which add the parts of a patch half and half and take
+// turns to map the 66 sums to w (X = H_z J, then J' X, J at most three entries per column) and
+// to add the result to the warp's shared accumulator; then the block is spread and added to the -KL terms that source_terms left in hess_out.
 // Latency-bound, so the patches of a source run side by side and a patch costs about 50 FP64
 // instructions; per-patch loops over the 44 x 44 entries with the KL and its Hessian in the
-// same CTA took 119 us for 500 sources and 49 us for 64.
+// same CTA took 119 us for 500 sources and 49 us for 64, this 31 and 22.
+// barrier of a band's two warps
+__device__ __forceinline__ void pair_barrier(int band) { asm volatile("bar.sync %0, 64;" ::"r"(band + 1) : "memory"); }
+
 constexpr int FH_SPLIT = 2, FH_WARPS = 5 * FH_SPLIT, FH_THREADS = 32 * FH_WARPS;
 constexpr int NPIX = P_K;                         // parameters that the pixels depend on
 constexpr int NPIXH = NPIX * (NPIX + 1) / 2;
 __device__ const PackedTriangle<NPIX> g_pix = packed_triangle<NPIX>();
 __device__ const PackedTriangle<NY> g_ypk = packed_triangle<NY>();
 
-__global__ void __launch_bounds__(FH_THREADS)
-k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __restrict__ patch_off,
+__global__ void __launch_bounds__(FH_THREADS, 4)
+k_finalize_hess(int n_src, int hchunk, const PatchGeo* __restrict__ geo, const int32_t* __restrict__ patch_off,
                 const ImgMeta* __restrict__ img, const double* __restrict__ part, const double* __restrict__ hsrc,
                 double* __restrict__ local_out, double* __restrict__ grad_out, double* __restrict__ hess_out,
                 const int32_t* __restrict__ src_active) {
@@ -982,15 +929,15 @@ k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __re
         const int pl = pb + lane;
         unsigned mine = __ballot_sync(0xffffffffu, pl < p1 && img[geo[pl < p1 ? pl : p0].img].band == band);
         for (; mine; mine &= mine - 1) {
-            if ((seen++ & (FH_SPLIT - 1)) != half) continue;
             const int p = pb + __ffs(mine) - 1;
             const PatchGeo g = geo[p];
             const double* A = img[g.img].A;
-            // the patch's records in order (items cut into HCHUNK-pixel parts, so one per HCHUNK
-            // pixels), loaded four at a time before any is added
+            // the patch's parts, each warp of the band half of them in order, loaded four at a
+            // time before any is added; the two sums meet in the warp whose turn the patch is
             double v[3] = {0.0, 0.0, 0.0};
-            const int r0 = g.item0 * HSPLIT, i1 = r0 + (g.w * g.h + HCHUNK - 1) / HCHUNK;
-            for (int i0 = r0; i0 < i1; i0 += 4) {
+            const int np = (g.w * g.h + hchunk - 1) / hchunk, mid = g.hpart0 + (np + 1) / 2;
+            const int i1 = half ? g.hpart0 + np : mid;
+            for (int i0 = half ? mid : g.hpart0; i0 < i1; i0 += 4) {
                 double x[4][3];
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
@@ -1004,6 +951,18 @@ k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __re
 #pragma unroll
                         for (int c = 0; c < 3; ++c) v[c] += x[u][c];
             }
+            const bool turn = (seen++ & 1) == half;
+            if (!turn)
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    if (lane + 32 * c < HV) sy[warp][lane + 32 * c] = v[c];
+            pair_barrier(band);
+            if (turn)
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    if (lane + 32 * c < HV) v[c] += sy[band + 5 * (1 - half)][lane + 32 * c];
+            pair_barrier(band);   // the other warp may write its sums of the next patch
+            if (!turn) continue;
             // the shape derivatives through the patch's map
             for (int i = lane; i < 36; i += 32)
                 sg[warp][i] = a_transform(A, rec + HR_DW + 3 * (i / 3), i % 3);
@@ -1117,22 +1076,50 @@ k_finalize_hess(int n_src, const PatchGeo* __restrict__ geo, const int32_t* __re
 template <class R>
 static cudaError_t hess_pixels(const DevProblem& P, const R* tbl, const double* d_theta, double* d_hess,
                                cudaStream_t st) {
-    const SourceTerms src{P.n_src, d_theta, P.model, P.hsrc, P.kl, d_hess, P.status};
-    const int grid = P.n_item * HSPLIT + (P.n_src + TERM_SRC - 1) / TERM_SRC;
+    HessArgs<R> a{};
+    a.parts = P.hitems;
+    a.n_part = P.n_hitem;
+    a.img = P.img;
+    a.geo = P.geo;
+    a.n_comp = P.npsf_max * P.nprof;
+    a.nprof = P.nprof;
+    a.n_exp = P.model_ne;
+    a.pixels = P.pixels;
+    a.sky_map = P.sky_map;
+    a.tbl = tbl;
+    a.hframe = (const float*)P.tbl64;
+    a.single = P.single;
+    a.emap = (const R*)P.emap;
+    a.vmap = (const R*)P.vmap;
+    a.part = P.item_part;
+    a.src_active = P.src_active;
+    a.queue = P.hqueue;
+    a.src = SourceTerms{P.n_src, d_theta, P.model, P.hsrc, P.kl, d_hess, P.status};
+    // resident CTAs per SM: the registers allow 4 (FP32) or 2, the shared memory (228 KB, 1 KB of
+    // it the system's per CTA) perhaps fewer
+    const int bytes = HessLay<R>(a.n_comp).bytes();
+    const int per_sm = std::max(1, std::min(sizeof(R) == 8 ? 2 : 4, 228 * 1024 / (bytes + 1024)));
+    const int64_t tasks = 2LL * P.n_src + P.n_hitem;
+    const int grid = (int)std::min<int64_t>((tasks + HESS_WARPS - 1) / HESS_WARPS, (int64_t)per_sm * sm_count());
     if (grid == 0) return cudaSuccess;
-    k_hess<R><<<grid, HCHUNK, HessLay<R>::bytes, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.pixels, P.sky_map,
-                                                      tbl, P.single, (const R*)P.emap, (const R*)P.vmap, P.item_part,
-                                                      P.src_active, src);
+    auto* fn = k_hess<R, 0, 0>;
+    if constexpr (sizeof(R) == 4)
+        if (P.model_ne == 6 && P.model_nd == 8) fn = k_hess<R, 6, 8>;
+    fn<<<grid, 32 * HESS_WARPS, bytes, st>>>(a);
     return cudaGetLastError();
 }
 
 // shared-memory limits of the Hessian kernels on the current device, set at problem
 // creation (outside any stream capture)
 cudaError_t prime_hess_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(k_hess<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         HessLay<float>::bytes);
+    constexpr int most = MAXPSF * MAXPROF;
+    cudaError_t e = cudaSuccess;
+    for (auto* fn : {k_hess<float, 0, 0>, k_hess<float, 6, 8>})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, HessLay<float>(most).bytes());
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_hess<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, HessLay<double>::bytes);
+        e = cudaFuncSetAttribute(k_hess<double, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 HessLay<double>(most).bytes());
     return e;
 }
 
@@ -1145,7 +1132,7 @@ cudaError_t launch_hess_pixels(const DevProblem& P, int precision, const double*
 cudaError_t launch_finalize_hess(const DevProblem& P, double* d_local, double* d_grad, double* d_hess,
                                  cudaStream_t st) {
     if (P.n_src == 0) return cudaSuccess;
-    k_finalize_hess<<<P.n_src, FH_THREADS, 0, st>>>(P.n_src, P.geo, P.patch_off, P.img, P.item_part, P.hsrc, d_local,
+    k_finalize_hess<<<P.n_src, FH_THREADS, 0, st>>>(P.n_src, P.hchunk, P.geo, P.patch_off, P.img, P.item_part, P.hsrc, d_local,
                                                     d_grad, d_hess, P.src_active);
     return cudaGetLastError();
 }

@@ -82,15 +82,18 @@ constexpr int H_A0 = 0, H_A1 = 1, H_EL0 = 2, H_EL20 = 3, H_EL1 = 4, H_EL21 = 5, 
 // component 12 + 12 per pair); each profile group padded to an even count
 constexpr int ZFULL_FLOATS = 16 + MAXPSF * (8 + ((MAXPROF + 2) / 2) * 8) + MAXPSF * (12 + ((MAXPROF + 2) / 2) * 12);
 constexpr int CHUNK = 256;   // pixels per work item (one CTA)
-// The Hessian pass takes an item in parts of HCHUNK pixels, a CTA and a record of item_part
-// each: its CTAs are heavy in registers, and small ones overlap one's set-up and reduction
-// with the others' pixels and even out the last wave.
-constexpr int HCHUNK = 128, HSPLIT = CHUNK / HCHUNK;
+// The Hessian pass cuts a patch into parts of hchunk pixels, a task of one warp each: as many
+// pixels as leave every resident warp (16 per SM) three parts or more, so that the last ones to
+// finish hold little, and at least a warp's 32.  (A part costs its table's copy and its rows.)
+inline int hess_chunk(int64_t n_sp, int n_sm) {
+    int c = 128;
+    while (c > 32 && n_sp / c < 3LL * 16 * n_sm) c /= 2;
+    return c;
+}
 // Its ten variables z per (source, patch) (hess_kernels.cu) and a part's record: ll, d/dz, the
 // packed upper triangle of d2/dz2
 enum : int { Z_K0 = 0, Z_K1, Z_Q0, Z_Q1, Z_MX, Z_MY, Z_ED, Z_GXX, Z_GXY, Z_GYY, NZ };
 constexpr int HV = 1 + NZ + NZ * (NZ + 1) / 2;
-constexpr int ITEM_PART = HSPLIT * HV > NPART ? HSPLIT * HV : NPART;   // doubles of item_part per item
 constexpr int ZIMAX = 512;   // most pixels per item of the FP32 value / gradient kernel
 constexpr int ZMAXC = 4;     // other covering patches named inline in such an item's queue record
 constexpr int ZSTAGE = 12;   // other covering patches whose value records an item stages (more are
@@ -128,11 +131,30 @@ struct PatchGeo {
     int32_t img, x0, y0, w, h, src;
     int64_t sp_off;          // offset in the per-(source, pixel) buffers
     int32_t item0, nitem;    // work items covering this patch
+    int32_t hpart0, pad;     // its first part of the Hessian pass (hchunk pixels each, in order)
 };
 
 struct WorkItem {
     int32_t patch, q0, n, src;
 };
+
+// One part of the Hessian pass: n <= hchunk pixels of a patch from q0, with what its kernel
+// needs of the patch and its image (w: the patch's width, W: the image's; m0: the patch's
+// origin in the pixel and map buffers; sp0: its per-(source, pixel) offset)
+struct alignas(16) HItem {
+    int32_t patch, q0, n, src;
+    int32_t w, W, npsf, pad;
+    int64_t m0, sp0;
+};
+// appends the parts of patch p (its hpart0 set to the first)
+template <class Vec>
+inline void push_parts(Vec& v, PatchGeo& g, int p, const ImgMeta& im, int hchunk) {
+    g.hpart0 = (int32_t)v.size();
+    const int npx = g.w * g.h;
+    for (int q0 = 0; q0 < npx; q0 += hchunk)
+        v.push_back(HItem{p, q0, npx - q0 < hchunk ? npx - q0 : hchunk, g.src, g.w, im.W, im.npsf, 0,
+                          im.px_off + (int64_t)g.y0 * im.W + g.x0, g.sp_off});
+}
 
 // One item of the FP32 value / gradient kernel: n <= ZIMAX consecutive pixel records of
 // one patch (from pix; the patch's multiply covered pixels come first, nm of them), its
@@ -288,6 +310,8 @@ struct DevProblem {
     const float* sky_map;
     const PatchGeo* geo;
     const WorkItem* items;
+    const HItem* hitems;     // the Hessian pass's parts
+    int32_t n_hitem, hchunk;
     const Tile* tiles;
     const int32_t* tile_list;
     const int32_t* tile_grid;
@@ -301,7 +325,7 @@ struct DevProblem {
     void* vmap;
     const uint8_t* single;   // per (source, pixel): 1 when no other patch covers the pixel (nullable)
     double* item_ll;         // per work item: ll summed over its singly covered pixels
-    double* item_part;
+    double* item_part;       // per item (value / gradient) or part (Hessian) sums
     double* tile_ll;
     double* kl;
     double* kl_grad;         // [n_src][44] KL gradient, written by k_prep (nullable: no KL in prep)
@@ -331,6 +355,7 @@ struct DevProblem {
     int32_t tune_items;          // item kernel variant, 1 .. 5 (pixels per thread, CTAs per SM,
                                  // unroll; item_kernels.cu); 0 = the default, 1
     int32_t model_ne, model_nd;     // exp / dev profile components of the model
+    int32_t* hqueue;         // [2] the Hessian pass's work queue (next part, finished CTAs), 0 between launches
     int32_t* queue;          // [2] work queue of the FP64 / Hessian map pass's persistent variants
                              // (next item, finished CTAs), 0 between launches (nullable: those
                              // variants fall back to one CTA per item)
@@ -398,10 +423,24 @@ cudaError_t prime_hess_kernels();
 // total = tile ll sums + item ll sums - KL (after the gather and every item ll)
 cudaError_t launch_total(const DevProblem& P, double* d_total, cudaStream_t st);
 // tables (and, with_kl, the KL value / gradient and the domain check) of every source
+// (hess, FP32: and the Hessian pass's frames, in the place of the FP64 tables)
 cudaError_t launch_prep(const DevProblem& P, const double* d_theta, int precision,
-                        cudaStream_t st, bool with_kl = true);
+                        cudaStream_t st, bool with_kl = true, bool hess = false);
+// multiprocessors of the current device
+inline int sm_count() {
+    static int n = 0;
+    if (n == 0) {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+            n = v;
+        else
+            n = 1;
+    }
+    return n;
+}
 // E_s and Var_s at every item pixel, singly covered ones (P.single) finished into the maps;
-// multi_only (FP64): at the multiply covered pixels alone, the others being left to the
+// multi_only: at the multiply covered pixels alone, the others being left to the
 // kernels that evaluate the source there anyway
 cudaError_t launch_contrib(const DevProblem& P, int precision, cudaStream_t st, bool multi_only = false);
 // The FP32 value (MODE_LL) or value + gradient (MODE_GRAD) evaluation (item_kernels.cu):

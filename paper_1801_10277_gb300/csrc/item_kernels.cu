@@ -1257,19 +1257,6 @@ cudaError_t items_launch(const ItemArgs& a, int code, int n_sm, cudaStream_t st)
     }
 }
 
-int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            n = v;
-        else
-            n = 1;
-    }
-    return n;
-}
-
 template <int MODE>
 cudaError_t items_setup_mode() {
     cudaError_t e = cudaSuccess;
