@@ -4,22 +4,24 @@
 // source's step is a Newton step with its exact Hessian inside a trust region
 // (Nocedal & Wright, Chapter 4).
 //
-// Per colour the batch runs in lock step; one iteration is
-//   k_prep / k_contrib   E_s, Var_s of every batch source at theta
+// Every source's E_s / Var_s are formed once per precision phase (k_prep, k_contrib) and kept
+// current: each batch writes back the ones it moved.  Per batch, k_batch_start (free
+// coordinates, trust-region state), E_other / Var_other at its pixels (k_other) and its own
+// tables and E_s / Var_s; then the sources run in lock step, one iteration being
 //   k_batch_maps         E = E_other + E_s and Var at the batch pixels (patches of one
-//                        colour are disjoint, so every pixel has one writer)
+//                        batch are disjoint, so every pixel has one writer); a source whose
+//                        last candidate was accepted first takes its E_s, Var_s and tables
 //   k_hess / k_finalize_hess   ELBO_s, gradient and Hessian (44 x 44)
 //   k_tr_step            one CTA per source: free coordinates (41), the trust-region
 //                        subproblem (More-Sorensen with Cholesky factorisations), the
 //                        candidate point
-//   k_prep / k_contrib   E_s, Var_s at the candidate
+//   k_prep / k_contrib   tables, E_s, Var_s at the candidate
 //   k_batch_dll          per-pixel change of the log-likelihood (stable difference form)
 //   k_tr_accept          actual / predicted gain, radius update, accept or reject
-// The iteration is captured once per colour as a CUDA graph and replayed; the host
-// reads one counter (sources still iterating) per replay.  A per-source mask
-// (k_mark_active, after the step and after the acceptance) lets every pixel kernel skip
-// the items of a source that has stopped iterating, so a replay costs in proportion to
-// the sources still active.
+// The iteration is captured once per batch as a CUDA graph and replayed; the host
+// reads one counter (sources still iterating) per replay.  A per-source mask (written by the
+// step and by the acceptance) lets every pixel kernel skip the items of a source that has
+// stopped iterating, so a replay costs in proportion to the sources still active.
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -31,6 +33,7 @@
 #include "internal.cuh"
 #include "problem.cuh"
 #include "source_math.cuh"
+#include "whiten.cuh"
 
 namespace cel {
 
@@ -76,31 +79,22 @@ __device__ void free_to_theta_warp(const double* t, double* th) {
     if (lane < 16) th[P_K + 8 * i + d] = K_LO + ex / den;
 }
 
-__device__ void theta_to_free(const double* th, double* t) {
+// free coordinate a of theta
+__device__ double theta_to_free(const double* th, int a) {
     // a fitted parameter can sit on its bound after rounding (the sigmoid of a large free
     // coordinate is 1 in FP64); the fraction is kept 1e-15 inside so the free coordinate
     // stays finite and a fit can resume from its own result
-    auto logit = [](double p) {
-        p = fmin(fmax(p, 1e-15), 1.0 - 1e-15);
+    if (a == 2 || a == 3 || a == 26) {
+        const double lo = a == 26 ? A_LO : BOX_LO, hi = a == 26 ? A_HI : BOX_HI;
+        const double p = fmin(fmax((th[a] - lo) / (hi - lo), 1e-15), 1.0 - 1e-15);
         return log(p / (1.0 - p));
-    };
-    t[0] = th[0];
-    t[1] = th[1];
-    t[2] = logit((th[P_EDEV] - BOX_LO) / (BOX_HI - BOX_LO));
-    t[3] = logit((th[P_AXIS] - BOX_LO) / (BOX_HI - BOX_LO));
-    t[4] = th[P_ANGLE];
-    t[5] = log(th[P_SCALE]);
-    t[6] = th[P_R1];
-    t[7] = th[P_R1 + 1];
-    t[8] = log(th[P_R2]);
-    t[9] = log(th[P_R2 + 1]);
-    for (int j = 0; j < 8; ++j) {
-        t[10 + j] = th[P_C1 + j];
-        t[18 + j] = log(th[P_C2 + j]);
     }
-    t[26] = logit((th[P_A] - A_LO) / (A_HI - A_LO));
-    for (int i = 0; i < 2; ++i)
-        for (int e = 0; e < 7; ++e) t[27 + 7 * i + e] = log(th[P_K + 8 * i + e] / th[P_K + 8 * i + 7]);
+    if (a >= 27) {
+        const int i = a >= 34, e = a - 27 - 7 * i;
+        return log(th[P_K + 8 * i + e] / th[P_K + 8 * i + 7]);
+    }
+    if (a == P_SCALE || a == P_R2 || a == P_R2 + 1 || a >= P_C2) return log(th[a]);
+    return th[a];
 }
 
 // ------------------------------------------------------------------------------------
@@ -155,25 +149,69 @@ __global__ void k_other(const WorkItem* __restrict__ bitems, const PatchGeo* __r
     vo[g.sp_off + q] = V;
 }
 
-// E, Var maps at the batch pixels from E_other and the batch sources' own terms
+struct TrState {
+    double delta;   // trust radius (free coordinates)
+    double pred;    // predicted gain of the candidate
+    double pnorm;   // |p|
+    double f;       // ELBO_s at theta
+    double kl;      // KL at theta
+    int32_t status; // ST_*
+    int32_t iters;
+    int32_t cand;   // a candidate was produced this iteration
+    int32_t moved;  // the last candidate was accepted: its E_s, Var_s and tables are theta's
+    double lam;     // multiplier of the last boundary step (warm start of the next), 0 inside
+};
+
+// E, Var maps at the batch pixels from E_other and the batch sources' own terms; a source
+// whose last candidate was accepted takes the candidate's terms (ce, cv), and its patches'
+// tables (n_tbl entries, FP32: and n_frame of the Hessian pass's frames), first
 template <class R>
 __global__ void k_batch_maps(const WorkItem* __restrict__ bitems, const PatchGeo* __restrict__ bgeo,
                              const ImgMeta* __restrict__ img, const R* __restrict__ eo,
-                             const R* __restrict__ vo, const R* __restrict__ se,
-                             const R* __restrict__ sv, R* __restrict__ emap, R* __restrict__ vmap,
-                             const int32_t* __restrict__ src_active) {
+                             const R* __restrict__ vo, R* __restrict__ se, R* __restrict__ sv,
+                             const R* __restrict__ ce, const R* __restrict__ cv, R* __restrict__ emap,
+                             R* __restrict__ vmap, const int32_t* __restrict__ src_active,
+                             const TrState* __restrict__ st, R* __restrict__ tbl, const R* __restrict__ ctbl,
+                             int n_tbl, float* __restrict__ frame, const float* __restrict__ cframe, int n_frame) {
     const WorkItem it = bitems[blockIdx.x];
     const int t = threadIdx.x;
-    if (t >= it.n) return;
     const PatchGeo g = bgeo[it.patch];
     if (!src_active[g.src]) return;   // a converged source's maps do not change
+    const bool moved = st[g.src].moved != 0;
+    if (moved && it.q0 == 0) {
+        const size_t o = (size_t)it.patch * TBL_STRIDE, h = (size_t)it.patch * HF_STRIDE;
+        for (int i = t; i < n_tbl; i += blockDim.x) tbl[o + i] = ctbl[o + i];
+        for (int i = t; i < n_frame; i += blockDim.x) frame[h + i] = cframe[h + i];
+    }
+    if (t >= it.n) return;
     const ImgMeta& im = img[g.img];
     const int q = it.q0 + t;
     const int yy = q / g.w, xx = q - yy * g.w;
     const int64_t m = im.px_off + (int64_t)(g.y0 + yy) * im.W + (g.x0 + xx);
     const int64_t b = g.sp_off + q;
-    emap[m] = eo[b] + se[b];
-    vmap[m] = vo[b] + sv[b];
+    const R e = moved ? ce[b] : se[b], v = moved ? cv[b] : sv[b];
+    if (moved) {
+        se[b] = e;
+        sv[b] = v;
+    }
+    emap[m] = eo[b] + e;
+    vmap[m] = vo[b] + v;
+}
+
+// the batch's E_s / Var_s at its final parameters into the whole problem's
+template <class R>
+__global__ void k_batch_end(const WorkItem* __restrict__ bitems, const PatchGeo* __restrict__ bgeo,
+                            const R* __restrict__ se, const R* __restrict__ sv, const R* __restrict__ ce,
+                            const R* __restrict__ cv, const TrState* __restrict__ st, R* __restrict__ spE,
+                            R* __restrict__ spV) {
+    const WorkItem it = bitems[blockIdx.x];
+    const int t = threadIdx.x;
+    if (t >= it.n) return;
+    const PatchGeo g = bgeo[it.patch];
+    const int64_t b = g.sp_off + it.q0 + t, o = g.whole_sp + it.q0 + t;
+    const bool moved = st[g.src].moved != 0;
+    spE[o] = moved ? ce[b] : se[b];
+    spV[o] = moved ? cv[b] : sv[b];
 }
 
 // per-item sum of ll(E', V') - ll(E, V) at the candidate, in a difference form that
@@ -214,9 +252,23 @@ __global__ void k_batch_dll(const WorkItem* __restrict__ bitems, const PatchGeo*
     }
 }
 
-__global__ void k_to_free(int nb, const double* __restrict__ th, double* __restrict__ t) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nb) theta_to_free(th + (size_t)NP * b, t + (size_t)NT * b);
+// A batch's start, one warp per source: its parameters, free coordinates (a lane each: the
+// logarithms side by side), trust-region state and mask
+__global__ void __launch_bounds__(32)
+k_batch_start(int nb, const int32_t* __restrict__ bsrc, const double* __restrict__ theta, double* __restrict__ bth,
+              double* __restrict__ t, TrState* __restrict__ st, int32_t* __restrict__ act, double delta0) {
+    const int b = blockIdx.x, lane = threadIdx.x;
+    if (b >= nb) return;
+    const double* th = theta + (size_t)NP * bsrc[b];
+    for (int i = lane; i < NP; i += 32) bth[(size_t)NP * b + i] = th[i];
+    for (int i = lane; i < NT; i += 32) t[(size_t)NT * b + i] = theta_to_free(th, i);
+    if (lane == 0) {
+        TrState S{};
+        S.delta = delta0;
+        S.status = ST_ACTIVE;
+        st[b] = S;
+        act[b] = 1;
+    }
 }
 
 // ------------------------------------------------------------------------------------
@@ -224,24 +276,12 @@ __global__ void k_to_free(int nb, const double* __restrict__ th, double* __restr
 
 constexpr int TR_THREADS = 128;
 constexpr int TRN = NT;   // 41
-// k_tr_step's dynamic shared memory: the source's 44 x 44 Hessian and H T (44 x 41)
+// k_tr_step's dynamic shared memory: the source's 44 x 44 Hessian and H T (44 x 41); later the
+// FP32 copies of the multiplier search
 constexpr size_t TR_DYN_BYTES = sizeof(double) * (NP * NP + NP * TRN);
 
-struct TrState {
-    double delta;   // trust radius (free coordinates)
-    double pred;    // predicted gain of the candidate
-    double pnorm;   // |p|
-    double f;       // ELBO_s at theta
-    double kl;      // KL at theta
-    int32_t status; // ST_*
-    int32_t iters;
-    int32_t cand;   // a candidate was produced this iteration
-    int32_t pad;
-    double lam;     // multiplier of the last boundary step (warm start of the next), 0 inside
-};
-
-// Packed lower-triangle order of side 40 (every trailing triangle of n = 41), copied
-// into shared memory by each CTA
+// Packed lower-triangle order of side 40 (the trailing triangles of the bordered matrix
+// below), copied into shared memory by each CTA
 constexpr int PK_N = (TRN - 1) * TRN / 2;
 __device__ const PackedTriangle<TRN - 1> g_pk = packed_triangle<TRN - 1>();
 
@@ -249,92 +289,127 @@ __device__ void packed_table(uint16_t* pk) {
     for (int idx = threadIdx.x; idx < PK_N; idx += blockDim.x) pk[idx] = g_pk.v[idx];
 }
 
-// Cholesky of (B + lam I) into L (lower, row-major n x n, n <= TRN); returns success to
-// all threads.  Right-looking, two barriers per column: step k scales column k by the
-// pivot's 1 / sqrt(d_k) (its diagonal becomes sqrt(d_k)), then updates the trailing
-// triangle with one FMA per entry, L_ij -= L_ik L_jk (entries dealt out in packed order,
-// pk).  The thread that updates (k + 1, k + 1), the next pivot, takes its FP64 rsqrt at
-// once, so the pivot is ready at the barrier.  On GB300's narrow FP64 pipe the
-// factorisation is bound by its FP64 instruction count (a warp instruction costs the
-// same however few lanes are active), so each pivot's square root and reciprocal come
-// from one thread and the update is a single FMA.
-// T = double, or float for the multiplier search (the same steps, FP32's reciprocal
-// square root).
-__device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
-__device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
-
-template <class T>
-__device__ bool block_chol(const T* B, T lam, T* L, int n, int* flag, T* rcp, const uint16_t* pk) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    auto pivot = [&](int k, T d) {
-        if (!(d > (T)0) || !isfinite(d)) {
-            *flag = 0;
-        } else {
-            const T r = rsqrt_t(d);
-            rcp[k] = r;           // 1 / sqrt(d)
-            rcp[n + k] = r * r;   // 1 / d
-        }
-    };
-    for (int i = tid; i < n * n; i += nt) {
-        const int r = i / n, c = i - r * n;
-        L[i] = (c <= r) ? B[i] + (r == c ? lam : (T)0) : (T)0;
-    }
-    if (tid == 0) {
-        *flag = 1;
-        pivot(0, L[0]);   // this thread wrote L[0]
-    }
-    __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        if (!*flag) return false;
-        const T r = rcp[k];
-        for (int i = k + tid; i < n; i += nt) L[i * n + k] *= r;
-        __syncthreads();
-        const int m = n - k - 1;
-        const int cnt = m * (m + 1) / 2;
-        for (int idx = tid; idx < cnt; idx += nt) {
-            const int ab = pk[idx];
-            const int i = k + 1 + (ab >> 8), j = k + 1 + (ab & 255);
-            const T v = fma(-L[i * n + k], L[j * n + k], L[i * n + j]);
-            L[i * n + j] = v;
-            if (idx == 0) pivot(k + 1, v);
-        }
-        __syncthreads();
-    }
-    return true;
+// 1 / d for d > 0.  FP64: from the FP32 reciprocal y of d's leading bits (integer
+// conversions: FP64 ones would queue on the FP64 pipe), 1 / d = y (1 + e + e^2) with
+// e = 1 - d y below 2^-22 (relative error e^3): three dependent FP64 operations.
+__device__ __forceinline__ double recip_pos(double d) {
+    const int hi = __double2hiint(d), ex = (hi >> 20) - 1023;
+    if (ex < -100 || ex > 100) return 1.0 / d;
+    const float m = __int_as_float(0x3F800000 | ((hi & 0xFFFFF) << 3) | ((unsigned)__double2loint(d) >> 29));
+    const int y = __float_as_int(__frcp_rn(m));   // of d 2^-ex, in (1/2, 1]
+    const double r = __hiloint2double(((y >> 3) + 0x38000000) - (ex << 20), y << 29);
+    const double e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
-// Warp-level triangular solves (every lane of the calling warp calls them): lane l holds
-// rows l and l + 32 of the right-hand side; one column of L per step (column-oriented
-// substitution), the solved entry broadcast by shuffle.  invd[k] = 1 / L[k][k].  The
-// arrays must not overlap.
+// Factorisation of B + lam I bordered by a right-hand side, n <= TRN: A has n + 1 rows of n
+// (lower part).  FP64: L D L', rd[k] = 1 / d_k, L's unit diagonal not stored; FP32: Cholesky,
+// rd[k] = 1 / L_kk.  Row n receives the solution of L D w = rhs (FP32: L w = rhs).  Returns
+// whether every pivot is positive (rd[k] = 0 marks one that is not: a slot of its own per
+// column, so that no warp can see the mark of a later column and leave the loop ahead of the
+// others).
+// Right-looking with the next column ahead of the rest: at step k warp 0 updates column
+// k + 1, takes its pivot's reciprocal (root) and scales the column while the other warps
+// update the columns after it, so a column costs one barrier and, in FP64, a chain of five
+// dependent operations (update, three for the reciprocal, scale) of about 70 cycles each:
+// that chain is the cost on GB300.  FP32 keeps the square root: its entries are formed by the
+// operations of a plain Cholesky factorisation, and the multipliers of the search with them.
+// cb: 2 (n + 1) entries, columns k and k + 1 as the updates multiply by them (FP64: unscaled).
+__device__ __forceinline__ double pivot_factor(double d) { return recip_pos(d); }
+__device__ __forceinline__ float pivot_factor(float d) { return rsqrtf(d); }
+
 template <class T>
-__device__ void warp_fwd(const T* __restrict__ L, const T* __restrict__ invd, const T* __restrict__ b,
+__device__ bool block_factor(const T* B, T lam, const T* rhs, T* A, T* cb, T* rd, int n, const uint16_t* pk) {
+    constexpr bool LDL = sizeof(T) == 8;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    for (int r = tid >> 5; r <= n; r += nt >> 5)   // a row per warp
+        for (int c = lane; c <= r && c < n; c += 32)
+            A[r * n + c] = r == n ? rhs[c] : r == c ? B[r * n + c] + lam : B[r * n + c];
+    __syncthreads();
+    // column k by warp 0: v0, v1 its entries at rows lane and lane + 32 (rows k .. n in use)
+    auto finish = [&](int k, T v0, T v1) {
+        const T d = __shfl_sync(0xffffffffu, k < 32 ? v0 : v1, k & 31);
+        const T r = d > (T)0 && isfinite(d) ? pivot_factor(d) : (T)0;
+        T* c = cb + (k & 1) * (n + 1);
+        if (lane > k && lane <= n) {
+            const T l = v0 * r;
+            c[lane] = LDL ? v0 : l;
+            A[lane * n + k] = l;
+        }
+        if (lane + 32 > k && lane + 32 <= n) {
+            const T l = v1 * r;
+            c[lane + 32] = LDL ? v1 : l;
+            A[(lane + 32) * n + k] = l;
+        }
+        if (lane == 0) rd[k] = r;
+    };
+    auto entry = [&](int i, int k) { return i >= k && i <= n ? A[i * n + k] : (T)0; };
+    if (tid < 32) finish(0, entry(lane, 0), entry(lane + 32, 0));
+    __syncthreads();
+    for (int k = 0; k < n - 1; ++k) {
+        if (rd[k] == (T)0) return false;
+        const T* c = cb + (k & 1) * (n + 1);
+        if (tid < 32) {
+            const T f = c[k + 1];
+            T v0 = entry(lane, k + 1), v1 = entry(lane + 32, k + 1);
+            if (lane > k && lane <= n) v0 = fma(-A[lane * n + k], f, v0);
+            if (lane + 32 > k && lane + 32 <= n) v1 = fma(-A[(lane + 32) * n + k], f, v1);
+            finish(k + 1, v0, v1);
+        } else {
+            // rows k + 2 .. n, columns k + 2 .. n - 1: the packed triangle but its last corner
+            const int m = n - k - 1, cnt = m * (m + 1) / 2 - 1, b0 = k + 2, step = nt - 32;
+            for (int idx = tid - 32; idx < cnt; idx += 2 * step) {
+                const int p0 = pk[idx], p1 = pk[min(idx + step, cnt - 1)];
+                const int i0 = b0 + (p0 >> 8), j0 = b0 + (p0 & 255), i1 = b0 + (p1 >> 8), j1 = b0 + (p1 & 255);
+                const T a0 = A[i0 * n + j0], l0 = A[i0 * n + k], c0 = c[j0];
+                const T a1 = A[i1 * n + j1], l1 = A[i1 * n + k], c1 = c[j1];
+                A[i0 * n + j0] = fma(-l0, c0, a0);
+                if (idx + step < cnt) A[i1 * n + j1] = fma(-l1, c1, a1);
+            }
+        }
+        __syncthreads();
+    }
+    return rd[n - 1] != (T)0;
+}
+
+// Warp-level triangular solves with that L (every lane of the calling warp calls them): lane
+// l holds rows l and l + 32 of the right-hand side; one column of L per step (column-oriented
+// substitution), the solved entry broadcast by shuffle (FP32: times 1 / L_kk).  The arrays
+// must not overlap.
+template <class T>
+__device__ void warp_fwd(const T* __restrict__ L, const T* __restrict__ rd, const T* __restrict__ b,
                          T* __restrict__ y, int n) {
+    constexpr bool LDL = sizeof(T) == 8;
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
     T r0 = lane < n ? b[lane] : (T)0, r1 = lane + 32 < n ? b[lane + 32] : (T)0;
     for (int k = 0; k < n; ++k) {
-        const T rk = __shfl_sync(full, k < 32 ? r0 : r1, k & 31);
-        const T yk = rk * invd[k];
+        const T l0 = lane > k && lane < n ? L[lane * n + k] : (T)0;
+        const T l1 = lane + 32 > k && lane + 32 < n ? L[(lane + 32) * n + k] : (T)0;
+        T yk = __shfl_sync(full, k < 32 ? r0 : r1, k & 31);
+        if (!LDL) yk *= rd[k];
         if (lane == (k & 31)) y[k] = yk;
-        if (lane > k && lane < n) r0 -= L[lane * n + k] * yk;
-        if (lane + 32 > k && lane + 32 < n) r1 -= L[(lane + 32) * n + k] * yk;
+        r0 = fma(-l0, yk, r0);
+        r1 = fma(-l1, yk, r1);
     }
     __syncwarp();
 }
 
 template <class T>
-__device__ void warp_bwd(const T* __restrict__ L, const T* __restrict__ invd, const T* __restrict__ y,
+__device__ void warp_bwd(const T* __restrict__ L, const T* __restrict__ rd, const T* __restrict__ y,
                          T* __restrict__ x, int n) {
+    constexpr bool LDL = sizeof(T) == 8;
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
     T r0 = lane < n ? y[lane] : (T)0, r1 = lane + 32 < n ? y[lane + 32] : (T)0;
     for (int k = n - 1; k >= 0; --k) {
-        const T rk = __shfl_sync(full, k < 32 ? r0 : r1, k & 31);
-        const T xk = rk * invd[k];
+        const T l0 = lane < k ? L[k * n + lane] : (T)0;
+        const T l1 = lane + 32 < k ? L[k * n + lane + 32] : (T)0;
+        T xk = __shfl_sync(full, k < 32 ? r0 : r1, k & 31);
+        if (!LDL) xk *= rd[k];
         if (lane == (k & 31)) x[k] = xk;
-        if (lane < k) r0 -= L[k * n + lane] * xk;
-        if (lane + 32 < k) r1 -= L[k * n + lane + 32] * xk;
+        r0 = fma(-l0, xk, r0);
+        r1 = fma(-l1, xk, r1);
     }
     __syncwarp();
 }
@@ -358,15 +433,14 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
           const double* __restrict__ f_in, const double* __restrict__ g_in,
           const double* __restrict__ h_in, const double* __restrict__ kl_in,
           double* __restrict__ theta_c, double* __restrict__ tfree_c, TrState* __restrict__ st,
-          celeste_fit_options o, int32_t* __restrict__ active) {
+          celeste_fit_options o, int32_t* __restrict__ act) {
     const int b = blockIdx.x;
     if (b >= nb) return;
     __shared__ TrState S;
-    __shared__ double gt[TRN], Ht[TRN * TRN], L[TRN * TRN], cvec[TRN], p[TRN], w[TRN];
+    __shared__ double gt[TRN], Ht[TRN * TRN], L[(TRN + 1) * TRN], cvec[TRN], p[TRN], w[TRN];
     __shared__ double th[NP], tt[TRN], g44[NP];
-    __shared__ int tn[TRN], tj[TRN][8];
-    __shared__ double tv[TRN][8];
-    __shared__ int flag, done;
+    __shared__ double f[P_A + 1], hb[2][NP], gb[2];
+    __shared__ int done;
     __shared__ double lam_s, pn_s;
     __shared__ uint16_t pk[PK_N];
     extern __shared__ double tr_dyn[];
@@ -376,7 +450,10 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     if (tid == 0) S = st[b];
     __syncthreads();
     if (S.status != ST_ACTIVE) {
-        if (tid == 0) st[b].cand = 0;
+        if (tid == 0) {
+            st[b].cand = 0;
+            act[b] = 0;
+        }
         return;
     }
     for (int i = tid; i < NP; i += blockDim.x) {
@@ -390,74 +467,71 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     }
     packed_table(pk);
     __syncthreads();
-    // columns of T = d theta / d t
-    if (tid < TRN) {
+    // T = d theta / d t: column a < 26 has the one entry f_a at theta_a, column 26 the entries
+    // f_26, -f_26 at the two types' probabilities, and column (i, e) of the softmax p_d
+    // (delta_de - p_e) at k_id.  So for any row x over theta, (x T)_a is f_a x_a, f_26 (x_a0 -
+    // x_a1) or p_e (x_e - x.p), with x.p summed over the type's eight weights first.
+    if (tid <= P_A) {
         const int a = tid;
-        int n = 0;
-        auto put = [&](int j, double v) {
-            tj[a][n] = j;
-            tv[a][n] = v;
-            ++n;
-        };
-        if (a == 2 || a == 3) {
+        double v = 1.0;
+        if (a == 2 || a == 3 || a == P_A) {
             const double s = sigm(tt[a]);
-            put(a, (BOX_HI - BOX_LO) * s * (1.0 - s));
-        } else if (a == 5 || a == 8 || a == 9 || (a >= 18 && a < 26)) {
-            put(a, th[a]);
-        } else if (a == 26) {
-            const double s = sigm(tt[26]);
-            const double d = (A_HI - A_LO) * s * (1.0 - s);
-            put(P_A, d);
-            put(P_A + 1, -d);
-        } else if (a >= 27) {
-            const int i = (a - 27) / 7, e = (a - 27) % 7;
-            const double pe = th[P_K + 8 * i + e];
-            for (int d = 0; d < 8; ++d) {
-                const double pd = th[P_K + 8 * i + d];
-                put(P_K + 8 * i + d, pd * ((d == e ? 1.0 : 0.0) - pe));
-            }
-        } else {
-            put(a, 1.0);
+            v = (a == P_A ? A_HI - A_LO : BOX_HI - BOX_LO) * s * (1.0 - s);
+        } else if (a == 5 || a == 8 || a == 9 || a >= 18) {
+            v = th[a];
         }
-        tn[a] = n;
-        double s = 0.0;
-        for (int u = 0; u < n; ++u) s += tv[a][u] * g44[tj[a][u]];
-        gt[a] = s;
+        f[a] = v;
+    } else if (tid >= 32 && tid < 32 + 2 * NP) {
+        const int r = (tid - 32) >> 1, i = tid & 1;
+        double v = 0.0;
+        for (int d = 0; d < 8; ++d) v += th[P_K + 8 * i + d] * Hs[r * NP + P_K + 8 * i + d];
+        hb[i][r] = v;
+    } else if (tid >= 126) {
+        const int i = tid & 1;
+        double v = 0.0;
+        for (int d = 0; d < 8; ++d) v += th[P_K + 8 * i + d] * g44[P_K + 8 * i + d];
+        gb[i] = v;
     }
     __syncthreads();
-    // Ht = T' H T + sum_j g_j d2 theta_j / dt dt, T' H T as two sparse products from
-    // shared memory: X = H T, then T' X
+    auto times_T = [&](int a, const double* x, int stride, double xp0, double xp1) {
+        if (a < P_A) return f[a] * x[a * stride];
+        if (a == P_A) return f[a] * (x[P_A * stride] - x[(P_A + 1) * stride]);
+        const int i = a >= 34, e = a - 27 - 7 * i, k = P_K + 8 * i + e;
+        return th[k] * (x[k * stride] - (i ? xp1 : xp0));
+    };
+    if (tid < TRN) gt[tid] = times_T(tid, g44, 1, gb[0], gb[1]);
     for (int idx = tid; idx < NP * TRN; idx += blockDim.x) {
-        const int r = idx / TRN, c = idx - r * TRN;
-        double x = 0.0;
-        for (int v = 0; v < tn[c]; ++v) x += Hs[r * NP + tj[c][v]] * tv[c][v];
-        X[idx] = x;
+        const int r = idx / TRN;
+        X[idx] = times_T(idx - r * TRN, Hs + r * NP, 1, hb[0][r], hb[1][r]);
     }
     __syncthreads();
+    if (tid < 2 * TRN) {
+        const int c = tid >> 1, i = tid & 1;
+        double v = 0.0;
+        for (int d = 0; d < 8; ++d) v += th[P_K + 8 * i + d] * X[(P_K + 8 * i + d) * TRN + c];
+        hb[i][c] = v;
+    }
+    __syncthreads();
+    // Ht = T' (H T) + sum_j g_j d2 theta_j / dt dt
     for (int idx = tid; idx < TRN * TRN; idx += blockDim.x) {
-        const int a = idx / TRN, c = idx % TRN;
-        double s = 0.0;
-        for (int u = 0; u < tn[a]; ++u) s += tv[a][u] * X[tj[a][u] * TRN + c];
+        const int a = idx / TRN, c = idx - a * TRN;
+        double s = times_T(a, X + c, TRN, hb[0][c], hb[1][c]);
         if (a == c) {
             if (a == 2 || a == 3) {
-                const double sg = sigm(tt[a]);
-                s += g44[a] * (BOX_HI - BOX_LO) * sg * (1.0 - sg) * (1.0 - 2.0 * sg);
+                s += g44[a] * f[a] * (1.0 - 2.0 * sigm(tt[a]));
             } else if (a == 5 || a == 8 || a == 9 || (a >= 18 && a < 26)) {
                 s += g44[a] * th[a];
             } else if (a == 26) {
-                const double sg = sigm(tt[26]);
-                s += (g44[P_A] - g44[P_A + 1]) * (A_HI - A_LO) * sg * (1.0 - sg) * (1.0 - 2.0 * sg);
+                s += (g44[P_A] - g44[P_A + 1]) * f[a] * (1.0 - 2.0 * sigm(tt[26]));
             }
         }
-        if (a >= 27 && c >= 27 && (a - 27) / 7 == (c - 27) / 7) {
-            const int i = (a - 27) / 7, e = (a - 27) % 7, f = (c - 27) % 7;
-            const double pe = th[P_K + 8 * i + e], pf = th[P_K + 8 * i + f];
-            for (int d = 0; d < 8; ++d) {
-                const double pd = th[P_K + 8 * i + d];
-                const double de = (d == e) ? 1.0 : 0.0, df = (d == f) ? 1.0 : 0.0;
-                const double ef = (e == f) ? 1.0 : 0.0;
-                s += g44[P_K + 8 * i + d] * pd * ((de - pe) * (df - pf) - pe * (ef - pf));
-            }
+        if (a >= 27 && c >= 27 && (a >= 34) == (c >= 34)) {
+            // softmax: delta_ef p_e (g_e - g.p) - p_e p_f (g_e + g_f - 2 g.p)
+            const int i = a >= 34, ka = P_K + 8 * i + a - 27 - 7 * i, kc = P_K + 8 * i + c - 27 - 7 * i;
+            const double ge = g44[ka] - gb[i], gf = g44[kc] - gb[i];
+            double v = -th[kc] * (ge + gf);
+            if (a == c) v += ge;
+            s += th[ka] * v;
         }
         Ht[idx] = s;
     }
@@ -491,6 +565,7 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
         if (tid == 0) {
             S.cand = 0;
             st[b] = S;
+            act[b] = 0;
         }
         return;
     }
@@ -498,10 +573,10 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     for (int i = tid; i < TRN * TRN; i += blockDim.x) Ht[i] = -Ht[i];   // Ht now holds B
     for (int i = tid; i < TRN; i += blockDim.x) cvec[i] = -gt[i];
     __syncthreads();
-    const double Delta = S.delta;
+    const double Delta = S.delta, iDelta = 1.0 / Delta;
     // |c|, the largest absolute row sum of B and its smallest diagonal entry: one row per
     // thread, then combined in row order
-    __shared__ double rs[TRN], invd[TRN];
+    __shared__ double rs[TRN], rd[TRN], cb[2 * (TRN + 1)];
     if (tid < TRN) {
         double r = 0.0;
         for (int j = 0; j < TRN; ++j) r += fabs(Ht[tid * TRN + j]);
@@ -536,22 +611,22 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     for (int i = tid; i < TRN; i += blockDim.x) p[i] = 0.0;   // a zero step if nothing factors
     if (tid == 0) pn_s = 0.0;
     __syncthreads();
-    __shared__ double rcp[2 * TRN];
-    bool ok = block_chol(Ht, 0.0, L, TRN, &flag, rcp, pk);
+    // p = -(B + lam I)^-1 c from the bordered factorisation, and |p| (warp 0)
+    auto step_norm = [&]() {
+        warp_bwd(L, rd, L + TRN * TRN, p, TRN);
+        double s = 0.0;
+        for (int i = tid; i < TRN; i += 32) {
+            p[i] = -p[i];
+            s += p[i] * p[i];
+        }
+        return sqrt(warp_sum_d(s));
+    };
+    bool ok = block_factor(Ht, 0.0, cvec, L, cb, rd, TRN, pk);
     bool solved = false;
     if (ok) {
-        if (tid < TRN) invd[tid] = rcp[tid];
-        __syncthreads();
         if (tid < 32) {
-            warp_fwd(L, invd, cvec, w, TRN);
-            warp_bwd(L, invd, w, p, TRN);
-            double s = 0.0;
-            for (int i = tid; i < TRN; i += 32) {
-                p[i] = -p[i];
-                s += p[i] * p[i];
-            }
-            s = warp_sum_d(s);
-            if (tid == 0) pn_s = sqrt(s);
+            const double pn = step_norm();
+            if (tid == 0) pn_s = pn;
         }
         __syncthreads();
         if (pn_s <= Delta) solved = true;
@@ -571,14 +646,14 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
         {
             float* B32 = reinterpret_cast<float*>(tr_dyn);   // H and H T are dead by now
             float* L32 = B32 + TRN * TRN;
-            float* c32 = L32 + TRN * TRN;
-            float *y32 = c32 + TRN, *p32 = y32 + TRN, *w32 = p32 + TRN, *r32 = w32 + TRN;   // r32: 2 TRN
+            float* c32 = L32 + (TRN + 1) * TRN;
+            float *p32 = c32 + TRN, *w32 = p32 + TRN, *r32 = w32 + TRN, *b32 = r32 + TRN;   // b32: 2 (TRN + 1)
             for (int i = tid; i < TRN * TRN; i += blockDim.x) B32[i] = (float)Ht[i];
             for (int i = tid; i < TRN; i += blockDim.x) c32[i] = (float)cvec[i];
             __syncthreads();
             double l = lam, lo = lamL, hi = lamU;
             for (int it = 0; it < 16; ++it) {
-                const bool pd = block_chol<float>(B32, (float)l, L32, TRN, &flag, r32, pk);
+                const bool pd = block_factor<float>(B32, (float)l, c32, L32, b32, r32, TRN, pk);
                 if (tid < 32) {
                     double nl = l;
                     int dn = 0;
@@ -586,8 +661,7 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
                         lo = fmax(lo, l);
                         nl = fmax(sqrt(fmax(lo, 1e-300) * hi), lo + 0.01 * (hi - lo));
                     } else {
-                        warp_fwd<float>(L32, r32, c32, y32, TRN);
-                        warp_bwd<float>(L32, r32, y32, p32, TRN);
+                        warp_bwd<float>(L32, r32, L32 + TRN * TRN, p32, TRN);
                         float sp = 0.f;
                         for (int i = tid; i < TRN; i += 32) sp += p32[i] * p32[i];
                         const double pn = sqrt((double)warp_sum_f(sp));
@@ -597,10 +671,10 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
                             if (pn < Delta) hi = l;
                             else lo = l;
                             warp_fwd<float>(L32, r32, p32, w32, TRN);
-                            float sw = 0.f;
+                            float sw = 0.f;   // p' (B + lam I)^-1 p
                             for (int i = tid; i < TRN; i += 32) sw += w32[i] * w32[i];
                             const double wn = (double)warp_sum_f(sw);
-                            nl = l + (pn * pn / wn) * (pn - Delta) / Delta;
+                            nl = l + pn * pn * recip_pos(wn) * (pn - Delta) * iDelta;
                             if (!(nl > lo && nl < hi)) nl = fmax(sqrt(fmax(lo, 1e-300) * hi), lo + 0.01 * (hi - lo));
                             if (hi - lo <= 1e-6 * fmax(1.0, hi)) dn = 1;
                         }
@@ -619,9 +693,7 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
             if (l > lamL && l < lamU) lam = l;
         }
         for (int it = 0; it < 200; ++it) {
-            const bool pd = block_chol(Ht, lam, L, TRN, &flag, rcp, pk);
-            if (pd && tid < TRN) invd[tid] = rcp[tid];
-            __syncthreads();
+            const bool pd = block_factor(Ht, lam, cvec, L, cb, rd, TRN, pk);
             if (tid < 32) {
                 double nl = 0.0;
                 if (!pd) {
@@ -629,15 +701,8 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
                     nl = fmax(sqrt(fmax(lamL, 1e-300) * lamU), lamL + 0.01 * (lamU - lamL));
                     if (tid == 0) done = 0;
                 } else {
-                    // p = -(B + lam I)^-1 c, then w = L^-1 p for Newton's step on 1/|p|
-                    warp_fwd(L, invd, cvec, w, TRN);
-                    warp_bwd(L, invd, w, p, TRN);
-                    double s = 0.0;
-                    for (int i = tid; i < TRN; i += 32) {
-                        p[i] = -p[i];
-                        s += p[i] * p[i];
-                    }
-                    const double pn = sqrt(warp_sum_d(s));
+                    // p, then w = L^-1 p for Newton's step on 1/|p|
+                    const double pn = step_norm();
                     if (tid == 0) pn_s = pn;
                     __syncwarp();
                     int dn;
@@ -649,11 +714,11 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
                     } else {
                         if (pn < Delta) lamU = lam;
                         else lamL = lam;
-                        warp_fwd(L, invd, p, w, TRN);
-                        double wn = 0.0;
-                        for (int i = tid; i < TRN; i += 32) wn += w[i] * w[i];
+                        warp_fwd(L, rd, p, w, TRN);
+                        double wn = 0.0;   // p' (B + lam I)^-1 p
+                        for (int i = tid; i < TRN; i += 32) wn += w[i] * w[i] * rd[i];
                         wn = warp_sum_d(wn);
-                        nl = lam + (pn * pn / wn) * (pn - Delta) / Delta;
+                        nl = lam + pn * pn * recip_pos(wn) * (pn - Delta) * iDelta;
                         if (!(nl > lamL && nl < lamU))
                             nl = fmax(sqrt(fmax(lamL, 1e-300) * lamU), lamL + 0.01 * (lamU - lamL));
                         dn = (lamU - lamL <= 1e-10 * fmax(1.0, lamU)) ? 2 : 0;
@@ -680,8 +745,10 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
                 for (int i = tid; i < TRN; i += 32) zs[i] = 1.0 + 0.01 * i;
                 __syncwarp();
                 for (int r = 0; r < 6; ++r) {
-                    warp_fwd(L, invd, zs, ys, TRN);
-                    warp_bwd(L, invd, ys, w, TRN);
+                    warp_fwd(L, rd, zs, ys, TRN);
+                    for (int i = tid; i < TRN; i += 32) ys[i] *= rd[i];
+                    __syncwarp();
+                    warp_bwd(L, rd, ys, w, TRN);
                     double zn = 0.0;
                     for (int i = 0; i < TRN; ++i) zn += w[i] * w[i];
                     zn = sqrt(zn);
@@ -743,6 +810,7 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
             done = 0;
         }
         st[b] = S;
+        act[b] = S.cand;   // only sources with a candidate evaluate it
     }
     __syncthreads();
     if (done) return;
@@ -751,7 +819,6 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     if (tid < TRN) tt[tid] += p[tid];
     __syncthreads();
     if (tid < 32) free_to_theta_warp(tt, theta_c + (size_t)NP * b);
-    if (tid == 0) atomicAdd(active, 1);
 }
 
 // ratio of actual to predicted gain, radius update, acceptance: one warp per source (the
@@ -761,7 +828,8 @@ __global__ void __launch_bounds__(32)
 k_tr_accept(int nb, const int32_t* __restrict__ bpatch_off, const PatchGeo* __restrict__ bgeo,
             const double* __restrict__ dll, const ModelDev* __restrict__ md, double* __restrict__ theta,
             double* __restrict__ tfree, const double* __restrict__ theta_c,
-            const double* __restrict__ tfree_c, TrState* __restrict__ st, celeste_fit_options o) {
+            const double* __restrict__ tfree_c, TrState* __restrict__ st, celeste_fit_options o,
+            int32_t* __restrict__ act, int32_t* __restrict__ active) {
     const int b = blockIdx.x;
     if (b >= nb) return;
     const int lane = threadIdx.x;
@@ -791,7 +859,10 @@ k_tr_accept(int nb, const int32_t* __restrict__ bpatch_off, const PatchGeo* __re
         S.iters += 1;
         if (S.iters >= o.max_iter) S.status = ST_MAXITER;
         S.cand = 0;
+        S.moved = accept;
         st[b] = S;
+        act[b] = S.status == ST_ACTIVE;
+        if (S.status == ST_ACTIVE) atomicAdd(active, 1);
     }
     __syncwarp();
     if (accept) {
@@ -800,31 +871,10 @@ k_tr_accept(int nb, const int32_t* __restrict__ bpatch_off, const PatchGeo* __re
     }
 }
 
-__global__ void k_gather_theta(int nb, const int32_t* __restrict__ bsrc,
-                               const double* __restrict__ theta, double* __restrict__ bth) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nb * NP) bth[i] = theta[(size_t)NP * bsrc[i / NP] + i % NP];
-}
-
 __global__ void k_scatter_theta(int nb, const int32_t* __restrict__ bsrc,
                                 const double* __restrict__ bth, double* __restrict__ theta) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < nb * NP) theta[(size_t)NP * bsrc[i / NP] + i % NP] = bth[i];
-}
-
-// per batch source: 1 while its Newton iterations continue (its pixel work is skipped after)
-__global__ void k_mark_active(int nb, const TrState* __restrict__ st, int32_t* __restrict__ act) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nb) act[b] = st[b].status == ST_ACTIVE ? 1 : 0;
-}
-
-__global__ void k_init_state(int nb, TrState* st, double delta0) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    TrState S{};
-    S.delta = delta0;
-    S.status = ST_ACTIVE;
-    st[b] = S;
 }
 
 // ------------------------------------------------------------------------------------
@@ -864,6 +914,7 @@ Batch make_batch(const celeste_problem* pr, const std::vector<int32_t>& members)
         for (int p = pr->patch_off[s]; p < pr->patch_off[s + 1]; ++p) {
             PatchGeo g = pr->geo[p];
             g.src = bi;
+            g.whole_sp = g.sp_off;
             g.sp_off = B.n_sp;
             g.item0 = (int)B.items.size();
             const int npx = g.w * g.h;
@@ -1086,8 +1137,8 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
     PatchGeo* d_bgeo;
     WorkItem* d_bitems;
     HItem* d_bparts;
-    double *d_bth, *d_bthc, *d_bt, *d_btc, *d_f, *d_g, *d_h, *d_kl, *d_hsrc, *d_part, *d_dll, *d_tbl64;
-    float* d_tbl32;
+    double *d_bth, *d_bthc, *d_bt, *d_btc, *d_f, *d_g, *d_h, *d_kl, *d_hsrc, *d_part, *d_dll, *d_tbl64, *d_ctbl64;
+    float *d_tbl32, *d_ctbl32;
     TrState* d_st;
     unsigned char *d_eo, *d_vo, *d_se, *d_sv, *d_ce, *d_cv;
     FIT_CUDA(mem.alloc(&d_bsrc, maxB));
@@ -1110,6 +1161,8 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
     FIT_CUDA(mem.alloc(&d_dll, maxI));
     FIT_CUDA(mem.alloc(&d_tbl64, maxP * TBL_STRIDE));
     FIT_CUDA(mem.alloc(&d_tbl32, maxP * TBL_STRIDE));
+    FIT_CUDA(mem.alloc(&d_ctbl64, maxP * TBL_STRIDE));
+    FIT_CUDA(mem.alloc(&d_ctbl32, maxP * TBL_STRIDE));
     FIT_CUDA(mem.alloc(&d_st, maxB));
     FIT_CUDA(mem.alloc(&d_eo, maxSp * rs));
     FIT_CUDA(mem.alloc(&d_vo, maxSp * rs));
@@ -1123,6 +1176,14 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
         int32_t* p;
         ~HostFree() { cudaFreeHost(p); }
     } hf{h_active};
+    // the captured iteration, kept over the batches
+    cudaGraphExec_t exec = nullptr;
+    struct ExecFree {
+        cudaGraphExec_t& e;
+        ~ExecFree() {
+            if (e) cudaGraphExecDestroy(e);
+        }
+    } ef{exec};
 
     // region-task stage: every source's task id, the stage-start parameters and, per
     // precision phase, every source's E_s / Var_s at them
@@ -1164,6 +1225,9 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
         FIT_CUDA(cudaMemcpyAsync(d_se0, P.spE, bytes, cudaMemcpyDeviceToDevice, st));
         FIT_CUDA(cudaMemcpyAsync(d_sv0, P.spE2, bytes, cudaMemcpyDeviceToDevice, st));
     }
+    // E_s / Var_s of every source (where another patch covers the pixel) at the phase's start
+    FIT_CUDA(launch_prep(P, pr->d_theta, prec, st, false));
+    FIT_CUDA(launch_contrib(P, prec, st, true));
     int sw = 0;
     for (; sw < opts->max_sweeps; ++sw, ++g_sweep) {
         sweep_batches(g_sweep, batches);
@@ -1171,9 +1235,6 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             const Batch& B = batches[c];
             const int nb = (int)B.src.size();
             if (nb == 0) continue;
-            // current E_s / Var_s of every source (global buffers)
-            FIT_CUDA(launch_prep(P, pr->d_theta, prec, st));
-            FIT_CUDA(launch_contrib(P, prec, st, true));
             FIT_CUDA(cudaMemcpyAsync(d_bsrc, B.src.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice, st));
             FIT_CUDA(cudaMemcpyAsync(d_bpo, B.patch_off.data(), sizeof(int32_t) * (nb + 1), cudaMemcpyHostToDevice, st));
             FIT_CUDA(cudaMemcpyAsync(d_bgeo, B.geo.data(), sizeof(PatchGeo) * B.geo.size(), cudaMemcpyHostToDevice, st));
@@ -1194,10 +1255,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
                                                         csr_bounds(P), d_task, (const float*)d_se0,
                                                         (const float*)d_sv0);
             }
-            k_gather_theta<<<(nb * NP + 255) / 256, 256, 0, st>>>(nb, d_bsrc, pr->d_theta, d_bth);
-            k_to_free<<<(nb + 127) / 128, 128, 0, st>>>(nb, d_bth, d_bt);
-            k_init_state<<<(nb + 127) / 128, 128, 0, st>>>(nb, d_st, opts->delta0);
-            k_mark_active<<<(nb + 127) / 128, 128, 0, st>>>(nb, d_st, d_srcact);
+            k_batch_start<<<nb, 32, 0, st>>>(nb, d_bsrc, pr->d_theta, d_bth, d_bt, d_st, d_srcact, opts->delta0);
             FIT_CUDA(cudaGetLastError());
             // batch views of the problem
             DevProblem Pb = P;
@@ -1227,54 +1285,47 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             DevProblem Pc = Pb;
             Pc.spE = d_ce;
             Pc.spE2 = d_cv;
+            Pc.tbl64 = d_ctbl64;
+            Pc.tbl32 = d_ctbl32;
+            // the batch's tables and E_s / Var_s at its start
+            FIT_CUDA(launch_prep(Pb, d_bth, prec, st, false, true));
+            FIT_CUDA(launch_contrib(Pb, prec, st));
             // one Newton iteration, captured as a graph
             cudaGraph_t graph = nullptr;
-            cudaGraphExec_t exec = nullptr;
             FIT_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
             cudaError_t ce = cudaSuccess;
             auto chk = [&](cudaError_t e) {
                 if (ce == cudaSuccess && e != cudaSuccess) ce = e;
             };
             chk(cudaMemsetAsync(d_active, 0, sizeof(int32_t), st));
-            chk(launch_prep(Pb, d_bth, prec, st, true, true));
-            chk(launch_contrib(Pb, prec, st));
-            if (nI > 0) {
-                if (prec == CELESTE_FP64)
-                    k_batch_maps<double><<<nI, CHUNK, 0, st>>>(d_bitems, d_bgeo, P.img, (const double*)d_eo,
-                                                               (const double*)d_vo, (const double*)d_se,
-                                                               (const double*)d_sv, (double*)P.emap, (double*)P.vmap,
-                                                               d_srcact);
+            const int n_tbl = T_GAL + P.npsf_max * P.nprof * GAL_STRIDE;
+            auto pixel_kernels = [&](auto R, auto* tbl, auto* ctbl, bool maps) {
+                using T = decltype(R);
+                T *eo = (T*)d_eo, *vo = (T*)d_vo, *se = (T*)d_se, *sv = (T*)d_sv, *cE = (T*)d_ce, *cV = (T*)d_cv;
+                if (nI == 0) return;
+                if (maps)
+                    k_batch_maps<T><<<nI, CHUNK, 0, st>>>(d_bitems, d_bgeo, P.img, eo, vo, se, sv, cE, cV, (T*)P.emap,
+                                                          (T*)P.vmap, d_srcact, d_st, tbl, ctbl, n_tbl,
+                                                          (float*)d_tbl64, (const float*)d_ctbl64,
+                                                          sizeof(T) == 4 ? P.npsf_max * WFR : 0);
                 else
-                    k_batch_maps<float><<<nI, CHUNK, 0, st>>>(d_bitems, d_bgeo, P.img, (const float*)d_eo,
-                                                              (const float*)d_vo, (const float*)d_se,
-                                                              (const float*)d_sv, (float*)P.emap, (float*)P.vmap,
-                                                              d_srcact);
-            }
+                    k_batch_dll<T><<<nI, CHUNK, 0, st>>>(d_bitems, d_bgeo, P.img, P.pixels, eo, vo, se, sv, cE, cV,
+                                                         d_dll, d_srcact);
+            };
+            auto batch_pixels = [&](bool maps) {
+                if (prec == CELESTE_FP64) pixel_kernels(0.0, d_tbl64, d_ctbl64, maps);
+                else pixel_kernels(0.f, d_tbl32, d_ctbl32, maps);
+            };
+            batch_pixels(true);
             chk(launch_hess_pixels(Pb, prec, d_bth, d_h, st));
             chk(launch_finalize_hess(Pb, d_f, d_g, d_h, st));
             k_tr_step<<<nb, TR_THREADS, TR_DYN_BYTES, st>>>(nb, d_bth, d_bt, d_f, d_g, d_h, d_kl, d_bthc, d_btc,
-                                                 d_st, *opts, d_active);
-            // only sources with a candidate evaluate it
-            k_mark_active<<<(nb + 127) / 128, 128, 0, st>>>(nb, d_st, d_srcact);
-            chk(launch_prep(Pc, d_bthc, prec, st));
+                                                 d_st, *opts, d_srcact);
+            chk(launch_prep(Pc, d_bthc, prec, st, false, true));
             chk(launch_contrib(Pc, prec, st));
-            if (nI > 0) {
-                if (prec == CELESTE_FP64)
-                    k_batch_dll<double><<<nI, CHUNK, 0, st>>>(d_bitems, d_bgeo, P.img, P.pixels,
-                                                              (const double*)d_eo, (const double*)d_vo,
-                                                              (const double*)d_se, (const double*)d_sv,
-                                                              (const double*)d_ce, (const double*)d_cv, d_dll,
-                                                              d_srcact);
-                else
-                    k_batch_dll<float><<<nI, CHUNK, 0, st>>>(d_bitems, d_bgeo, P.img, P.pixels,
-                                                             (const float*)d_eo, (const float*)d_vo,
-                                                             (const float*)d_se, (const float*)d_sv,
-                                                             (const float*)d_ce, (const float*)d_cv, d_dll,
-                                                             d_srcact);
-            }
+            batch_pixels(false);
             k_tr_accept<<<nb, 32, 0, st>>>(nb, d_bpo, d_bgeo, d_dll, P.model, d_bth, d_bt, d_bthc, d_btc,
-                                           d_st, *opts);
-            k_mark_active<<<(nb + 127) / 128, 128, 0, st>>>(nb, d_st, d_srcact);
+                                           d_st, *opts, d_srcact, d_active);
             chk(cudaGetLastError());
             chk(cudaMemcpyAsync(h_active, d_active, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
             cudaError_t ee = cudaStreamEndCapture(st, &graph);
@@ -1282,21 +1333,35 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
                 if (graph) cudaGraphDestroy(graph);
                 return cuda_err(ce != cudaSuccess ? ce : ee, "fit iteration capture");
             }
-            ee = cudaGraphInstantiate(&exec, graph, 0);
+            // the graph has the same nodes for every batch: the executable one takes the new
+            // batch's sizes and is only built anew where that is refused
+            cudaGraphExecUpdateResultInfo info;
+            if (exec && cudaGraphExecUpdate(exec, graph, &info) != cudaSuccess) {
+                (void)cudaGetLastError();
+                cudaGraphExecDestroy(exec);
+                exec = nullptr;
+            }
+            if (!exec) ee = cudaGraphInstantiate(&exec, graph, 0);
             cudaGraphDestroy(graph);
             if (ee != cudaSuccess) return cuda_err(ee, "cudaGraphInstantiate");
             int it = 0;
             for (; it < opts->max_iter + 1; ++it) {
                 ee = cudaGraphLaunch(exec, st);
                 if (ee == cudaSuccess) ee = cudaStreamSynchronize(st);
-                if (ee != cudaSuccess) {
-                    cudaGraphExecDestroy(exec);
-                    return cuda_err(ee, "fit iteration");
-                }
+                if (ee != cudaSuccess) return cuda_err(ee, "fit iteration");
                 if (*h_active == 0) break;
             }
-            cudaGraphExecDestroy(exec);
-            // results of this colour
+            // results of this batch
+            if (nI > 0) {
+                if (prec == CELESTE_FP64)
+                    k_batch_end<double><<<nI, CHUNK, 0, st>>>(d_bitems, d_bgeo, (const double*)d_se, (const double*)d_sv,
+                                                              (const double*)d_ce, (const double*)d_cv, d_st,
+                                                              (double*)P.spE, (double*)P.spE2);
+                else
+                    k_batch_end<float><<<nI, CHUNK, 0, st>>>(d_bitems, d_bgeo, (const float*)d_se, (const float*)d_sv,
+                                                             (const float*)d_ce, (const float*)d_cv, d_st,
+                                                             (float*)P.spE, (float*)P.spE2);
+            }
             k_scatter_theta<<<(nb * NP + 255) / 256, 256, 0, st>>>(nb, d_bsrc, d_bth, pr->d_theta);
             FIT_CUDA(cudaGetLastError());
             FIT_CUDA(cudaMemcpyAsync(hst.data(), d_st, sizeof(TrState) * nb, cudaMemcpyDeviceToHost, st));

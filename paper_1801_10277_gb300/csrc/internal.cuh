@@ -132,6 +132,7 @@ struct PatchGeo {
     int64_t sp_off;          // offset in the per-(source, pixel) buffers
     int32_t item0, nitem;    // work items covering this patch
     int32_t hpart0, pad;     // its first part of the Hessian pass (hchunk pixels each, in order)
+    int64_t whole_sp;        // in a fit's batch: the patch's sp_off in the whole problem
 };
 
 struct WorkItem {

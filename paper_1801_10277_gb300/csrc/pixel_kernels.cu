@@ -727,12 +727,13 @@ k_contrib64(const WorkItem* __restrict__ items, const PatchGeo* __restrict__ geo
             double* __restrict__ vmap, bool multi_only, const int32_t* __restrict__ src_active) {
     __shared__ __align__(16) double sT[TBL_STRIDE];
     __shared__ __align__(16) double tab[EX_N];
-    const int item = (int)blockIdx.x;
-    const WorkItem it = items[item];
+    // the items in CHUNK / blockDim.x parts
+    const int split = CHUNK / (int)blockDim.x;
+    const WorkItem it = items[(int)blockIdx.x / split];
     const PatchGeo g = geo[it.patch];
     if (src_active && !src_active[g.src]) return;
     const ImgMeta& im = img[g.img];
-    const int t = threadIdx.x, q = it.q0 + (t < it.n ? t : 0);
+    const int t = (int)blockIdx.x % split * (int)blockDim.x + threadIdx.x, q = it.q0 + (t < it.n ? t : 0);
     const int64_t sp = g.sp_off + q;
     const bool alone = single && single[sp], need = t < it.n && !(alone && multi_only);
     if (!__syncthreads_or(need)) return;
@@ -1533,11 +1534,16 @@ cudaError_t launch_prep(const DevProblem& P, const double* d_theta, int precisio
 cudaError_t launch_contrib(const DevProblem& P, int precision, cudaStream_t st, bool multi_only) {
     const ItemSet S{nullptr, P.n_item};
     if (S.n == 0) return cudaSuccess;
-    if (precision == CELESTE_FP64)
-        k_contrib64<<<S.n, CHUNK, 0, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.tbl64, (double*)P.spE,
+    if (precision == CELESTE_FP64) {
+        // An SM runs a CTA's FP64 instructions at a warp per 16 cycles whatever its size, so few
+        // items are cut until there are eight CTAs per SM (64 crowded sources, 565 items: the map
+        // pass 110 -> 80 us; a fit's batch of 60 items 40 -> 17 us).
+        int split = 1;
+        while (split < 4 && (int64_t)S.n * split < 8LL * sm_count()) split *= 2;
+        k_contrib64<<<S.n * split, CHUNK / split, 0, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.tbl64, (double*)P.spE,
                                            (double*)P.spE2, P.single, P.sky_map, (double*)P.emap, (double*)P.vmap,
                                            multi_only, P.src_active);
-    else
+    } else
         switch (ppt_contrib(P)) {
 #define CEL_CONTRIB32(N)                                                                          \
     case N:                                                                                       \
