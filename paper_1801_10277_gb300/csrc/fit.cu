@@ -302,58 +302,52 @@ __device__ __forceinline__ double recip_pos(double d) {
     return fma(r, fma(e, e, e), r);
 }
 
-// Factorisation of B + lam I bordered by a right-hand side, n <= TRN: A has n + 1 rows of n
-// (lower part).  FP64: L D L', rd[k] = 1 / d_k, L's unit diagonal not stored; FP32: Cholesky,
-// rd[k] = 1 / L_kk.  Row n receives the solution of L D w = rhs (FP32: L w = rhs).  Returns
-// whether every pivot is positive (rd[k] = 0 marks one that is not: a slot of its own per
-// column, so that no warp can see the mark of a later column and leave the loop ahead of the
-// others).
+// L D L' factorisation of B + lam I bordered by a right-hand side, n <= TRN: A has n + 1 rows
+// of n (lower part).  The strict lower part of rows 0 .. n - 1 receives L, rd[k] = 1 / d_k, and
+// row n the solution w of L D w = rhs.  Returns whether every pivot is positive (rd[k] = 0
+// marks one that is not: a slot of its own per column, so that no warp can see the mark of a
+// later column and leave the loop ahead of the others).
 // Right-looking with the next column ahead of the rest: at step k warp 0 updates column
-// k + 1, takes its pivot's reciprocal (root) and scales the column while the other warps
-// update the columns after it, so a column costs one barrier and, in FP64, a chain of five
-// dependent operations (update, three for the reciprocal, scale) of about 70 cycles each:
-// that chain is the cost on GB300.  FP32 keeps the square root: its entries are formed by the
-// operations of a plain Cholesky factorisation, and the multipliers of the search with them.
-// cb: 2 (n + 1) entries, columns k and k + 1 as the updates multiply by them (FP64: unscaled).
-__device__ __forceinline__ double pivot_factor(double d) { return recip_pos(d); }
-__device__ __forceinline__ float pivot_factor(float d) { return rsqrtf(d); }
-
-template <class T>
-__device__ bool block_factor(const T* B, T lam, const T* rhs, T* A, T* cb, T* rd, int n, const uint16_t* pk) {
-    constexpr bool LDL = sizeof(T) == 8;
+// k + 1, takes its pivot's reciprocal and scales the column while the other warps update the
+// columns after it, so a column costs one barrier and a chain of five dependent FP64
+// operations (update, three for the reciprocal, scale) of about 70 cycles each: that chain is
+// the cost on GB300.  cb: 2 (n + 1) entries, the unscaled columns k and k + 1.
+__device__ __noinline__ bool block_factor(const double* B, double lam, const double* rhs, double* A, double* cb, double* rd,
+                             int n, const uint16_t* pk) {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
     for (int r = tid >> 5; r <= n; r += nt >> 5)   // a row per warp
         for (int c = lane; c <= r && c < n; c += 32)
             A[r * n + c] = r == n ? rhs[c] : r == c ? B[r * n + c] + lam : B[r * n + c];
     __syncthreads();
-    // column k by warp 0: v0, v1 its entries at rows lane and lane + 32 (rows k .. n in use)
-    auto finish = [&](int k, T v0, T v1) {
-        const T d = __shfl_sync(0xffffffffu, k < 32 ? v0 : v1, k & 31);
-        const T r = d > (T)0 && isfinite(d) ? pivot_factor(d) : (T)0;
-        T* c = cb + (k & 1) * (n + 1);
-        if (lane > k && lane <= n) {
-            const T l = v0 * r;
-            c[lane] = LDL ? v0 : l;
-            A[lane * n + k] = l;
+    // column k by warp 0: lane l holds its row k + l in v0 and, while there are more than 32 rows
+    // left, row k + 32 + l in v1 (rows k .. n)
+    auto finish = [&](int k, double v0, double v1) {
+        const double d = __shfl_sync(0xffffffffu, v0, 0);
+        const double r = d > 0.0 && isfinite(d) ? recip_pos(d) : 0.0;
+        double* c = cb + (k & 1) * (n + 1);
+        const int i = k + lane;
+        if (lane > 0 && i <= n) {
+            c[i] = v0;
+            A[i * n + k] = v0 * r;
         }
-        if (lane + 32 > k && lane + 32 <= n) {
-            const T l = v1 * r;
-            c[lane + 32] = LDL ? v1 : l;
-            A[(lane + 32) * n + k] = l;
+        if (k + 32 <= n && i + 32 <= n) {
+            c[i + 32] = v1;
+            A[(i + 32) * n + k] = v1 * r;
         }
         if (lane == 0) rd[k] = r;
     };
-    auto entry = [&](int i, int k) { return i >= k && i <= n ? A[i * n + k] : (T)0; };
+    auto entry = [&](int i, int k) { return i <= n ? A[i * n + k] : 0.0; };
     if (tid < 32) finish(0, entry(lane, 0), entry(lane + 32, 0));
     __syncthreads();
     for (int k = 0; k < n - 1; ++k) {
-        if (rd[k] == (T)0) return false;
-        const T* c = cb + (k & 1) * (n + 1);
+        if (rd[k] == 0.0) return false;
+        const double* c = cb + (k & 1) * (n + 1);
         if (tid < 32) {
-            const T f = c[k + 1];
-            T v0 = entry(lane, k + 1), v1 = entry(lane + 32, k + 1);
-            if (lane > k && lane <= n) v0 = fma(-A[lane * n + k], f, v0);
-            if (lane + 32 > k && lane + 32 <= n) v1 = fma(-A[(lane + 32) * n + k], f, v1);
+            const double f = c[k + 1];
+            const int i = k + 1 + lane;
+            double v0 = 0.0, v1 = 0.0;
+            if (i <= n) v0 = fma(-A[i * n + k], f, A[i * n + k + 1]);
+            if (k + 33 <= n && i + 32 <= n) v1 = fma(-A[(i + 32) * n + k], f, A[(i + 32) * n + k + 1]);
             finish(k + 1, v0, v1);
         } else {
             // rows k + 2 .. n, columns k + 2 .. n - 1: the packed triangle but its last corner
@@ -361,55 +355,147 @@ __device__ bool block_factor(const T* B, T lam, const T* rhs, T* A, T* cb, T* rd
             for (int idx = tid - 32; idx < cnt; idx += 2 * step) {
                 const int p0 = pk[idx], p1 = pk[min(idx + step, cnt - 1)];
                 const int i0 = b0 + (p0 >> 8), j0 = b0 + (p0 & 255), i1 = b0 + (p1 >> 8), j1 = b0 + (p1 & 255);
-                const T a0 = A[i0 * n + j0], l0 = A[i0 * n + k], c0 = c[j0];
-                const T a1 = A[i1 * n + j1], l1 = A[i1 * n + k], c1 = c[j1];
+                const double a0 = A[i0 * n + j0], l0 = A[i0 * n + k], c0 = c[j0];
+                const double a1 = A[i1 * n + j1], l1 = A[i1 * n + k], c1 = c[j1];
                 A[i0 * n + j0] = fma(-l0, c0, a0);
                 if (idx + step < cnt) A[i1 * n + j1] = fma(-l1, c1, a1);
             }
         }
         __syncthreads();
     }
-    return rd[n - 1] != (T)0;
+    return rd[n - 1] != 0.0;
 }
 
-// Warp-level triangular solves with that L (every lane of the calling warp calls them): lane
-// l holds rows l and l + 32 of the right-hand side; one column of L per step (column-oriented
-// substitution), the solved entry broadcast by shuffle (FP32: times 1 / L_kk).  The arrays
-// must not overlap.
-template <class T>
-__device__ void warp_fwd(const T* __restrict__ L, const T* __restrict__ rd, const T* __restrict__ b,
-                         T* __restrict__ y, int n) {
-    constexpr bool LDL = sizeof(T) == 8;
+// Solves with that unit-diagonal L by one warp (every lane calls them): lane l holds rows l and
+// l + 32 of the right-hand side; one column of L per step (column-oriented substitution), the
+// solved entry broadcast by shuffle.  The arrays must not overlap.
+__device__ __noinline__ void warp_fwd(const double* __restrict__ L, const double* __restrict__ b, double* __restrict__ y, int n) {
+    __syncwarp();   // a solve entered by a diverged warp issues each step several times (8.7 -> 31 us)
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    T r0 = lane < n ? b[lane] : (T)0, r1 = lane + 32 < n ? b[lane + 32] : (T)0;
+    double r0 = lane < n ? b[lane] : 0.0, r1 = lane + 32 < n ? b[lane + 32] : 0.0;
+#pragma unroll 2
     for (int k = 0; k < n; ++k) {
-        const T l0 = lane > k && lane < n ? L[lane * n + k] : (T)0;
-        const T l1 = lane + 32 > k && lane + 32 < n ? L[(lane + 32) * n + k] : (T)0;
-        T yk = __shfl_sync(full, k < 32 ? r0 : r1, k & 31);
-        if (!LDL) yk *= rd[k];
-        if (lane == (k & 31)) y[k] = yk;
-        r0 = fma(-l0, yk, r0);
+        const double l0 = lane > k && lane < n ? L[lane * n + k] : 0.0;
+        const double l1 = lane + 32 > k && lane + 32 < n ? L[(lane + 32) * n + k] : 0.0;
+        const double yk = __shfl_sync(full, k < 32 ? r0 : r1, k & 31);
+        if (k < 31) r0 = fma(-l0, yk, r0);
         r1 = fma(-l1, yk, r1);
     }
+    if (lane < n) y[lane] = r0;
+    if (lane + 32 < n) y[lane + 32] = r1;
     __syncwarp();
 }
 
-template <class T>
-__device__ void warp_bwd(const T* __restrict__ L, const T* __restrict__ rd, const T* __restrict__ y,
-                         T* __restrict__ x, int n) {
-    constexpr bool LDL = sizeof(T) == 8;
+__device__ __noinline__ void warp_bwd(const double* __restrict__ L, const double* __restrict__ y, double* __restrict__ x, int n) {
+    __syncwarp();
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    T r0 = lane < n ? y[lane] : (T)0, r1 = lane + 32 < n ? y[lane + 32] : (T)0;
+    double r0 = lane < n ? y[lane] : 0.0, r1 = lane + 32 < n ? y[lane + 32] : 0.0;
+#pragma unroll 2
     for (int k = n - 1; k >= 0; --k) {
-        const T l0 = lane < k ? L[k * n + lane] : (T)0;
-        const T l1 = lane + 32 < k ? L[k * n + lane + 32] : (T)0;
-        T xk = __shfl_sync(full, k < 32 ? r0 : r1, k & 31);
-        if (!LDL) xk *= rd[k];
-        if (lane == (k & 31)) x[k] = xk;
+        const double l0 = lane < k ? L[k * n + lane] : 0.0;
+        const double l1 = lane + 32 < k ? L[k * n + lane + 32] : 0.0;
+        const double xk = __shfl_sync(full, k < 32 ? r0 : r1, k & 31);
         r0 = fma(-l0, xk, r0);
-        r1 = fma(-l1, xk, r1);
+        if (k > 32) r1 = fma(-l1, xk, r1);
+    }
+    if (lane < n) x[lane] = r0;
+    if (lane + 32 < n) x[lane + 32] = r1;
+    __syncwarp();
+}
+
+// The FP32 multiplier search's factorisation, by one warp with the matrix in registers: lane l
+// holds row l in a0 and row 32 + l in a1 (the bordering right-hand side is row TRN).  Cholesky
+// with the operations of the textbook right-looking form in its order (the multiplier at which
+// the search stops decides how a step ends on the boundary, so its arithmetic is kept).
+// The current column is always entry 0: an update writes entry j + 1's new value to entry j, so
+// that one loop body serves every column (W entries wide; two widths).  The code is kept small
+// on purpose: a step's kernels run one after another and each call fetches its instructions
+// anew, which cost a fully unrolled factorisation (40 KB) more than its arithmetic.
+// L receives the factor (rows of TRN; the solution of L w = rhs in row TRN), rd 1 / L_kk; cb: 44
+// floats, 16-byte aligned.
+template <int W>
+__device__ __forceinline__ bool chol32_columns(float (&a0)[TRN], float (&a1)[TRN], int k0, int k1, float* L,
+                                               float* rd, float* cb) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k) {
+        const float d = __shfl_sync(0xffffffffu, k < 32 ? a0[0] : a1[0], k & 31);
+        if (!(d > 0.f) || !isfinite(d)) return false;
+        const float q = rsqrtf(d);
+        const float l0 = a0[0] * q, l1 = a1[0] * q;
+        __syncwarp();   // cb was last read in the previous column
+        if (lane == 0) rd[k] = q;
+        if (lane > k) {
+            L[lane * TRN + k] = l0;
+            cb[lane - k] = l0;
+        }
+        if (lane + 32 > k && lane + 32 <= TRN) {
+            L[(lane + 32) * TRN + k] = l1;
+            cb[lane + 32 - k] = l1;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < W; j += 4) {
+            const float4 c = *reinterpret_cast<const float4*>(cb + j);
+            const float cj[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (j + u >= 1 && j + u < W) {
+                    a0[j + u - 1] = fmaf(-l0, cj[u], a0[j + u]);
+                    a1[j + u - 1] = fmaf(-l1, cj[u], a1[j + u]);
+                }
+        }
+    }
+    return true;
+}
+__device__ __noinline__ bool chol32(const float* B, float lam, const float* rhs, float* L, float* rd, float* cb) {
+    __syncwarp();
+    const int lane = threadIdx.x & 31, i = lane + 32;
+    float a0[TRN], a1[TRN];
+#pragma unroll
+    for (int j = 0; j < TRN; ++j) {
+        a0[j] = B[lane * TRN + j];
+        a1[j] = i < TRN ? B[i * TRN + j] : i == TRN ? rhs[j] : 0.f;
+        if (j == lane) a0[j] += lam;
+        if (j == i) a1[j] += lam;
+    }
+    constexpr int HALF = 20;
+    const bool ok = chol32_columns<TRN>(a0, a1, 0, HALF, L, rd, cb) &&
+                    chol32_columns<TRN - HALF>(a0, a1, HALF, TRN, L, rd, cb);
+    __syncwarp();
+    return ok;
+}
+__device__ __noinline__ void warp_fwd32(const float* __restrict__ L, const float* __restrict__ rd, const float* __restrict__ b,
+                           float* __restrict__ y) {
+    __syncwarp();
+    const int lane = threadIdx.x & 31;
+    float r0 = b[lane], r1 = lane + 32 < TRN ? b[lane + 32] : 0.f;
+#pragma unroll 2
+    for (int k = 0; k < TRN; ++k) {
+        const float l0 = lane > k ? L[lane * TRN + k] : 0.f;
+        const float l1 = lane + 32 > k && lane + 32 < TRN ? L[(lane + 32) * TRN + k] : 0.f;
+        const float yk = __shfl_sync(0xffffffffu, k < 32 ? r0 : r1, k & 31) * rd[k];
+        if (lane == (k & 31)) y[k] = yk;
+        r0 = fmaf(-l0, yk, r0);
+        r1 = fmaf(-l1, yk, r1);
+    }
+    __syncwarp();
+}
+__device__ __noinline__ void warp_bwd32(const float* __restrict__ L, const float* __restrict__ rd, const float* __restrict__ y,
+                           float* __restrict__ x) {
+    __syncwarp();
+    const int lane = threadIdx.x & 31;
+    float r0 = y[lane], r1 = lane + 32 < TRN ? y[lane + 32] : 0.f;
+#pragma unroll 2
+    for (int k = TRN - 1; k >= 0; --k) {
+        const float l0 = lane < k ? L[k * TRN + lane] : 0.f;
+        const float l1 = lane + 32 < k ? L[k * TRN + lane + 32] : 0.f;
+        const float xk = __shfl_sync(0xffffffffu, k < 32 ? r0 : r1, k & 31) * rd[k];
+        if (lane == (k & 31)) x[k] = xk;
+        r0 = fmaf(-l0, xk, r0);
+        r1 = fmaf(-l1, xk, r1);
     }
     __syncwarp();
 }
@@ -428,6 +514,11 @@ __device__ __forceinline__ float warp_sum_f(float v) {
     return v;
 }
 
+// Bound by chains of dependent operations, not by rates (4 warps of a CTA per source): per call
+// with an active source 260 us with a plain Cholesky factor and solves behind it, 192 us with
+// the bordered factor, 155 us with the FP32 search in one warp's registers (5 factorisations,
+// 47 us; FP64: 2 or 3, 44 us; the set-up of T'HT 21 us; the solves 40 us).  An iteration ends
+// when its slowest source does, so more CTAs per source would not help either.
 __global__ void __launch_bounds__(TR_THREADS)
 k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ tfree,
           const double* __restrict__ f_in, const double* __restrict__ g_in,
@@ -439,7 +530,7 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     __shared__ TrState S;
     __shared__ double gt[TRN], Ht[TRN * TRN], L[(TRN + 1) * TRN], cvec[TRN], p[TRN], w[TRN];
     __shared__ double th[NP], tt[TRN], g44[NP];
-    __shared__ double f[P_A + 1], hb[2][NP], gb[2];
+    __shared__ double f[P_A + 1], f2[P_A + 1], hb[2][NP], gb[2];
     __shared__ int done;
     __shared__ double lam_s, pn_s;
     __shared__ uint16_t pk[PK_N];
@@ -473,14 +564,16 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     // x_a1) or p_e (x_e - x.p), with x.p summed over the type's eight weights first.
     if (tid <= P_A) {
         const int a = tid;
-        double v = 1.0;
+        double v = 1.0, v2 = 0.0;   // d theta_a / dt, d2 theta_a / dt2
         if (a == 2 || a == 3 || a == P_A) {
             const double s = sigm(tt[a]);
             v = (a == P_A ? A_HI - A_LO : BOX_HI - BOX_LO) * s * (1.0 - s);
+            v2 = v * (1.0 - 2.0 * s);
         } else if (a == 5 || a == 8 || a == 9 || a >= 18) {
-            v = th[a];
+            v = v2 = th[a];
         }
         f[a] = v;
+        f2[a] = v2;
     } else if (tid >= 32 && tid < 32 + 2 * NP) {
         const int r = (tid - 32) >> 1, i = tid & 1;
         double v = 0.0;
@@ -516,15 +609,7 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     for (int idx = tid; idx < TRN * TRN; idx += blockDim.x) {
         const int a = idx / TRN, c = idx - a * TRN;
         double s = times_T(a, X + c, TRN, hb[0][c], hb[1][c]);
-        if (a == c) {
-            if (a == 2 || a == 3) {
-                s += g44[a] * f[a] * (1.0 - 2.0 * sigm(tt[a]));
-            } else if (a == 5 || a == 8 || a == 9 || (a >= 18 && a < 26)) {
-                s += g44[a] * th[a];
-            } else if (a == 26) {
-                s += (g44[P_A] - g44[P_A + 1]) * f[a] * (1.0 - 2.0 * sigm(tt[26]));
-            }
-        }
+        if (a == c && a <= P_A) s += (a == P_A ? g44[P_A] - g44[P_A + 1] : g44[a]) * f2[a];
         if (a >= 27 && c >= 27 && (a >= 34) == (c >= 34)) {
             // softmax: delta_ef p_e (g_e - g.p) - p_e p_f (g_e + g_f - 2 g.p)
             const int i = a >= 34, ka = P_K + 8 * i + a - 27 - 7 * i, kc = P_K + 8 * i + c - 27 - 7 * i;
@@ -574,15 +659,21 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     for (int i = tid; i < TRN; i += blockDim.x) cvec[i] = -gt[i];
     __syncthreads();
     const double Delta = S.delta, iDelta = 1.0 / Delta;
-    // |c|, the largest absolute row sum of B and its smallest diagonal entry: one row per
-    // thread, then combined in row order
-    __shared__ double rs[TRN], rd[TRN], cb[2 * (TRN + 1)];
-    if (tid < TRN) {
-        double r = 0.0;
-        for (int j = 0; j < TRN; ++j) r += fabs(Ht[tid * TRN + j]);
-        rs[tid] = r;
-    }
-    __syncthreads();
+    // |c|, the largest absolute row sum of B and its smallest diagonal entry
+    __shared__ double rs[TRN], rp[3][TRN], rd[TRN], cb[2 * (TRN + 1)];
+    // sum over j of f(i, j) for every row i, three threads a row (their sums added in order)
+    auto row_sums = [&](auto f) {
+        if (tid < 3 * TRN) {
+            const int i = tid % TRN, part = tid / TRN;
+            double r = 0.0;
+            for (int j = 14 * part; j < min(14 * part + 14, TRN); ++j) r += f(i, j);
+            rp[part][i] = r;
+        }
+        __syncthreads();
+        if (tid < TRN) rs[tid] = rp[0][tid] + rp[1][tid] + rp[2][tid];
+        __syncthreads();
+    };
+    row_sums([&](int i, int j) { return fabs(Ht[i * TRN + j]); });
     __shared__ double bnd[3];
     if (tid < 32) {
         double c2 = 0.0, bn = 0.0, bd = 1e300;
@@ -613,7 +704,7 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     __syncthreads();
     // p = -(B + lam I)^-1 c from the bordered factorisation, and |p| (warp 0)
     auto step_norm = [&]() {
-        warp_bwd(L, rd, L + TRN * TRN, p, TRN);
+        warp_bwd(L, L + TRN * TRN, p, TRN);
         double s = 0.0;
         for (int i = tid; i < TRN; i += 32) {
             p[i] = -p[i];
@@ -647,49 +738,44 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
             float* B32 = reinterpret_cast<float*>(tr_dyn);   // H and H T are dead by now
             float* L32 = B32 + TRN * TRN;
             float* c32 = L32 + (TRN + 1) * TRN;
-            float *p32 = c32 + TRN, *w32 = p32 + TRN, *r32 = w32 + TRN, *b32 = r32 + TRN;   // b32: 2 (TRN + 1)
+            float *p32 = c32 + TRN, *w32 = p32 + TRN, *r32 = w32 + TRN;
+            float* cb32 = B32 + 4 * TRN * TRN;   // 16-byte aligned, past the others
             for (int i = tid; i < TRN * TRN; i += blockDim.x) B32[i] = (float)Ht[i];
             for (int i = tid; i < TRN; i += blockDim.x) c32[i] = (float)cvec[i];
             __syncthreads();
-            double l = lam, lo = lamL, hi = lamU;
-            for (int it = 0; it < 16; ++it) {
-                const bool pd = block_factor<float>(B32, (float)l, c32, L32, b32, r32, TRN, pk);
-                if (tid < 32) {
-                    double nl = l;
-                    int dn = 0;
-                    if (!pd) {
+            if (tid < 32) {
+                double l = lam, lo = lamL, hi = lamU;
+                for (int it = 0; it < 16; ++it) {
+                    bool dn = false;
+                    if (!chol32(B32, (float)l, c32, L32, r32, cb32)) {
                         lo = fmax(lo, l);
-                        nl = fmax(sqrt(fmax(lo, 1e-300) * hi), lo + 0.01 * (hi - lo));
+                        l = fmax(sqrt(fmax(lo, 1e-300) * hi), lo + 0.01 * (hi - lo));
                     } else {
-                        warp_bwd<float>(L32, r32, L32 + TRN * TRN, p32, TRN);
+                        warp_bwd32(L32, r32, L32 + TRN * TRN, p32);
                         float sp = 0.f;
                         for (int i = tid; i < TRN; i += 32) sp += p32[i] * p32[i];
                         const double pn = sqrt((double)warp_sum_f(sp));
                         if (fabs(pn - Delta) <= 1e-4 * Delta) {
-                            dn = 1;
+                            dn = true;
                         } else {
                             if (pn < Delta) hi = l;
                             else lo = l;
-                            warp_fwd<float>(L32, r32, p32, w32, TRN);
+                            warp_fwd32(L32, r32, p32, w32);
                             float sw = 0.f;   // p' (B + lam I)^-1 p
                             for (int i = tid; i < TRN; i += 32) sw += w32[i] * w32[i];
                             const double wn = (double)warp_sum_f(sw);
-                            nl = l + pn * pn * recip_pos(wn) * (pn - Delta) * iDelta;
+                            double nl = l + pn * pn * recip_pos(wn) * (pn - Delta) * iDelta;
                             if (!(nl > lo && nl < hi)) nl = fmax(sqrt(fmax(lo, 1e-300) * hi), lo + 0.01 * (hi - lo));
-                            if (hi - lo <= 1e-6 * fmax(1.0, hi)) dn = 1;
+                            if (hi - lo <= 1e-6 * fmax(1.0, hi)) dn = true;
+                            l = nl;
                         }
                     }
-                    if (tid == 0) {
-                        done = dn;
-                        lam_s = nl;
-                    }
+                    if (dn) break;
                 }
-                __syncthreads();
-                l = lam_s;
-                const int stop = done;
-                __syncthreads();   // every thread has read done and lam_s
-                if (stop) break;
+                if (tid == 0) lam_s = l;
             }
+            __syncthreads();
+            const double l = lam_s;
             if (l > lamL && l < lamU) lam = l;
         }
         for (int it = 0; it < 200; ++it) {
@@ -714,7 +800,7 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
                     } else {
                         if (pn < Delta) lamU = lam;
                         else lamL = lam;
-                        warp_fwd(L, rd, p, w, TRN);
+                        warp_fwd(L, p, w, TRN);
                         double wn = 0.0;   // p' (B + lam I)^-1 p
                         for (int i = tid; i < TRN; i += 32) wn += w[i] * w[i] * rd[i];
                         wn = warp_sum_d(wn);
@@ -745,10 +831,10 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
                 for (int i = tid; i < TRN; i += 32) zs[i] = 1.0 + 0.01 * i;
                 __syncwarp();
                 for (int r = 0; r < 6; ++r) {
-                    warp_fwd(L, rd, zs, ys, TRN);
+                    warp_fwd(L, zs, ys, TRN);
                     for (int i = tid; i < TRN; i += 32) ys[i] *= rd[i];
                     __syncwarp();
-                    warp_bwd(L, rd, ys, w, TRN);
+                    warp_bwd(L, ys, w, TRN);
                     double zn = 0.0;
                     for (int i = 0; i < TRN; ++i) zn += w[i] * w[i];
                     zn = sqrt(zn);
@@ -759,8 +845,7 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
             }
             __syncthreads();
             if (tid == 0) {
-                double z[TRN];
-                for (int i = 0; i < TRN; ++i) z[i] = zs[i];
+                const double* z = zs;
                 double pz = 0.0, pp = 0.0;
                 for (int i = 0; i < TRN; ++i) {
                     pz += p[i] * z[i];
@@ -785,13 +870,8 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
         }
     }
     // predicted gain of the maximisation: g.p + p.H p / 2 = -(c.p + p.B p / 2); the rows
-    // of B p one per thread, the sum in row order
-    if (tid < TRN) {
-        double s = 0.0;
-        for (int j = 0; j < TRN; ++j) s += Ht[tid * TRN + j] * p[j];
-        rs[tid] = s;
-    }
-    __syncthreads();
+    // of B p three threads a row
+    row_sums([&](int i, int j) { return Ht[i * TRN + j] * p[j]; });
     double pred = 0.0;
     if (tid < 32) {
         for (int i = tid; i < TRN; i += 32) pred -= cvec[i] * p[i] + 0.5 * p[i] * rs[i];
