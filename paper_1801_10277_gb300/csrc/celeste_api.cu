@@ -216,6 +216,16 @@ celeste_status ensure_out(celeste_problem* pr) {
     return CELESTE_OK;
 }
 
+// FP32 value / gradient evaluations: the item kernels, which write the status word themselves
+// (every other path starts from a status word that the caller sets to 0)
+bool items_path(const DevProblem& P, int precision, int mode) {
+    return precision == CELESTE_FP32_ACC64 && mode != MODE_HESS && P.ztasks;
+}
+cudaError_t reset_status(const DevProblem& P, int precision, int mode, cudaStream_t st) {
+    if (items_path(P, precision, mode) && P.n_src > 0) return cudaSuccess;
+    return cudaMemsetAsync(P.status, 0, sizeof(int32_t), st);
+}
+
 celeste_status run(celeste_problem* pr, const double* d_theta, int precision, int mode,
                    double* d_total, double* d_local, double* d_grad, double* d_hess,
                    cudaStream_t st) {
@@ -228,8 +238,7 @@ celeste_status run(celeste_problem* pr, const double* d_theta, int precision, in
     // the items (a programmatic dependent of the tables), the per-source epilogues and
     // the total (a programmatic dependent of the items); timed as three stages when
     // profiling.  FP64 and the Hessian: the map / gather / adjoint pipeline below.
-    const bool fused = precision == CELESTE_FP32_ACC64 && mode != MODE_HESS && P.ztasks;
-    if (fused) {
+    if (items_path(P, precision, mode)) {
         static const char* const names[3] = {"tables", "items", "finish"};
         for (int stage = 0; stage < 3; ++stage)
             CEL_CUDA(timed(pr, names[stage], st, [&] {
@@ -253,7 +262,7 @@ celeste_status run(celeste_problem* pr, const double* d_theta, int precision, in
 }
 
 // run() through the graph cache: the first call with an argument set captures the
-// evaluation (with the status reset when reset_status) on the private capture stream and
+// evaluation (with its status reset) on the private capture stream and
 // instantiates it; every call launches the graph on st.  With profiling on, run() is
 // called directly (its per-kernel events are recorded at launch time).
 constexpr size_t MAX_GRAPHS = 8;
@@ -265,22 +274,21 @@ void drop_graphs(celeste_problem* pr) {
 
 celeste_status run_cached(celeste_problem* pr, const double* d_theta, int precision, int mode,
                           double* d_total, double* d_local, double* d_grad, double* d_hess,
-                          cudaStream_t st, bool reset_status) {
+                          cudaStream_t st) {
     const DevProblem& P = pr->P;
     if (pr->profile || !pr->capture) {
-        if (reset_status) CEL_CUDA(cudaMemsetAsync(P.status, 0, sizeof(int32_t), st));
+        CEL_CUDA(reset_status(P, precision, mode, st));
         return run(pr, d_theta, precision, mode, d_total, d_local, d_grad, d_hess, st);
     }
     celeste_problem::GraphKey key{precision, mode, P.tune_contrib, P.tune_adjoint, P.tune_items,
                                   {d_theta, d_total, d_local, d_grad, d_hess}};
-    if (!reset_status) key.mode |= 0x100;
     cudaGraphExec_t exec = nullptr;
     for (auto& g : pr->graphs)
         if (g.first == key) exec = g.second;
     if (!exec) {
         cudaStream_t cs = pr->capture;
         CEL_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-        cudaError_t ce = reset_status ? cudaMemsetAsync(P.status, 0, sizeof(int32_t), cs) : cudaSuccess;
+        const cudaError_t ce = reset_status(P, precision, mode, cs);
         celeste_status rs = ce == cudaSuccess
                                 ? run(pr, d_theta, precision, mode, d_total, d_local, d_grad, d_hess, cs)
                                 : CELESTE_ERR_CUDA;
@@ -322,7 +330,7 @@ celeste_status run_host(celeste_problem* pr, const double* theta, int precision,
                              pr->stream));
     s = run_cached(pr, pr->d_theta, precision, mode, o_total, o_local,
                    mode >= MODE_GRAD ? o_grad : nullptr, mode >= MODE_HESS ? o_hess : nullptr,
-                   pr->stream, true);
+                   pr->stream);
     if (s) return s;
     if (total) CEL_CUDA(cudaMemcpyAsync(total, o_total, sizeof(double), cudaMemcpyDeviceToHost, pr->stream));
     if (local) CEL_CUDA(cudaMemcpyAsync(local, o_local, sizeof(double) * n, cudaMemcpyDeviceToHost, pr->stream));
@@ -818,12 +826,13 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
         void* q;
         if ((st = dalloc(pr, &q, sizeof(double) * ZPCOLS * (size_t)P.n_sitem))) return bail(st);
         P.spart = (double*)q;
-        if ((st = dalloc(pr, &q, sizeof(int32_t)))) return bail(st);
+        if ((st = dalloc(pr, &q, 2 * sizeof(int32_t)))) return bail(st);
         P.zf_done = (int32_t*)q;
-        if (cudaMemset(P.zf_done, 0, sizeof(int32_t)) != cudaSuccess)
-            return bail(fail(CELESTE_ERR_CUDA, "memset"));
         if ((st = dalloc(pr, &q, sizeof(int32_t) * ((size_t)n_patch + 2)))) return bail(st);
         P.zready = (int32_t*)q;
+        if (cudaMemset(P.zf_done, 0, 2 * sizeof(int32_t)) != cudaSuccess ||
+            cudaMemset(P.zready, 0, sizeof(int32_t) * ((size_t)n_patch + 2)) != cudaSuccess)
+            return bail(fail(CELESTE_ERR_CUDA, "memset"));
         if ((st = dalloc(pr, &q, sizeof(float4) * NP * (size_t)n_patch))) return bail(st);
         P.zchain = (float4*)q;
     }
@@ -917,7 +926,7 @@ static celeste_status run_device(celeste_problem* pr, const double* d_theta, int
     cudaStream_t st = (cudaStream_t)stream;
     CEL_CUDA(cudaSetDevice(pr->device));
     // the status word (checked on the device) is reset first
-    return run_cached(pr, d_theta, precision, mode, d_total, d_local, d_grad, d_hess, st, true);
+    return run_cached(pr, d_theta, precision, mode, d_total, d_local, d_grad, d_hess, st);
 }
 
 celeste_status celeste_elbo_device(celeste_problem* pr, const double* d_theta, int32_t precision,
@@ -1033,14 +1042,13 @@ celeste_status celeste_grad_device(celeste_problem* pr, const double* d_theta, i
     CEL_CUDA(cudaSetDevice(pr->device));
     pr->last_stream = st;
     const DevProblem& P = pr->P;
-    CEL_CUDA(cudaMemsetAsync(P.status, 0, sizeof(int32_t), st));
+    CEL_CUDA(reset_status(P, precision, MODE_GRAD, st));
     // FP64: the mixture tables and the E / Var maps of the preceding celeste_elbo_device
     // call are reused; the mixture terms themselves are recomputed by the adjoint.  FP32:
     // the item kernel of celeste_elbo_grad runs again (it recomputes its tables, E and Var
     // from theta; the KL of the preceding forward call is reused), so the gradient is
     // bit-identical to the one-call gradient.
-    const bool fused = precision == CELESTE_FP32_ACC64 && P.ztasks;
-    if (fused) {
+    if (items_path(P, precision, MODE_GRAD)) {
         static const char* const names[3] = {"tables", "items", "finish"};
         for (int stage = 0; stage < 3; ++stage)
             CEL_CUDA(timed(pr, names[stage], st, [&] {
@@ -1101,12 +1109,12 @@ celeste_status celeste_autotune(celeste_problem* pr, const double* theta, int32_
         for (int code = 1; code <= 5 && e == cudaSuccess; ++code) {
             P.tune_items = code;
             celeste_status rs = run_cached(pr, pr->d_theta, CELESTE_FP32_ACC64, MODE_GRAD, o, o + 1,
-                                           o + 1 + P.n_src, nullptr, st, false);
+                                           o + 1 + P.n_src, nullptr, st);
             float t = 0.f;
             if (rs == CELESTE_OK) e = cudaEventRecord(a, st);
             for (int r = 0; r < 2 * reps && rs == CELESTE_OK && e == cudaSuccess; ++r)
                 rs = run_cached(pr, pr->d_theta, CELESTE_FP32_ACC64, MODE_GRAD, o, o + 1, o + 1 + P.n_src,
-                                nullptr, st, false);
+                                nullptr, st);
             if (rs != CELESTE_OK) e = cudaErrorUnknown;
             if (e == cudaSuccess) e = cudaEventRecord(b, st);
             if (e == cudaSuccess) e = cudaEventSynchronize(b);

@@ -340,7 +340,8 @@ struct DevProblem {
     const int32_t* sitem_off;    // [n_src + 1]
     int n_sitem, n_smulti;       // items; those holding multiply covered pixels
     double* spart;               // [n_sitem][ZPCOLS] per-item partials
-    int32_t* zf_done;            // finished sources of the FP32 epilogue kernel, 0 between launches
+    int32_t* zf_done;            // finished sources of the FP32 epilogue kernel, the evaluation's status; 0 between
+                                 // evaluations
     const int32_t* src_active;   // per source: 0 = skip its work (the fit's converged batch
                                  // sources); nullable = every source works
     // the FP32 value / gradient item kernel (item_kernels.cu)
@@ -352,7 +353,7 @@ struct DevProblem {
     float* ztbl;                 // [n_patch][ZFULL_FLOATS] whitened-frame tables (FP32)
     float4* zchain;              // [n_patch][NP] chain-rule records of the patches
     int32_t* zready;             // [n_patch] table ready flags, then the queue counter and the
-                                 // count of built tables (reset before each launch)
+                                 // count of built tables; 0 between evaluations
     int32_t tune_items;          // item kernel variant, 1 .. 5 (pixels per thread, CTAs per SM,
                                  // unroll; item_kernels.cu); 0 = the default, 1
     int32_t model_ne, model_nd;     // exp / dev profile components of the model

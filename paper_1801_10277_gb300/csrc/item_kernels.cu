@@ -655,7 +655,7 @@ struct ItemArgs {
     float* ztbl;               // [patch][ZFULL] tables
     float4* zchain;            // [patch][NP] chain-rule records
     int32_t* ready;            // [patch] table ready flags, then the queue counter and the
-                               // count of built tables; all 0 before the launch
+                               // count of built tables; all 0 between evaluations
     const PatchGeo* geo_tab;
     const ImgMeta* img_tab;
     double* part;              // [item][ZPCOLS]
@@ -665,10 +665,11 @@ struct ItemArgs {
     int n_zcand, n_sitem, n_img_rec;
     double* kl;
     double* kl_grad;
-    int32_t* status;
+    int32_t* status;           // the evaluation's status, 0 between evaluations
+    int32_t* status_out;       // where the epilogue kernel leaves it
     int mode;
     const int32_t* sitem_off;
-    int32_t* grp_done;         // [0]: finished sources of the epilogue kernel, 0 between launches
+    int32_t* grp_done;         // [0]: finished sources of the epilogue kernel, 0 between evaluations
     double* src_total;         // [n_src] each source's share of the total (epilogue kernel)
     double* local_out;
     double* grad_out;
@@ -1033,12 +1034,17 @@ __global__ void __launch_bounds__(128) k_tables(ItemArgs a) {
 // CTA then adds the warps' sums in warp order and subtracts the KL: the local objective
 // and gradient, and the source's share of the total (the ll of the pixels its items own,
 // minus its KL).  The last CTA to finish adds the shares in source order (its warps over
-// contiguous ranges, lanes strided, then warp order) and resets the counter.
+// contiguous ranges, lanes strided, then warp order).  The kernel leaves the flags, counters
+// and the status word of the evaluation at 0 for the next one (the status goes to the
+// caller's word), so an evaluation is three kernels and nothing else: two fills of a few bytes
+// ahead of them cost an evaluation FILL_US.
 constexpr int FIN_W = 4, FIN_WIN = 16;
 __global__ void __launch_bounds__(32 * FIN_W) k_finish(ItemArgs a) {
     __shared__ double sh[FIN_W][64];
     __shared__ int s_last;
     pdl_wait();
+    for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < a.n_patch + 2; i += (int)(gridDim.x * blockDim.x))
+        a.ready[i] = 0;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, s = (int)blockIdx.x;
     const bool grad = a.mode >= MODE_GRAD;
     const int ncol = grad ? ZPCOLS : 2;
@@ -1079,14 +1085,19 @@ __global__ void __launch_bounds__(32 * FIN_W) k_finish(ItemArgs a) {
             if (cA >= 2) a.grad_out[(size_t)NP * s + cA - 2] = tA - __ldcg(a.kl_grad + (size_t)NP * s + cA - 2);
             if (cB < ncol) a.grad_out[(size_t)NP * s + cB - 2] = tB - __ldcg(a.kl_grad + (size_t)NP * s + cB - 2);
         }
-        if (lane == 1 && a.total_out) {
-            a.src_total[s] = tA - klv;   // column 1: owned ll
+        if (lane == 1) {
+            if (a.total_out) a.src_total[s] = tA - klv;   // column 1: owned ll
             s_last = arrive_acq_rel(a.grp_done) == (int)gridDim.x - 1;
         }
     }
-    if (!a.total_out) return;
     __syncthreads();
     if (!s_last) return;
+    if (threadIdx.x == 0) {
+        *a.status_out = *reinterpret_cast<volatile int32_t*>(a.status);
+        *a.status = 0;
+        a.grp_done[0] = 0;
+    }
+    if (!a.total_out) return;
     const int n = a.n_src, per = (n + FIN_W - 1) / FIN_W;
     const int b0 = w * per, b1 = min(n, b0 + per);
     double acc = 0.0;
@@ -1108,7 +1119,6 @@ __global__ void __launch_bounds__(32 * FIN_W) k_finish(ItemArgs a) {
         double t = 0.0;
         for (int v = 0; v < FIN_W; ++v) t += sh[v][0];
         *a.total_out = t;
-        a.grp_done[0] = 0;
     }
 }
 
@@ -1305,7 +1315,8 @@ cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStr
     a.n_img_rec = P.n_img_rec;
     a.kl = P.kl;
     a.kl_grad = P.kl_grad;
-    a.status = P.status;
+    a.status = P.zf_done + 1;
+    a.status_out = P.status;
     a.mode = mode;
     a.sitem_off = P.sitem_off;
     a.grp_done = P.zf_done;
@@ -1314,9 +1325,6 @@ cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStr
     a.grad_out = mode >= MODE_GRAD ? d_grad : nullptr;
     a.total_out = d_total;
     if (stage == 0) {
-        // ready flags, the queue counter and the built-table count start at 0
-        cudaError_t e = cudaMemsetAsync(P.zready, 0, sizeof(int32_t) * ((size_t)P.n_patch + 2), st);
-        if (e != cudaSuccess) return e;
         k_tables<<<(P.n_patch + P.n_src + 3) / 4, 128, 0, st>>>(a);
         return cudaGetLastError();
     }
