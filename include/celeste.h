@@ -327,9 +327,9 @@ celeste_status celeste_grad_device(celeste_problem* prob, const double* d_theta,
  *     256-pixel work items), 3, 5 two or four pixels per thread in packed FP32x2
  *     instructions, 6, 7 the same as persistent CTAs taking items from a work queue.
  *   items_code: the variant of the persistent FP32 value / gradient item kernel (CTAs
- *     of four compute warps and one producer warp), as (pixels per thread, CTAs per SM,
- *     unroll of the loop over profile-component pairs): 1 (2, 2, 7), 2 (3, 2, 3),
- *     3 (2, 3, 2), 4 (3, 2, 7), 5 (3, 2, 2); timed on whole FP32 value + gradient
+ *     of four warps, two pixels per thread), as (CTAs per SM, unroll of the loop over
+ *     profile-component pairs): 1 (4, 7), 2 (3, 7), 3 (4, 2), 4 (4, 3), 5 (3, 3); timed
+ *     on whole FP32 value + gradient
  *     evaluations as the calls run them (the captured CUDA graph).
  * The choices are kept for later FP32 calls and returned (nullable outputs);
  * celeste_set_tuning restores them (contrib 0 .. 7, items 0 .. 5; 0 = the built-in

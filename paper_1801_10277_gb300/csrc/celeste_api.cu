@@ -509,52 +509,6 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
                         c[(size_t)(g.y0 + yy) * im[g.img].W + g.x0 + xx] == 1;
         }
     }
-    // The FP32 value / gradient kernel's items: per source, per patch, the patch's pixels
-    // with the multiply covered ones first (row-major), then the singly covered ones, cut
-    // into ceil(n / cap) items of near-equal size.  cap = ZIMAX, or for a problem too small
-    // to give two items to each of the kernel's resident CTAs (two per SM), the pixel count
-    // that would, rounded up to 64 and at least 128.
-    int item_cap = ZIMAX;
-    {
-        int dev = 0, n_sm = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm <= 0)
-            n_sm = 152;
-        const int64_t per = (n_sp + 4LL * n_sm - 1) / (4LL * n_sm);
-        item_cap = (int)std::min<int64_t>(ZIMAX, std::max<int64_t>(128, (per + 63) / 64 * 64));
-    }
-    struct SItem {
-        int32_t patch, src, n, nm;
-        int64_t q0;   // first pixel (spix)
-    };
-    std::vector<SItem> sitems;
-    std::vector<int32_t> spix, sitem_off(1, 0);
-    int n_smulti = 0;
-    spix.reserve((size_t)n_sp);
-    int64_t sp_single = 0;
-    for (int s = 0; s < n_src; ++s) {
-        for (int p = patch_offsets[s]; p < patch_offsets[s + 1]; ++p) {
-            const PatchGeo& g = geo[p];
-            const uint8_t* f = single.data() + g.sp_off;
-            const int64_t first = (int64_t)spix.size();
-            const int npx = g.w * g.h;
-            for (int q = 0; q < npx; ++q)
-                if (!f[q]) spix.push_back(((q / g.w) << 16) | (q % g.w));
-            const int nm_all = (int)((int64_t)spix.size() - first);
-            for (int q = 0; q < npx; ++q)
-                if (f[q]) spix.push_back(((q / g.w) << 16) | (q % g.w));
-            sp_single += npx - nm_all;
-            const int k = (npx + item_cap - 1) / item_cap, base = npx / k, rem = npx % k;
-            for (int j = 0, o = 0; j < k; ++j) {
-                const int n = base + (j < rem ? 1 : 0);
-                const int nm = std::max(0, std::min(n, nm_all - o));
-                sitems.push_back({p, s, n, nm, first + o});
-                if (nm > 0) ++n_smulti;
-                o += n;
-            }
-        }
-        sitem_off.push_back((int32_t)sitems.size());
-    }
     // tiles: per image a dense grid of TILE x TILE cells, each with its covering patches
     std::vector<Tile> tiles;
     std::vector<int32_t> tile_list;
@@ -588,6 +542,99 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
                 }
         }
     }
+    // The FP32 value / gradient kernel's items: per source, per patch, the patch's pixels
+    // with the multiply covered ones first, then the singly covered ones (row-major), cut
+    // into ceil(n / cap) items of near-equal numbers of whole 64-pixel warp chunks (a patch of
+    // 560 pixels is 9 chunks in two items; two items of 280 pixels are 10).  The multiply covered
+    // ones are grouped by the set of patches that cover them (row-major within a group): a warp
+    // evaluates another patch for a whole chunk if it covers any of its pixels, and in a crowded
+    // field that is a fifth to a quarter less often than in row-major order.  cap = ZIMAX, or for a
+    // problem too small to give an item to each of the kernel's resident CTAs (four per SM), the
+    // pixel count that would, rounded up to a chunk and at least 128 (64 sources, 119,000
+    // source-pixels: 256 pixels 33 us, 128 36 us, 512 37 us; 910,000: 512 pixels 53 us, 256 55 us).
+    int item_cap = ZIMAX;
+    {
+        int dev = 0, n_sm = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm <= 0)
+            n_sm = 152;
+        const int64_t per = (n_sp + 4LL * n_sm - 1) / (4LL * n_sm);
+        item_cap = (int)std::min<int64_t>(ZIMAX, std::max<int64_t>(128, (per + 63) / 64 * 64));
+    }
+    struct SItem {
+        int32_t patch, src, n, nm;
+        int64_t q0;   // first pixel (spix)
+    };
+    std::vector<SItem> sitems;
+    std::vector<int32_t> spix, zitem_off(1, 0);
+    int n_smulti = 0;
+    // a patch's multiply covered pixels (not f), grouped by a bit mask of the other patches that
+    // cover them (patches past the 64th share bits: the groups only order the pixels)
+    std::vector<std::pair<uint64_t, std::vector<int32_t>>> groups;
+    std::vector<uint64_t> mask;
+    std::vector<int32_t> over;
+    auto cover_groups = [&](int p, const uint8_t* f) {
+        const PatchGeo& g = geo[p];
+        const ImgMeta& M = im[g.img];
+        groups.clear();
+        over.clear();
+        for (int ty = g.y0 / TILE; ty <= (g.y0 + g.h - 1) / TILE; ++ty)
+            for (int tx = g.x0 / TILE; tx <= (g.x0 + g.w - 1) / TILE; ++tx) {
+                const int t = tile_grid[M.tg_off + (size_t)ty * M.tgw + tx];
+                if (t < 0) continue;
+                for (int e = 0; e < tiles[t].list_n; ++e)
+                    if (tile_list[tiles[t].list_off + e] != p) over.push_back(tile_list[tiles[t].list_off + e]);
+            }
+        std::sort(over.begin(), over.end());
+        over.erase(std::unique(over.begin(), over.end()), over.end());
+        mask.assign((size_t)g.w * g.h, 0);
+        for (size_t e = 0; e < over.size(); ++e) {
+            const PatchGeo& G = geo[over[e]];
+            const int xa = std::max(0, G.x0 - g.x0), xb = std::min<int>(g.w, G.x0 + G.w - g.x0);
+            const int ya = std::max(0, G.y0 - g.y0), yb = std::min<int>(g.h, G.y0 + G.h - g.y0);
+            for (int y = ya; y < yb; ++y)
+                for (int x = xa; x < xb; ++x) mask[(size_t)y * g.w + x] |= 1ull << (e & 63);
+        }
+        size_t last = 0;
+        for (int q = 0; q < g.w * g.h; ++q) {
+            if (f[q]) continue;
+            if (last >= groups.size() || groups[last].first != mask[q]) {
+                last = 0;
+                while (last < groups.size() && groups[last].first != mask[q]) ++last;
+                if (last == groups.size()) groups.push_back({mask[q], {}});
+            }
+            groups[last].second.push_back(q);
+        }
+        std::sort(groups.begin(), groups.end(),
+                  [](const auto& a, const auto& b) { return a.first < b.first; });
+    };
+    spix.reserve((size_t)n_sp);
+    int64_t sp_single = 0;
+    for (int s = 0; s < n_src; ++s) {
+        for (int p = patch_offsets[s]; p < patch_offsets[s + 1]; ++p) {
+            const PatchGeo& g = geo[p];
+            const uint8_t* f = single.data() + g.sp_off;
+            const int64_t first = (int64_t)spix.size();
+            const int npx = g.w * g.h;
+            cover_groups(p, f);
+            for (const auto& gr : groups)
+                for (int q : gr.second) spix.push_back(((q / g.w) << 16) | (q % g.w));
+            const int nm_all = (int)((int64_t)spix.size() - first);
+            for (int q = 0; q < npx; ++q)
+                if (f[q]) spix.push_back(((q / g.w) << 16) | (q % g.w));
+            sp_single += npx - nm_all;
+            const int k = (npx + item_cap - 1) / item_cap, chunks = (npx + ZCHUNK - 1) / ZCHUNK;
+            const int base = chunks / k, rem = chunks % k;
+            for (int j = 0, o = 0; j < k; ++j) {
+                const int n = std::min(ZCHUNK * (base + (j < rem ? 1 : 0)), npx - o);
+                const int nm = std::max(0, std::min(n, nm_all - o));
+                sitems.push_back({p, s, n, nm, first + o});
+                if (nm > 0) ++n_smulti;
+                o += n;
+            }
+            zitem_off.push_back((int32_t)sitems.size());
+        }
+    }
     // Per item, the other patches covering any of its multiply covered pixels (ascending
     // patch id = ascending source id within an image) and its cost: its pixels plus about
     // a third of a pixel per (64-pixel warp chunk, other patch touching the chunk).
@@ -602,9 +649,9 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
             const ImgMeta& M = im[g.img];
             cand.clear();
             double extra = 0.0;
-            for (int c0 = 0; c0 < it.nm; c0 += 64) {
+            for (int c0 = 0; c0 < it.nm; c0 += ZCHUNK) {
                 chunk.clear();
-                for (int l = c0; l < std::min(it.nm, c0 + 64); ++l) {
+                for (int l = c0; l < std::min(it.nm, c0 + ZCHUNK); ++l) {
                     const int xx = spix[it.q0 + l] & 0xffff, yy = spix[it.q0 + l] >> 16;
                     const int gx = g.x0 + xx, gy = g.y0 + yy;
                     const int tid = tile_grid[M.tg_off + (size_t)(gy / TILE) * M.tgw + gx / TILE];
@@ -799,12 +846,12 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     if ((st = dupload(pr, &d_single, single.data(), single.size()))) return bail(st);
     P.single = d_single;
     if (!sitems.empty()) {
-        int32_t* d_soff = nullptr;
+        int32_t* d_ioff = nullptr;
         ZBuild* d_tord = nullptr;
         ZTask* d_zt = nullptr;
         ZCand* d_zc = nullptr;
         float4* d_zpx = nullptr;
-        if ((st = dupload(pr, &d_soff, sitem_off.data(), sitem_off.size()))) return bail(st);
+        if ((st = dupload(pr, &d_ioff, zitem_off.data(), zitem_off.size()))) return bail(st);
         // build records from the final patch geometry (a patch with its own linearised map
         // refers to the image copy that carries it)
         std::vector<ZBuild> zb;
@@ -815,7 +862,7 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
         if ((st = dupload(pr, &d_zt, ztasks.data(), ztasks.size()))) return bail(st);
         if (!zcands.empty() && (st = dupload(pr, &d_zc, zcands.data(), zcands.size()))) return bail(st);
         if ((st = dupload(pr, &d_zpx, zpx.data(), zpx.size()))) return bail(st);
-        P.sitem_off = d_soff;
+        P.zitem_off = d_ioff;
         P.ztorder = d_tord;
         P.ztasks = d_zt;
         P.n_task = (int32_t)ztasks.size();
@@ -824,8 +871,8 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
         P.n_sitem = (int)sitems.size();
         P.n_smulti = n_smulti;
         void* q;
-        if ((st = dalloc(pr, &q, sizeof(double) * ZPCOLS * (size_t)P.n_sitem))) return bail(st);
-        P.spart = (double*)q;
+        if ((st = dalloc(pr, &q, sizeof(double) * 16 * (size_t)P.n_sitem))) return bail(st);
+        P.zpart = (double*)q;
         if ((st = dalloc(pr, &q, 2 * sizeof(int32_t)))) return bail(st);
         P.zf_done = (int32_t*)q;
         if ((st = dalloc(pr, &q, sizeof(int32_t) * ((size_t)n_patch + 2)))) return bail(st);
@@ -833,7 +880,7 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
         if (cudaMemset(P.zf_done, 0, 2 * sizeof(int32_t)) != cudaSuccess ||
             cudaMemset(P.zready, 0, sizeof(int32_t) * ((size_t)n_patch + 2)) != cudaSuccess)
             return bail(fail(CELESTE_ERR_CUDA, "memset"));
-        if ((st = dalloc(pr, &q, sizeof(float4) * NP * (size_t)n_patch))) return bail(st);
+        if ((st = dalloc(pr, &q, sizeof(float4) * ZCHAIN * (size_t)n_patch))) return bail(st);
         P.zchain = (float4*)q;
     }
     pr->sp_single = sp_single;
@@ -1142,8 +1189,7 @@ celeste_status celeste_set_tuning(celeste_problem* pr, int32_t contrib_code, int
                     "pixels), 6 / 7 the same as persistent CTAs on a work queue");
     if (items_code < 0 || items_code > 5)
         return fail(CELESTE_ERR_ARG,
-                    "items code: 0 default, 1 .. 5 the item kernel's variant (pixels per thread, CTAs per SM, "
-                    "unroll)");
+                    "items code: 0 default, 1 .. 5 the item kernel's variant (CTAs per SM, unroll)");
     pr->P.tune_contrib = contrib_code;
     pr->P.tune_items = items_code;
     return CELESTE_OK;

@@ -45,10 +45,6 @@ constexpr int NYH = NY * (NY + 1) / 2;   // packed upper triangle of the y-Hessi
 // the item's pixels, [1..44] gradient wrt theta (the chain rule applied per item).
 constexpr int PART_LL = 0, PART_TH = 1;
 constexpr int NPART = 1 + NP;
-// Per-item partial record of the FP32 value / gradient kernel (doubles): [0] ll of the
-// item's pixels, [1] ll of the pixels the item owns (its share of the total), [2 .. 2 + NP)
-// d ll / d theta of its source (the patch's chain rule applied per item).
-constexpr int ZPCOLS = 2 + NP;
 // A source's record in the Hessian pass (doubles; hess_kernels.cu): KL, its gradient, the bands'
 // brightness moments, the world-frame shape derivatives
 constexpr int HREC = 104;
@@ -96,7 +92,9 @@ enum : int { Z_K0 = 0, Z_K1, Z_Q0, Z_Q1, Z_MX, Z_MY, Z_ED, Z_GXX, Z_GXY, Z_GYY, 
 constexpr int HV = 1 + NZ + NZ * (NZ + 1) / 2;
 constexpr int ZIMAX = 512;   // most pixels per item of the FP32 value / gradient kernel
 constexpr int ZMAXC = 4;     // other covering patches named inline in such an item's queue record
-constexpr int ZSTAGE = 12;   // other covering patches whose value records an item stages (more are
+constexpr int ZCHUNK = 64;   // pixels of a warp's pass over such an item
+constexpr int ZCHAIN = P_K;  // theta columns that the pixels depend on (the first ones)
+constexpr int ZSTAGE = 8;    // other covering patches whose value records an item stages (more are
                              // read in place)
 constexpr int TILE = 16;     // gather tiles are TILE x TILE pixels
 
@@ -335,11 +333,11 @@ struct DevProblem {
     int32_t* done;           // k_finalize completion counter, 0 between launches
     double* tot_part;        // [64] k_total slice sums
     int32_t* tot_done;       // k_total completion counter, 0 between launches
-    // The FP32 value / gradient kernel's work (item_kernels.cu): a source's items are
-    // contiguous in partial order (sitem_off); ztasks null when there is none.
-    const int32_t* sitem_off;    // [n_src + 1]
+    // The FP32 value / gradient kernel's work (item_kernels.cu): a patch's items are
+    // contiguous, the patches in order; ztasks null when there is none.
+    const int32_t* zitem_off;    // [n_patch + 1] first item of each patch
     int n_sitem, n_smulti;       // items; those holding multiply covered pixels
-    double* spart;               // [n_sitem][ZPCOLS] per-item partials
+    double* zpart;               // [n_sitem][16] per-item sums
     int32_t* zf_done;            // finished sources of the FP32 epilogue kernel, the evaluation's status; 0 between
                                  // evaluations
     const int32_t* src_active;   // per source: 0 = skip its work (the fit's converged batch
@@ -351,11 +349,11 @@ struct DevProblem {
     const ZCand* zcands;
     const float4* zpx;           // per item pixel: (column, row in the patch, counts, sky)
     float* ztbl;                 // [n_patch][ZFULL_FLOATS] whitened-frame tables (FP32)
-    float4* zchain;              // [n_patch][NP] chain-rule records of the patches
+    float4* zchain;              // [n_patch][ZCHAIN] chain-rule records of the patches
     int32_t* zready;             // [n_patch] table ready flags, then the queue counter and the
                                  // count of built tables; 0 between evaluations
-    int32_t tune_items;          // item kernel variant, 1 .. 5 (pixels per thread, CTAs per SM,
-                                 // unroll; item_kernels.cu); 0 = the default, 1
+    int32_t tune_items;          // item kernel variant, 1 .. 5 (CTAs per SM, unroll;
+                                 // item_kernels.cu); 0 = the default, 1
     int32_t model_ne, model_nd;     // exp / dev profile components of the model
     int32_t* hqueue;         // [2] the Hessian pass's work queue (next part, finished CTAs), 0 between launches
     int32_t* queue;          // [2] work queue of the FP64 / Hessian map pass's persistent variants

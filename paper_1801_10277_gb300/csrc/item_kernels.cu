@@ -20,21 +20,20 @@
 // Work.  Three launches.  k_tables builds every patch's table and chain-rule record (one
 // warp per patch, FP32 with the position in FP64), publishing each with a ready flag, and
 // every source's KL terms (one warp per source).  k_items, its programmatic dependent,
-// runs on persistent CTAs of four compute warps and a producer warp that take items from
-// a queue (a global counter over the items in decreasing cost): up to ZIMAX pixels of one
-// patch, the multiply covered ones first.  The producer waits for the tables an item
-// reads and copies its patch's table and chain-rule record, its pixel records and the
-// value records of up to ZSTAGE other patches covering its pixels into a shared-memory
-// stage with bulk asynchronous copies (two stages, completing on mbarriers), while the
-// compute warps run the item in the other stage.  They evaluate the mixture and its
-// derivatives at the item's pixels; where other patches cover a pixel, E = sky + sum_s
+// runs on persistent CTAs of four warps that take items from a queue (a global counter over
+// the items in decreasing cost): up to ZIMAX pixels of one patch, the multiply covered ones
+// first.  An item's patch table, its pixel records and the value records of up to ZSTAGE other
+// patches covering its pixels are copied into a shared-memory stage with bulk asynchronous
+// copies (two stages, completing on mbarriers; the warp that finishes an item last waits for
+// the tables that the item after the next reads and starts its copies), while the warps take the
+// chunks of 64 pixels of the item in the other stage in turn.  They evaluate the mixture and its
+// derivatives at the chunk's pixels; where other patches cover a pixel, E = sky + sum_s
 // E_s and Var = sum_s Var_s are summed over every covering source in ascending source
-// order (every covering item forms the same sum, bit for bit).  Per warp FP32 sums; the
-// producer adds the warps in FP64, applies the patch's chain rule dy/dtheta and writes the
-// item's record.  k_finish, k_items' programmatic dependent, runs every
-// source's epilogue once the items are done (one CTA per source: FP64 sums of its item
-// records in a fixed order, minus the KL); the last CTA to finish adds the sources' shares
-// of the total in source order.
+// order (every covering item forms the same sum, bit for bit).  FP32 sums per chunk, added
+// in FP64 to the item's record (ll and d ll / d y).  k_finish, k_items' programmatic
+// dependent, runs every source's epilogue once the items are done (FP64 sums of each patch's
+// item records in a fixed order, the patch's chain rule dy/dtheta, minus the KL); the last
+// CTA to finish adds the sources' shares of the total in source order.
 // Every wait is bounded (~1 s), after which the kernel records CELESTE_ERR_TIMEOUT and
 // ends.
 #include <math.h>
@@ -67,7 +66,8 @@ constexpr float HL = -0.72134752044448170368f;   // -log2(e) / 2
 //   (s = sign(alpha_k) (1 - e_dev) for exp components, sign(alpha_k) e_dev for dev ones);
 //   exp components fill pairs 0 .. npe-1, dev components pairs npe .. npe+npd-1, each
 //   group padded to an even count with a component of weight zero (C = -1e30).
-// Chain-rule record of a patch: per theta column j, (k0, k1, k2, y0 | y1 << 4 | y2 << 8):
+// Chain-rule record of a patch: per theta column j < ZCHAIN (the pixels do not depend on the
+// others), (k0, k1, k2, y0 | y1 << 4 | y2 << 8):
 // d y_{y_e} / d theta_j = k_e (unused pairs y = 0, k = 0).
 constexpr int ZMAXPAIR = (MAXPROF + 2) / 2;
 constexpr int VH = 16, VKH = 8, VPAIR = 8, VK = VKH + ZMAXPAIR * VPAIR, VFULL = VH + MAXPSF * VK;
@@ -76,48 +76,48 @@ constexpr int ZFULL = VFULL + GFULL;
 static_assert(ZFULL == ZFULL_FLOATS, "table size");
 static_assert(VFULL % 4 == 0 && ZFULL % 4 == 0, "tables are copied in 16-byte units");
 
-// CTA shape: four compute warps and the producer warp
+// CTA shape: four warps
 constexpr int NWC = 4;
 constexpr int NTC = 32 * NWC;
-constexpr int IT_THREADS = NTC + 32;
 
-// One shared-memory stage (bytes): the item's table, its patch's chain-rule record, its
-// pixel records, and its first ZSTAGE candidates' records and value tables.
+// One shared-memory stage (bytes): the item's table, its pixel records, and its first
+// ZSTAGE candidates' records and value tables.
 constexpr int ST_TBL = 0;
-constexpr int ST_CHAIN = ST_TBL + ZFULL * 4;
-constexpr int ST_PX = ST_CHAIN + NP * 16;
+constexpr int ST_PX = ST_TBL + ZFULL * 4;
 constexpr int ST_ZC = ST_PX + ZIMAX * 16;
 constexpr int ST_VREC = ST_ZC + ZSTAGE * (int)sizeof(ZCand);
 constexpr int ST_BYTES = ST_VREC + ZSTAGE * VFULL * 4;
-static_assert(ST_CHAIN % 16 == 0 && ST_PX % 16 == 0 && ST_ZC % 16 == 0 && ST_VREC % 16 == 0 && ST_BYTES % 16 == 0,
+static_assert(ST_PX % 16 == 0 && ST_ZC % 16 == 0 && ST_VREC % 16 == 0 && ST_BYTES % 16 == 0,
               "bulk copies land on 16-byte boundaries");
 static_assert(sizeof(ZCand) == 32 && sizeof(ZTask) == 64, "record sizes");
 
 constexpr int PG_F = 10;                 // floats of a ProfileGrad
-constexpr int NSUM = 2 + NY;             // per-thread sums: ll, d ll / d y, owned ll
 constexpr int SCR_W = 880;               // bytes per warp of the table kernel: KL arrays (2 x 44
                                          // doubles, 44 floats) or the table builder's 96 floats
-constexpr int RED_W = 16;                // floats per warp of an item's warp sums
+
+// Pixels per thread; a chunk is the 32 PX pixels of one pass of a warp
+constexpr int PX = 2;
+static_assert(32 * PX == ZCHUNK, "chunk size");
 
 // the rest of the item kernel's shared memory (bytes), after the two stages
-template <int PX>
 struct Lay {
-    static constexpr int vs = 2 * ST_BYTES;                        // running sums [NSUM][NTC]
-    static constexpr int pg = vs + NSUM * NTC * 4;                 // stashed derivatives [PX PG_F][NTC]
-    static constexpr int red = pg + PX * PG_F * NTC * 4;           // [2][NWC][RED_W] warp sums
-    static constexpr int bar = red + 2 * NWC * RED_W * 4;          // full[2], reduced[2]
-    static constexpr int task = bar + 4 * 8;                       // [2] ZTask
-    static constexpr int bytes = task + 2 * (int)sizeof(ZTask);
+    static constexpr int pg = 2 * ST_BYTES;                        // stashed derivatives [PX PG_F][NTC]
+    static constexpr int nch = ZIMAX / ZCHUNK;                     // most chunks of an item
+    static constexpr int red = pg + PX * PG_F * NTC * 4;           // [2][nch][16] chunk sums
+    static constexpr int bar = red + 2 * nch * 16 * 4;             // full[2], fetched[2]
+    static constexpr int task = bar + 4 * 8;                       // [2] ZTask: the stages' items
+    static constexpr int next = task + 2 * (int)sizeof(ZTask);     // [2] ZTask: records fetched ahead
+    static constexpr int cnt = next + 2 * (int)sizeof(ZTask);      // [2] warps done with the stage's item,
+                                                                   // [2] its chunks taken
+    static constexpr int bytes = cnt + 16;
     static_assert(task % 16 == 0 && bar % 8 == 0, "alignment");
 };
 
-// Registers per thread with MINB CTAs of IT_THREADS threads per SM: the SM's 64K
-// registers, and each of its four sub-partitions' 16K over the warps it holds (warps are
-// spread evenly), in multiples of 8.
+// Registers per thread with MINB CTAs of four warps per SM (one per sub-partition, whose 16K
+// registers its MINB warps share), in multiples of 8.
 constexpr int regs_for(int minb) {
-    const int warps = minb * (IT_THREADS / 32), per_part = (warps + 3) / 4;
-    const int a = 65536 / (minb * IT_THREADS), b = 16384 / (per_part * 32);
-    return (a < b ? a : b) & ~7;
+    const int r = (16384 / (minb * 32)) & ~7;
+    return r < 248 ? r : 248;
 }
 
 __device__ __forceinline__ float ex2f(float x) {
@@ -329,11 +329,11 @@ __device__ __forceinline__ void build_patch_table(const double* __restrict__ the
     float dG[3][3];
 #pragma unroll
     for (int e = 0; e < 9; ++e) dG[e / 3][e % 3] = dgs[e];
-    for (int j = lane; j < NP; j += 32) {
+    if (lane < ZCHAIN) {
         int y0, y1, y2;
         float k0, k1, k2;
-        chain_column<float>(j, band, Af, el, el2, dG, &y0, &k0, &y1, &k1, &y2, &k2);
-        zchain[(size_t)patch * NP + j] = make_float4(k0, k1, k2, __int_as_float(y0 | (y1 << 4) | (y2 << 8)));
+        chain_column<float>(lane, band, Af, el, el2, dG, &y0, &k0, &y1, &k1, &y2, &k2);
+        zchain[(size_t)patch * ZCHAIN + lane] = make_float4(k0, k1, k2, __int_as_float(y0 | (y1 << 4) | (y2 << 8)));
     }
 }
 
@@ -431,7 +431,7 @@ __device__ __forceinline__ void source_ev(const float* H, float G0, float G1, fl
 
 // the profile sums g0 (star), g1 (galaxy) of one patch at PX pixels from its value part
 // (an item's own table or another patch's value record: the same layout)
-template <int PX, int NPE, int NPD>
+template <int NPE, int NPD>
 __device__ __forceinline__ void profile_value(const float* H, int npsf, int npe_rt, int npd_rt,
                                               const float (&X)[PX], const float (&Y)[PX], float (&G0)[PX],
                                               float (&G1)[PX]) {
@@ -490,7 +490,7 @@ static_assert(sizeof(ProfileGrad) == PG_F * sizeof(float), "ProfileGrad layout")
 // the profile sums and their derivatives of the item's own patch at PX pixels; g0 and g1
 // are formed with exactly the operations of profile_value (UNR: unroll factor of the
 // loop over component pairs)
-template <int PX, int NPE, int NPD, int UNR>
+template <int NPE, int NPD, int UNR>
 __device__ __forceinline__ void profile_grad(const float* H, int npsf, int npe_rt, int npd_rt,
                                              const float (&X)[PX], const float (&Y)[PX],
                                              ProfileGrad (&o)[PX]) {
@@ -593,17 +593,17 @@ __device__ __forceinline__ void pix_weights(float x, float E, float V, float& cE
 
 // the item's own source at this thread's pixels: E_s, Var_s, f_i and (gradient) the
 // profile sums with their derivatives
-template <int MODE, int PX, int NPE, int NPD, int UNR>
+template <int MODE, int NPE, int NPD, int UNR>
 __device__ __forceinline__ void own_source(const float* H, int npsf, int npe, int npd, const float (&X)[PX],
                                            const float (&Y)[PX], float (&Es)[PX], float (&Vs)[PX],
                                            float (&f0)[PX], float (&f1)[PX], ProfileGrad (&pg)[PX]) {
     if constexpr (MODE == MODE_LL) {
         float G0[PX], G1[PX];
-        profile_value<PX, NPE, NPD>(H, npsf, npe, npd, X, Y, G0, G1);
+        profile_value<NPE, NPD>(H, npsf, npe, npd, X, Y, G0, G1);
 #pragma unroll
         for (int p = 0; p < PX; ++p) source_ev(H, G0[p], G1[p], f0[p], f1[p], Es[p], Vs[p]);
     } else {
-        profile_grad<PX, NPE, NPD, UNR>(H, npsf, npe, npd, X, Y, pg);
+        profile_grad<NPE, NPD, UNR>(H, npsf, npe, npd, X, Y, pg);
 #pragma unroll
         for (int p = 0; p < PX; ++p) source_ev(H, pg[p].g0, pg[p].g1, f0[p], f1[p], Es[p], Vs[p]);
     }
@@ -653,12 +653,13 @@ struct ItemArgs {
     const ModelDev* md;
     const double* theta;
     float* ztbl;               // [patch][ZFULL] tables
-    float4* zchain;            // [patch][NP] chain-rule records
+    float4* zchain;            // [patch][ZCHAIN] chain-rule records
     int32_t* ready;            // [patch] table ready flags, then the queue counter and the
                                // count of built tables; all 0 between evaluations
     const PatchGeo* geo_tab;
     const ImgMeta* img_tab;
-    double* part;              // [item][ZPCOLS]
+    double* part;              // [item][16] sums: ll, owned ll, d ll / d y
+    const int32_t* item_off;   // [n_patch + 1] first item of each patch
     int ne, nd;                // exp / dev profile components
     int n_patch, n_src;
     int64_t n_sp;              // pixel records (bounds checks)
@@ -668,7 +669,7 @@ struct ItemArgs {
     int32_t* status;           // the evaluation's status, 0 between evaluations
     int32_t* status_out;       // where the epilogue kernel leaves it
     int mode;
-    const int32_t* sitem_off;
+    const int32_t* patch_off;  // [n_src + 1] first patch of each source
     int32_t* grp_done;         // [0]: finished sources of the epilogue kernel, 0 between evaluations
     double* src_total;         // [n_src] each source's share of the total (epilogue kernel)
     double* local_out;
@@ -698,16 +699,62 @@ __device__ __forceinline__ int arrive_acq_rel(int32_t* ctr) {
 // ---------------------------------------------------------------------------------
 // tasks of the compute warps
 
-// One item on the four compute warps: warp w takes the chunks of 32 PX pixels w, w + 4,
-// ... (PX consecutive pixels per thread); the thread's running sums wait in shared memory
-// between chunks; a chunk that holds multiply covered pixels (warp-uniform) stashes its
-// derivatives in shared memory while the other covering patches are evaluated.  Each
-// warp leaves its FP32 sums (ll, d ll / d y, owned ll) in red (lane 0).
-template <int MODE, int PX, int NPE, int NPD, int UNR>
-__device__ __forceinline__ void item_compute(const ItemArgs& a, const ZItem& it, const uint8_t* stage,
-                                             float* vs, float* spg, float* red) {
+// The sums over a warp's lanes of N <= 16 values, each along the same tree (FP32); value j is
+// returned on the lanes 2 j and 2 j + 1.  Halving the values with each exchange takes 16 shuffles
+// for 16 values instead of 80.
+template <int N>
+__device__ __forceinline__ float warp_sums(const float (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    float r[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) r[j] = j < N ? v[j] : 0.f;
+#pragma unroll
+    for (int h = 8; h >= 1; h >>= 1) {
+        const bool up = lane & (2 * h);
+#pragma unroll
+        for (int j = 0; j < h; ++j) {
+            const float keep = up ? r[j + h] : r[j], send = up ? r[j] : r[j + h];
+            r[j] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, 2 * h));
+        }
+    }
+    return __fadd_rn(r[0], __shfl_xor_sync(0xffffffffu, r[0], 1));
+}
+
+// float -> double without the FP64 pipe (whose conversions take as long as its arithmetic)
+// unless a lane holds a denormal, an infinity or a NaN.  Every lane calls it.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned b = __float_as_uint(f), e = b & 0x7f800000u;
+    if (__any_sync(0xffffffffu, e == 0x7f800000u || (e == 0 && (b << 1) != 0))) return (double)f;
+    const unsigned hi = ((b & 0x7fffffffu) >> 3) + 0x38000000u;
+    return __hiloint2double((int)((b & 0x80000000u) | (e ? hi : 0u)), (int)(b << 29));
+}
+
+// An item's record from its chunks' sums: FP64, lanes c and c + 16 column c of every other
+// chunk, then the two added
+template <int MODE>
+__device__ __forceinline__ void item_record(const ItemArgs& a, int out, const float* red, int nch) {
+    const int lane = threadIdx.x & 31, col = lane & 15, half = lane >> 4;
+    constexpr int NS = (MODE == MODE_LL) ? 2 : 2 + NY;
+    float r[Lay::nch / 2];
+#pragma unroll
+    for (int u = 0; u < Lay::nch / 2; ++u) r[u] = col < NS && 2 * u + half < nch ? red[(2 * u + half) * 16 + col] : 0.f;
+    double y = widen(r[0]);
+#pragma unroll
+    for (int u = 1; u < Lay::nch / 2; ++u)
+        if (2 * u < nch) y += widen(r[u]);
+    y += __shfl_xor_sync(0xffffffffu, y, 16);
+    if (lane < NS) a.part[(size_t)out * 16 + lane] = y;
+}
+
+// One chunk of an item on a warp: the 32 PX pixels from c0 on (PX consecutive ones per
+// thread).  A chunk that holds multiply covered pixels (warp-uniform) stashes its derivatives
+// in shared memory while the other covering patches are evaluated.  The chunk's FP32 sums
+// (ll, owned ll, d ll / d y) go to rec.
+template <int MODE, int NPE, int NPD, int UNR>
+__device__ __forceinline__ void chunk_compute(const ItemArgs& a, const ZItem& it, const uint8_t* stage, int c0,
+                                              float* spg, float* rec) {
     constexpr int NV = (MODE == MODE_LL) ? 1 : 1 + NY;   // ll (+ d ll / d y)
-    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    const int lane = threadIdx.x & 31;
     const int n = it.n_nm & 0xffff, nm = it.n_nm >> 16;
     const int npsf = it.nc_npsf >> 24, nc = it.nc_npsf & 0xffffff;
     const int npe = (a.ne + 1) >> 1, npd = (a.nd + 1) >> 1;
@@ -715,126 +762,119 @@ __device__ __forceinline__ void item_compute(const ItemArgs& a, const ZItem& it,
     const float4* pxr = reinterpret_cast<const float4*>(stage + ST_PX);
     const ZCand* zc = reinterpret_cast<const ZCand*>(stage + ST_ZC);
     const float* vrec = reinterpret_cast<const float*>(stage + ST_VREC);
+    float X[PX], Y[PX], xv[PX], sky[PX];
+    bool ok[PX];
 #pragma unroll
-    for (int i = 0; i <= NV; ++i) vs[i * NTC] = 0.f;
-    for (int c0 = w * 32 * PX; c0 < n; c0 += NWC * 32 * PX) {
-        float X[PX], Y[PX], xv[PX], sky[PX];
-        bool ok[PX];
-#pragma unroll
-        for (int p = 0; p < PX; ++p) {
-            const int l = c0 + lane * PX + p;
-            ok[p] = l < n;
-            const float4 r = pxr[ok[p] ? l : n - 1];
-            X[p] = r.x;
-            Y[p] = r.y;
-            xv[p] = r.z;
-            sky[p] = r.w;
-        }
-        float Es[PX], Vs[PX], f0[PX], f1[PX];
-        ProfileGrad pg[PX];
-        own_source<MODE, PX, NPE, NPD, UNR>(T, npsf, npe, npd, X, Y, Es, Vs, f0, f1, pg);
-        float E[PX], V[PX];
-        bool owner[PX];
-        if (c0 < nm) {
-            // E and Var over every covering source in ascending source order; the item's
-            // own source enters at its place
-            if constexpr (MODE >= MODE_GRAD) {
-#pragma unroll
-                for (int p = 0; p < PX; ++p) {
-                    const float* q = reinterpret_cast<const float*>(&pg[p]);
-#pragma unroll
-                    for (int f = 0; f < PG_F; ++f) spg[(p * PG_F + f) * NTC] = q[f];
-                }
-            }
-            bool added = false;
+    for (int p = 0; p < PX; ++p) {
+        const int l = c0 + lane * PX + p;
+        ok[p] = l < n;
+        const float4 r = pxr[ok[p] ? l : n - 1];
+        X[p] = r.x;
+        Y[p] = r.y;
+        xv[p] = r.z;
+        sky[p] = r.w;
+    }
+    float Es[PX], Vs[PX], f0[PX], f1[PX];
+    ProfileGrad pg[PX];
+    own_source<MODE, NPE, NPD, UNR>(T, npsf, npe, npd, X, Y, Es, Vs, f0, f1, pg);
+    float E[PX], V[PX];
+    bool owner[PX];
+    if (c0 < nm) {
+        // E and Var over every covering source in ascending source order; the item's
+        // own source enters at its place
+        if constexpr (MODE >= MODE_GRAD) {
 #pragma unroll
             for (int p = 0; p < PX; ++p) {
-                E[p] = sky[p];
-                V[p] = 0.f;
-                owner[p] = true;
+                const float* q = reinterpret_cast<const float*>(&pg[p]);
+#pragma unroll
+                for (int f = 0; f < PG_F; ++f) spg[(p * PG_F + f) * NTC] = q[f];
             }
-            for (int ci = 0; ci < nc; ++ci) {
-                const ZCand c = ci < ZSTAGE ? zc[ci] : a.cands[it.c0 + ci];
-                const float* R = ci < ZSTAGE ? vrec + ci * VFULL : a.ztbl + (size_t)c.patch * ZFULL;
-                if (!added && c.src > it.src) {
+        }
+        bool added = false;
 #pragma unroll
-                    for (int p = 0; p < PX; ++p) {
-                        E[p] = __fadd_rn(E[p], Es[p]);
-                        V[p] = __fadd_rn(V[p], Vs[p]);
-                    }
-                    added = true;
-                }
-                float Xc[PX], Yc[PX];
-                bool in[PX], any = false;
-#pragma unroll
-                for (int p = 0; p < PX; ++p) {
-                    const int xx = (int)X[p] - c.dx, yy = (int)Y[p] - c.dy;
-                    in[p] = ok[p] && xx >= 0 && xx < c.w && yy >= 0 && yy < c.h;
-                    Xc[p] = (float)xx;
-                    Yc[p] = (float)yy;
-                    any = any || in[p];
-                    if (in[p] && c.src < it.src) owner[p] = false;
-                }
-                if (!__any_sync(0xffffffffu, any)) continue;
-                float G0[PX], G1[PX];
-                profile_value<PX, NPE, NPD>(R, c.npsf, npe, npd, Xc, Yc, G0, G1);
-#pragma unroll
-                for (int p = 0; p < PX; ++p) {
-                    float q0, q1, ec, vc;
-                    source_ev(R, G0[p], G1[p], q0, q1, ec, vc);
-                    if (in[p]) {
-                        E[p] = __fadd_rn(E[p], ec);
-                        V[p] = __fadd_rn(V[p], vc);
-                    }
-                }
-            }
-            if (!added)
+        for (int p = 0; p < PX; ++p) {
+            E[p] = sky[p];
+            V[p] = 0.f;
+            owner[p] = true;
+        }
+        for (int ci = 0; ci < nc; ++ci) {
+            const ZCand c = ci < ZSTAGE ? zc[ci] : a.cands[it.c0 + ci];
+            const float* R = ci < ZSTAGE ? vrec + ci * VFULL : a.ztbl + (size_t)c.patch * ZFULL;
+            if (!added && c.src > it.src) {
 #pragma unroll
                 for (int p = 0; p < PX; ++p) {
                     E[p] = __fadd_rn(E[p], Es[p]);
                     V[p] = __fadd_rn(V[p], Vs[p]);
                 }
-            if constexpr (MODE >= MODE_GRAD) {
-#pragma unroll
-                for (int p = 0; p < PX; ++p) {
-                    float* q = reinterpret_cast<float*>(&pg[p]);
-#pragma unroll
-                    for (int f = 0; f < PG_F; ++f) q[f] = spg[(p * PG_F + f) * NTC];
-                }
+                added = true;
             }
-        } else {
+            float Xc[PX], Yc[PX];
+            bool in[PX], any = false;
 #pragma unroll
             for (int p = 0; p < PX; ++p) {
-                E[p] = __fadd_rn(sky[p], Es[p]);
-                V[p] = Vs[p];
-                owner[p] = true;
+                const int xx = (int)X[p] - c.dx, yy = (int)Y[p] - c.dy;
+                in[p] = ok[p] && xx >= 0 && xx < c.w && yy >= 0 && yy < c.h;
+                Xc[p] = (float)xx;
+                Yc[p] = (float)yy;
+                any = any || in[p];
+                if (in[p] && c.src < it.src) owner[p] = false;
+            }
+            if (!__any_sync(0xffffffffu, any)) continue;
+            float G0[PX], G1[PX];
+            profile_value<NPE, NPD>(R, c.npsf, npe, npd, Xc, Yc, G0, G1);
+#pragma unroll
+            for (int p = 0; p < PX; ++p) {
+                float q0, q1, ec, vc;
+                source_ev(R, G0[p], G1[p], q0, q1, ec, vc);
+                if (in[p]) {
+                    E[p] = __fadd_rn(E[p], ec);
+                    V[p] = __fadd_rn(V[p], vc);
+                }
             }
         }
-        float v[NV + 1];
+        if (!added)
 #pragma unroll
-        for (int i = 0; i <= NV; ++i) v[i] = vs[i * NTC];
+            for (int p = 0; p < PX; ++p) {
+                E[p] = __fadd_rn(E[p], Es[p]);
+                V[p] = __fadd_rn(V[p], Vs[p]);
+            }
+        if constexpr (MODE >= MODE_GRAD) {
+#pragma unroll
+            for (int p = 0; p < PX; ++p) {
+                float* q = reinterpret_cast<float*>(&pg[p]);
+#pragma unroll
+                for (int f = 0; f < PG_F; ++f) q[f] = spg[(p * PG_F + f) * NTC];
+            }
+        }
+    } else {
 #pragma unroll
         for (int p = 0; p < PX; ++p) {
-            if (!ok[p]) continue;
-            float vv[NV], ll;
-#pragma unroll
-            for (int i = 0; i < NV; ++i) vv[i] = v[i];
-            pixel_terms<MODE, NV>(T, xv[p], E[p], V[p], Es[p], f0[p], f1[p], pg[p], vv, ll);
-#pragma unroll
-            for (int i = 0; i < NV; ++i) v[i] = vv[i];
-            if (owner[p]) v[NV] += ll;
+            E[p] = __fadd_rn(sky[p], Es[p]);
+            V[p] = Vs[p];
+            owner[p] = true;
         }
-#pragma unroll
-        for (int i = 0; i <= NV; ++i) vs[i * NTC] = v[i];
     }
-    // the warp's sums (FP32 shuffle tree) to red
+    float v[NV + 1];
 #pragma unroll
-    for (int i = 0; i <= NV; ++i) {
-        float s = vs[i * NTC];
+    for (int i = 0; i <= NV; ++i) v[i] = 0.f;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) red[i] = s;
+    for (int p = 0; p < PX; ++p) {
+        if (!ok[p]) continue;
+        float vv[NV], ll;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) vv[i] = v[i];
+        pixel_terms<MODE, NV>(T, xv[p], E[p], V[p], Es[p], f0[p], f1[p], pg[p], vv, ll);
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] = vv[i];
+        if (owner[p]) v[NV] += ll;
     }
+    float c[NV + 1];
+    c[0] = v[0];
+    c[1] = v[NV];
+#pragma unroll
+    for (int i = 1; i < NV; ++i) c[1 + i] = v[i];
+    const float r = warp_sums(c);
+    if (!(lane & 1) && (lane >> 1) <= NV) rec[lane >> 1] = r;
 }
 
 // the KL value and gradient of source s on one warp (with the domain check of its theta)
@@ -856,64 +896,8 @@ __device__ __forceinline__ void kl_task(const ItemArgs& a, int s, float* scr) {
     for (int i = lane; i < NP; i += 32) a.kl_grad[(size_t)NP * s + i] = kg[i];
 }
 
-// After an item, on the producer warp: the compute warps' sums added in warp order
-// (FP64), the patch's chain rule applied (column j of d ll / d theta =
-// sum_e k_e d ll / d y_{y_e}, FP64) and the item's record written.  In two parts: what
-// the record needs from the item's stage and warp sums, read into registers (so that the
-// stage can take its next item at once), then the FP64 arithmetic and the stores.
-struct ItemSums {
-    float r[NWC];       // lane < NS: the warps' sums of column lane
-    float4 ch[2];       // the chain-rule columns lane, lane + 32
-};
-
-template <int MODE>
-__device__ __forceinline__ ItemSums finish_load(const uint8_t* stage, const float* red) {
-    const int lane = threadIdx.x & 31;
-    constexpr int NS = (MODE == MODE_LL) ? 2 : 2 + NY;   // ll, (d ll / d y), owned ll
-    ItemSums q;
-#pragma unroll
-    for (int w = 0; w < NWC; ++w) q.r[w] = lane < NS ? red[w * RED_W + lane] : 0.f;
-    if constexpr (MODE >= MODE_GRAD) {
-        const float4* ch = reinterpret_cast<const float4*>(stage + ST_CHAIN);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int c = lane + 32 * h;
-            q.ch[h] = ch[c < NP ? c : 0];
-        }
-    }
-    return q;
-}
-
-template <int MODE>
-__device__ __forceinline__ void finish_store(const ItemArgs& a, int out, const ItemSums& q) {
-    const int lane = threadIdx.x & 31;
-    constexpr int NS = (MODE == MODE_LL) ? 2 : 2 + NY;
-    double y = 0.0;
-    if (lane < NS)
-#pragma unroll
-        for (int w = 0; w < NWC; ++w) y += (double)q.r[w];
-    double* rec = a.part + (size_t)out * ZPCOLS;
-    if (lane == 0) rec[0] = y;
-    if (lane == NS - 1) rec[1] = y;
-    if constexpr (MODE >= MODE_GRAD) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int c = lane + 32 * h;
-            const float4 r = q.ch[h];
-            const int yy = __float_as_int(r.w);
-            const double y0 = __shfl_sync(0xffffffffu, y, 1 + (yy & 15));
-            const double y1 = __shfl_sync(0xffffffffu, y, 1 + ((yy >> 4) & 15));
-            const double y2 = __shfl_sync(0xffffffffu, y, 1 + ((yy >> 8) & 15));
-            double g = (double)r.x * y0;
-            g = fma((double)r.y, y1, g);
-            g = fma((double)r.z, y2, g);
-            if (c < NP) rec[2 + c] = g;
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------------
-// the producer warp
+// staging the items
 
 // the 64-byte record of queue slot q, a quarter per lane 0 .. 3 (past the end: an end
 // marker)
@@ -981,10 +965,9 @@ __device__ void prepare(const ItemArgs& a, int4 rec, uint8_t* stage, ZTask* tk, 
     __syncwarp();
     // lane 0 announces the bytes before any copy is issued
     const unsigned tbl_bytes = MODE == MODE_LL ? VFULL * 4 : ZFULL * 4;
-    const unsigned chain_bytes = MODE == MODE_LL ? 0u : NP * 16;
     if (lane == 0) {
         const unsigned bytes =
-            tbl_bytes + chain_bytes + (unsigned)n * 16u + (unsigned)nc0 * (unsigned)(sizeof(ZCand) + VFULL * 4);
+            tbl_bytes + (unsigned)n * 16u + (unsigned)nc0 * (unsigned)(sizeof(ZCand) + VFULL * 4);
         mbar_expect_arrive(full, bytes);
     }
     __syncwarp();
@@ -992,7 +975,6 @@ __device__ void prepare(const ItemArgs& a, int4 rec, uint8_t* stage, ZTask* tk, 
     fence_proxy_async_smem();   // the stage was last read through the generic proxy
     if (lane == 0) {
         bulk_g2s_tx(stage + ST_TBL, a.ztbl + (size_t)it.patch * ZFULL, tbl_bytes, full);
-        if (chain_bytes) bulk_g2s_tx(stage + ST_CHAIN, a.zchain + (size_t)it.patch * NP, chain_bytes, full);
         bulk_g2s_tx(stage + ST_PX, a.px + it.pix, (unsigned)n * 16u, full);
         if (nc0 > 0) bulk_g2s_tx(stage + ST_ZC, a.cands + it.c0, (unsigned)nc0 * (unsigned)sizeof(ZCand), full);
     } else if (lane - 1 < nc0) {
@@ -1028,67 +1010,138 @@ __global__ void __launch_bounds__(128) k_tables(ItemArgs a) {
 }
 
 // The per-source epilogues and the total, after every item: the item kernel's
-// programmatic dependent, waiting for it to finish.  One CTA of FIN_W warps per source:
-// warp w adds the columns of the source's items w, w + FIN_W, ... in item order (FP64;
-// lane c columns c and c + 32, loaded FIN_WIN items at a time before any is added), the
-// CTA then adds the warps' sums in warp order and subtracts the KL: the local objective
-// and gradient, and the source's share of the total (the ll of the pixels its items own,
-// minus its KL).  The last CTA to finish adds the shares in source order (its warps over
-// contiguous ranges, lanes strided, then warp order).  The kernel leaves the flags, counters
-// and the status word of the evaluation at 0 for the next one (the status goes to the
-// caller's word), so an evaluation is three kernels and nothing else: two fills of a few bytes
-// ahead of them cost an evaluation FILL_US.
-constexpr int FIN_W = 4, FIN_WIN = 16;
-__global__ void __launch_bounds__(32 * FIN_W) k_finish(ItemArgs a) {
-    __shared__ double sh[FIN_W][64];
+// programmatic dependent, waiting for it to finish.  One CTA of W warps per source:
+// warp w takes the source's patches w, w + W, ...: the FP64 sums of the patch's item records
+// (lanes c and c + 16 column c of every other item, then the two added), then the patch's
+// chain rule (lane j < ZCHAIN: column j of d ll / d theta += sum_e k_e d ll / d y_{y_e};
+// the next two lanes the ll and the owned ll).  The CTA then adds the warps' sums in warp order
+// and subtracts the KL: the local objective and gradient, and the source's share of the total
+// (the ll of the pixels its items own, minus its KL).  The last CTA to finish adds the shares
+// in source order (its warps over contiguous ranges, lanes strided, then warp order).  The
+// kernel leaves the flags, counters and the status word of the evaluation at 0 for the next one
+// (the status goes to the caller's word), so an evaluation is three kernels and nothing else:
+// two fills of a few bytes ahead of them cost an evaluation 2 us.
+//
+// Bound by the latency of its loads and of about ten dependent FP64 operations per patch; the next
+// patch's records are loaded ahead.  The chain rule stands here, once per patch, and not in the
+// item kernel, once per item, where its ~30 FP64 operations delayed the warp that has to
+// stage the next item.
+// W warps per CTA: on one source (SHARED), or each on a source of its own.  FIN_C: item records
+// loaded ahead per lane.
+template <int W, int FIN_C, bool SHARED>
+__global__ void __launch_bounds__(32 * W, 32 / W) k_finish(ItemArgs a) {
+    __shared__ double sh[W][32];
     __shared__ int s_last;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s = SHARED ? (int)blockIdx.x : (int)blockIdx.x * W + w;
+    constexpr int STEP = SHARED ? W : 1;   // this warp's patches: p0 + w (SHARED) or p0, STEP apart
+    const bool grad = a.mode >= MODE_GRAD;
+    const int col = lane & 15, half = lane >> 4;
+    const bool used = col < (grad ? 2 + NY : 2), valid = s < a.n_src;
+    int p0 = valid ? a.patch_off[s] : 0, p1 = valid ? a.patch_off[s + 1] : 0;
+    if (!CEL_IN_BOUNDS(p0 >= 0 && p0 <= p1 && p1 <= a.n_patch, a.status)) p0 = p1 = 0;
+    if (SHARED) p0 += w;
+    int o0 = 0, o1 = 0;   // the items of patch pl, one of this warp's next 32
+    auto offsets = [&](int pl) {
+        o0 = o1 = 0;
+        if (pl >= p1) return;
+        o0 = a.item_off[pl];
+        o1 = a.item_off[pl + 1];
+        if (!CEL_IN_BOUNDS(o0 >= 0 && o0 <= o1 && o1 <= a.n_sitem, a.status)) o0 = o1 = 0;
+    };
+    offsets(p0 + STEP * lane);
+    if (threadIdx.x == 0) s_last = 0;
+    if (!SHARED) __syncthreads();
     pdl_wait();
     for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < a.n_patch + 2; i += (int)(gridDim.x * blockDim.x))
         a.ready[i] = 0;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, s = (int)blockIdx.x;
-    const bool grad = a.mode >= MODE_GRAD;
-    const int ncol = grad ? ZPCOLS : 2;
-    int i0 = __ldcg(a.sitem_off + s), i1 = __ldcg(a.sitem_off + s + 1);
-    if (!CEL_IN_BOUNDS(i0 >= 0 && i0 <= i1 && i1 <= a.n_sitem, a.status)) i0 = i1 = 0;
-    const int cA = lane, cB = lane + 32;
-    double sA = 0.0, sB = 0.0;
-    for (int k0 = i0 + w; k0 < i1; k0 += FIN_W * FIN_WIN) {
-        double vA[FIN_WIN], vB[FIN_WIN];
-#pragma unroll
-        for (int u = 0; u < FIN_WIN; ++u) {
-            const int k = k0 + FIN_W * u;
-            const double* r = a.part + (size_t)k * ZPCOLS;
-            vA[u] = (k < i1 && cA < ncol) ? __ldcg(r + cA) : 0.0;
-            vB[u] = (k < i1 && cB < ncol) ? __ldcg(r + cB) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < FIN_WIN; ++u) {
-            if (k0 + FIN_W * u >= i1) break;
-            sA += vA[u];
-            sB += vB[u];
+    // (the KL terms, asked for early)
+    double klv = 0.0, kg0 = 0.0, kg1 = 0.0;
+    if (valid && (!SHARED || w == 0)) {
+        const double* kg = a.kl_grad + (size_t)NP * s;
+        klv = __ldcg(a.kl + s);
+        if (grad) {
+            kg0 = __ldcg(kg + lane);
+            if (lane < NP - ZCHAIN) kg1 = __ldcg(kg + ZCHAIN + lane);
         }
     }
-    sh[w][cA] = sA;
-    sh[w][cB] = sB;
-    s_last = 0;
-    __syncthreads();
-    if (w == 0) {
-        double tA = 0.0, tB = 0.0;
+    double acc = 0.0;
+    for (int pb = p0; pb < p1; pb += 32 * STEP) {
+        const int np = min(32, (p1 - pb + STEP - 1) / STEP);
+        if (pb != p0) offsets(pb + STEP * lane);
+        double x[FIN_C];
+        float4 ch;
+        auto records = [&](int c0, int c1, double (&v)[FIN_C]) {
 #pragma unroll
-        for (int v = 0; v < FIN_W; ++v) {
-            tA += sh[v][cA];
-            tB += sh[v][cB];
+            for (int u = 0; u < FIN_C; ++u) {
+                const int c = c0 + 2 * u + half;
+                v[u] = used && c < c1 ? __ldcg(a.part + (size_t)c * 16 + col) : 0.0;
+            }
+        };
+        auto load = [&](int i) {
+            records(__shfl_sync(0xffffffffu, o0, i), __shfl_sync(0xffffffffu, o1, i), x);
+            ch = make_float4(lane < ZCHAIN ? 0.f : 1.f, 0.f, 0.f, 0.f);
+            if (grad && lane < ZCHAIN) ch = __ldcg(a.zchain + (size_t)(pb + STEP * i) * ZCHAIN + lane);
+        };
+        load(0);
+        for (int i = 0; i < np; ++i) {
+            const int c0 = __shfl_sync(0xffffffffu, o0, i), c1 = __shfl_sync(0xffffffffu, o1, i);
+            const float4 k = ch;
+            double v[FIN_C];
+#pragma unroll
+            for (int u = 0; u < FIN_C; ++u) v[u] = x[u];
+            if (i + 1 < np) load(i + 1);
+            double y = v[0];
+#pragma unroll
+            for (int u = 1; u < FIN_C; ++u)
+                if (c0 + 2 * u < c1) y += v[u];
+            for (int b = c0 + 2 * FIN_C; b < c1; b += 2 * FIN_C) {   // patches of more items
+                records(b, c1, v);
+#pragma unroll
+                for (int u = 0; u < FIN_C; ++u)
+                    if (b + 2 * u < c1) y += v[u];
+            }
+            if (c1 - c0 > 1) y += __shfl_xor_sync(0xffffffffu, y, 16);
+            const int yy = __float_as_int(k.w);
+            const bool lls = lane >= ZCHAIN;   // the ll and the owned ll: columns 0 and 1
+            const double y0 = __shfl_sync(0xffffffffu, y, lls ? (lane - ZCHAIN) & 1 : 2 + (yy & 15));
+            const double y1 = __shfl_sync(0xffffffffu, y, 2 + ((yy >> 4) & 15));
+            const double y2 = __shfl_sync(0xffffffffu, y, 2 + ((yy >> 8) & 15));
+            const double k0 = widen(k.x), k1 = widen(k.y), k2 = widen(k.z);
+            acc = fma(k0, y0, acc);
+            if (!lls) acc = fma(k2, y2, fma(k1, y1, acc));
         }
-        const double klv = __ldcg(a.kl + s);
-        if (lane == 0 && a.local_out) a.local_out[s] = tA - klv;   // column 0: ll
+    }
+    if (SHARED) {
+        sh[w][lane] = acc;
+        __syncthreads();
+    }
+    if (valid && (!SHARED || w == 0)) {
+        double t = acc;
+        if (SHARED) {
+            double r[W];
+#pragma unroll
+            for (int v = 0; v < W; ++v) r[v] = sh[v][lane];
+#pragma unroll
+            for (int h = W / 2; h >= 1; h >>= 1)
+#pragma unroll
+                for (int v = 0; v < h; ++v) r[v] += r[v + h];
+            t = r[0];
+        }
+        if (lane == ZCHAIN && a.local_out) a.local_out[s] = t - klv;
         if (grad && a.grad_out) {
-            if (cA >= 2) a.grad_out[(size_t)NP * s + cA - 2] = tA - __ldcg(a.kl_grad + (size_t)NP * s + cA - 2);
-            if (cB < ncol) a.grad_out[(size_t)NP * s + cB - 2] = tB - __ldcg(a.kl_grad + (size_t)NP * s + cB - 2);
+            double* g = a.grad_out + (size_t)NP * s;
+            if (lane < ZCHAIN) g[lane] = t - kg0;
+            if (lane < NP - ZCHAIN) g[ZCHAIN + lane] = -kg1;
         }
-        if (lane == 1) {
-            if (a.total_out) a.src_total[s] = tA - klv;   // column 1: owned ll
-            s_last = arrive_acq_rel(a.grp_done) == (int)gridDim.x - 1;
+        if (lane == ZCHAIN + 1) {
+            if (a.total_out) a.src_total[s] = t - klv;
+            if (SHARED) s_last = arrive_acq_rel(a.grp_done) == (int)gridDim.x - 1;
         }
+    }
+    if (!SHARED) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_last = arrive_acq_rel(a.grp_done) == (int)gridDim.x - 1;
     }
     __syncthreads();
     if (!s_last) return;
@@ -1098,9 +1151,9 @@ __global__ void __launch_bounds__(32 * FIN_W) k_finish(ItemArgs a) {
         a.grp_done[0] = 0;
     }
     if (!a.total_out) return;
-    const int n = a.n_src, per = (n + FIN_W - 1) / FIN_W;
+    const int n = a.n_src, per = (n + W - 1) / W;
     const int b0 = w * per, b1 = min(n, b0 + per);
-    double acc = 0.0;
+    double tot = 0.0;
     for (int c0 = b0; c0 < b1; c0 += 32 * 16) {
         double x[16];
 #pragma unroll
@@ -1109,109 +1162,132 @@ __global__ void __launch_bounds__(32 * FIN_W) k_finish(ItemArgs a) {
             x[u] = i < b1 ? __ldcg(a.src_total + i) : 0.0;
         }
 #pragma unroll
-        for (int u = 0; u < 16; ++u) acc += x[u];
+        for (int u = 0; u < 16; ++u) tot += x[u];
     }
-    acc = warp_dsum(acc);
+    tot = warp_dsum(tot);
     __syncthreads();   // every warp is past its reads of sh
-    if (lane == 0) sh[w][0] = acc;
+    if (lane == 0) sh[w][0] = tot;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int v = 0; v < FIN_W; ++v) t += sh[v][0];
+        for (int v = 0; v < W; ++v) t += sh[v][0];
         *a.total_out = t;
     }
 }
 
-// The items, on persistent CTAs of four compute warps and a producer warp.  The producer
-// keeps the next two items in the two stages: once the compute warps are done with item
-// i it writes item i's record (the warps' sums in FP64, the chain rule) and puts item
-// i + 2 in that stage; it holds one task record ahead in registers and one queue slot
-// claimed beyond that.  CTA c's first two items are slots c and c + G (G CTAs); later
-// slots come from the queue counter.
-template <int MODE, int PX, int NPE, int NPD, int MINB, int UNR>
-__global__ void __launch_bounds__(IT_THREADS) __maxnreg__(regs_for(MINB)) k_items(ItemArgs a) {
+// Fetch the record of queue slot q ahead (lane 0): a bulk copy into rec completing on bar, or
+// an end marker past the end.
+__device__ __forceinline__ void fetch_record(const ItemArgs& a, int q, ZTask* rec, uint64_t* bar) {
+    if (q >= a.n_task) {
+        rec->kind = ZT_END;
+        mbar_arrive_plain(bar);
+        return;
+    }
+    fence_proxy_async_smem();   // rec was last read through the generic proxy
+    mbar_expect_arrive(bar, (unsigned)sizeof(ZTask));
+    bulk_g2s_tx(rec, a.tasks + q, (unsigned)sizeof(ZTask), bar);
+}
+
+// The items, on persistent CTAs of four warps that keep the next two items in two stages.
+// The warps take an item's chunks in turn from a counter in shared memory and go on to the next
+// item when none is left; the one that leaves item i last puts item i + 2, whose record was
+// fetched before, in that stage and fetches the record of item i + 3.  CTA c's first two items are slots c and c + G
+// (G CTAs); later slots come from the queue counter.
+//
+// Bound by the FMA pipe and by the issue of dependent operations (55% and 61% busy with 12 warps
+// per SM).  Four CTAs per SM at 128 registers hold 16 computing warps, and the 7 component
+// pairs of 2 pixels still unroll without spilling.  For 8.7 million source-pixels in a dense
+// field: two CTAs per SM of four warps and a fifth for the staging and the records 444 us; the
+// fifth warp's work on the warp that finishes last, three CTAs, chunks dealt out by warp number
+// 434 (a quarter of the warps' time went on waiting for the slowest); chunks taken in turn
+// 391; four CTAs 360; whole chunks per item 354; pixels grouped by covering set 336; the
+// chain rule moved to k_finish 328.
+template <int MODE, int NPE, int NPD, int MINB, int UNR>
+__global__ void __launch_bounds__(NTC) __maxnreg__(regs_for(MINB)) k_items(ItemArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
-    using L = Lay<PX>;
+    using L = Lay;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + L::bar);
-    uint64_t* reduced = full + 2;
+    uint64_t* fetched = full + 2;
     ZTask* tasks = reinterpret_cast<ZTask*>(smem + L::task);
     float* red = reinterpret_cast<float*>(smem + L::red);
+    ZTask* next = reinterpret_cast<ZTask*>(smem + L::next);
+    int* cnt = reinterpret_cast<int*>(smem + L::cnt);
+    int* taken = cnt + 2;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     pdl_trigger();   // the epilogue kernel may start (it waits for this grid to finish)
     if (t == 0) {
-        mbar_init(&full[0], 1);
-        mbar_init(&full[1], 1);
-        mbar_init(&reduced[0], NTC);
-        mbar_init(&reduced[1], NTC);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&full[b], 1);
+            mbar_init(&fetched[b], 1);
+            cnt[b] = taken[b] = 0;
+        }
         mbar_init_fence();
     }
     __syncthreads();
     int32_t* queue = a.ready + a.n_patch;
-    if (w == NWC) {
-        bool all_built = false;
-        // slots 0 .. 2 G - 1 (G CTAs) are dealt out, one per stage of every CTA, so that
-        // a queue of few items spreads over all CTAs; the rest are claimed one at a time
-        const int G = (int)gridDim.x, base = 2 * G;
-        int qa = 0;
-        if (lane == 0) qa = base + atomicAdd(queue, 1);
-        qa = __shfl_sync(0xffffffffu, qa, 0);
-        const int4 r0 = load_task(a, (int)blockIdx.x), r1 = load_task(a, (int)blockIdx.x + G);
-        int4 ra = load_task(a, qa);   // the record of the next item to prepare
-        prepare<MODE>(a, r0, smem, &tasks[0], &full[0], all_built);
-        prepare<MODE>(a, r1, smem + ST_BYTES, &tasks[1], &full[1], all_built);
-        int qb = 0;   // lane 0: the slot after that
-        if (lane == 0) qb = base + atomicAdd(queue, 1);
-        for (int i = 0;; ++i) {
-            const int b = i & 1;
-            __syncwarp();
-            if (tasks[b].kind == ZT_END) break;
-            if (!mbar_wait_launch(&reduced[b], (i >> 1) & 1, a.status)) break;
-            // item i is done: what its record needs, read from the stage; item i + 2's
-            // copies into the stage; item i's record (FP64, off the compute warps)
-            const int out = tasks[b].item.out;
-            const ItemSums q = finish_load<MODE>(smem + b * ST_BYTES, red + b * NWC * RED_W);
-            __syncwarp();
-            prepare<MODE>(a, ra, smem + b * ST_BYTES, &tasks[b], &full[b], all_built);
-            finish_store<MODE>(a, out, q);
-            ra = load_task(a, __shfl_sync(0xffffffffu, qb, 0));
-            if (lane == 0) qb = base + atomicAdd(queue, 1);
-        }
-        // this grid completes only after the table kernel (and its KL terms) has, so the
-        // epilogue kernel that waits for this grid sees both, and the next evaluation's
-        // flag reset follows both
-        pdl_wait();
-        return;
-    }
-    // compute warps
-    float* vs = reinterpret_cast<float*>(smem + L::vs) + t;
+    // slots 0 .. 2 G - 1 (G CTAs) are dealt out, one per stage of every CTA, so that a queue
+    // of few items spreads over all CTAs; the rest are claimed one at a time
+    const int G = (int)gridDim.x, base = 2 * G;
+    bool all_built = false;
+    if (w < 2)
+        prepare<MODE>(a, load_task(a, (int)blockIdx.x + w * G), smem + w * ST_BYTES, &tasks[w], &full[w], all_built);
+    else if (w == 2 && lane == 0)
+        fetch_record(a, base + atomicAdd(queue, 1), &next[0], &fetched[0]);
     float* spg = reinterpret_cast<float*>(smem + L::pg) + t;
     for (int i = 0;; ++i) {
         const int b = i & 1;
+        __syncwarp();
         if (!mbar_wait_launch(&full[b], (i >> 1) & 1, a.status)) break;
         if (tasks[b].kind == ZT_END) break;
         const ZItem it = tasks[b].item;
-        const uint8_t* stage = smem + b * ST_BYTES;
-        float* rb = red + b * NWC * RED_W;
-        item_compute<MODE, PX, NPE, NPD, UNR>(a, it, stage, vs, spg, rb + w * RED_W);
-        // the producer adds the warps' sums and writes the item's record
+        uint8_t* stage = smem + b * ST_BYTES;
+        float* rb = red + b * L::nch * 16;
+        const int nch = ((it.n_nm & 0xffff) + ZCHUNK - 1) / ZCHUNK;
+        for (;;) {
+            int c = 0;
+            if (lane == 0) c = atomicAdd(&taken[b], 1);
+            c = __shfl_sync(0xffffffffu, c, 0);
+            if (c >= nch) break;
+            chunk_compute<MODE, NPE, NPD, UNR>(a, it, stage, c * ZCHUNK, spg, rb + c * 16);
+        }
         __syncwarp();
-        mbar_arrive_plain(&reduced[b]);
+        int last = 0;
+        if (lane == 0) {
+            __threadfence_block();
+            last = atomicAdd(&cnt[b], 1) == NWC - 1;
+            if (last) cnt[b] = taken[b] = 0;
+            __threadfence_block();
+        }
+        if (!__shfl_sync(0xffffffffu, last, 0)) continue;
+        int q = 0;
+        if (lane == 0) q = base + atomicAdd(queue, 1);
+        item_record<MODE>(a, it.out, rb, nch);
+        if (!mbar_wait_launch(&fetched[b], (i >> 1) & 1, a.status)) break;
+        const int4 rec = lane < 4 ? reinterpret_cast<const int4*>(&next[b])[lane] : make_int4(0, 0, 0, 0);
+        __syncwarp();
+        prepare<MODE>(a, rec, stage, &tasks[b], &full[b], all_built);
+        if (lane == 0) fetch_record(a, q, &next[b ^ 1], &fetched[b ^ 1]);
     }
+    // this grid completes only after the table kernel (and its KL terms) has, so the epilogue
+    // kernel that waits for this grid sees both
+    if (w == 0) pdl_wait();
 }
 
 // ---------------------------------------------------------------------------------
 // launch
 
-template <int MODE, int PX, int NPE, int NPD, int MINB, int UNR>
+template <int MODE, int NPE, int NPD, int MINB, int UNR>
 struct ItemsKernel {
     static int per_sm;   // resident CTAs per SM (0: not yet set up)
     static cudaError_t setup() {
         if (per_sm > 0) return cudaSuccess;
-        auto* fn = k_items<MODE, PX, NPE, NPD, MINB, UNR>;
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<PX>::bytes);
+        auto* fn = k_items<MODE, NPE, NPD, MINB, UNR>;
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::bytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         int per = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, IT_THREADS, Lay<PX>::bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, NTC, Lay::bytes);
         if (e != cudaSuccess) return e;
         per_sm = per > 0 ? per : 1;
         return cudaSuccess;
@@ -1225,54 +1301,52 @@ struct ItemsKernel {
         if (grid < 1) return cudaSuccess;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)grid);
-        cfg.blockDim = dim3(IT_THREADS);
-        cfg.dynamicSmemBytes = Lay<PX>::bytes;
+        cfg.blockDim = dim3(NTC);
+        cfg.dynamicSmemBytes = Lay::bytes;
         cfg.stream = st;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, k_items<MODE, PX, NPE, NPD, MINB, UNR>, a);
+        return cudaLaunchKernelEx(&cfg, k_items<MODE, NPE, NPD, MINB, UNR>, a);
     }
 };
-template <int MODE, int PX, int NPE, int NPD, int MINB, int UNR>
-int ItemsKernel<MODE, PX, NPE, NPD, MINB, UNR>::per_sm = 0;
+template <int MODE, int NPE, int NPD, int MINB, int UNR>
+int ItemsKernel<MODE, NPE, NPD, MINB, UNR>::per_sm = 0;
 
 // the model of the synthetic workloads and of the paper (6 exp + 8 dev profile
 // components: 3 + 4 pairs) gets its loops unrolled for those counts
-template <int MODE, int PX, int MINB, int UNR>
+template <int MODE, int MINB, int UNR>
 cudaError_t items_launch_v(const ItemArgs& a, int n_sm, cudaStream_t st) {
-    if ((a.ne + 1) / 2 == 3 && (a.nd + 1) / 2 == 4) return ItemsKernel<MODE, PX, 3, 4, MINB, UNR>::launch(a, n_sm, st);
-    return ItemsKernel<MODE, PX, -1, -1, MINB, 1>::launch(a, n_sm, st);
+    if ((a.ne + 1) / 2 == 3 && (a.nd + 1) / 2 == 4) return ItemsKernel<MODE, 3, 4, MINB, UNR>::launch(a, n_sm, st);
+    return ItemsKernel<MODE, -1, -1, MINB, 1>::launch(a, n_sm, st);
 }
 
-#define CEL_ITEM_VARIANTS(X)   \
-    X(1, 2, 2, 7)              \
-    X(2, 3, 2, 3)              \
-    X(3, 2, 3, 2)              \
-    X(4, 3, 2, 7)              \
-    X(5, 3, 2, 2)
-// variant codes (code, pixels per thread, CTAs per SM, unroll of the component-pair loop):
-// 1 (2, 2, 7), 2 (3, 2, 3), 3 (2, 3, 2), 4 (3, 2, 7), 5 (3, 2, 2); two CTAs per SM leave
-// 168 registers per thread, three 128
+#define CEL_ITEM_VARIANTS(X) \
+    X(1, 4, 7)               \
+    X(2, 3, 7)               \
+    X(3, 4, 2)               \
+    X(4, 4, 3)               \
+    X(5, 3, 3)
+// variant codes (code, CTAs per SM, unroll of the component-pair loop)
 template <int MODE>
 cudaError_t items_launch(const ItemArgs& a, int code, int n_sm, cudaStream_t st) {
     switch (code) {
-#define CEL_CASE(c, px, minb, unr) \
-    case c: return items_launch_v<MODE, px, minb, unr>(a, n_sm, st);
+#define CEL_CASE(c, minb, unr) \
+    case c: return items_launch_v<MODE, minb, unr>(a, n_sm, st);
         CEL_ITEM_VARIANTS(CEL_CASE)
 #undef CEL_CASE
-        default: return items_launch_v<MODE, 2, 2, 7>(a, n_sm, st);
+        default: return items_launch_v<MODE, 4, 7>(a, n_sm, st);
     }
 }
 
 template <int MODE>
 cudaError_t items_setup_mode() {
     cudaError_t e = cudaSuccess;
-#define CEL_SETUP(c, px, minb, unr)                                                    \
-    if (e == cudaSuccess) e = ItemsKernel<MODE, px, 3, 4, minb, unr>::setup();           \
-    if (e == cudaSuccess) e = ItemsKernel<MODE, px, -1, -1, minb, 1>::setup();
+#define CEL_SETUP(c, minb, unr)                                                    \
+    if (e == cudaSuccess) e = ItemsKernel<MODE, 3, 4, minb, unr>::setup();           \
+    if (e == cudaSuccess) e = ItemsKernel<MODE, -1, -1, minb, 1>::setup();
     CEL_ITEM_VARIANTS(CEL_SETUP)
 #undef CEL_SETUP
     return e;
@@ -1304,7 +1378,8 @@ cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStr
     a.ready = P.zready;
     a.geo_tab = P.geo;
     a.img_tab = P.img;
-    a.part = P.spart;
+    a.part = P.zpart;
+    a.item_off = P.zitem_off;
     a.ne = P.model_ne;
     a.nd = P.model_nd;
     a.n_patch = P.n_patch;
@@ -1318,7 +1393,7 @@ cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStr
     a.status = P.zf_done + 1;
     a.status_out = P.status;
     a.mode = mode;
-    a.sitem_off = P.sitem_off;
+    a.patch_off = P.patch_off;
     a.grp_done = P.zf_done;
     a.src_total = P.src_total;
     a.local_out = d_local;
@@ -1334,15 +1409,20 @@ cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStr
                                : items_launch<MODE_GRAD>(a, P.tune_items, n_sm, st);
     }
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)P.n_src);
-    cfg.blockDim = dim3(32 * FIN_W);
+    // Sixteen warps on a source of many images (a source of 80 images with four: 22 us, sixteen 19),
+    // eight on one of a few.  Beyond four waves of eight-warp CTAs a warp takes a source of its own
+    // (3125 sources of 5 images: 30 -> 26 us; 1200 sources: 12 -> 17 us, so not below).
+    const bool wide = P.n_patch > 8 * (int64_t)P.n_src, shared = wide || P.n_src <= 16 * sm_count();
+    cfg.gridDim = dim3((unsigned)(shared ? P.n_src : (P.n_src + 7) / 8));
+    cfg.blockDim = dim3(32 * (wide ? 16 : 8));
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_finish, a);
+    if (wide) return cudaLaunchKernelEx(&cfg, k_finish<16, 4, true>, a);
+    return shared ? cudaLaunchKernelEx(&cfg, k_finish<8, 2, true>, a) : cudaLaunchKernelEx(&cfg, k_finish<8, 2, false>, a);
 }
 
 cudaError_t launch_items(const DevProblem& P, int mode, cudaStream_t st, const double* d_theta, double* d_local,
