@@ -17,12 +17,13 @@ class ELBO(torch.autograd.Function):
         if not (theta.is_cuda and theta.dtype == torch.float64):
             raise TypeError("theta must be a CUDA float64 tensor")
         th = theta.detach().contiguous()
-        total = torch.zeros(1, dtype=torch.float64, device=theta.device)
+        # (written by the evaluation of any source: no fill, and no view of it to return)
+        total = (torch.empty if problem.n_src else torch.zeros)((), dtype=torch.float64, device=theta.device)
         problem.elbo_device(th, total, None, precision=precision)
         ctx.problem, ctx.precision = problem, precision
         ctx.generation = problem.generation
         ctx.save_for_backward(th)
-        return total[0]
+        return total
 
     @staticmethod
     def backward(ctx, grad_out):

@@ -399,8 +399,10 @@ class Problem:
     # ---- device-pointer calls (torch tensors on the problem's device)
     @staticmethod
     def _stream():
+        # the current stream's handle without a torch.cuda.Stream object around it (3.1 -> 0.6 us
+        # of the 8 us that a device call takes on the host)
         import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
     @staticmethod
     def _dp(t):
