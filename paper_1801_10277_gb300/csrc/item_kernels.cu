@@ -17,8 +17,8 @@
 // arithmetic pairs two mixture components per instruction (coefficients of adjacent
 // components side by side in the table).
 //
-// Work.  Three launches.  k_tables builds every patch's table and chain-rule record (one
-// warp per patch, FP32 with the position in FP64), publishing each with a ready flag, and
+// Work.  Three launches.  k_tables builds every patch's table and chain-rule record (a
+// warp per patch or per four, FP32 with the position in FP64), publishing each with a ready flag, and
 // every source's KL terms (one warp per source).  k_items, its programmatic dependent,
 // runs on persistent CTAs of four warps that take items from a queue (a global counter over
 // the items in decreasing cost): up to ZIMAX pixels of one patch, the multiply covered ones
@@ -130,9 +130,10 @@ __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
 // ---------------------------------------------------------------------------------
-// table construction: one warp per patch, written to the table in global memory
+// table construction: LP lanes per patch, written to the table in global memory
 
-// One patch's table and chain-rule record, built by one warp.  Every lane first converts
+// A patch's table and chain-rule record, built by LP lanes (32 or 8: one or four patches per
+// warp; every lane of the warp calls it, live: its patch is one to build).  Every lane first converts
 // a share of theta to FP32 (FP64 -> FP32 conversions and FP64 arithmetic have ~70-cycle
 // latencies on GB300's narrow FP64 pipe, so each is done once); lane 0 forms the position
 // in FP64 (relative to the patch origin, so FP32 offsets stay exact).  Then every lane
@@ -140,13 +141,15 @@ __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast
 // brightness moments of each type (lanes npsf, npsf + 1), the weights (lane npsf + 2)
 // and the shape Jacobian (lane npsf + 3);
 // finally one lane per (PSF component, component slot) the slot's coefficients and one
-// lane per theta column its chain-rule pairs.  sm: 96 floats of this warp's shared memory.
+// lane per theta column its chain-rule pairs.  sm: 96 floats of this patch's shared memory.
 
-__device__ __forceinline__ void build_patch_table(const double* __restrict__ theta, const ZBuild& g,
+template <int LP>
+__device__ __forceinline__ void build_patch_table(const double* __restrict__ theta, const ZBuild& g, bool live,
                                                   const ImgMeta* __restrict__ img, const ModelDev& md,
                                                   float* __restrict__ ztbl, float4* __restrict__ zchain,
                                                   float* sm) {
-    const int lane = threadIdx.x & 31;
+    static_assert(LP >= MAXPSF + 4, "a lane per part of phase one");
+    const int lane = threadIdx.x & (LP - 1);
     const int patch = g.patch;
     const ImgMeta& im = img[g.img];
     const double* th = theta + (size_t)NP * g.src;
@@ -154,8 +157,9 @@ __device__ __forceinline__ void build_patch_table(const double* __restrict__ the
     float* thf = sm;        // [44] theta in FP32
     float* dscr = sm + 44;  // [8] D1, D2 per PSF component
     float* mu = sm + 52;    // [2] position relative to the patch origin
-    float* elv = sm + 56;   // [4] el0, el20, el1, el21
+    float* elv = sm + 56;   // [4] el0, el1, el20, el21
     float* dgs = sm + 60;   // [9] dG
+    float* Af = sm + 69;    // [4] A
     // every global value this lane reads below, loaded together (one memory round trip)
     const int npsf = im.npsf, band = im.band;
     const float a0 = im.A_f[0], a1 = im.A_f[1], a2 = im.A_f[2], a3 = im.A_f[3];
@@ -164,8 +168,9 @@ __device__ __forceinline__ void build_patch_table(const double* __restrict__ the
     const float ps1 = im.psf_f[kk][1], ps2 = im.psf_f[kk][2], csk = im.psf_cs[kk], sgk = im.psf_sg[kk];
     const float iota = im.iota_f;
     const int n_exp = md.n_exp, n_dev = md.n_dev;
-    thf[lane] = (float)th[lane];
-    if (lane + 32 < NP) thf[lane + 32] = (float)th[lane + 32];
+#pragma unroll
+    for (int i = 0; i < (NP + LP - 1) / LP; ++i)
+        if (lane + LP * i < NP) thf[lane + LP * i] = (float)th[lane + LP * i];
     if (lane == 0) {
         const double u0 = th[0], u1 = th[1];
         mu[0] = (float)fma(im.A[0], u0, fma(im.A[1], u1, g.ox));
@@ -208,7 +213,7 @@ __device__ __forceinline__ void build_patch_table(const double* __restrict__ the
         d1 = fmaxf(d1, 0.f);
         d2 = fmaxf(d2, 0.f);
         const float t11 = cs * a - sn * b, t12 = -sn * c, t21 = sn * a + cs * b, t22 = cs * c;
-        if (lane < npsf) {
+        if (live && lane < npsf) {
             const int k = lane;
             float4* K = reinterpret_cast<float4*>(T + VH + k * VK);
             K[0] = make_float4(-(mu[0] + ps1), -(mu[1] + ps2), csk, sgk);
@@ -233,15 +238,18 @@ __device__ __forceinline__ void build_patch_table(const double* __restrict__ the
             v += bb * bb * thf[P_C2 + 4 * i + j];
         }
         const float el = expf(m + 0.5f * v), el2 = expf(2.f * m + 2.f * v), em = expm1f(v);
-        if (lane == npsf || lane == npsf + 1) {
+        if (live && (lane == npsf || lane == npsf + 1)) {
             T[2 + 2 * i] = el;
             T[3 + 2 * i] = el2;
             T[8 + i] = em;
-            elv[2 * i] = el;
-            elv[2 * i + 1] = el2;
+            elv[i] = el;
+            elv[2 + i] = el2;
         }
     }
     if (lane == npsf + 2) {
+        Af[0] = a0; Af[1] = a1; Af[2] = a2; Af[3] = a3;
+    }
+    if (live && lane == npsf + 2) {
         T[0] = thf[P_A];
         T[1] = thf[P_A + 1];
         T[6] = iota;
@@ -259,7 +267,7 @@ __device__ __forceinline__ void build_patch_table(const double* __restrict__ the
         dW[1][0] = -2.f * bh * s2; dW[1][1] = 2.f * bh * c2; dW[1][2] = 2.f * bh * s2;
         da = sg * (1.f + rho * rho); db = sg * (1.f - rho * rho);
         dW[2][0] = da + db * c2; dW[2][1] = db * s2; dW[2][2] = da - db * c2;
-        if (lane == npsf + 3) {
+        if (live && lane == npsf + 3) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 const float ux = dW[q][0], uxy = dW[q][1], uy = dW[q][2];
@@ -270,36 +278,44 @@ __device__ __forceinline__ void build_patch_table(const double* __restrict__ the
         }
     }
     // the coefficients of each (PSF component k, component slot): lane r takes slots r,
-    // r + 32, ..., whose constants are read before the wait for phase one
+    // r + LP, ..., whose constants are read before the wait for phase one (LP = 32)
     const int npe = (n_exp + 1) >> 1, nslot = 2 * (npe + ((n_dev + 1) >> 1));
-    constexpr int NR = (MAXPSF * 2 * ZMAXPAIR + 31) / 32;   // rounds of 32 slots
-    int sj[NR], sk[NR];
-    float snu[NR], slw[NR], ssg[NR], scs[NR];
-#pragma unroll
-    for (int u = 0; u < NR; ++u) {
-        const int r = lane + 32 * u;
-        const int k = r / nslot, slot = r - k * nslot, q = slot >> 1;
+    constexpr int NR = (MAXPSF * 2 * ZMAXPAIR + LP - 1) / LP;   // rounds of LP slots
+    constexpr int NA = LP == 32 ? NR : 1;                       // rounds read ahead
+    const float inv_nslot = __frcp_rn((float)nslot);
+    int sk[NA], ss[NA], sj[NA];
+    float snu[NA], slw[NA], ssg[NA], scs[NA];
+    auto constants = [&](int u, int e) {
+        const int r = lane + LP * u;
+        // r / nslot (r + 1/2 is no multiple of nslot and r < 2^7, so the product cannot round across one)
+        const int k = (int)(((float)r + 0.5f) * inv_nslot), slot = r - k * nslot;
         int j = -1;   // slot -> profile component j (or a padding slot)
         if (r < npsf * nslot) {
-            if (q < npe) {
+            if (slot < 2 * npe) {
                 if (slot < n_exp) j = slot;
             } else if (slot - 2 * npe < n_dev) {
                 j = n_exp + slot - 2 * npe;
             }
         }
-        sj[u] = j;
-        sk[u] = k;
-        snu[u] = j >= 0 ? md.prof_nu_f[j] : 0.f;
-        slw[u] = j >= 0 ? md.prof_lw_f[j] : 0.f;
-        ssg[u] = r < npsf * nslot ? im.psf_sg[k] : 0.f;
-        scs[u] = r < npsf * nslot ? im.psf_cs[k] : 0.f;
+        sk[e] = k;
+        ss[e] = slot;
+        sj[e] = j;
+        snu[e] = j >= 0 ? md.prof_nu_f[j] : 0.f;
+        slw[e] = j >= 0 ? md.prof_lw_f[j] : 0.f;
+        ssg[e] = r < npsf * nslot ? im.psf_sg[k] : 0.f;
+        scs[e] = r < npsf * nslot ? im.psf_cs[k] : 0.f;
+    };
+    if (NA > 1) {
+#pragma unroll
+        for (int u = 0; u < NA; ++u) constants(u, u);
     }
     __syncwarp();
-#pragma unroll
-    for (int u = 0; u < NR; ++u) {
-        const int r = lane + 32 * u;
-        if (r >= npsf * nslot) break;
-        const int k = sk[u], slot = r - k * nslot, q = slot >> 1, h = slot & 1, j = sj[u];
+#pragma unroll(NA > 1 ? NR : 1)
+    for (int u_ = 0; u_ < NR; ++u_) {
+        const int u = NA > 1 ? u_ : 0;
+        if (!live || lane + LP * u_ >= npsf * nslot) break;
+        if (NA == 1) constants(u_, 0);
+        const int k = sk[u], slot = ss[u], q = slot >> 1, h = slot & 1, j = sj[u];
         const bool dev = j >= n_exp;
         float A = 0.f, B = 0.f, C = -1e30f, U1 = 0.f, U2 = 0.f, Wa = 0.f, Wb = 0.f, W12 = 0.f, Va = 0.f, Vb = 0.f;
         if (j >= 0) {
@@ -324,16 +340,12 @@ __device__ __forceinline__ void build_patch_table(const double* __restrict__ the
         pq[0] = U2; pq[2] = Wa; pq[4] = Wb; pq[6] = W12; pq[8] = Va; pq[10] = Vb;
     }
     // the chain-rule record: column j of dy/dtheta for this patch
-    const float Af[4] = {a0, a1, a2, a3};
-    const float el[2] = {elv[0], elv[2]}, el2[2] = {elv[1], elv[3]};
-    float dG[3][3];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) dG[e / 3][e % 3] = dgs[e];
-    if (lane < ZCHAIN) {
+#pragma unroll 1
+    for (int j = lane; live && j < ZCHAIN; j += LP) {
         int y0, y1, y2;
         float k0, k1, k2;
-        chain_column<float>(lane, band, Af, el, el2, dG, &y0, &k0, &y1, &k1, &y2, &k2);
-        zchain[(size_t)patch * ZCHAIN + lane] = make_float4(k0, k1, k2, __int_as_float(y0 | (y1 << 4) | (y2 << 8)));
+        chain_column<float>(j, band, Af, elv, elv + 2, reinterpret_cast<const float(*)[3]>(dgs), &y0, &k0, &y1, &k1, &y2, &k2);
+        zchain[(size_t)patch * ZCHAIN + j] = make_float4(k0, k1, k2, __int_as_float(y0 | (y1 << 4) | (y2 << 8)));
     }
 }
 
@@ -985,27 +997,42 @@ __device__ void prepare(const ItemArgs& a, int4 rec, uint8_t* stage, ZTask* tk, 
 // ---------------------------------------------------------------------------------
 // the kernels
 
-// Tables and KL terms: warp u < n_patch builds the table and chain-rule record of the
-// patch of torder[u] (the patches in the order the items first read them) and publishes
-// it; warp n_patch + s computes the KL terms of source s (with the domain check of its
-// theta).  The item kernel is launched as this kernel's programmatic dependent and waits
-// for each table's flag, not for this kernel.
+// Tables and KL terms, a warp each in turn while there are both: the tables and chain-rule
+// records of the patches torder[0 .. n_patch) (the patches in the order the items first read
+// them), 32 / LP per warp, published when built; the KL terms of a source (with the domain check
+// of its theta).  The item kernel is launched as this kernel's programmatic dependent and
+// waits for each table's flag, not for this kernel.
+// Bound by instruction issue where a warp builds one table (most of its lanes repeat the same
+// set-up) and, once the patches are more than the chip's warps, by the KL terms' FP64 pipe time,
+// which therefore runs beside the tables and not behind them.  A warp for four patches takes 2.4
+// times fewer instructions per patch but is slower for each.  Stage times: 15,625 patches of
+// 3,125 sources 47 us with a warp per patch and the KL terms last, 38 with both in turn, 31 with
+// four patches per warp too; 8,000 patches of 100 sources 26, 21, 20; 2,500 patches of 500
+// sources 15.4 with one patch per warp, 16.7 with four.
+template <int LP>
 __global__ void __launch_bounds__(128) k_tables(ItemArgs a) {
-    __shared__ __align__(16) float scr[4][SCR_W / 4];
+    __shared__ __align__(16) float scr[4][SCR_W / 4 * (LP == 32 ? 1 : 2)];
+    constexpr int PW = 32 / LP;   // patches per warp
+    static_assert(PW * 96 * 4 <= sizeof(scr[0]), "scratch of the warp's patches");
     pdl_trigger();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int u = (int)blockIdx.x * 4 + w;
-    if (u < a.n_patch) {
-        const ZBuild g = a.torder[u];
-        if (!CEL_IN_BOUNDS(g.patch >= 0 && g.patch < a.n_patch && g.img >= 0 && g.img < a.n_img_rec && g.src >= 0 &&
-                               g.src < a.n_src,
-                           a.status))
-            return;
-        build_patch_table(a.theta, g, a.img_tab, *a.md, a.ztbl, a.zchain, scr[w]);
+    const int n_warp = (a.n_patch + PW - 1) / PW, both = 2 * min(n_warp, a.n_src), v = (int)blockIdx.x * 4 + w;
+    const bool table = v < both ? !(v & 1) : n_warp > a.n_src;
+    const int u = v < both ? v >> 1 : v - (both >> 1);
+    if (table && u < n_warp) {
+        const int t = u * PW + lane / LP;
+        const ZBuild g = a.torder[min(t, a.n_patch - 1)];
+        const bool live = t < a.n_patch && CEL_IN_BOUNDS(g.patch >= 0 && g.patch < a.n_patch && g.img >= 0 &&
+                                                             g.img < a.n_img_rec && g.src >= 0 && g.src < a.n_src,
+                                                         a.status);
+        if (!__any_sync(0xffffffffu, live)) return;
+        ZBuild gs = g;
+        if (!live) gs = ZBuild{0, 0, 0, 0, 0.0, 0.0};   // (indices in range; nothing is stored)
+        build_patch_table<LP>(a.theta, gs, live, a.img_tab, *a.md, a.ztbl, a.zchain, scr[w] + 96 * (lane / LP));
         __syncwarp();
-        if (lane == 0) publish_ready(a.ready + g.patch, a.ready + a.n_patch + 1);
-    } else if (u < a.n_patch + a.n_src) {
-        kl_task(a, u - a.n_patch, scr[w]);
+        if (live && lane % LP == 0) publish_ready(a.ready + g.patch, a.ready + a.n_patch + 1);
+    } else if (!table && u < a.n_src) {
+        kl_task(a, u, scr[w]);
     }
 }
 
@@ -1400,7 +1427,10 @@ cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStr
     a.grad_out = mode >= MODE_GRAD ? d_grad : nullptr;
     a.total_out = d_total;
     if (stage == 0) {
-        k_tables<<<(P.n_patch + P.n_src + 3) / 4, 128, 0, st>>>(a);
+        // a warp per patch up to one wave of warps (36 per SM), four patches per warp beyond
+        const int pw = P.n_patch > 36 * sm_count() ? 4 : 1, n_warp = (P.n_patch + pw - 1) / pw + P.n_src;
+        if (pw == 4) k_tables<8><<<(n_warp + 3) / 4, 128, 0, st>>>(a);
+        else k_tables<32><<<(n_warp + 3) / 4, 128, 0, st>>>(a);
         return cudaGetLastError();
     }
     if (stage == 1) {
