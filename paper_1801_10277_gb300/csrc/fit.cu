@@ -1006,7 +1006,9 @@ Batch make_batch(const celeste_problem* pr, const std::vector<int32_t>& members)
         }
         B.patch_off.push_back((int)B.geo.size());
     }
-    B.hchunk = hess_chunk(B.n_sp, sm_count());
+    // by the problem, not by the batch: the FP32 sums, and with them a source's iterates, must not
+    // depend on which other sources share its batch (a batch is an eighth of the problem or so)
+    B.hchunk = hess_chunk(pr->P.n_sp / 8, sm_count());
     for (int p = 0; p < (int)B.geo.size(); ++p)
         push_parts(B.parts, B.geo[p], p, pr->imgs[B.geo[p].img], B.hchunk);
     return B;

@@ -86,3 +86,19 @@ def test_larger_parts(n_src, side):
         for prec in (cel.FP64, cel.FP32):
             _check(P, prec, prob.theta, [s], loc[k:k + 1], grad[k:k + 1], hess[k:k + 1])
     P.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_fit_does_not_depend_on_batch_sizes(prec):
+    """One Cyclades sweep of the 500-source field in one sample (batches of 0.8 million
+    source-pixels) and in samples of 32 (0.07 million): the same random order, so the same
+    iterates bit for bit."""
+    from paper_1801_10277_gb300 import celeste as cel
+    prob = synth.config(1)
+    order = np.random.default_rng(3).permutation(prob.n_src).astype(np.int32)[None]
+    P = cel.Problem(prob)
+    fits = [P.fit(prob.theta, precision=prec, max_sweeps=1, max_iter=2, refine_fp64=0, schedule="cyclades", order=order,
+                  sample_size=size) for size in (prob.n_src, 32)]
+    np.testing.assert_array_equal(fits[0][0], fits[1][0])
+    np.testing.assert_array_equal(fits[0][1], fits[1][1])
+    P.close()
