@@ -1221,14 +1221,13 @@ __device__ __forceinline__ void fetch_record(const ItemArgs& a, int q, ZTask* re
 // fetched before, in that stage and fetches the record of item i + 3.  CTA c's first two items are slots c and c + G
 // (G CTAs); later slots come from the queue counter.
 //
-// Bound by the FMA pipe and by the issue of dependent operations (55% and 61% busy with 12 warps
-// per SM).  Four CTAs per SM at 128 registers hold 16 computing warps, and the 7 component
-// pairs of 2 pixels still unroll without spilling.  For 8.7 million source-pixels in a dense
-// field: two CTAs per SM of four warps and a fifth for the staging and the records 444 us; the
-// fifth warp's work on the warp that finishes last, three CTAs, chunks dealt out by warp number
-// 434 (a quarter of the warps' time went on waiting for the slowest); chunks taken in turn
-// 391; four CTAs 360; whole chunks per item 354; pixels grouped by covering set 336; the
-// chain rule moved to k_finish 328.
+// Bound by the FMA pipe and by instruction issue (60% and 67% busy).  Four CTAs per SM at 128
+// registers hold 16 computing warps, and the 7 component pairs of 2 pixels still unroll without
+// spilling.  For 8.7 million source-pixels in a dense field: two CTAs per SM of four warps and a
+// fifth for the staging and the records 444 us; the fifth warp's work on the warp that finishes
+// last, three CTAs, chunks dealt out by warp number 434 (a quarter of the warps' time went on
+// waiting for the slowest); chunks taken in turn 391; four CTAs 360; whole chunks per item 354;
+// pixels grouped by covering set 336; the chain rule moved to k_finish 328.
 template <int MODE, int NPE, int NPD, int MINB, int UNR>
 __global__ void __launch_bounds__(NTC) __maxnreg__(regs_for(MINB)) k_items(ItemArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -1389,8 +1388,8 @@ cudaError_t prime_items_kernels() {
     return e;
 }
 
-cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStream_t st, const double* d_theta,
-                               double* d_local, double* d_grad, double* d_total) {
+static cudaError_t launch_stage(const DevProblem& P, int stage, int mode, cudaStream_t st, const double* d_theta,
+                                double* d_local, double* d_grad, double* d_total) {
     if (P.n_src == 0 || !P.ztasks) return cudaSuccess;
     ItemArgs a{};
     a.tasks = P.ztasks;
@@ -1453,6 +1452,17 @@ cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStr
     cfg.numAttrs = 1;
     if (wide) return cudaLaunchKernelEx(&cfg, k_finish<16, 4, true>, a);
     return shared ? cudaLaunchKernelEx(&cfg, k_finish<8, 2, true>, a) : cudaLaunchKernelEx(&cfg, k_finish<8, 2, false>, a);
+}
+
+cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStream_t st, const double* d_theta,
+                               double* d_local, double* d_grad, double* d_total) {
+    const cudaError_t e = launch_stage(P, stage, mode, st, d_theta, d_local, d_grad, d_total);
+    // tables published without an epilogue kernel behind them must not pass for the next call's
+    if (e != cudaSuccess && stage > 0) {
+        cudaMemsetAsync(P.zready, 0, sizeof(int32_t) * ((size_t)P.n_patch + 2), st);
+        cudaMemsetAsync(P.zf_done, 0, 2 * sizeof(int32_t), st);
+    }
+    return e;
 }
 
 cudaError_t launch_items(const DevProblem& P, int mode, cudaStream_t st, const double* d_theta, double* d_local,
