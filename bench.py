@@ -51,7 +51,7 @@ SM_COUNT = 152
 # DRAM bytes (read + write) per launch of the item kernel on the one-field workload, from one
 # ncu capture (profiles/k_items_field_500src.md); emptied whenever the kernel changes after
 # the capture.
-DRAM_BYTES_PER_LAUNCH = {"items": 26240256}
+DRAM_BYTES_PER_LAUNCH = {"items": 24471808}
 DRAM_BYTES_SOURCE = "ncu capture of one k_items launch, profiles/k_items_field_500src.md (imported, not measured here)"
 FP32_LANES = 128
 XU_LANES = 16   # MUFU ex2 results per SM per clock
@@ -106,7 +106,9 @@ def hess_pass_flops_per_source_pixel(npsf, n_exp, n_dev):
     galaxy component's exponent and value (5) and its 35 weighted sums (70), and the sums'
     map back to the pixel frame (329: the z-monomials, the whitened gradient and Hessian
     blocks, their transforms through T and K); per pixel the 78 packed y-Hessian entries,
-    the gradient and the likelihood weights (600)."""
+    the gradient and the likelihood weights (600).  (The kernel forms 16 of the 35 sums from
+    the other 19 and 66 pixel sums in place of 78; the count stays that of the formulas, so
+    that rates compare across versions.)"""
     nprof = n_exp + n_dev
     return npsf * (5 + 31 + 8 + 329 + 75 * nprof) + 600
 
@@ -121,7 +123,8 @@ def hess_flops_per_source_pixel(npsf, n_exp, n_dev):
 def hess64_flops_per_source_pixel(npsf, n_exp, n_dev):
     """The same for the FP64 Hessian path, which evaluates the mixture's first and second
     derivatives component by component in the pixel frame (per PSF component 20 + 42, each
-    galaxy component 140; per pixel 600)."""
+    galaxy component 140; per pixel 600).  (The kernel works in the whitened frame with about
+    half of these operations, so its rate by this count can exceed the FP64 peak.)"""
     nprof = n_exp + n_dev
     return npsf * (5 + 8 + 8 * nprof) + 30 + npsf * (20 + 42 + 140 * nprof) + 600
 

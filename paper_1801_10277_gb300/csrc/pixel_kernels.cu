@@ -407,7 +407,7 @@ __device__ __forceinline__ bool any_multi(const WorkItem& it, const PatchGeo& g,
 // expected log-likelihood go straight to the maps and to the item's ll sum; only
 // pixels covered by several patches keep E_s / Var_s for k_gather.  multi_only: items
 // without such pixels are skipped (the Hessian pass forms E and Var at the others itself;
-// 500 sources, 92 % of the source-pixels singly covered: 23 -> 11 us).
+// 500 sources, 92 % of the source-pixels singly covered: 23 -> 16 us).
 
 template <class R, int PPT>
 __global__ void __launch_bounds__(CHUNK / PPT) k_contrib(const WorkItem* __restrict__ items,
@@ -1537,7 +1537,7 @@ cudaError_t launch_contrib(const DevProblem& P, int precision, cudaStream_t st, 
     if (precision == CELESTE_FP64) {
         // An SM runs a CTA's FP64 instructions at a warp per 16 cycles whatever its size, so few
         // items are cut until there are eight CTAs per SM (64 crowded sources, 565 items: the map
-        // pass 110 -> 80 us; a fit's batch of 60 items 40 -> 17 us).
+        // pass 115 -> 107 us; a fit's batch of 60 items 40 -> 31 us).
         int split = 1;
         while (split < 4 && (int64_t)S.n * split < 8LL * sm_count()) split *= 2;
         k_contrib64<<<S.n * split, CHUNK / split, 0, st>>>(P.items, P.geo, P.img, P.nprof, P.model_ne, P.tbl64, (double*)P.spE,
