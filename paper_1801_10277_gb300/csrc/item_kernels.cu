@@ -1457,8 +1457,9 @@ static cudaError_t launch_stage(const DevProblem& P, int stage, int mode, cudaSt
 cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStream_t st, const double* d_theta,
                                double* d_local, double* d_grad, double* d_total) {
     const cudaError_t e = launch_stage(P, stage, mode, st, d_theta, d_local, d_grad, d_total);
-    // tables published without an epilogue kernel behind them must not pass for the next call's
-    if (e != cudaSuccess && stage > 0) {
+    // tables published without an epilogue kernel behind them must not pass for the next call's (the
+    // first stage too: the error that it reports can be one that an earlier call left)
+    if (e != cudaSuccess && P.ztasks) {
         cudaMemsetAsync(P.zready, 0, sizeof(int32_t) * ((size_t)P.n_patch + 2), st);
         cudaMemsetAsync(P.zf_done, 0, 2 * sizeof(int32_t), st);
     }

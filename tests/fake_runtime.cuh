@@ -1,0 +1,82 @@
+// A stand-in for the CUDA runtime calls that the library's host code makes around its
+// launches, so that a host check can include a .cu file and drive that code without a GPU:
+// devices with multiprocessor counts of their own, recorded attributes and memory calls,
+// errors on demand.  (The <<< >>> launches themselves go to the real runtime, which must
+// see no device: main starts with no_real_device().)
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstdio>
+#include <cstdlib>
+#include <map>
+#include <set>
+#include <vector>
+
+namespace fake {
+
+inline int device = 0;                               // current device
+inline std::vector<int> sm_of_device = {152, 132};   // multiprocessors
+inline cudaError_t last_error = cudaSuccess;         // what cudaGetLastError returns (once)
+inline cudaError_t launch_error = cudaSuccess;       // what cudaLaunchKernelEx returns
+inline std::set<std::pair<const void*, int>> smem_set;   // (kernel, device) with its shared-memory limit raised
+inline bool launched_unset = false;                  // a launch over 48 KB on a device without the limit
+inline unsigned grid = 0;                            // of the last cudaLaunchKernelEx
+struct Set {
+    void* p;
+    size_t bytes;
+};
+inline std::vector<Set> sets;                        // cudaMemsetAsync calls
+
+inline void no_real_device() {
+    int n = 0;
+    if (cudaGetDeviceCount(&n) == cudaSuccess && n > 0) {
+        printf("a GPU is visible: run with CUDA_VISIBLE_DEVICES=\n");
+        exit(2);
+    }
+    (void)cudaGetLastError();
+}
+
+inline cudaError_t get_device(int* d) {
+    *d = device;
+    return cudaSuccess;
+}
+inline cudaError_t get_attribute(int* v, cudaDeviceAttr a, int d) {
+    *v = a == cudaDevAttrMultiProcessorCount ? sm_of_device[d] : 0;
+    return cudaSuccess;
+}
+template <class F>
+cudaError_t func_set_attribute(F* f, cudaFuncAttribute a, int) {
+    if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) smem_set.insert({(const void*)f, device});
+    return cudaSuccess;
+}
+template <class F>
+cudaError_t occupancy(int* n, F*, int, size_t) {
+    *n = 4;
+    return cudaSuccess;
+}
+inline cudaError_t get_last_error() {
+    const cudaError_t e = last_error;
+    last_error = cudaSuccess;
+    return e;
+}
+template <class... A, class... B>
+cudaError_t launch_ex(const cudaLaunchConfig_t* c, void (*f)(A...), B&&...) {
+    grid = c->gridDim.x;
+    if (c->dynamicSmemBytes > 48 * 1024 && !smem_set.count({(const void*)f, device})) launched_unset = true;
+    return launch_error;
+}
+inline cudaError_t memset_async(void* p, int, size_t n, cudaStream_t) {
+    sets.push_back({p, n});
+    return cudaSuccess;
+}
+
+}  // namespace fake
+
+#define cudaGetDevice fake::get_device
+#define cudaDeviceGetAttribute fake::get_attribute
+#define cudaFuncSetAttribute fake::func_set_attribute
+#define cudaOccupancyMaxActiveBlocksPerMultiprocessor fake::occupancy
+#define cudaGetLastError fake::get_last_error
+#define cudaLaunchKernelEx fake::launch_ex
+#define cudaMemsetAsync fake::memset_async

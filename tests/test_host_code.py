@@ -1,0 +1,40 @@
+"""The library's host code around its kernels, compiled into small check programs that run on
+the CPU with a stand-in for the CUDA runtime (fake_runtime.cuh)."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+CSRC = os.path.join(ROOT, "paper_1801_10277_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def check(tmp_path_factory):
+    """check(program, *arguments): tests/<program>.cu compiled once and run with no GPU visible."""
+    nvcc = os.environ.get("NVCC") or shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not found")
+    where, built = tmp_path_factory.mktemp("checks"), {}
+
+    def run(program, *args):
+        if program not in built:
+            exe = str(where / program)
+            r = subprocess.run([nvcc, "-std=c++17", "--expt-relaxed-constexpr", "-gencode",
+                                "arch=compute_103a,code=compute_103a", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
+                                "-I", HERE, os.path.join(HERE, program + ".cu"), "-o", exe],
+                               capture_output=True, text=True)
+            assert r.returncode == 0, r.stdout + r.stderr
+            built[program] = exe
+        r = subprocess.run([built[program], *map(str, args)], capture_output=True, text=True, timeout=300,
+                           env=dict(os.environ, CUDA_VISIBLE_DEVICES=""))
+        assert r.returncode == 0, r.stdout + r.stderr
+        return r.stdout
+
+    return run
+
+
+def test_a_failed_launch_leaves_no_ready_flags(check):
+    check("item_launch_check", "flags")
