@@ -399,6 +399,20 @@ __device__ __forceinline__ bool mbar_wait_launch(uint64_t* bar, unsigned parity,
     return false;
 }
 
+// A warp that gave up on a wait at item i: let the copies that its CTA has in flight (the stages and
+// the records ahead of items i and i + 1) land before it leaves, as the shared memory is another
+// CTA's next.  A barrier that nothing is on its way to costs the limit, about 10 ms.
+__device__ __forceinline__ void drain(uint64_t* full, uint64_t* fetched, int i) {
+#pragma unroll 1
+    for (int e = 0; e < 4; ++e) {
+        const int x = i + (e >> 1);
+        uint64_t* bar = (e & 1 ? fetched : full) + (x & 1);
+        const long long t0 = clock64();
+        for (int n = 0; n < MBAR_MAX_POLLS && clock64() - t0 < MBAR_MAX_CYCLES / 100; ++n)
+            if (mbar_try_wait(bar, (x >> 1) & 1)) break;
+    }
+}
+
 __device__ __forceinline__ void mbar_arrive_plain(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
@@ -1260,10 +1274,14 @@ __global__ void __launch_bounds__(NTC) __maxnreg__(regs_for(MINB)) k_items(ItemA
     else if (w == 2 && lane == 0)
         fetch_record(a, base + atomicAdd(queue, 1), &next[0], &fetched[0]);
     float* spg = reinterpret_cast<float*>(smem + L::pg) + t;
+    int stopped = -1;   // the item at which a wait gave up
     for (int i = 0;; ++i) {
         const int b = i & 1;
         __syncwarp();
-        if (!mbar_wait_launch(&full[b], (i >> 1) & 1, a.status)) break;
+        if (!mbar_wait_launch(&full[b], (i >> 1) & 1, a.status)) {
+            stopped = i;
+            break;
+        }
         if (tasks[b].kind == ZT_END) break;
         const ZItem it = tasks[b].item;
         uint8_t* stage = smem + b * ST_BYTES;
@@ -1288,12 +1306,16 @@ __global__ void __launch_bounds__(NTC) __maxnreg__(regs_for(MINB)) k_items(ItemA
         int q = 0;
         if (lane == 0) q = base + atomicAdd(queue, 1);
         item_record<MODE>(a, it.out, rb, nch);
-        if (!mbar_wait_launch(&fetched[b], (i >> 1) & 1, a.status)) break;
+        if (!mbar_wait_launch(&fetched[b], (i >> 1) & 1, a.status)) {
+            stopped = i;
+            break;
+        }
         const int4 rec = lane < 4 ? reinterpret_cast<const int4*>(&next[b])[lane] : make_int4(0, 0, 0, 0);
         __syncwarp();
         prepare<MODE>(a, rec, stage, &tasks[b], &full[b], all_built);
         if (lane == 0) fetch_record(a, q, &next[b ^ 1], &fetched[b ^ 1]);
     }
+    if (stopped >= 0) drain(full, fetched, stopped);
     // this grid completes only after the table kernel (and its KL terms) has, so the epilogue
     // kernel that waits for this grid sees both
     if (w == 0) pdl_wait();
