@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <cmath>
 
 #include "celeste.h"
@@ -426,18 +427,30 @@ cudaError_t launch_total(const DevProblem& P, double* d_total, cudaStream_t st);
 // (hess, FP32: and the Hessian pass's frames, in the place of the FP64 tables)
 cudaError_t launch_prep(const DevProblem& P, const double* d_theta, int precision,
                         cudaStream_t st, bool with_kl = true, bool hess = false);
+// An int of each device, filled where it is first asked for (0: not yet); devices past the last
+// slot share none and ask each time
+struct PerDevice {
+    static constexpr int N = 64;
+    std::atomic<int> v[N];
+    template <class F>
+    int get(F&& ask) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= N) return ask(dev);
+        int n = v[dev].load(std::memory_order_acquire);
+        if (n == 0) {
+            n = ask(dev);
+            v[dev].store(n, std::memory_order_release);
+        }
+        return n;
+    }
+};
 // multiprocessors of the current device
 inline int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            n = v;
-        else
-            n = 1;
-    }
-    return n;
+    static PerDevice sms;
+    return sms.get([](int dev) {
+        int n = 0;
+        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 1;
+    });
 }
 // E_s and Var_s at every item pixel, singly covered ones (P.single) finished into the maps;
 // multi_only: at the multiply covered pixels alone, the others being left to the

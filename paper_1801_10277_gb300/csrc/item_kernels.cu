@@ -1326,25 +1326,27 @@ __global__ void __launch_bounds__(NTC) __maxnreg__(regs_for(MINB)) k_items(ItemA
 
 template <int MODE, int NPE, int NPD, int MINB, int UNR>
 struct ItemsKernel {
-    static int per_sm;   // resident CTAs per SM (0: not yet set up)
-    static cudaError_t setup() {
-        if (per_sm > 0) return cudaSuccess;
-        auto* fn = k_items<MODE, NPE, NPD, MINB, UNR>;
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::bytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        int per = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, NTC, Lay::bytes);
-        if (e != cudaSuccess) return e;
-        per_sm = per > 0 ? per : 1;
-        return cudaSuccess;
+    // Resident CTAs per SM on the current device, its shared-memory limit raised first (both are
+    // a device's own: the limit holds on the device it was set on).  0: an error, in *err.
+    static int per_sm(cudaError_t* err) {
+        static PerDevice on;
+        *err = cudaSuccess;
+        return on.get([&](int) {
+            auto* fn = k_items<MODE, NPE, NPD, MINB, UNR>;
+            cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::bytes);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+            int per = 0;
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, NTC, Lay::bytes);
+            *err = e;
+            return e != cudaSuccess ? 0 : per > 0 ? per : 1;
+        });
     }
     // a programmatic dependent launch of the table kernel before it on st
     static cudaError_t launch(const ItemArgs& a, int n_sm, cudaStream_t st) {
-        cudaError_t e = setup();
+        cudaError_t e;
+        int grid = per_sm(&e) * n_sm;
         if (e != cudaSuccess) return e;
-        int grid = per_sm * n_sm;
         if (grid > a.n_task) grid = a.n_task;
         if (grid < 1) return cudaSuccess;
         cudaLaunchConfig_t cfg{};
@@ -1360,9 +1362,6 @@ struct ItemsKernel {
         return cudaLaunchKernelEx(&cfg, k_items<MODE, NPE, NPD, MINB, UNR>, a);
     }
 };
-template <int MODE, int NPE, int NPD, int MINB, int UNR>
-int ItemsKernel<MODE, NPE, NPD, MINB, UNR>::per_sm = 0;
-
 // the model of the synthetic workloads and of the paper (6 exp + 8 dev profile
 // components: 3 + 4 pairs) gets its loops unrolled for those counts
 template <int MODE, int MINB, int UNR>
@@ -1393,8 +1392,8 @@ template <int MODE>
 cudaError_t items_setup_mode() {
     cudaError_t e = cudaSuccess;
 #define CEL_SETUP(c, minb, unr)                                                    \
-    if (e == cudaSuccess) e = ItemsKernel<MODE, 3, 4, minb, unr>::setup();           \
-    if (e == cudaSuccess) e = ItemsKernel<MODE, -1, -1, minb, 1>::setup();
+    if (e == cudaSuccess) ItemsKernel<MODE, 3, 4, minb, unr>::per_sm(&e);            \
+    if (e == cudaSuccess) ItemsKernel<MODE, -1, -1, minb, 1>::per_sm(&e);
     CEL_ITEM_VARIANTS(CEL_SETUP)
 #undef CEL_SETUP
     return e;
@@ -1402,8 +1401,8 @@ cudaError_t items_setup_mode() {
 
 }  // namespace
 
-// shared-memory limits and resident CTAs of every item-kernel variant, set once outside
-// any stream capture
+// shared-memory limits and resident CTAs of every item-kernel variant on the current device, set
+// once per device outside any stream capture
 cudaError_t prime_items_kernels() {
     cudaError_t e = items_setup_mode<MODE_LL>();
     if (e == cudaSuccess) e = items_setup_mode<MODE_GRAD>();

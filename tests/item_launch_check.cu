@@ -3,6 +3,8 @@
 //   flags   An evaluation whose k-th launch fails leaves the tables' ready flags, the queue
 //           counter and the status word cleared: tables published by a kernel with no epilogue
 //           kernel behind it must not pass for the next evaluation's.
+//   devices After problems on two devices were set up, the item kernel has its shared-memory
+//           limit raised on both, and its grid is that of the device it is launched on.
 #include "fake_runtime.cuh"
 
 #include "item_kernels.cu"
@@ -48,10 +50,31 @@ static int check_flags() {
     return 0;
 }
 
+static int check_devices() {
+    std::vector<int32_t> ready;
+    int32_t done[2];
+    cel::ZTask task;
+    const cel::DevProblem P = problem(ready, done, &task);
+    for (int d : {0, 1, 0}) {
+        fake::device = d;
+        fake::launched_unset = false;
+        if (cel::prime_items_kernels() != cudaSuccess) return printf("set-up failed on device %d\n", d), 1;
+        for (int mode : {cel::MODE_LL, cel::MODE_GRAD}) {
+            const cudaError_t e = cel::launch_items_stage(P, 1, mode, nullptr, nullptr, nullptr, nullptr, nullptr);
+            const unsigned want = 4u * fake::sm_of_device[d];   // the stand-in's four CTAs per multiprocessor
+            if (e != cudaSuccess || fake::launched_unset || fake::grid != want)
+                return printf("device %d, mode %d: error %d, limit missing %d, grid %u (expected %u)\n", d, mode, (int)e,
+                              fake::launched_unset, fake::grid, want), 1;
+        }
+    }
+    return 0;
+}
+
 int main(int argc, char** argv) {
     fake::no_real_device();
     const char* what = argc > 1 ? argv[1] : "";
     if (!strcmp(what, "flags")) return check_flags();
+    if (!strcmp(what, "devices")) return check_devices();
     printf("unknown check %s\n", what);
     return 1;
 }

@@ -38,3 +38,7 @@ def check(tmp_path_factory):
 
 def test_a_failed_launch_leaves_no_ready_flags(check):
     check("item_launch_check", "flags")
+
+
+def test_a_second_device_gets_its_own_set_up(check):
+    check("item_launch_check", "devices")
