@@ -276,9 +276,21 @@ k_batch_start(int nb, const int32_t* __restrict__ bsrc, const double* __restrict
 
 constexpr int TR_THREADS = 128;
 constexpr int TRN = NT;   // 41
-// k_tr_step's dynamic shared memory: the source's 44 x 44 Hessian and H T (44 x 41); later the
-// FP32 copies of the multiplier search
-constexpr size_t TR_DYN_BYTES = sizeof(double) * (NP * NP + NP * TRN);
+// k_tr_step's dynamic shared memory: the source's Hessian and H T; once these are dead, the FP32
+// copies of the multiplier search
+struct alignas(16) TrShared {
+    struct Step {
+        double H[NP * NP], X[NP * TRN];
+    };
+    struct Search {
+        float B[TRN * TRN], L[(TRN + 1) * TRN], c[TRN], p[TRN], w[TRN], rd[TRN];
+        alignas(16) float cb[44];   // chol32's column, read as float4
+    };
+    union {
+        Step step;
+        Search search;
+    };
+};
 
 // Packed lower-triangle order of side 40 (the trailing triangles of the bordered matrix
 // below), copied into shared memory by each CTA
@@ -534,9 +546,9 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
     __shared__ int done;
     __shared__ double lam_s, pn_s;
     __shared__ uint16_t pk[PK_N];
-    extern __shared__ double tr_dyn[];
-    double* Hs = tr_dyn;             // [NP][NP] the source's Hessian
-    double* X = tr_dyn + NP * NP;    // [NP][TRN] H T
+    extern __shared__ TrShared tr_dyn[];
+    double* Hs = tr_dyn->step.H;   // [NP][NP] the source's Hessian
+    double* X = tr_dyn->step.X;    // [NP][TRN] H T
     const int tid = threadIdx.x;
     if (tid == 0) S = st[b];
     __syncthreads();
@@ -735,11 +747,8 @@ k_tr_step(int nb, const double* __restrict__ theta, const double* __restrict__ t
         // which then needs one or two.  The FP32 bracket is not kept: FP32 rounding can
         // misjudge definiteness near the smallest eigenvalue.
         {
-            float* B32 = reinterpret_cast<float*>(tr_dyn);   // H and H T are dead by now
-            float* L32 = B32 + TRN * TRN;
-            float* c32 = L32 + (TRN + 1) * TRN;
-            float *p32 = c32 + TRN, *w32 = p32 + TRN, *r32 = w32 + TRN;
-            float* cb32 = B32 + 4 * TRN * TRN;   // 16-byte aligned, past the others
+            TrShared::Search& S32 = tr_dyn->search;   // H and H T are dead by now
+            float *B32 = S32.B, *L32 = S32.L, *c32 = S32.c, *p32 = S32.p, *w32 = S32.w, *r32 = S32.rd, *cb32 = S32.cb;
             for (int i = tid; i < TRN * TRN; i += blockDim.x) B32[i] = (float)Ht[i];
             for (int i = tid; i < TRN; i += blockDim.x) c32[i] = (float)cvec[i];
             __syncthreads();
@@ -1280,7 +1289,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
         FIT_CUDA(cudaMemcpyAsync(d_task, task_of, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
         FIT_CUDA(cudaMemcpyAsync(d_th0, theta, sizeof(double) * NP * n, cudaMemcpyHostToDevice, st));
     }
-    FIT_CUDA(cudaFuncSetAttribute(k_tr_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TR_DYN_BYTES));
+    FIT_CUDA(cudaFuncSetAttribute(k_tr_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrShared)));
     FIT_CUDA(cudaMemcpyAsync(pr->d_theta, theta, sizeof(double) * NP * n, cudaMemcpyHostToDevice, st));
     std::vector<int32_t> iters(n, 0), status(n, ST_CONVERGED);
     double prev = 0.0;
@@ -1401,7 +1410,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             batch_pixels(true);
             chk(launch_hess_pixels(Pb, prec, d_bth, d_h, st));
             chk(launch_finalize_hess(Pb, d_f, d_g, d_h, st));
-            k_tr_step<<<nb, TR_THREADS, TR_DYN_BYTES, st>>>(nb, d_bth, d_bt, d_f, d_g, d_h, d_kl, d_bthc, d_btc,
+            k_tr_step<<<nb, TR_THREADS, sizeof(TrShared), st>>>(nb, d_bth, d_bt, d_f, d_g, d_h, d_kl, d_bthc, d_btc,
                                                  d_st, *opts, d_srcact);
             chk(launch_prep(Pc, d_bthc, prec, st, false, true));
             chk(launch_contrib(Pc, prec, st));

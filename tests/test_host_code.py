@@ -42,3 +42,7 @@ def test_a_failed_launch_leaves_no_ready_flags(check):
 
 def test_a_second_device_gets_its_own_set_up(check):
     check("item_launch_check", "devices")
+
+
+def test_trust_region_shared_memory_alignment(check):
+    check("fit_layout_check")
