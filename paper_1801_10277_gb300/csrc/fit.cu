@@ -994,6 +994,11 @@ struct Batch {
     int hchunk = 0;                  // pixels of a part
 };
 
+// Pixels of a part of the Hessian pass in a fit: by the problem, not by the batch, as the FP32 sums,
+// and with them a source's iterates, must not depend on which other sources share its batch (a
+// batch is an eighth of the problem or so)
+int batch_hchunk(const celeste_problem* pr) { return hess_chunk(pr->P.n_sp / 8, sm_count()); }
+
 Batch make_batch(const celeste_problem* pr, const std::vector<int32_t>& members) {
     Batch B;
     B.src = members;
@@ -1015,9 +1020,7 @@ Batch make_batch(const celeste_problem* pr, const std::vector<int32_t>& members)
         }
         B.patch_off.push_back((int)B.geo.size());
     }
-    // by the problem, not by the batch: the FP32 sums, and with them a source's iterates, must not
-    // depend on which other sources share its batch (a batch is an eighth of the problem or so)
-    B.hchunk = hess_chunk(pr->P.n_sp / 8, sm_count());
+    B.hchunk = batch_hchunk(pr);
     for (int p = 0; p < (int)B.geo.size(); ++p)
         push_parts(B.parts, B.geo[p], p, pr->imgs[B.geo[p].img], B.hchunk);
     return B;
@@ -1174,6 +1177,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             maxSp = std::max(maxSp, B.n_sp);
         }
     } else {
+        const int hchunk = batch_hchunk(pr);
         std::vector<int64_t> np_, ni_, nh_, nsp_;
         for (int s : moving) {
             int64_t a = 0, b = 0, h = 0, c = 0;
@@ -1181,7 +1185,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
                 const int64_t npx = (int64_t)pr->geo[p].w * pr->geo[p].h;
                 ++a;
                 b += (npx + CHUNK - 1) / CHUNK;
-                h += (npx + 31) / 32;   // the smallest parts a batch may have
+                h += (npx + hchunk - 1) / hchunk;
                 c += npx;
             }
             np_.push_back(a);
@@ -1228,8 +1232,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
     PatchGeo* d_bgeo;
     WorkItem* d_bitems;
     HItem* d_bparts;
-    double *d_bth, *d_bthc, *d_bt, *d_btc, *d_f, *d_g, *d_h, *d_kl, *d_hsrc, *d_part, *d_dll, *d_tbl64, *d_ctbl64;
-    float *d_tbl32, *d_ctbl32;
+    double *d_bth, *d_bthc, *d_bt, *d_btc, *d_f, *d_g, *d_h, *d_kl, *d_hsrc, *d_part, *d_dll, *d_ctbl;
     TrState* d_st;
     unsigned char *d_eo, *d_vo, *d_se, *d_sv, *d_ce, *d_cv;
     FIT_CUDA(mem.alloc(&d_bsrc, maxB));
@@ -1250,10 +1253,12 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
     FIT_CUDA(mem.alloc(&d_part, maxH * HV));
     FIT_CUDA(mem.alloc(&d_bparts, maxH));
     FIT_CUDA(mem.alloc(&d_dll, maxI));
-    FIT_CUDA(mem.alloc(&d_tbl64, maxP * TBL_STRIDE));
-    FIT_CUDA(mem.alloc(&d_tbl32, maxP * TBL_STRIDE));
-    FIT_CUDA(mem.alloc(&d_ctbl64, maxP * TBL_STRIDE));
-    FIT_CUDA(mem.alloc(&d_ctbl32, maxP * TBL_STRIDE));
+    // The tables of a batch's patches at theta take the place of the problem's (which every
+    // evaluation of the problem builds anew); these are the candidates': FP64 tables, or (FP32)
+    // FP32 tables with the Hessian pass's frames behind them.
+    const bool any64 = opts->precision == CELESTE_FP64 || opts->refine_fp64;
+    static_assert((TBL_STRIDE + HF_STRIDE) * sizeof(float) <= TBL_STRIDE * sizeof(double), "one buffer for both");
+    FIT_CUDA(mem.alloc(&d_ctbl, any64 ? maxP * TBL_STRIDE : maxP * (TBL_STRIDE + HF_STRIDE) / 2));
     FIT_CUDA(mem.alloc(&d_st, maxB));
     FIT_CUDA(mem.alloc(&d_eo, maxSp * rs));
     FIT_CUDA(mem.alloc(&d_vo, maxSp * rs));
@@ -1360,8 +1365,6 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             Pb.n_hitem = (int)B.parts.size();
             Pb.hchunk = B.hchunk;
             Pb.patch_off = d_bpo;
-            Pb.tbl64 = d_tbl64;
-            Pb.tbl32 = d_tbl32;
             Pb.spE = d_se;
             Pb.spE2 = d_sv;
             Pb.item_part = d_part;
@@ -1376,8 +1379,8 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             DevProblem Pc = Pb;
             Pc.spE = d_ce;
             Pc.spE2 = d_cv;
-            Pc.tbl64 = d_ctbl64;
-            Pc.tbl32 = d_ctbl32;
+            Pc.tbl32 = (float*)d_ctbl;
+            Pc.tbl64 = prec == CELESTE_FP64 ? d_ctbl : (double*)(Pc.tbl32 + maxP * TBL_STRIDE);
             // the batch's tables and E_s / Var_s at its start
             FIT_CUDA(launch_prep(Pb, d_bth, prec, st, false, true));
             FIT_CUDA(launch_contrib(Pb, prec, st));
@@ -1397,15 +1400,15 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
                 if (maps)
                     k_batch_maps<T><<<nI, CHUNK, 0, st>>>(d_bitems, d_bgeo, P.img, eo, vo, se, sv, cE, cV, (T*)P.emap,
                                                           (T*)P.vmap, d_srcact, d_st, tbl, ctbl, n_tbl,
-                                                          (float*)d_tbl64, (const float*)d_ctbl64,
+                                                          (float*)Pb.tbl64, (const float*)Pc.tbl64,
                                                           sizeof(T) == 4 ? P.npsf_max * WFR : 0);
                 else
                     k_batch_dll<T><<<nI, CHUNK, 0, st>>>(d_bitems, d_bgeo, P.img, P.pixels, eo, vo, se, sv, cE, cV,
                                                          d_dll, d_srcact);
             };
             auto batch_pixels = [&](bool maps) {
-                if (prec == CELESTE_FP64) pixel_kernels(0.0, d_tbl64, d_ctbl64, maps);
-                else pixel_kernels(0.f, d_tbl32, d_ctbl32, maps);
+                if (prec == CELESTE_FP64) pixel_kernels(0.0, Pb.tbl64, Pc.tbl64, maps);
+                else pixel_kernels(0.f, Pb.tbl32, Pc.tbl32, maps);
             };
             batch_pixels(true);
             chk(launch_hess_pixels(Pb, prec, d_bth, d_h, st));

@@ -9,6 +9,7 @@
 
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <map>
 #include <set>
 #include <vector>
@@ -27,6 +28,9 @@ struct Set {
     size_t bytes;
 };
 inline std::vector<Set> sets;                        // cudaMemsetAsync calls
+
+inline size_t live_bytes = 0;                        // device memory held
+inline std::map<void*, size_t> blocks;
 
 inline void no_real_device() {
     int n = 0;
@@ -71,6 +75,36 @@ inline cudaError_t memset_async(void* p, int, size_t n, cudaStream_t) {
     return cudaSuccess;
 }
 
+// device memory is host memory, so that copies work; its bytes are counted
+template <class T>
+cudaError_t device_malloc(T** p, size_t n) {
+    *p = (T*)calloc(n ? n : 1, 1);
+    blocks[(void*)*p] = n;
+    live_bytes += n;
+    return *p ? cudaSuccess : cudaErrorMemoryAllocation;
+}
+inline cudaError_t device_free(void* p) {
+    auto b = blocks.find(p);
+    if (b == blocks.end()) return p ? cudaErrorInvalidValue : cudaSuccess;
+    live_bytes -= b->second;
+    blocks.erase(b);
+    free(p);
+    return cudaSuccess;
+}
+template <class T>
+cudaError_t host_malloc(T** p, size_t n) {
+    *p = (T*)calloc(n, 1);
+    return cudaSuccess;
+}
+inline cudaError_t host_free(void* p) {
+    free(p);
+    return cudaSuccess;
+}
+inline cudaError_t copy_async(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+    memcpy(d, s, n);
+    return cudaSuccess;
+}
+
 }  // namespace fake
 
 #define cudaGetDevice fake::get_device
@@ -80,3 +114,8 @@ inline cudaError_t memset_async(void* p, int, size_t n, cudaStream_t) {
 #define cudaGetLastError fake::get_last_error
 #define cudaLaunchKernelEx fake::launch_ex
 #define cudaMemsetAsync fake::memset_async
+#define cudaMalloc fake::device_malloc
+#define cudaFree fake::device_free
+#define cudaMallocHost fake::host_malloc
+#define cudaFreeHost fake::host_free
+#define cudaMemcpyAsync fake::copy_async

@@ -46,3 +46,9 @@ def test_a_second_device_gets_its_own_set_up(check):
 
 def test_trust_region_shared_memory_alignment(check):
     check("fit_layout_check")
+
+
+@pytest.mark.parametrize("schedule", ["colour", "cyclades"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp32only"])
+def test_device_memory_of_a_fit(check, precision, schedule):
+    check("fit_memory_check", precision, schedule)
