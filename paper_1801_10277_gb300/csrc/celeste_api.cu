@@ -901,12 +901,15 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     P.tbl32 = (float*)p;
     if ((st = dalloc(pr, &p, sizeof(float) * ZFULL_FLOATS * (size_t)n_patch))) return bail(st);
     P.ztbl = (float*)p;
-    if ((st = dalloc(pr, &P.spE, sizeof(double) * (size_t)n_sp))) return bail(st);
-    if ((st = dalloc(pr, &P.spE2, sizeof(double) * (size_t)n_sp))) return bail(st);
+    // E_s and Var_s side by side (the second on a 256-byte boundary); the Hessian pass's part records
+    // take their place, as its map passes are done with them when its pixel pass starts
+    const size_t sp_bytes = (sizeof(double) * (size_t)n_sp + 255) / 256 * 256;
+    if ((st = dalloc(pr, &P.spE, std::max(2 * sp_bytes, sizeof(double) * HV * (size_t)P.n_hitem)))) return bail(st);
+    P.spE2 = (char*)P.spE + sp_bytes;
+    P.hpart = (double*)P.spE;
     if ((st = dalloc(pr, &P.emap, sizeof(double) * (size_t)n_px))) return bail(st);
     if ((st = dalloc(pr, &P.vmap, sizeof(double) * (size_t)n_px))) return bail(st);
-    if ((st = dalloc(pr, &p, sizeof(double) * std::max(NPART * (size_t)P.n_item, HV * (size_t)P.n_hitem))))
-        return bail(st);
+    if ((st = dalloc(pr, &p, sizeof(double) * NPART * (size_t)P.n_item))) return bail(st);
     P.item_part = (double*)p;
     if ((st = dalloc(pr, &p, sizeof(double) * (size_t)P.n_tile))) return bail(st);
     P.tile_ll = (double*)p;

@@ -1367,7 +1367,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             Pb.patch_off = d_bpo;
             Pb.spE = d_se;
             Pb.spE2 = d_sv;
-            Pb.item_part = d_part;
+            Pb.hpart = d_part;
             Pb.kl = d_kl;
             Pb.hsrc = d_hsrc;
             Pb.kl_grad = nullptr;   // the Hessian pass and k_tr_accept take the KL themselves

@@ -1091,7 +1091,7 @@ static cudaError_t hess_pixels(const DevProblem& P, const R* tbl, const double* 
     a.single = P.single;
     a.emap = (const R*)P.emap;
     a.vmap = (const R*)P.vmap;
-    a.part = P.item_part;
+    a.part = P.hpart;
     a.src_active = P.src_active;
     a.queue = P.hqueue;
     a.src = SourceTerms{P.n_src, d_theta, P.model, P.hsrc, P.kl, d_hess, P.status};
@@ -1132,7 +1132,7 @@ cudaError_t launch_hess_pixels(const DevProblem& P, int precision, const double*
 cudaError_t launch_finalize_hess(const DevProblem& P, double* d_local, double* d_grad, double* d_hess,
                                  cudaStream_t st) {
     if (P.n_src == 0) return cudaSuccess;
-    k_finalize_hess<<<P.n_src, FH_THREADS, 0, st>>>(P.n_src, P.hchunk, P.geo, P.patch_off, P.img, P.item_part, P.hsrc, d_local,
+    k_finalize_hess<<<P.n_src, FH_THREADS, 0, st>>>(P.n_src, P.hchunk, P.geo, P.patch_off, P.img, P.hpart, P.hsrc, d_local,
                                                     d_grad, d_hess, P.src_active);
     return cudaGetLastError();
 }

@@ -325,7 +325,8 @@ struct DevProblem {
     void* vmap;
     const uint8_t* single;   // per (source, pixel): 1 when no other patch covers the pixel (nullable)
     double* item_ll;         // per work item: ll summed over its singly covered pixels
-    double* item_part;       // per item (value / gradient) or part (Hessian) sums
+    double* item_part;       // per item sums (value / gradient)
+    double* hpart;           // the Hessian pass's per-part sums (a problem's: over spE, spE2)
     double* tile_ll;
     double* kl;
     double* kl_grad;         // [n_src][44] KL gradient, written by k_prep (nullable: no KL in prep)

@@ -7,6 +7,7 @@
 
 #include <cuda_runtime.h>
 
+#include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -105,6 +106,39 @@ inline cudaError_t copy_async(void* d, const void* s, size_t n, cudaMemcpyKind, 
     return cudaSuccess;
 }
 
+inline cudaError_t copy(void* d, const void* s, size_t n, cudaMemcpyKind) {
+    memcpy(d, s, n);
+    return cudaSuccess;
+}
+// every other call succeeds; handles are numbered
+inline size_t handles = 0;
+template <class H, class... A>
+cudaError_t make_handle(H* h, A...) {
+    *h = (H)(uintptr_t)++handles;
+    return cudaSuccess;
+}
+template <class S, class H>
+cudaError_t make_second(S, H* h) {
+    return make_handle(h);
+}
+template <class... A>
+cudaError_t done(A...) {
+    return cudaSuccess;
+}
+inline cudaError_t priority_range(int* least, int* greatest) {
+    *least = *greatest = 0;
+    return cudaSuccess;
+}
+inline float elapsed_ms = 1.f;   // what every pair of events is apart
+inline cudaError_t elapsed(float* t, cudaEvent_t, cudaEvent_t) {
+    *t = elapsed_ms;
+    return cudaSuccess;
+}
+inline cudaError_t set_bytes(void* p, int v, size_t n) {
+    memset(p, v, n);
+    return cudaSuccess;
+}
+
 }  // namespace fake
 
 #define cudaGetDevice fake::get_device
@@ -119,3 +153,24 @@ inline cudaError_t copy_async(void* d, const void* s, size_t n, cudaMemcpyKind, 
 #define cudaMallocHost fake::host_malloc
 #define cudaFreeHost fake::host_free
 #define cudaMemcpyAsync fake::copy_async
+#define cudaMemcpy fake::copy
+#define cudaMemset fake::set_bytes
+#define cudaSetDevice fake::done
+#define cudaDeviceSynchronize fake::done
+#define cudaStreamSynchronize fake::done
+#define cudaStreamCreateWithFlags fake::make_handle
+#define cudaStreamCreateWithPriority fake::make_handle
+#define cudaStreamDestroy fake::done
+#define cudaStreamBeginCapture fake::done
+#define cudaStreamEndCapture fake::make_second
+#define cudaDeviceGetStreamPriorityRange fake::priority_range
+#define cudaEventCreate fake::make_handle
+#define cudaEventCreateWithFlags fake::make_handle
+#define cudaEventDestroy fake::done
+#define cudaEventRecord fake::done
+#define cudaEventSynchronize fake::done
+#define cudaEventElapsedTime fake::elapsed
+#define cudaGraphInstantiate fake::make_handle
+#define cudaGraphDestroy fake::done
+#define cudaGraphExecDestroy fake::done
+#define cudaGraphLaunch fake::done

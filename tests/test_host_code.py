@@ -52,3 +52,7 @@ def test_trust_region_shared_memory_alignment(check):
 @pytest.mark.parametrize("precision", ["fp64", "fp32", "fp32only"])
 def test_device_memory_of_a_fit(check, precision, schedule):
     check("fit_memory_check", precision, schedule)
+
+
+def test_device_memory_of_a_problem(check):
+    check("api_check", "memory")
