@@ -950,6 +950,9 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     if ((st = dalloc(pr, &p, sizeof(double) * NP * (size_t)n_src))) return bail(st);
     pr->d_theta = (double*)p;
     if ((st = ensure_out(pr))) return bail(st);
+    // the counters and flags that the kernels leave at 0 for each other are filled on the default
+    // stream; evaluations run on streams that do not wait for it
+    if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return bail(fail(CELESTE_ERR_CUDA, "synchronize"));
     *out = pr;
     return CELESTE_OK;
 }

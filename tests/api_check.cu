@@ -3,6 +3,8 @@
 // Argument: which check.  Exit status 1 on a failure.
 //   memory   The device memory of a problem: the Hessian pass's part records take the place of
 //            the per-pixel E_s / Var_s, which its map passes are done with by then.
+//   settled  A problem's counters and flags are filled when its creation returns: the fills are
+//            on the default stream, which an evaluation on a non-blocking stream does not wait for.
 #include "fake_runtime.cuh"
 
 #include "celeste_api.cu"
@@ -93,10 +95,20 @@ static int check_memory() {
     return held <= may && fake::live_bytes == 0 ? 0 : 1;
 }
 
+static int check_settled() {
+    celeste_problem* pr = create(128, 4, 9, 20);
+    if (!pr) return 1;
+    const int n = fake::unsettled;
+    if (n) printf("%d fills under way\n", n);
+    celeste_problem_destroy(pr);
+    return n != 0;
+}
+
 int main(int argc, char** argv) {
     fake::no_real_device();
     const char* what = argc > 1 ? argv[1] : "";
     if (!strcmp(what, "memory")) return check_memory();
+    if (!strcmp(what, "settled")) return check_settled();
     printf("unknown check %s\n", what);
     return 1;
 }

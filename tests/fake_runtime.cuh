@@ -106,6 +106,8 @@ inline cudaError_t copy_async(void* d, const void* s, size_t n, cudaMemcpyKind, 
     return cudaSuccess;
 }
 
+// cudaMemset returns before the fill: unsettled until the host has waited for the stream or device
+inline int unsettled = 0;
 inline cudaError_t copy(void* d, const void* s, size_t n, cudaMemcpyKind) {
     memcpy(d, s, n);
     return cudaSuccess;
@@ -136,6 +138,15 @@ inline cudaError_t elapsed(float* t, cudaEvent_t, cudaEvent_t) {
 }
 inline cudaError_t set_bytes(void* p, int v, size_t n) {
     memset(p, v, n);
+    ++unsettled;
+    return cudaSuccess;
+}
+inline cudaError_t stream_synchronize(cudaStream_t st) {
+    if (st == nullptr || st == cudaStreamLegacy) unsettled = 0;
+    return cudaSuccess;
+}
+inline cudaError_t device_synchronize() {
+    unsettled = 0;
     return cudaSuccess;
 }
 
@@ -156,8 +167,8 @@ inline cudaError_t set_bytes(void* p, int v, size_t n) {
 #define cudaMemcpy fake::copy
 #define cudaMemset fake::set_bytes
 #define cudaSetDevice fake::done
-#define cudaDeviceSynchronize fake::done
-#define cudaStreamSynchronize fake::done
+#define cudaDeviceSynchronize fake::device_synchronize
+#define cudaStreamSynchronize fake::stream_synchronize
 #define cudaStreamCreateWithFlags fake::make_handle
 #define cudaStreamCreateWithPriority fake::make_handle
 #define cudaStreamDestroy fake::done

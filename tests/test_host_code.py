@@ -56,3 +56,7 @@ def test_device_memory_of_a_fit(check, precision, schedule):
 
 def test_device_memory_of_a_problem(check):
     check("api_check", "memory")
+
+
+def test_a_new_problem_is_settled(check):
+    check("api_check", "settled")
