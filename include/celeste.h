@@ -323,7 +323,8 @@ celeste_status celeste_grad_device(celeste_problem* prob, const double* d_theta,
 /*
  * Autotuner, at theta (host), with CUDA events on the problem's stream.
  *   contrib_code: the FP32 map-pass kernel of the Hessian and fit paths, timed over reps
- *     launches: 1, 2, 4 pixels per thread (CTAs of 256, 128, 64 threads over the same
+ *     passes of each (the Hessian's at the multiply covered pixels, the fit's at every
+ *     one): 1, 2, 4 pixels per thread (CTAs of 256, 128, 64 threads over the same
  *     256-pixel work items), 3, 5 two or four pixels per thread in packed FP32x2
  *     instructions, 6, 7 the same as persistent CTAs taking items from a work queue.
  *   items_code: the variant of the persistent FP32 value / gradient item kernel (CTAs

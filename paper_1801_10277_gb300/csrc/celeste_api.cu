@@ -1135,18 +1135,26 @@ celeste_status celeste_autotune(celeste_problem* pr, const double* theta, int32_
     CEL_CUDA(cudaEventCreate(&a));
     CEL_CUDA(cudaEventCreate(&b));
     cudaError_t e = cudaSuccess;
-    // the FP32 map pass of the Hessian and fit paths: 1, 2, 4 pixels per thread; 3, 5: two
-    // and four pixels per thread in packed FP32x2; 6, 7: the packed kernels as persistent
-    // CTAs on a work queue
+    // the FP32 map pass: 1, 2, 4 pixels per thread; 3, 5: two and four pixels per thread in packed
+    // FP32x2; 6, 7: the packed kernels as persistent CTAs on a work queue.  Timed as its two users
+    // run it: a Hessian evaluation at the multiply covered pixels alone, a fit's batches at
+    // every pixel of theirs, into the per-pixel buffers.
+    auto map_passes = [&]() {
+        DevProblem F = P;
+        F.single = nullptr;
+        F.item_ll = nullptr;
+        const cudaError_t h = launch_contrib(P, CELESTE_FP32_ACC64, st, true);
+        return h != cudaSuccess ? h : launch_contrib(F, CELESTE_FP32_ACC64, st);
+    };
     const int cands[7] = {1, 2, 4, 3, 5, 6, 7};
     float best_c = 1e30f;
     int pick_c = 2;
     for (int ci = 0; ci < 7 && e == cudaSuccess; ++ci) {
         P.tune_contrib = cands[ci];
         float tc = 0.f;
-        e = launch_contrib(P, CELESTE_FP32_ACC64, st);   // warm
+        e = map_passes();   // warm
         if (e == cudaSuccess) e = cudaEventRecord(a, st);
-        for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch_contrib(P, CELESTE_FP32_ACC64, st);
+        for (int r = 0; r < reps && e == cudaSuccess; ++r) e = map_passes();
         if (e == cudaSuccess) e = cudaEventRecord(b, st);
         if (e == cudaSuccess) e = cudaEventSynchronize(b);
         if (e == cudaSuccess) e = cudaEventElapsedTime(&tc, a, b);

@@ -5,13 +5,19 @@
 //            the per-pixel E_s / Var_s, which its map passes are done with by then.
 //   settled  A problem's counters and flags are filled when its creation returns: the fills are
 //            on the default stream, which an evaluation on a non-blocking stream does not wait for.
+//   autotune The map pass is timed as the paths that take the choice run it: at the multiply
+//            covered pixels (the Hessian evaluation) and at every pixel without the maps (a fit's batches).
 #include "fake_runtime.cuh"
 
 #include "celeste_api.cu"
 
 namespace cel {
 cudaError_t launch_prep(const DevProblem&, const double*, int, cudaStream_t, bool, bool) { return cudaSuccess; }
-cudaError_t launch_contrib(const DevProblem&, int, cudaStream_t, bool) { return cudaSuccess; }
+static std::map<int, int> hess_passes, fit_passes, other_passes;   // by kernel code
+cudaError_t launch_contrib(const DevProblem& P, int, cudaStream_t, bool multi_only) {
+    ++(P.single && multi_only ? hess_passes : !P.single && !multi_only ? fit_passes : other_passes)[P.tune_contrib];
+    return cudaSuccess;
+}
 cudaError_t launch_gather(const DevProblem&, int, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_adjoint(const DevProblem&, int, int, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_hess_pixels(const DevProblem&, int, const double*, double*, cudaStream_t) { return cudaSuccess; }
@@ -104,11 +110,25 @@ static int check_settled() {
     return n != 0;
 }
 
+static int check_autotune() {
+    celeste_problem* pr = create(128, 4, 9, 20);
+    if (!pr) return 1;
+    std::vector<double> theta((size_t)pr->P.n_src * NP, 0.5);
+    const celeste_status st = celeste_autotune(pr, theta.data(), 3, nullptr, nullptr);
+    bool ok = st == CELESTE_OK && cel::other_passes.empty() && cel::hess_passes.size() == 7 &&
+              cel::hess_passes == cel::fit_passes;
+    printf("status %d, codes: Hessian %zu, fit %zu, neither %zu\n", st, cel::hess_passes.size(), cel::fit_passes.size(),
+           cel::other_passes.size());
+    celeste_problem_destroy(pr);
+    return ok ? 0 : 1;
+}
+
 int main(int argc, char** argv) {
     fake::no_real_device();
     const char* what = argc > 1 ? argv[1] : "";
     if (!strcmp(what, "memory")) return check_memory();
     if (!strcmp(what, "settled")) return check_settled();
+    if (!strcmp(what, "autotune")) return check_autotune();
     printf("unknown check %s\n", what);
     return 1;
 }

@@ -60,3 +60,7 @@ def test_device_memory_of_a_problem(check):
 
 def test_a_new_problem_is_settled(check):
     check("api_check", "settled")
+
+
+def test_autotune_times_the_map_passes_that_run(check):
+    check("api_check", "autotune")
