@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "cover_order.cuh"
 #include "internal.cuh"
 
 using namespace cel;
@@ -570,13 +571,12 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     int n_smulti = 0;
     // a patch's multiply covered pixels (not f), grouped by a bit mask of the other patches that
     // cover them (patches past the 64th share bits: the groups only order the pixels)
-    std::vector<std::pair<uint64_t, std::vector<int32_t>>> groups;
+    std::vector<CoverRun> runs;
     std::vector<uint64_t> mask;
     std::vector<int32_t> over;
     auto cover_groups = [&](int p, const uint8_t* f) {
         const PatchGeo& g = geo[p];
         const ImgMeta& M = im[g.img];
-        groups.clear();
         over.clear();
         for (int ty = g.y0 / TILE; ty <= (g.y0 + g.h - 1) / TILE; ++ty)
             for (int tx = g.x0 / TILE; tx <= (g.x0 + g.w - 1) / TILE; ++tx) {
@@ -595,18 +595,7 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
             for (int y = ya; y < yb; ++y)
                 for (int x = xa; x < xb; ++x) mask[(size_t)y * g.w + x] |= 1ull << (e & 63);
         }
-        size_t last = 0;
-        for (int q = 0; q < g.w * g.h; ++q) {
-            if (f[q]) continue;
-            if (last >= groups.size() || groups[last].first != mask[q]) {
-                last = 0;
-                while (last < groups.size() && groups[last].first != mask[q]) ++last;
-                if (last == groups.size()) groups.push_back({mask[q], {}});
-            }
-            groups[last].second.push_back(q);
-        }
-        std::sort(groups.begin(), groups.end(),
-                  [](const auto& a, const auto& b) { return a.first < b.first; });
+        cover_order(f, mask.data(), g.w * g.h, runs);
     };
     spix.reserve((size_t)n_sp);
     int64_t sp_single = 0;
@@ -617,8 +606,8 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
             const int64_t first = (int64_t)spix.size();
             const int npx = g.w * g.h;
             cover_groups(p, f);
-            for (const auto& gr : groups)
-                for (int q : gr.second) spix.push_back(((q / g.w) << 16) | (q % g.w));
+            for (const CoverRun& r : runs)
+                for (int q = r.q0; q < r.q1; ++q) spix.push_back(((q / g.w) << 16) | (q % g.w));
             const int nm_all = (int)((int64_t)spix.size() - first);
             for (int q = 0; q < npx; ++q)
                 if (f[q]) spix.push_back(((q / g.w) << 16) | (q % g.w));

@@ -64,3 +64,7 @@ def test_a_new_problem_is_settled(check):
 
 def test_autotune_times_the_map_passes_that_run(check):
     check("api_check", "autotune")
+
+
+def test_order_of_multiply_covered_pixels(check):
+    check("cover_order_check")
