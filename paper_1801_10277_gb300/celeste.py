@@ -364,6 +364,7 @@ class Problem:
     def render(self, theta):
         """The model's expected image E[F] and variance Var[F] at theta, one [H][W] array
         per image (FP64)."""
+        self.generation += 1   # the problem's tables now belong to this call
         th = self._theta(theta)
         npx = sum(h * w for h, w in self.shapes)
         e = np.zeros(npx, np.float64)
