@@ -42,7 +42,7 @@ constexpr int WS_N = 0,    // N
 // dev and the exp components' sums at unit weight.  So the kernel accumulates 19 sums over
 // the exp components, then over the dev components, and forms the 35 once per (pixel, k).
 constexpr int BS_LL = 0, BS_C = 3, BS_D2 = 7, BS_D3 = 10, BS_D4 = 14, NBS = 19;
-constexpr int WROW = 40;   // a full row: exponent coefficients of z1^2, z2^2, constant; 35 weights; pad
+constexpr int WROW = 40;   // a full row (whiten_row): exponent coefficients of z1^2, z2^2, constant; 35 weights; pad
 constexpr int BROW = 24;   // a kernel row: the exponent's three coefficients, (FP32: a pad,) 19 weights, pad
 constexpr int WFR = 16;    // entries per k: T (row-major), K (3 x 3), g1, g2, pad
 // K[e][p] = (T E_e T')_p for the pixel-frame shape directions E_e = (xx, xy + yx, yy)
@@ -99,7 +99,8 @@ __host__ __device__ inline void whiten_frame(const float* sT, int k, float* fr) 
     whiten_shape_map(fr);
 }
 
-// lam1^(deg - i) lam2^i, i = 0 .. deg, times w
+// The 35 sums' weights one by one, the plain form that the host test of the frame sums (no kernel
+// does: they take the 19 of base_row): lam1^(deg - i) lam2^i, i = 0 .. deg, times w
 template <class R>
 __host__ __device__ __forceinline__ void monomials(R w, R l1, R l2, int deg, R* c) {
 #pragma unroll
@@ -111,7 +112,7 @@ __host__ __device__ __forceinline__ void monomials(R w, R l1, R l2, int deg, R* 
     }
 }
 
-// the row of galaxy component (k, j): exponent in z and the 35 monomial weights
+// ... and the row of galaxy component (k, j): exponent in z and the 35 monomial weights
 __host__ __device__ inline void whiten_row(const float* G, const float* fr, float* row) {
     const float nu = G[9], w = G[7], dw = G[8];
     const float l1 = 1.f / (1.f + nu * fr[WF_G]), l2 = 1.f / (1.f + nu * fr[WF_G + 1]);

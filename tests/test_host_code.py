@@ -68,3 +68,14 @@ def test_autotune_times_the_map_passes_that_run(check):
 
 def test_order_of_multiply_covered_pixels(check):
     check("cover_order_check")
+
+
+def test_hessian_sums_match_the_pixel_frame(check):
+    """As accurate as the pixel-frame formulas in the same type: at most twice their worst error of
+    a quantity's scale (and 1e-6, or that many rounding units in FP64, for none at all).  A wrong
+    index or a dropped term gives order one."""
+    rows = {tuple(line.split()[:2]): tuple(map(float, line.split()[2:]))
+            for line in check("base_sums_check").splitlines()}
+    assert len(rows) == 10
+    for (kind, name), (kernel, formulas) in rows.items():
+        assert kernel <= 2.0 * formulas + 1e-6 * (1.0 if kind == "float" else 2.0 ** -29), (kind, name, kernel, formulas)
