@@ -334,7 +334,9 @@ celeste_status celeste_grad_device(celeste_problem* prob, const double* d_theta,
  *     evaluations as the calls run them (the captured CUDA graph).
  * The choices are kept for later FP32 calls and returned (nullable outputs);
  * celeste_set_tuning restores them (contrib 0 .. 7, items 0 .. 5; 0 = the built-in
- * defaults 2 and 1; anything else is CELESTE_ERR_ARG).
+ * defaults 2 and 1; anything else is CELESTE_ERR_ARG).  A code names a kernel of this
+ * build: one kept from a build with other variants is accepted and picks another kernel,
+ * with the same results at another speed.
  */
 celeste_status celeste_autotune(celeste_problem* prob, const double* theta, int32_t reps,
                                 int32_t* contrib_code, int32_t* items_code);
@@ -346,14 +348,12 @@ celeste_status celeste_device_status(celeste_problem* prob);
 
 /*
  * Per-kernel timing (tracing aid).  With profiling on, every stage launch of the
- * calls above (prep, contrib, gather, adjoint / ll_sum / hess_adjoint, finalize) is
- * bracketed by CUDA events on its launch stream.  on = 1: the stages run as in a
- * normal call (the FP32 value / gradient path's fused pass and total on a second
- * stream, concurrently with the others), so a stage's time includes waiting for SM
- * slots that the concurrent stages hold; on = 2: every stage runs on the calling
- * stream, one after another, so the times add up to a serialised evaluation (results
- * identical to the concurrent order's); on = 0: off; anything else is CELESTE_ERR_ARG.
- * celeste_profile_read waits for the
+ * calls above (prep, contrib, gather, adjoint / ll_sum / hess_adjoint, finalize; the FP32
+ * value / gradient path: tables, items, finish) is bracketed by CUDA events on its launch
+ * stream.  on = 1 or 2: the stages run on the calling stream, one after another (without the
+ * captured graph and the overlap of the FP32 path's launches), so the times add up to a
+ * serialised evaluation with the same results; on = 0: off; anything else is
+ * CELESTE_ERR_ARG.  celeste_profile_read waits for the
  * recorded events, writes up to max_kernels entries (names[k*32 .. k*32+31]
  * NUL-terminated, total milliseconds, kernel launches), resets the accumulators and
  * returns the number of distinct stages (negative status on error).

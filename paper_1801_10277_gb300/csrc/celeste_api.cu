@@ -378,10 +378,7 @@ void celeste_problem_destroy(celeste_problem* pr) {
     for (cudaEvent_t e : pr->pool) cudaEventDestroy(e);
     drop_graphs(pr);
     for (void* p : pr->owned) cudaFree(p);
-    if (pr->side) cudaStreamDestroy(pr->side);
     if (pr->capture) cudaStreamDestroy(pr->capture);
-    for (cudaEvent_t e : {pr->ev_prep, pr->ev_fused, pr->ev_gather, pr->ev_join})
-        if (e) cudaEventDestroy(e);
     if (pr->stream) cudaStreamDestroy(pr->stream);
     if (pr->h_status) cudaFreeHost(pr->h_status);
     delete pr;
@@ -568,7 +565,6 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     };
     std::vector<SItem> sitems;
     std::vector<int32_t> spix, zitem_off(1, 0);
-    int n_smulti = 0;
     // a patch's multiply covered pixels (not f), grouped by a bit mask of the other patches that
     // cover them (patches past the 64th share bits: the groups only order the pixels)
     std::vector<CoverRun> runs;
@@ -618,7 +614,6 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
                 const int n = std::min(ZCHUNK * (base + (j < rem ? 1 : 0)), npx - o);
                 const int nm = std::max(0, std::min(n, nm_all - o));
                 sitems.push_back({p, s, n, nm, first + o});
-                if (nm > 0) ++n_smulti;
                 o += n;
             }
             zitem_off.push_back((int32_t)sitems.size());
@@ -769,16 +764,12 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
     if (cudaStreamCreateWithFlags(&pr->stream, cudaStreamNonBlocking) != cudaSuccess)
         return bail(fail(CELESTE_ERR_CUDA, "cudaStreamCreate failed"));
     {
-        int least = 0, greatest = 0;   // numerically greatest = lowest priority
+        // the evaluations' graphs are captured on a stream of the highest priority and instantiated
+        // to keep it
+        int least = 0, greatest = 0;
         cudaDeviceGetStreamPriorityRange(&least, &greatest);
-        // graphs are captured with the critical chain on the highest-priority stream and the
-        // fused pass on the lowest, and instantiated to keep those per-node priorities
-        if (cudaStreamCreateWithPriority(&pr->side, cudaStreamNonBlocking, least) != cudaSuccess ||
-            cudaStreamCreateWithPriority(&pr->capture, cudaStreamNonBlocking, greatest) != cudaSuccess)
+        if (cudaStreamCreateWithPriority(&pr->capture, cudaStreamNonBlocking, greatest) != cudaSuccess)
             return bail(fail(CELESTE_ERR_CUDA, "cudaStreamCreate failed"));
-        for (cudaEvent_t* e : {&pr->ev_prep, &pr->ev_fused, &pr->ev_gather, &pr->ev_join})
-            if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess)
-                return bail(fail(CELESTE_ERR_CUDA, "cudaEventCreate failed"));
     }
     pr->last_stream = pr->stream;
     if (cudaMallocHost((void**)&pr->h_status, sizeof(int32_t)) != cudaSuccess)
@@ -858,7 +849,6 @@ celeste_status celeste_problem_create_ex(const celeste_image* imgs, int32_t n_im
         P.zcands = d_zc;
         P.zpx = d_zpx;
         P.n_sitem = (int)sitems.size();
-        P.n_smulti = n_smulti;
         void* q;
         if ((st = dalloc(pr, &q, sizeof(double) * 16 * (size_t)P.n_sitem))) return bail(st);
         P.zpart = (double*)q;
@@ -967,7 +957,6 @@ static celeste_status run_device(celeste_problem* pr, const double* d_theta, int
     if (!pr || !d_theta) return fail(CELESTE_ERR_ARG, "null problem or theta");
     cudaStream_t st = (cudaStream_t)stream;
     CEL_CUDA(cudaSetDevice(pr->device));
-    // the status word (checked on the device) is reset first
     return run_cached(pr, d_theta, precision, mode, d_total, d_local, d_grad, d_hess, st);
 }
 
@@ -1035,7 +1024,6 @@ celeste_status celeste_profile_enable(celeste_problem* pr, int32_t on) {
     if (!pr) return fail(CELESTE_ERR_ARG, "null problem");
     if (on < 0 || on > 2) return fail(CELESTE_ERR_ARG, "profiling mode must be 0, 1 or 2");
     pr->profile = on != 0;
-    pr->profile_serial = on == 2;
     return CELESTE_OK;
 }
 
@@ -1088,8 +1076,7 @@ celeste_status celeste_grad_device(celeste_problem* pr, const double* d_theta, i
     // FP64: the mixture tables and the E / Var maps of the preceding celeste_elbo_device
     // call are reused; the mixture terms themselves are recomputed by the adjoint.  FP32:
     // the item kernel of celeste_elbo_grad runs again (it recomputes its tables, E and Var
-    // from theta; the KL of the preceding forward call is reused), so the gradient is
-    // bit-identical to the one-call gradient.
+    // and the KL terms from theta), so the gradient is bit-identical to the one-call gradient.
     if (items_path(P, precision, MODE_GRAD)) {
         static const char* const names[3] = {"tables", "items", "finish"};
         for (int stage = 0; stage < 3; ++stage)

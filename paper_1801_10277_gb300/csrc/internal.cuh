@@ -338,7 +338,7 @@ struct DevProblem {
     // The FP32 value / gradient kernel's work (item_kernels.cu): a patch's items are
     // contiguous, the patches in order; ztasks null when there is none.
     const int32_t* zitem_off;    // [n_patch + 1] first item of each patch
-    int n_sitem, n_smulti;       // items; those holding multiply covered pixels
+    int n_sitem;                 // items
     double* zpart;               // [n_sitem][16] per-item sums
     int32_t* zf_done;            // finished sources of the FP32 epilogue kernel, the evaluation's status; 0 between
                                  // evaluations
@@ -457,14 +457,11 @@ inline int sm_count() {
 // multi_only: at the multiply covered pixels alone, the others being left to the
 // kernels that evaluate the source there anyway
 cudaError_t launch_contrib(const DevProblem& P, int precision, cudaStream_t st, bool multi_only = false);
-// The FP32 value (MODE_LL) or value + gradient (MODE_GRAD) evaluation (item_kernels.cu):
-// the patches' whitened-frame tables, the KL value / gradient and the domain check of
-// theta, every item, the per-source epilogue (local objective, gradient; each nullable)
-// and the total (nullable); launch_items_stage below launches them one stage at a time
-cudaError_t launch_items(const DevProblem& P, int mode, cudaStream_t st, const double* d_theta, double* d_local,
-                         double* d_grad, double* d_total);
-// its three launches one at a time: stage 0 the tables and KL terms (after resetting the
-// ready flags), 1 the items, 2 the per-source epilogues and the total
+// The FP32 value (MODE_LL) or value + gradient (MODE_GRAD) evaluation (item_kernels.cu) one launch
+// at a time: stage 0 the patches' whitened-frame tables, the KL value / gradient and the domain
+// check of theta (nothing is reset: the last evaluation's stage 2 left the flags at 0), 1 every
+// item, 2 the per-source epilogue (local objective, gradient; each nullable) and the total
+// (nullable)
 cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStream_t st, const double* d_theta,
                                double* d_local, double* d_grad, double* d_total);
 cudaError_t launch_gather(const DevProblem& P, int precision, cudaStream_t st);

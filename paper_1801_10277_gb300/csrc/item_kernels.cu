@@ -682,7 +682,6 @@ struct ItemArgs {
     float4* zchain;            // [patch][ZCHAIN] chain-rule records
     int32_t* ready;            // [patch] table ready flags, then the queue counter and the
                                // count of built tables; all 0 between evaluations
-    const PatchGeo* geo_tab;
     const ImgMeta* img_tab;
     double* part;              // [item][16] sums: ll, owned ll, d ll / d y
     const int32_t* item_off;   // [n_patch + 1] first item of each patch
@@ -1423,7 +1422,6 @@ static cudaError_t launch_stage(const DevProblem& P, int stage, int mode, cudaSt
     a.ztbl = P.ztbl;
     a.zchain = P.zchain;
     a.ready = P.zready;
-    a.geo_tab = P.geo;
     a.img_tab = P.img;
     a.part = P.zpart;
     a.item_off = P.zitem_off;
@@ -1485,15 +1483,6 @@ cudaError_t launch_items_stage(const DevProblem& P, int stage, int mode, cudaStr
         cudaMemsetAsync(P.zf_done, 0, 2 * sizeof(int32_t), st);
     }
     return e;
-}
-
-cudaError_t launch_items(const DevProblem& P, int mode, cudaStream_t st, const double* d_theta, double* d_local,
-                         double* d_grad, double* d_total) {
-    for (int stage = 0; stage < 3; ++stage) {
-        const cudaError_t e = launch_items_stage(P, stage, mode, st, d_theta, d_local, d_grad, d_total);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
 }
 
 }  // namespace cel

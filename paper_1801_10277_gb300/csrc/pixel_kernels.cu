@@ -102,7 +102,7 @@ __device__ __forceinline__ double lg2(double x) { return log2(x); }
 
 // Per-pixel FP32 quantities with every rounding written out (no contraction left to the
 // compiler), so that every kernel that forms them -- the value-only and the gradient
-// variants, the fused pass and the gather / adjoint passes -- gets the same bits.
+// variants of the map and adjoint passes -- gets the same bits.
 //   f_i = iota E[l_i] g_i,  E_s = a0 f0 + a1 f1,
 //   Var_s = a0 f0^2 em0 + a1 f1^2 em1 + a0 (1 - a0) f0^2 + a1 (1 - a1) f1^2 - 2 a0 a1 f0 f1
 //   (em_i = E[l_i^2] / E[l_i]^2 - 1)

@@ -14,12 +14,7 @@ struct celeste_problem {
     DevProblem P{};
     cudaStream_t stream = nullptr;       // stream of the host-pointer entry points
     cudaStream_t last_stream = nullptr;  // stream of the last enqueued call
-    // the fused FP32 pass and the total run on a low-priority side stream, forked from and
-    // joined back into the caller's stream by these events
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_prep = nullptr, ev_fused = nullptr, ev_gather = nullptr, ev_join = nullptr;
-    // one evaluation (status reset + every launch of both streams) captured as a CUDA graph
-    // per argument set, replayed by later calls with the same arguments
+    // one evaluation (status reset + every launch) captured as a CUDA graph per argument set, replayed by later calls with the same arguments
     struct GraphKey {
         int precision, mode, tune_c, tune_a, cap;
         const void* ptr[5];   // theta, total, local, grad, hess
@@ -50,7 +45,6 @@ struct celeste_problem {
     size_t scr_cap = 0;
     // per-kernel CUDA-event timing (celeste_profile_*)
     bool profile = false;
-    bool profile_serial = false;   // every stage on the calling stream, one after another
     struct Rec { std::string name; cudaEvent_t a, b; int n_kernels; };
     std::vector<Rec> pending;
     std::vector<cudaEvent_t> pool;
