@@ -1412,7 +1412,7 @@ celeste_status cel::fit_sources_impl(celeste_problem* pr, double* theta, const i
             };
             batch_pixels(true);
             chk(launch_hess_pixels(Pb, prec, d_bth, d_h, st));
-            chk(launch_finalize_hess(Pb, d_f, d_g, d_h, st));
+            chk(launch_finalize_hess(Pb, prec, d_f, d_g, d_h, st));
             k_tr_step<<<nb, TR_THREADS, sizeof(TrShared), st>>>(nb, d_bth, d_bt, d_f, d_g, d_h, d_kl, d_bthc, d_btc,
                                                  d_st, *opts, d_srcact);
             chk(launch_prep(Pc, d_bthc, prec, st, false, true));

@@ -9,10 +9,13 @@
 //                    added to the KL Hessian; the full symmetric 44 x 44 matrix, the
 //                    gradient and the local objective.
 //
-// The pixel terms depend on theta through ten variables z of the (source, patch): with
-// k_i = a_i iota E[l_i] and q_i = a_i iota^2 E[l_i^2] (i = star, galaxy),
-//   E_s = k_0 g_0 + k_1 g_1,  E2_s = q_0 g_0^2 + q_1 g_1^2,  Var_s = E2_s - E_s^2,
-// z = (k_0, k_1, q_0, q_1, the mean, e_dev, G).  (The twelve y of the gradient passes hold
+// The pixel terms depend on theta through ten variables z of the (source, patch).  With
+// E_s = k_0 g_0 + k_1 g_1,  E2_s = q_0 g_0^2 + q_1 g_1^2,  Var_s = E2_s - E_s^2,
+// k_i = a_i iota E[l_i] and q_i = a_i iota^2 E[l_i^2] (i = star, galaxy), the first four are A_i and
+// Q_i with k_i = K_i A_i, q_i = L_i (A_i + Q_i), K_i = iota E[l_i] and L_i = iota^2 E[l_i^2] held at theta,
+// where A_i = a_i and Q_i = 0.  (d/dA_i is d/da_i, whose parts K_i d/dk_i and L_i d/dq_i cancel
+// in part: they are added at the pixel, before the sums are rounded.)
+// z = (A_0, A_1, Q_0, Q_1, the mean, e_dev, G).  (The twelve y of the gradient passes hold
 // a_i, E[l_i] and E[l_i^2] apart: their rows of the Hessian are multiples of each other.)
 // With e = dE_s/dz, v = dVar_s/dz = dE2_s/dz - 2 E_s e and the second derivatives
 // DE = d2E_s/dz2, DE2 = d2E2_s/dz2:
@@ -606,6 +609,28 @@ __global__ void __launch_bounds__(32 * HESS_WARPS, sizeof(R) == 8 ? 2 : 4) k_hes
         }
         for (int i = lane; i < HV; i += 32) sums[i] = 0.0;
         __syncwarp();
+        // a_i, K_i, L_i, a_i K_i, a_i L_i: once per part in FP64 (for all of its pixels' FP64 instructions),
+        // per pixel in FP32, where the registers are short
+        struct Light {
+            R a0, a1, K0, K1, L0, L1, k0, k1, l0, l1;
+        };
+        auto light = [&]() {
+            const R iota = sT[H_IOTA];
+            Light p;
+            p.a0 = sT[H_A0];
+            p.a1 = sT[H_A1];
+            p.K0 = iota * sT[H_EL0];
+            p.K1 = iota * sT[H_EL1];
+            p.L0 = iota * iota * sT[H_EL20];
+            p.L1 = iota * iota * sT[H_EL21];
+            p.k0 = p.a0 * p.K0;
+            p.k1 = p.a1 * p.K1;
+            p.l0 = p.a0 * p.L0;
+            p.l1 = p.a1 * p.L1;
+            return p;
+        };
+        Light part_light;
+        if constexpr (DBL) part_light = light();
         for (int c0 = 0; c0 < it.n; c0 += 32) {
             // the pixel's data, asked for before the mixture
             const bool ok = c0 + lane < it.n;
@@ -644,24 +669,37 @@ __global__ void __launch_bounds__(32 * HESS_WARPS, sizeof(R) == 8 ? 2 : 4) k_hes
                         f1 = (float)z1s;
                         f2 = (float)z2s;
                     }
-                    {
-                        // P d = T' z and P = T' T
-                        R n;
-                        if constexpr (DBL)
-                            n = ex2_quad(EX_HALF, z1s, EX_HALF, z2s, (float)EX_HALF, f1, (float)EX_HALF, f2, tab);
-                        else
-                            n = ex2h((float)(-0.5 * LOG2E_W) * (z1s + z2s));
-                        n *= fr[15];
-                        const R qx = fr[0] * z1 + fr[2] * z2, qy = fr[1] * z1 + fr[3] * z2;
-                        const R pxx = fr[WF_K] + fr[WF_K + 2], pxy = (R)0.5 * (fr[WF_K + 3] + fr[WF_K + 5]),
-                                pyy = fr[WF_K + 6] + fr[WF_K + 8];
+                    auto star = [&]() {
+                        R n, qx, qy, pxx, pxy, pyy;
+                        if constexpr (DBL) {
+                            // P d = T' z and P = T' T
+                            n = fr[15] *
+                                ex2_quad(EX_HALF, z1s, EX_HALF, z2s, (float)EX_HALF, f1, (float)EX_HALF, f2, tab);
+                            qx = fr[0] * z1 + fr[2] * z2;
+                            qy = fr[1] * z1 + fr[3] * z2;
+                            pxx = fr[WF_K] + fr[WF_K + 2];
+                            pxy = (R)0.5 * (fr[WF_K + 3] + fr[WF_K + 5]);
+                            pyy = fr[WF_K + 6] + fr[WF_K + 8];
+                        } else {
+                            // in the pixel frame: with z in FP32 a source's gradient and Hessian were off
+                            // by a quarter more (500 sources, the medians of their errors against 64
+                            // bits: 2.5e-7 and 1.7e-7, here 1.9e-7 and 1.3e-7)
+                            const R* S = sT + T_STAR + k * STAR_STRIDE;
+                            pxx = S[4];
+                            pxy = S[5];
+                            pyy = S[6];
+                            qx = pxx * dx + pxy * dy;
+                            qy = pxy * dx + pyy * dy;
+                            n = S[7] * ex2h(fmaf((float)(-0.5 * LOG2E_W), fmaf(dx, qx, dy * qy), S[3]));
+                        }
                         g0 += n;
                         d0[0] += n * qx;
                         d0[1] += n * qy;
                         h0[0] += n * (qx * qx - pxx);
                         h0[1] += n * (qx * qy - pxy);
                         h0[2] += n * (qy * qy - pyy);
-                    }
+                    };
+                    if (DBL) star();   // (behind the galaxy's terms in FP32: fewer registers spill)
                     const R* row = rows + k * nprof * BROW;
                     // the base sums over one group's components (N of them where N > 0, else n)
                     auto group = [&](auto N, int n, R (&b)[NBS]) {
@@ -721,11 +759,11 @@ __global__ void __launch_bounds__(32 * HESS_WARPS, sizeof(R) == 8 ? 2 : 4) k_hes
                     group(std::integral_constant<int, ND>{}, nprof - n_exp, bd);
                     combine_groups(be, bd, fr[WF_G], fr[WF_G + 1], edev, s);
                     whitened_add(s, z1, z2, fr, g1, d1, de, h1, he);
+                    if (!DBL) star();
                 }
                 // ---- E, Var and the pixel's weights
-                const R iota = sT[H_IOTA], a0 = sT[H_A0], a1 = sT[H_A1];
-                const R k0 = a0 * iota * sT[H_EL0], k1 = a1 * iota * sT[H_EL1];
-                const R q0 = a0 * iota * iota * sT[H_EL20], q1 = a1 * iota * iota * sT[H_EL21];
+                const Light p = DBL ? part_light : light();
+                const R a0 = p.a0, a1 = p.a1, K0 = p.K0, K1 = p.K1, L0 = p.L0, L1 = p.L1, k0 = p.k0, k1 = p.k1;
                 const R Es = k0 * g0 + k1 * g1;
                 if (alone) {
                     if constexpr (DBL) {
@@ -735,7 +773,7 @@ __global__ void __launch_bounds__(32 * HESS_WARPS, sizeof(R) == 8 ? 2 : 4) k_hes
                         E += es;
                     } else {
                         // Var_s in the form that does not cancel (k_contrib's)
-                        const float f0 = iota * sT[H_EL0] * g0, f1 = iota * sT[H_EL1] * g1;
+                        const float f0 = K0 * g0, f1 = K1 * g1;
                         const float em0 = sT[H_EL20] / (sT[H_EL0] * sT[H_EL0]) - 1.f;
                         const float em1 = sT[H_EL21] / (sT[H_EL1] * sT[H_EL1]) - 1.f;
                         V = a0 * f0 * f0 * (em0 + (1.f - a0)) + a1 * f1 * f1 * (em1 + (1.f - a1)) -
@@ -746,7 +784,6 @@ __global__ void __launch_bounds__(32 * HESS_WARPS, sizeof(R) == 8 ? 2 : 4) k_hes
                 const R iE = (R)1 / E, iE2 = iE * iE;
                 const R cE = x * (iE + V * iE2 * iE) - (R)1;
                 const R cV = (R)-0.5 * x * iE2;
-                const R hEE = -x * iE2 * ((R)1 + (R)3 * V * iE2);
                 const R hEV = x * iE2 * iE;
                 out[0] = x * (lgh(E) - (R)0.5 * V * iE2) - E;
                 // ---- assemble the pixel's z-derivatives (entries known to be zero are left out: a
@@ -754,13 +791,14 @@ __global__ void __launch_bounds__(32 * HESS_WARPS, sizeof(R) == 8 ? 2 : 4) k_hes
                 const R w1 = cE - (R)2 * cV * Es, w2 = cV;
                 // gradient of g_1 over (mx, my, e_dev, Gxx, Gxy, Gyy); g_0's is (d0[0], d0[1], 0, 0, 0, 0)
                 const R dg1[6] = {d1[0], d1[1], de, d1[2], d1[3], d1[4]};
-                // e = dE_s/dz (0 for q), v2 = dE2_s/dz (0 for k)
+                // e = dE_s/dz (0 for Q_i), v2 = dE2_s/dz
                 R e[NZ], v2[NZ];
-                e[Z_K0] = g0;
-                e[Z_K1] = g1;
-                v2[Z_Q0] = g0 * g0;
-                v2[Z_Q1] = g1 * g1;
-                const R m0 = (R)2 * q0, m1 = (R)2 * q1, n0 = m0 * g0, n1 = m1 * g1;
+                e[Z_A0] = K0 * g0;
+                e[Z_A1] = K1 * g1;
+                v2[Z_A0] = v2[Z_Q0] = L0 * g0 * g0;
+                v2[Z_A1] = v2[Z_Q1] = L1 * g1 * g1;
+                // L_i g_i twice, and with a_i
+                const R m0 = (R)2 * L0 * g0, m1 = (R)2 * L1 * g1, n0 = a0 * m0, n1 = a1 * m1;
 #pragma unroll
                 for (int z = 0; z < 6; ++z) {
                     e[Z_MX + z] = k1 * dg1[z];
@@ -771,20 +809,16 @@ __global__ void __launch_bounds__(32 * HESS_WARPS, sizeof(R) == 8 ? 2 : 4) k_hes
                     }
                 }
                 auto has_e = [](int z) { return z != Z_Q0 && z != Z_Q1; };
-                auto has_v2 = [](int z) { return z != Z_K0 && z != Z_K1; };
                 // gradient, and the outer-product part of the Hessian: with v = v2 - 2 E_s e,
                 //   (h_EE - 2 c_V) e e' + h_EV (e v' + v e') = e p' + p e',
-                //   p = (h_EE / 2 - c_V - 2 h_EV E_s) e + h_EV v2
-                const R c1 = (R)0.5 * hEE - cV - (R)2 * hEV * Es;
+                //   p = (h_EE / 2 - c_V - 2 h_EV E_s) e + h_EV v2,  h_EE / 2 - c_V = -3 h_EV Var / (2 E)
+                const R c1 = -hEV * ((R)1.5 * V * iE + (R)2 * Es);
                 R pv[NZ];
 #pragma unroll
                 for (int z = 0; z < NZ; ++z) {
                     if (!has_e(z)) {
                         out[1 + z] = w2 * v2[z];
                         pv[z] = hEV * v2[z];
-                    } else if (!has_v2(z)) {
-                        out[1 + z] = w1 * e[z];
-                        pv[z] = c1 * e[z];
                     } else {
                         out[1 + z] = w1 * e[z] + w2 * v2[z];
                         pv[z] = c1 * e[z] + hEV * v2[z];
@@ -802,16 +836,16 @@ __global__ void __launch_bounds__(32 * HESS_WARPS, sizeof(R) == 8 ? 2 : 4) k_hes
                         H[sym<NZ>(a, b)] = h;
                     }
                 // second-derivative part  w1 DE + w2 DE2
-                const R b0 = w2 * m0, b1 = w2 * m1;
-                const R u0 = w1 * k0 + b0 * g0, u1 = w1 * k1 + b1 * g1;
-                const R r0 = (R)2 * w2 * g0, r1 = (R)2 * w2 * g1;
+                const R r0 = w2 * m0, r1 = w2 * m1, s0 = w1 * K0 + r0, s1 = w1 * K1 + r1;
+                const R u0 = a0 * s0, u1 = a1 * s1;
+                const R b0 = (R)2 * w2 * p.l0, b1 = (R)2 * w2 * p.l1;
                 R bd1[6];
 #pragma unroll
                 for (int z = 0; z < 6; ++z) {
-                    H[sym<NZ>(Z_K1, Z_MX + z)] += w1 * dg1[z];
+                    H[sym<NZ>(Z_A1, Z_MX + z)] += s1 * dg1[z];
                     H[sym<NZ>(Z_Q1, Z_MX + z)] += r1 * dg1[z];
                     if (z < 2) {
-                        H[sym<NZ>(Z_K0, Z_MX + z)] += w1 * d0[z];
+                        H[sym<NZ>(Z_A0, Z_MX + z)] += s0 * d0[z];
                         H[sym<NZ>(Z_Q0, Z_MX + z)] += r0 * d0[z];
                     }
                     bd1[z] = b1 * dg1[z];
@@ -905,9 +939,9 @@ __device__ const PackedTriangle<NY> g_ypk = packed_triangle<NY>();
 
 __global__ void __launch_bounds__(FH_THREADS, 4)
 k_finalize_hess(int n_src, int hchunk, const PatchGeo* __restrict__ geo, const int32_t* __restrict__ patch_off,
-                const ImgMeta* __restrict__ img, const double* __restrict__ part, const double* __restrict__ hsrc,
-                double* __restrict__ local_out, double* __restrict__ grad_out, double* __restrict__ hess_out,
-                const int32_t* __restrict__ src_active) {
+                const ImgMeta* __restrict__ img, const float* __restrict__ tbl32, const double* __restrict__ part,
+                const double* __restrict__ hsrc, double* __restrict__ local_out, double* __restrict__ grad_out,
+                double* __restrict__ hess_out, const int32_t* __restrict__ src_active) {
     const int s = blockIdx.x;
     if (s >= n_src || (src_active && !src_active[s])) return;
     constexpr int NACC = 1 + NY + NYH;
@@ -918,6 +952,7 @@ k_finalize_hess(int n_src, int hchunk, const PatchGeo* __restrict__ geo, const i
     __shared__ double sj[FH_WARPS][NY][3];   // J: column w's entries ...
     __shared__ uint8_t si[FH_WARPS][NY][3];  // ... and their z
     __shared__ double sg[FH_WARPS][36];      // dG, d2G of the patch
+    __shared__ double sr[FH_WARPS][4];       // r_K, r_L of each type (below)
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int band = warp % 5, half = warp / 5;
     for (int i = t; i < HREC; i += FH_THREADS) rec[i] = hsrc[(size_t)HREC * s + i];
@@ -932,6 +967,11 @@ k_finalize_hess(int n_src, int hchunk, const PatchGeo* __restrict__ geo, const i
             const int p = pb + __ffs(mine) - 1;
             const PatchGeo g = geo[p];
             const double* A = img[g.img].A;
+            float el = 0.f, el_iota = 0.f;   // FP32: the moments that the pass had (lanes 0 .. 3)
+            if (tbl32 && lane < 4) {
+                el = tbl32[(size_t)p * TBL_STRIDE + H_EL0 + lane];
+                el_iota = tbl32[(size_t)p * TBL_STRIDE + H_IOTA];
+            }
             // the patch's parts, each warp of the band half of them in order, loaded four at a
             // time before any is added; the two sums meet in the warp whose turn the patch is
             double v[3] = {0.0, 0.0, 0.0};
@@ -970,10 +1010,22 @@ k_finalize_hess(int n_src, int hchunk, const PatchGeo* __restrict__ geo, const i
             for (int c = 0; c < 3; ++c)
                 if (lane + 32 * c < HV) sy[warp][lane + 32 * c] = v[c];
             __syncwarp();
-            // iota E[l_i] and iota^2 E[l_i^2] of type i
-            const double iota = img[g.img].iota;
-            const double* mom = rec + HR_MOM + 4 * band;
-            const double m[4] = {iota * mom[0], iota * iota * mom[1], iota * mom[2], iota * iota * mom[3]};
+            // K_0, L_0, K_1, L_1 over the ones that the FP32 pass had, for the rows of the log brightness.
+            // (Not for those of a_i: the pass's rounding is in its E_s and Var_s too, and with
+            // the FP64 moments against these the a_i's gradient and Hessian entries were off by
+            // 1.3 to 2.3 times as much against 64 bits.)
+            if (lane < 4) {
+                double r = 1.0;
+                if (tbl32) {
+                    const double iota = img[g.img].iota;
+                    const double k = (lane & 1 ? iota * iota : iota) * rec[HR_MOM + 4 * band + lane];
+                    const float pass = (lane & 1 ? el_iota * el_iota : el_iota) * el;
+                    const float off = (float)(k - (double)pass) / pass;
+                    if (fabsf(off) < 1e-3f) r += (double)off;   // (rounding, not a denormal or an overflow)
+                }
+                sr[warp][lane] = r;
+            }
+            __syncwarp();
             const double* Gz = sy[warp] + 1;
             const double* Hz = sy[warp] + 1 + NZ;
             if (lane < NY) {
@@ -981,15 +1033,14 @@ k_finalize_hess(int n_src, int hchunk, const PatchGeo* __restrict__ geo, const i
                 int z0 = Z_ED, z1 = 0, z2 = 0;
                 double c0 = 1.0, c1 = 0.0, c2 = 0.0;
                 if (w <= Y_EL21) {
-                    // k_i = a_i iota E[l_i], q_i = a_i iota^2 E[l_i^2] over a_i, m_i, v_i
+                    // A_i and Q_i over a_i, m_i, v_i: A = a r_K e^{dm + dv/2}, A + Q = a r_L e^{2 dm + 2 dv}
                     const int i = w == Y_A1 || w >= Y_EL1;
-                    z0 = Z_K0 + i;
+                    z0 = Z_A0 + i;
                     z1 = Z_Q0 + i;
-                    c0 = i ? m[2] : m[0];
-                    c1 = i ? m[3] : m[1];
                     if (w >= Y_EL0) {
-                        c0 *= rec[HR_A + i] * ((w - Y_EL0) & 1 ? 0.5 : 1.0);
-                        c1 *= 2.0 * rec[HR_A + i];
+                        const double f = (w - Y_EL0) & 1 ? 0.5 : 1.0;
+                        c0 = f * sr[warp][2 * i] * rec[HR_A + i];
+                        c1 = 2.0 * sr[warp][2 * i + 1] * rec[HR_A + i] - c0;
                     }
                 } else if (w == Y_MX || w == Y_MY) {
                     z0 = Z_MX;
@@ -1020,10 +1071,12 @@ k_finalize_hess(int n_src, int hchunk, const PatchGeo* __restrict__ geo, const i
                 double h = 0.0;
 #pragma unroll
                 for (int e = 0; e < 3; ++e) h += sj[warp][a][e] * sx[warp][si[warp][a][e]][b];
-                // second derivatives of z over w: k = a iota e^{m + v/2}, q = a iota^2 e^{2m + 2v}, and G
+                // second derivatives of z over w: A = a r_K e^{dm + dv/2}, A + Q = a r_L e^{2 dm + 2 dv}, and G
                 const int ia = a == Y_A1 || a >= Y_EL1, ib = b == Y_A1 || b >= Y_EL1;
                 if (b <= Y_EL21 && b >= Y_EL0 && ia == ib) {
-                    const double Gk = Gz[Z_K0 + ia] * (ia ? m[2] : m[0]), Gq = Gz[Z_Q0 + ia] * (ia ? m[3] : m[1]);
+                    // K d/dk and L d/dq
+                    const double Gk = (Gz[Z_A0 + ia] - Gz[Z_Q0 + ia]) * sr[warp][2 * ia];
+                    const double Gq = Gz[Z_Q0 + ia] * sr[warp][2 * ia + 1];
                     const double fb = (b - Y_EL0) & 1 ? 0.5 : 1.0;
                     if (a >= Y_EL0) {
                         const double fa = (a - Y_EL0) & 1 ? 0.5 : 1.0;
@@ -1129,11 +1182,12 @@ cudaError_t launch_hess_pixels(const DevProblem& P, int precision, const double*
                                      : hess_pixels<float>(P, P.tbl32, d_theta, d_hess, st);
 }
 
-cudaError_t launch_finalize_hess(const DevProblem& P, double* d_local, double* d_grad, double* d_hess,
+cudaError_t launch_finalize_hess(const DevProblem& P, int precision, double* d_local, double* d_grad, double* d_hess,
                                  cudaStream_t st) {
     if (P.n_src == 0) return cudaSuccess;
-    k_finalize_hess<<<P.n_src, FH_THREADS, 0, st>>>(P.n_src, P.hchunk, P.geo, P.patch_off, P.img, P.hpart, P.hsrc, d_local,
-                                                    d_grad, d_hess, P.src_active);
+    const float* tbl32 = precision == CELESTE_FP64 ? nullptr : P.tbl32;
+    k_finalize_hess<<<P.n_src, FH_THREADS, 0, st>>>(P.n_src, P.hchunk, P.geo, P.patch_off, P.img, tbl32, P.hpart, P.hsrc,
+                                                    d_local, d_grad, d_hess, P.src_active);
     return cudaGetLastError();
 }
 

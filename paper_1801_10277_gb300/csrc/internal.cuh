@@ -89,7 +89,7 @@ inline int hess_chunk(int64_t n_sp, int n_sm) {
 }
 // Its ten variables z per (source, patch) (hess_kernels.cu) and a part's record: ll, d/dz, the
 // packed upper triangle of d2/dz2
-enum : int { Z_K0 = 0, Z_K1, Z_Q0, Z_Q1, Z_MX, Z_MY, Z_ED, Z_GXX, Z_GXY, Z_GYY, NZ };
+enum : int { Z_A0 = 0, Z_A1, Z_Q0, Z_Q1, Z_MX, Z_MY, Z_ED, Z_GXX, Z_GXY, Z_GYY, NZ };
 constexpr int HV = 1 + NZ + NZ * (NZ + 1) / 2;
 constexpr int ZIMAX = 512;   // most pixels per item of the FP32 value / gradient kernel
 constexpr int ZMAXC = 4;     // other covering patches named inline in such an item's queue record
@@ -470,7 +470,7 @@ cudaError_t launch_adjoint(const DevProblem& P, int precision, int mode, cudaStr
 // P.kl, -KL'' into d_hess); launch_finalize_hess then adds the pixel part
 cudaError_t launch_hess_pixels(const DevProblem& P, int precision, const double* d_theta, double* d_hess,
                                cudaStream_t st);
-cudaError_t launch_finalize_hess(const DevProblem& P, double* d_local, double* d_grad, double* d_hess,
+cudaError_t launch_finalize_hess(const DevProblem& P, int precision, double* d_local, double* d_grad, double* d_hess,
                                  cudaStream_t st);
 cudaError_t launch_finalize(const DevProblem& P, const double* d_theta, int precision, int mode,
                             double* d_total, double* d_local, double* d_grad, double* d_hess,

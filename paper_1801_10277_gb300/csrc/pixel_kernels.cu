@@ -378,7 +378,7 @@ k_prep(const double* __restrict__ theta, const PatchGeo* __restrict__ geo,
             T[base + 6] = pyy;
             T[base + 7] = w;
             if constexpr (!WHITE)
-                if (j < 0 && hframe) hess_frame(T, k, hframe + (size_t)(p0 + r0 + pj) * HF_STRIDE + k * WFR);
+                if (j < 0 && hframe) whiten_frame(T, k, hframe + (size_t)(p0 + r0 + pj) * HF_STRIDE + k * WFR);
             if (j >= 0) {
                 T[base + 8] = dw;
                 T[base + 9] = nu;

@@ -43,7 +43,7 @@ cudaError_t launch_finalize(const DevProblem& P, const double* d_theta, int prec
                             double* d_total, double* d_local, double* d_grad, double* d_hess,
                             cudaStream_t st) {
     if (mode == MODE_HESS) {
-        cudaError_t e = launch_finalize_hess(P, d_local, d_grad, d_hess, st);
+        cudaError_t e = launch_finalize_hess(P, precision, d_local, d_grad, d_hess, st);
         if (e != cudaSuccess) return e;
     } else if (P.n_src > 0) {
         // the KL value and gradient come from k_prep of the same theta

@@ -161,14 +161,9 @@ __host__ __device__ __forceinline__ void base_row(R w, R nu, R l1, R l2, R* c) {
     c[BS_D4 + 4] = c[BS_D3 + 3] * l2;
 }
 
-// The FP32 Hessian pass's frames of a patch (MAXPSF of them, entry 15: alpha_k / (2 pi
-// sqrt(det Sigma_k))) take the place of the FP64 tables, which an FP32 evaluation does not use.
+// The FP32 Hessian pass's frames of a patch (MAXPSF of them) take the place of the FP64 tables,
+// which an FP32 evaluation does not use.
 constexpr int HF_STRIDE = MAXPSF * WFR;   // floats per patch
 static_assert(HF_STRIDE * sizeof(float) <= TBL_STRIDE * sizeof(double), "in the place of a table");
-__device__ __forceinline__ void hess_frame(const float* T, int k, float* fr) {
-    whiten_frame(T, k, fr);
-    const float* S = T + T_STAR + k * STAR_STRIDE;
-    fr[15] = S[7] * exp2f(S[3]);
-}
 
 }  // namespace cel

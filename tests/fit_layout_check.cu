@@ -17,7 +17,7 @@ namespace cel {
 cudaError_t launch_prep(const DevProblem&, const double*, int, cudaStream_t, bool, bool) STUB
 cudaError_t launch_contrib(const DevProblem&, int, cudaStream_t, bool) STUB
 cudaError_t launch_hess_pixels(const DevProblem&, int, const double*, double*, cudaStream_t) STUB
-cudaError_t launch_finalize_hess(const DevProblem&, double*, double*, double*, cudaStream_t) STUB
+cudaError_t launch_finalize_hess(const DevProblem&, int, double*, double*, double*, cudaStream_t) STUB
 void set_last_error(const char*) {}
 }  // namespace cel
 
