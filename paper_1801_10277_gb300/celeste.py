@@ -403,8 +403,10 @@ class Problem:
         # the current stream's handle without a torch.cuda.Stream object around it (3.1 -> 0.6 us
         # of the 8 us that a device call takes on the host), where PyTorch has that call
         import torch
-        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-        return C.c_void_p(raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream)
+        try:
+            return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        except AttributeError:
+            return C.c_void_p(torch.cuda.current_stream().cuda_stream)
 
     @staticmethod
     def _dp(t):
