@@ -490,8 +490,8 @@ __device__ __forceinline__ void copy16_async(void* dst, const void* src) {
 // record and table are on their way to the warp's other stage.  A warp goes through its part 32
 // pixels at a time and shares nothing with the others, so it waits neither for memory nor at a
 // barrier; one CTA per part had its warps waiting for loads and barriers 40 % of the time.
-// 500 sources, FP32: 125 -> 112 us (issue slots 63 % used, FMA pipe 52 %; 56 us at that pipe's
-// peak); 64 crowded sources, FP64: 608 -> 584 us (FP64 pipe 88 %).
+// 500 sources, FP32: 125 -> 112 us back to back (117 alone with cold caches: issue slots 62 % used,
+// FMA pipe 48 %; 56 us at that pipe's peak); 64 crowded sources, FP64: 608 -> 587 us (FP64 pipe 88 %).
 // Bound by the FP32 or the FP64 pipe: 12 (packed) / 25 of its instructions per component, where
 // the 35 sums accumulated one by one took 38 and the pixel-frame formulas about 140.
 template <class R>
@@ -924,10 +924,11 @@ __device__ __forceinline__ int w_factor(int band, int j) {
 
 // One CTA per source, two warps per band, which add the parts of a patch half and half and take
 // turns to map the 66 sums to w (X = H_z J, then J' X, J at most three entries per column) and
-// to add the result to the warp's shared accumulator; then the block is spread and added to the -KL terms that source_terms left in hess_out.
+// to add the result to the warp's shared accumulator; then the block is spread and added to the
+// -KL terms that source_terms left in hess_out.
 // Latency-bound, so the patches of a source run side by side and a patch costs about 50 FP64
 // instructions; per-patch loops over the 44 x 44 entries with the KL and its Hessian in the
-// same CTA took 119 us for 500 sources and 49 us for 64, this 31 and 22.
+// same CTA took 119 us for 500 sources and 49 us for 64, this 36 and 26 (alone, cold caches).
 // barrier of a band's two warps
 __device__ __forceinline__ void pair_barrier(int band) { asm volatile("bar.sync %0, 64;" ::"r"(band + 1) : "memory"); }
 
